@@ -1053,20 +1053,6 @@ __device__ SegOut team_run_pipe(const typename Num<T>::RecJ* __restrict__ rec, i
     return out;
 }
 
-// ------------------------------------------------------------------------------------
-// team_run_pipe with each lane's columns split in two halves that advance side by side:
-// column q of the first half and column N/2 + q of the second sit in one float2 and share
-// a packed FFMA2 / FMUL2 (PACKED) or go through two scalar instructions (two independent
-// dependency chains per lane).  Both halves run the D-hat chains
-// of phase B at once, each from its own carry: the first half's comes from the left lane
-// (as in team_run_pipe), the second half's is the first half's D-hat at its last column,
-// formed after the scan.  The lane's scan aggregate joins the two half chains with
-// g^(N/2).  Phase A is not a separate pass here: row i's partials U and insertions J are
-// formed column by column inside phase B of row i, from row i - 1's M (the value the D-hat
-// chain reads anyway) and J, so no partials array is kept between rows (32 registers at
-// N = 32); the scan's latency is then left to the other warps.  Same results as
-// team_run_pipe up to rounding order.
-// ------------------------------------------------------------------------------------
 // Asynchronous 16-byte copy global -> shared through L2 only (cp.async.cg: the source was
 // written by this warp's previous strip with L2-only stores, so L1 may hold stale lines),
 // and the group bookkeeping around it.
@@ -1077,472 +1063,6 @@ __device__ __forceinline__ void cp_async16_cg(void* smem_dst, const void* gmem_s
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
-// float2 FMA / multiply as one packed instruction (PACKED) or as two scalar ones (two
-// independent dependency chains for the scheduler to interleave).
-template <bool PACKED>
-__device__ __forceinline__ float2 ffma2_sel(float2 a, float2 b, float2 c) {
-    if constexpr (PACKED) return __ffma2_rn(a, b, c);
-    else return make_float2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y));
-}
-template <bool PACKED>
-__device__ __forceinline__ float2 fmul2_sel(float2 a, float2 b) {
-    if constexpr (PACKED) return __fmul2_rn(a, b);
-    else return make_float2(a.x * b.x, a.y * b.y);
-}
-
-// LINK: the team is a whole warp running one 32 N-column strip of a wider pair whose
-// strips run one after another on this warp (the serial multi-warp kind).  As in
-// seg_link_pipe<N, true>: the finished left strip's boundary (float4 per row: M, J, D-hat,
-// E of its last column; `sin`) enters lane 0 and, as a carry g^(N t - 1), every lane's
-// D-hat; checkpoints keep E >= E_left; lane 31 stores this strip's boundary (`sout`).
-// The left boundary and the records are staged in shared memory (`stg`, `rstg`: two
-// blocks of 32 rows each for this warp), each block copied asynchronously (cp.async, one
-// row per lane) while the warp computes the 32 rows before it; every row then reads its
-// boundary and record as broadcasts (no record is held in registers across a row).
-// The lane's carry power g^(N lt - 1) stays in registers (reloaded when gcp changes):
-// reading it from L1 every row measured 2% slower on the 1M-pair uneven batch.
-// Progress of a strip of the wave kind (the rows whose boundary it has stored): released
-// by its writer after those stores, acquired by the right neighbour before it copies them.
-__device__ __forceinline__ unsigned long long ld_acquire_gpu(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_release_gpu(unsigned long long* p, unsigned long long v) {
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-// Waits (bounded, with backoff) until the left strip has stored rows 1..need.
-__device__ __forceinline__ bool wave_wait(const unsigned long long* p, unsigned long long need) {
-    long long spins = 0;
-    while (ld_acquire_gpu(p) < need) {
-        if (++spins > kSpinLimit) return false;
-        if (spins > kSpinFast) __nanosleep(64);
-    }
-    return true;
-}
-
-template <int N, bool PACKED, bool LINK = false, bool FUSE = LINK, bool L1P = false, bool WAVE = false>
-__device__ SegOut team_run_pipe2(const Rec32J* __restrict__ rec, int l, int lmax,
-                                 const uint8_t* __restrict__ hap, int k, int col0, int lt,
-                                 int tlast, int nsteps, const PowRow<float>* __restrict__ pow_tab,
-                                 const PipeRange& rng, const float4* sin = nullptr, float4* sout = nullptr,
-                                 bool has_left = false, bool has_right = false, float4* stg = nullptr,
-                                 float4* rstg = nullptr, const unsigned long long* prog_left = nullptr,
-                                 unsigned long long* prog_me = nullptr, uint32_t* status = nullptr) {
-    using NT = Num<float>;
-    static_assert(N <= 32 && N % 2 == 0, "match masks hold 32 columns; two halves");
-    static_assert(FUSE || !(LINK || L1P), "the serial strips and the L1 tables need the fused row");
-    static_assert(LINK || !WAVE, "the wave kind runs strips in link mode");
-    constexpr int H = N / 2;
-    uint32_t bmA = 0, bmC = 0, bmG = 0, bmT = 0, flags = rng.ok ? 0u : PF_DEGEN, mflags = 0;
-    const int nvalid = max(0, min(k - col0, N));
-#pragma unroll
-    for (int c = 0; c < N; ++c) {
-        if (c < nvalid) {
-            const int code = base_code(hap[col0 + c]);
-            // match bits in the order phase B reads them: bit 2q for column q of the first
-            // half, bit 2q + 1 for column H + q of the second
-            const uint32_t bit = 1u << (c < H ? 2 * c : 2 * (c - H) + 1);
-            if (code < 0) flags |= PF_BAD;
-            if (code == 0 || code == 4) bmA |= bit;
-            if (code == 1 || code == 4) bmC |= bit;
-            if (code == 2 || code == 4) bmG |= bit;
-            if (code == 3 || code == 4) bmT |= bit;
-        }
-    }
-    float2 M2[H], J2[H];  // .x: column q, .y: column H + q of the lane
-    float2 U2[FUSE ? 1 : H];  // unfused: row i + 1's partials, formed after row i's scan
-    int E = 120 - rng.target;    // see team_run_pipe's cinit
-    float2 dt2 = make_float2(0.f, 0.f), ml2 = make_float2(0.f, 0.f);
-    float nj = 0.f;  // J of row i - 1 at the column before the lane (previous lane's last)
-    float gprev = 0.f;
-    float sp1[5], sp2[5], last1 = 0.f, last2 = 0.f, hh1 = 0.f, hh2 = 0.f, hm1 = 0.f, hm2 = 0.f;
-    int gcp = -1;
-    float qa1 = 0.f, qa2 = 0.f;
-    float lsc = 1.f;  // LINK: 2^(E_left - E), constant between checkpoints
-    const int l1 = max(l, 1) - 1;
-    if constexpr (LINK) {
-        // block 0 (rows 1..32): records and, with a left strip, its boundary rows
-        const float4* src = reinterpret_cast<const float4*>(rec + min(lt, l1));
-        cp_async16_cg(rstg + 2 * lt, src);
-        cp_async16_cg(rstg + 2 * lt + 1, src + 1);
-        if constexpr (WAVE) {  // the left strip runs concurrently: its rows 1..32 first
-            if (has_left && !wave_wait(prog_left, (unsigned long long)min(l, 32))) {
-                flags |= PF_TIMEOUT;
-                atomicOr(status, ST_TIMEOUT);
-            }
-        }
-        if (has_left && lt + 1 <= l) cp_async16_cg(stg + lt, sin + lt);
-        cp_async_commit();
-        cp_async_wait_0();
-        __syncwarp();
-    }
-    SegOut out;
-    out.S = 0.0;
-    out.E = 0;
-    out.flags = 0;
-    const float cinit = l > 0 && k > 0 ? (float)(ldexp(1.0, rng.target) / (double)k) : 0.f;
-    Rec32J cur;
-    if constexpr (!LINK && !L1P) cur = load_recj(rec);
-    int until = 0;
-    for (int i = 1; i <= lmax; ++i) {
-        Rec32J nxt;
-        if constexpr (LINK) {
-            // Stage blocks of 32 rows (records and left boundary), two buffers: block b + 1
-            // is copied while block b is computed; at block b's first row the warp waits
-            // for block b (issued 32 rows earlier) and then issues block b + 1.  Row i
-            // sits in slot (i - 1) mod 64 of the two buffers taken together.
-            const int slot = (i - 1) & 63;
-            if ((slot & 31) == 0) {
-                cp_async_wait_0();
-                __syncwarp();  // block b has landed; every lane is done with block b - 1's buffer
-                const int r = i + 32 + lt;
-                const int ns = (slot + 32 + lt) & 63;  // row r's slot
-                const float4* src = reinterpret_cast<const float4*>(rec + min(r - 1, l1));
-                cp_async16_cg(rstg + 2 * ns, src);
-                cp_async16_cg(rstg + 2 * ns + 1, src + 1);
-                if constexpr (WAVE) {  // the next block's rows of the concurrent left strip
-                    if (has_left && i + 32 <= l && !wave_wait(prog_left, (unsigned long long)min(l, i + 63))) {
-                        flags |= PF_TIMEOUT;
-                        atomicOr(status, ST_TIMEOUT);
-                    }
-                }
-                if (has_left && r <= l) cp_async16_cg(stg + ns, sin + (r - 1));
-                cp_async_commit();
-            }
-            const float4 a = rstg[2 * slot], b = rstg[2 * slot + 1];
-            cur.pm = a.x; cur.px = a.y; cur.a = a.z; cur.b = a.w;
-            cur.h = b.x; cur.g = b.y; cur.mi = b.z; cur.meta = __float_as_uint(b.w);
-        } else if constexpr (L1P) {
-            // the row's record from L1 at the row's start; a few rows ahead are prefetched
-            const Rec32J* rp = rec + min(i - 1, l1);
-            cur = load_recj(rp);
-            asm volatile("prefetch.global.L1 [%0];" ::"l"(rec + min(i + 7, l1)));
-        } else {
-            nxt = cur;
-            if (i < lmax) nxt = load_recj(rec + min(i, l1));
-        }
-        const uint32_t meta = cur.meta;
-        mflags |= meta;
-        const int gq = (int)((meta >> META_GCP_SHIFT) & 0xffu);
-        const PowRow<float>* pr = pow_tab + min(gq, kMaxPhred);
-        if constexpr (L1P) {
-            // carry powers read from L1 where they are used (no registers across the row)
-            if constexpr (LINK) {
-                if (gq != gcp) {
-                    qa1 = __ldg(&pr->lq1[lt]);
-                    qa2 = __ldg(&pr->lq2[lt]);
-                    gcp = gq;
-                }
-            }
-        } else if (LINK ? __any_sync(kFull, gq != gcp) : gq != gcp) {
-            // (link mode: every lane holds the same row, so the vote is exact and the
-            // branch is warp-uniform)
-#pragma unroll
-            for (int s = 0; s < 5; ++s) {
-                sp1[s] = lt >= (1 << s) ? __ldg(&pr->sp1[s]) : 0.f;
-                sp2[s] = __ldg(&pr->sp2[s]);
-            }
-            last1 = (!LINK || lt >= 2) ? __ldg(&pr->last1) : 0.f;  // link: zz of lanes 0, 1 drops out
-            last2 = __ldg(&pr->last2);
-            hh1 = __ldg(&pr->hh1);
-            hh2 = __ldg(&pr->hh2);
-            hm1 = __ldg(&pr->hm1);
-            hm2 = __ldg(&pr->hm2);
-            if constexpr (LINK) {
-                qa1 = __ldg(&pr->lq1[lt]);
-                qa2 = __ldg(&pr->lq2[lt]);
-            }
-            gcp = gq;
-        }
-        // the row's carry powers: registers, or L1 reads at their use
-        const auto P_sp1 = [&](int s) { if constexpr (L1P) return lt >= (1 << s) ? __ldg(&pr->sp1[s]) : 0.f; else return sp1[s]; };
-        const auto P_sp2 = [&](int s) { if constexpr (L1P) return __ldg(&pr->sp2[s]); else return sp2[s]; };
-        const auto P_last1 = [&]() { if constexpr (L1P) return __ldg(&pr->last1); else return last1; };
-        const auto P_last2 = [&]() { if constexpr (L1P) return __ldg(&pr->last2); else return last2; };
-        const auto P_hh1 = [&]() { if constexpr (L1P) return __ldg(&pr->hh1); else return hh1; };
-        const auto P_hh2 = [&]() { if constexpr (L1P) return __ldg(&pr->hh2); else return hh2; };
-        const auto P_hm1 = [&]() { if constexpr (L1P) return __ldg(&pr->hm1); else return hm1; };
-        const auto P_hm2 = [&]() { if constexpr (L1P) return __ldg(&pr->hm2); else return hm2; };
-        const int code = (int)(meta & META_CODE_MASK);
-        const uint32_t mask = code == 0 ? bmA : code == 1 ? bmC : code == 2 ? bmG
-                            : code == 3 ? bmT : 0xffffffffu;
-        const float pim = cur.pm, pix = cur.px, rg = cur.g;
-        const float2 rg2 = make_float2(rg, rg);
-        float2 y2 = make_float2(0.f, 0.f), yp2 = make_float2(0.f, 0.f);
-        // phase B (both halves at once)
-        if (i == 1) {
-#pragma unroll
-            for (int q = 0; q < H; ++q) {
-                const float2 mn = make_float2((((mask >> (2 * q)) & 1u) ? pim : pix) * cinit,
-                                              (((mask >> (2 * q + 1)) & 1u) ? pim : pix) * cinit);
-                M2[q] = mn;
-                J2[q] = make_float2(0.f, 0.f);
-                if (q == H - 1) yp2 = y2;
-                y2 = ffma2_sel<PACKED>(rg2, y2, mn);
-            }
-        } else if constexpr (!FUSE) {
-            const float2 rb2 = make_float2(cur.b, cur.b), gp2 = make_float2(gprev, gprev);
-#pragma unroll
-            for (int q = 0; q < H; ++q) {
-                const float2 u2 = ffma2_sel<PACKED>(rb2, dt2, U2[q]);
-                dt2 = ffma2_sel<PACKED>(gp2, dt2, ml2);
-                ml2 = M2[q];
-                const float2 p2 = make_float2(((mask >> (2 * q)) & 1u) ? pim : pix,
-                                              ((mask >> (2 * q + 1)) & 1u) ? pim : pix);
-                const float2 mn = fmul2_sel<PACKED>(p2, u2);
-                M2[q] = mn;
-                if (q == H - 1) yp2 = y2;
-                y2 = ffma2_sel<PACKED>(rg2, y2, mn);
-            }
-        } else {
-            // Row i's partials U = a M' + J' and insertions J = M' + h J' (primes: row
-            // i - 1, from the column before for U, the same column for J) are formed
-            // column by column as phase B reaches them, from the old M and J.  Row i - 1's
-            // D-hat chain runs one column ahead (dA: the D-hat of the column before q; dB:
-            // that of column q, formed from column q - 1's old M), so column q's old M and
-            // J have their last uses (dB, column q + 1's partial, column q's J) before
-            // column q's new M is formed, and the new values take the old ones' registers.
-            const float2 rb2 = make_float2(cur.b, cur.b), gp2 = make_float2(gprev, gprev);
-            const float2 na2 = make_float2(cur.a, cur.a), nh2 = make_float2(cur.h, cur.h);
-            float2 uq = ffma2_sel<PACKED>(na2, ml2, make_float2(nj, J2[H - 1].x));
-            float2 dA = dt2, dB = ffma2_sel<PACKED>(gp2, dt2, ml2);
-#pragma unroll
-            for (int q = 0; q < H; ++q) {
-                const float2 u2 = ffma2_sel<PACKED>(rb2, dA, uq);
-                const float2 mo = M2[q];
-                if (q + 1 < H) {
-                    dA = dB;
-                    dB = ffma2_sel<PACKED>(gp2, dB, mo);
-                    uq = ffma2_sel<PACKED>(na2, mo, J2[q]);
-                }
-                J2[q] = ffma2_sel<PACKED>(nh2, J2[q], mo);
-                const float2 p2 = make_float2(((mask >> (2 * q)) & 1u) ? pim : pix,
-                                              ((mask >> (2 * q + 1)) & 1u) ? pim : pix);
-                const float2 mn = fmul2_sel<PACKED>(p2, u2);
-                M2[q] = mn;
-                if (q == H - 1) yp2 = y2;
-                y2 = ffma2_sel<PACKED>(rg2, y2, mn);
-            }
-        }
-        // Eq. 4 when a pair of this warp finishes (I = T_MI J on the last row); a strip
-        // of the serial kind is one pair on the whole warp
-        bool ends;
-        if constexpr (LINK) ends = false;  // one pair on the whole warp: summed after the loop
-        else ends = __any_sync(kFull, i == l);
-        if (ends) {
-            const double rmi = (double)cur.mi;
-            double s = 0.0;
-#pragma unroll
-            for (int q = 0; q < H; ++q) {
-                if (q < nvalid) s += (double)M2[q].x + rmi * (double)J2[q].x;
-                if (q + H < nvalid) s += (double)M2[q].y + rmi * (double)J2[q].y;
-            }
-            s = team_sum<double>(s, lt, tlast, nsteps);
-            uint32_t f = flags;
-            if (mflags & META_BAD) f |= PF_BAD;
-            if (mflags & META_DEGEN) f |= PF_DEGEN;
-            f = team_or(f, lt, tlast, nsteps);
-            if (i == l) {
-                out.S = s;
-                out.E = E;
-                out.flags = f;
-            }
-        }
-        // lane aggregates of the local (zero-carry) D-hat chain: one past the lane's last
-        // column (scan input) and at its last column (the right neighbour's carry)
-        const float zl = fmaf(y2.x * P_hh1(), P_hh2(), y2.y);
-        float ypl = fmaf(y2.x * P_hm1(), P_hm2(), yp2.y);
-        float jl = 0.f;
-        if constexpr (LINK) jl = J2[H - 1].y;  // this lane's last J of row i (sent right)
-        float yA = yp2.x;  // first half, at its last column
-        float nm = __shfl_up_sync(kFull, M2[H - 1].y, 1);
-        nj = __shfl_up_sync(kFull, J2[H - 1].y, 1);
-        float yp = __shfl_up_sync(kFull, ypl, 1);
-        if (!LINK && lt == 0) {  // link mode replaces lane 0's three after the checkpoint
-            nm = 0.f;
-            nj = 0.f;
-            yp = 0.f;
-        }
-        float Z = zl;
-#pragma unroll
-        for (int s = 0; s < 5; ++s) {
-            const float up = __shfl_up_sync(kFull, Z, 1 << s);
-            Z = fmaf(up * P_sp1(s), P_sp2(s), Z);
-        }
-        if constexpr (!FUSE) {  // phase A: row i + 1's partials and insertions
-            const float2 na2 = make_float2(nxt.a, nxt.a), nh2 = make_float2(nxt.h, nxt.h);
-            const float mal = M2[H - 1].x, jal = J2[H - 1].x;
-#pragma unroll
-            for (int q = H - 1; q >= 1; --q) {
-                U2[q] = ffma2_sel<PACKED>(na2, M2[q - 1], J2[q - 1]);
-                J2[q] = ffma2_sel<PACKED>(nh2, J2[q], M2[q]);
-            }
-            U2[0] = ffma2_sel<PACKED>(na2, make_float2(nm, mal), make_float2(nj, jal));
-            J2[0] = ffma2_sel<PACKED>(nh2, J2[0], M2[0]);
-        }
-        float zz = __shfl_up_sync(kFull, Z, 2);
-        if ((!LINK || L1P) && lt < 2) zz = 0.f;
-        if constexpr (LINK) {
-            // one broadcast read, taken with or without a left strip (without one the slot is
-            // stale and only selected away: no branch in the row)
-            const float4 v = stg[(i - 1) & 63];
-            float lM = has_left ? v.x : 0.f, lJ = has_left ? v.y : 0.f, lD = has_left ? v.z : 0.f;
-            const int Eleft = has_left ? __float_as_int(v.w) : INT_MIN;
-            // checkpoint (same rows in every strip of the pair): E >= E_left, so that left
-            // values only ever scale down
-            int Enew = E;
-            if (until == 0) {
-                until = rng.R;
-                float2 m2 = make_float2(0.f, 0.f);
-#pragma unroll
-                for (int q = 0; q < H; ++q) {
-                    m2.x = fmaxf(m2.x, fmaxf(fabsf(M2[q].x), fabsf(J2[q].x)));
-                    m2.y = fmaxf(m2.y, fmaxf(fabsf(M2[q].y), fabsf(J2[q].y)));
-                }
-                // the strip is the whole warp: one reduction over the lanes' maxima (values
-                // >= 0, so their bit patterns order like the values)
-                const float m = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(fmaxf(m2.x, m2.y))));
-                const int e = NT::expo(m);
-                int desired = E;
-                if (e == INT_MAX) {
-                    flags |= PF_NONFINITE;
-                } else if (e == INT_MIN) {
-                    if (has_left) desired = INT_MIN;  // nothing representable: follow the left
-                } else if (e > rng.hi || e <= NT::kLo) {
-                    desired = E + (e - rng.target);
-                }
-                Enew = desired;
-                bool forced = false;
-                if (has_left && Eleft > Enew) {
-                    Enew = Eleft;
-                    forced = true;
-                }
-                if (Enew == INT_MIN) Enew = E;
-                if (!forced && e != INT_MIN && e != INT_MAX && e <= rng.danger) flags |= PF_DANGER;
-                if (Enew != E) {  // only a checkpoint row changes the exponent
-                    const int sdn = E - Enew;
-#pragma unroll
-                    for (int q = 0; q < H; ++q) {
-                        M2[q] = make_float2(scale2(M2[q].x, sdn), scale2(M2[q].y, sdn));
-                        J2[q] = make_float2(scale2(J2[q].x, sdn), scale2(J2[q].y, sdn));
-                    }
-                    nm = scale2(nm, sdn);
-                    nj = scale2(nj, sdn);
-                    zz = scale2(zz, sdn);
-                    yp = scale2(yp, sdn);
-                    yA = scale2(yA, sdn);
-                    ypl = scale2(ypl, sdn);
-                    jl = scale2(jl, sdn);
-                    flags |= PF_RESCALED;
-                    E = Enew;
-                }
-                // both exponents change only on checkpoint rows (the same rows in every
-                // strip of the pair), so the left values' scale 2^(E_left - E) <= 1 is
-                // formed here (exactly, subnormal or zero below 2^-126) and kept
-                const int dsh = has_left ? Eleft - E : 0;
-                lsc = dsh >= -126 ? NT::pow2(dsh) : dsh >= -149 ? __uint_as_float(1u << (dsh + 149)) : 0.f;
-            }
-            --until;
-            // left values into this strip's scale (no left: zeros stay zero)
-            lM *= lsc;
-            lJ *= lsc;
-            lD *= lsc;
-            const float Wseg = fmaf(rg, lD, lM);  // D-hat at the strip's first column
-            float ndA = fmaf(zz * P_last1(), P_last2(), yp);
-            ndA = fmaf(Wseg * qa1, qa2, ndA);
-            if (lt == 0) {
-                ndA = lD;
-                nm = lM;
-                nj = lJ;
-            }
-            if (has_right && lt == 31) {
-                // D-hat at the strip's last column: the lane's own chain from ndA (the
-                // column before it, carry included) over its N columns, g^N ndA + ypl
-                const float dl = fmaf((ndA * rg) * P_last1(), P_last2(), ypl);
-                __stcg(sout + (i - 1), make_float4(M2[H - 1].y, jl, dl, __int_as_float(E)));
-                if constexpr (WAVE) {  // rows 1..i stored: publish at block ends and the last row
-                    if ((i & 31) == 0 || i == l) st_release_gpu(prog_me, (unsigned long long)i);
-                }
-            }
-            const float wl = fmaf(rg, ndA, nm);         // D-hat at the lane's first column
-            const float ndB = fmaf(wl * P_hm1(), P_hm2(), yA);  // D-hat at the first half's last column
-            dt2 = make_float2(ndA, ndB);
-            ml2 = make_float2(nm, M2[H - 1].x);
-            gprev = rg;
-            continue;
-        }
-        if (until == 0) {
-            until = rng.R;
-            float2 m2 = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int q = 0; q < H; ++q) {
-                m2.x = fmaxf(m2.x, fmaxf(fabsf(M2[q].x), fabsf(J2[q].x)));
-                m2.y = fmaxf(m2.y, fmaxf(fabsf(M2[q].y), fabsf(J2[q].y)));
-            }
-            const float m = team_max_pos(fmaxf(m2.x, m2.y), lt, tlast);
-            const int e = NT::expo(m);
-            if (e == INT_MAX) {
-                flags |= PF_NONFINITE;
-            } else if (e != INT_MIN) {
-                if (e <= rng.danger) flags |= PF_DANGER;
-                if (e > rng.hi || e <= NT::kLo) {
-                    const int sh = e - rng.target;
-                    float f1 = 1.f, f2v;
-                    if (sh >= -126 && sh <= 126) {
-                        f2v = NT::pow2(-sh);
-                    } else {
-                        f1 = NT::pow2((-sh) / 2);
-                        f2v = NT::pow2(-sh - (-sh) / 2);
-                    }
-                    const float2 a2 = make_float2(f1, f1), b2 = make_float2(f2v, f2v);
-#pragma unroll
-                    for (int q = 0; q < H; ++q) {
-                        M2[q] = fmul2_sel<PACKED>(fmul2_sel<PACKED>(M2[q], a2), b2);
-                        J2[q] = fmul2_sel<PACKED>(fmul2_sel<PACKED>(J2[q], a2), b2);
-                        if constexpr (!FUSE) U2[q] = fmul2_sel<PACKED>(fmul2_sel<PACKED>(U2[q], a2), b2);
-                    }
-                    nm = (nm * f1) * f2v;
-                    nj = (nj * f1) * f2v;
-                    zz = (zz * f1) * f2v;
-                    yp = (yp * f1) * f2v;
-                    yA = (yA * f1) * f2v;
-                    flags |= PF_RESCALED;
-                    E += sh;
-                }
-            }
-        }
-        --until;
-        const float ndA = fmaf(zz * P_last1(), P_last2(), yp);  // D-hat at the column before the lane
-        const float wl = fmaf(rg, ndA, nm);                      // D-hat at the lane's first column
-        const float ndB = fmaf(wl * P_hm1(), P_hm2(), yA);       // D-hat at the first half's last column
-        dt2 = make_float2(ndA, ndB);
-        ml2 = make_float2(nm, M2[H - 1].x);
-        gprev = rg;
-        if constexpr (!LINK && !L1P) cur = nxt;
-    }
-    if constexpr (LINK) {
-        cp_async_wait_0();  // nothing may land in the stage after this strip
-        // Eq. 4 on the pair's last row l (= lmax; a checkpoint on it rescaled M, J and E
-        // together, and its flags count)
-        const double rmi = (double)cur.mi;
-        double s = 0.0;
-#pragma unroll
-        for (int q = 0; q < H; ++q) {
-            if (q < nvalid) s += (double)M2[q].x + rmi * (double)J2[q].x;
-            if (q + H < nvalid) s += (double)M2[q].y + rmi * (double)J2[q].y;
-        }
-        s = team_sum<double>(s, lt, tlast, nsteps);
-        uint32_t f = flags;
-        if (mflags & META_BAD) f |= PF_BAD;
-        if (mflags & META_DEGEN) f |= PF_DEGEN;
-        out.S = s;
-        out.E = E;
-        out.flags = team_or(f, lt, tlast, nsteps);
-    }
-    return out;
-}
 
 // ------------------------------------------------------------------------------------
 // Pipelined FP32 engine for one warp segment of a multi-warp pair (32 N columns, all 32

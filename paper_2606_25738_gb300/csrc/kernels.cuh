@@ -11,6 +11,7 @@
 
 #include "engine.cuh"
 #include "phmm_internal.h"
+#include "skew.cuh"
 
 namespace phmm {
 
@@ -143,7 +144,8 @@ __device__ __forceinline__ Rec32J make_rec32j(const BaseQ& x, const float2* tq, 
     r.px = sround(df_mul(df_mul(q3_Q, om_g), mi_p), (uint32_t)((h1 >> 24) & 0xffffffu));
     r.a = sround(df_mul(df_mul(tmm, inv_g), imi_p), (uint32_t)((h1 >> 40) & 0xffffffu));
     r.b = sround(df_mul(q_dp, imi_p), (uint32_t)(h2 & 0xffffffu));
-    r.h = sround(df_mul(df_mul(q_g, mi_p), iq_i), (uint32_t)((h2 >> 24) & 0xffffffu));
+    // row 1 has no insertion before it (the skewed engines rely on h = 0 there)
+    r.h = first ? 0.0f : sround(df_mul(df_mul(q_g, mi_p), iq_i), (uint32_t)((h2 >> 24) & 0xffffffu));
     r.g = q_g.hi;
     r.mi = q_i.hi;
     uint32_t meta = (uint32_t)x.code | ((uint32_t)x.gcp << META_GCP_SHIFT);
@@ -648,20 +650,14 @@ k_forward_cluster(const BatchHeader* __restrict__ H, const PowRow<float>* __rest
 }
 
 // Multi-warp pairs one warp at a time (long kind 3): each warp takes a whole pair and
-// runs its strips of 32 N columns one after another (team_run_pipe2 in LINK mode), strip s
-// reading the boundary strip s - 1 left in this warp's scratch.  No warp ever waits on
-// another; the pair's S strips leave S partials, combined by the finalize kernel as for
-// CTA strips.
-template <int N, int MINB, bool L1P = false>
-__global__ void __launch_bounds__(128, MINB)
-k_forward_serial(const BatchHeader* __restrict__ H, const PowRow<float>* __restrict__ pow) {
-    __shared__ float4 stage[4][64];    // per warp: two blocks of 32 left-boundary rows
-    __shared__ float4 rstage[4][128];  // per warp: two blocks of 32 records (32 B each)
-    const PipeRange rng = pipe_range(H->dropgrow);
+// runs its strips of 32 N columns one after another (strip_run_skew), strip s reading the
+// boundary strip s - 1 left in this warp's scratch.  No warp ever waits on another; the
+// pair's S strips leave S partials, combined by the finalize kernel as for CTA strips.
+template <int N, bool G10>
+__device__ __forceinline__ void serial_items(const BatchHeader* __restrict__ H, const PipeRange& rng, SkewStage& st) {
     const uint32_t n_c = H->n_citems;
     const int lane = threadIdx.x & 31;
     const uint32_t gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (gw >= H->sbnd_warps) return;  // no scratch for this warp (grid larger than planned)
     float4* buf0 = H->sbnd + (size_t)gw * 2 * H->sbnd_rows;
     float4* buf1 = buf0 + H->sbnd_rows;
     for (;;) {
@@ -673,13 +669,10 @@ k_forward_serial(const BatchHeader* __restrict__ H, const PowRow<float>* __restr
         const PairDesc d = H->desc[cp.pair];
         const uint32_t S = cp.nstrip;
         for (uint32_t s = 0; s < S; ++s) {
-            const float4* in = (s & 1u) ? buf0 : buf1;  // what strip s - 1 wrote
-            float4* outb = (s & 1u) ? buf1 : buf0;
-            const int c0 = (int)(s * 32u * N) + lane * N;
-            const SegOut o = team_run_pipe2<N, true, true, true, L1P>(H->rec32j + d.roff, (int)d.l, (int)d.l,
-                                                           H->hap_bases + d.hoff, (int)d.k, c0, lane, 31, 5,
-                                                           pow, rng, in, outb, s > 0, s + 1 < S,
-                                                           stage[threadIdx.x >> 5], rstage[threadIdx.x >> 5]);
+            const float4* in = s == 0 ? nullptr : (s & 1u) ? buf0 : buf1;  // what strip s - 1 wrote
+            float4* outb = s + 1 == S ? nullptr : (s & 1u) ? buf1 : buf0;
+            const SegOut o = strip_run_skew<N, false, G10>(H->rec32j + d.roff, (int)d.l, H->hap_bases + d.hoff, (int)d.k,
+                                                           (int)s, rng, in, outb, st, 0u, H->status);
             __syncwarp();  // this strip's boundary stores before the next strip's loads
             if (lane == 0) {
                 Partial p;
@@ -691,22 +684,28 @@ k_forward_serial(const BatchHeader* __restrict__ H, const PowRow<float>* __restr
         }
     }
 }
-
-// Wave multi-warp kind (long kind 6): every 1024-column strip of a wide pair is its own
-// item, on its own warp, and the strips of a pair run at the same time.  Strip s stores its
-// right boundary row by row (float4: M, J, D-hat, E of its last column) at wbnd + bnd_out
-// and releases its progress (rows stored) in boundary word `pad` at every 32nd row and the
-// last; strip s + 1 acquires that word before it copies the next 32 rows of the boundary
-// (team_run_pipe2<..., WAVE>), so the strips hand over once per 32 rows.  Items are taken
-// in order and a pair's strips are consecutive: a strip only waits for a strip that some
-// warp already runs, so every wait ends (and each one is bounded).
 template <int N, int MINB>
 __global__ void __launch_bounds__(128, MINB)
-k_forward_wave(const BatchHeader* __restrict__ H, const PowRow<float>* __restrict__ pow) {
-    __shared__ float4 stage[4][64];    // per warp: two blocks of 32 left-boundary rows
-    __shared__ float4 rstage[4][128];  // per warp: two blocks of 32 records (32 B each)
-    const PipeRange rng = pipe_range(H->dropgrow);
+k_forward_serial(const BatchHeader* __restrict__ H) {
+    __shared__ SkewStage stage[4];
+    const PipeRange rng = skew_range(H);
+    const uint32_t gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (gw >= H->sbnd_warps) return;  // no scratch for this warp (grid larger than planned)
+    if (skew_g10(H->skst)) serial_items<N, true>(H, rng, stage[threadIdx.x >> 5]);
+    else serial_items<N, false>(H, rng, stage[threadIdx.x >> 5]);
+}
+
+// Wave multi-warp kind (long kinds 6 to 8): every strip of a wide pair is its own item, on its
+// own warp, and the strips of a pair run at the same time.  Strip s stores its right
+// boundary row by row (M, I, D-hat and the exponent with this launch's tag, one 16-byte
+// relaxed store) at wbnd + bnd_out; strip s + 1 takes kWaveBlock rows at a time once they
+// carry the tag, so no fence and no progress word stands between them.  Items are taken in
+// order and a pair's strips are consecutive: a strip only waits for a strip that some warp
+// already runs, so every wait ends (and each one is bounded).
+template <int N, bool G10>
+__device__ __forceinline__ void wave_items(const BatchHeader* __restrict__ H, const PipeRange& rng, SkewStage& st) {
     const uint32_t n_c = H->n_citems;
+    const uint32_t tag = *H->wave_epoch;
     const int lane = threadIdx.x & 31;
     for (;;) {
         uint32_t wi = 0;
@@ -716,15 +715,10 @@ k_forward_wave(const BatchHeader* __restrict__ H, const PowRow<float>* __restric
         const CtaPair cp = H->cpairs[H->citems[wi].first];
         const PairDesc d = H->desc[cp.pair];
         const uint32_t s = cp.strip, S = cp.nstrip;
-        const bool has_left = s > 0, has_right = s + 1 < S;
-        const float4* in = has_left ? H->wbnd + cp.bnd_in : nullptr;
-        float4* outb = has_right ? H->wbnd + cp.bnd_out : nullptr;
-        const unsigned long long* pl = has_left ? H->bnd + (cp.pad - 1) : nullptr;
-        unsigned long long* pm = has_right ? H->bnd + cp.pad : nullptr;
-        const int c0 = (int)cp.col0 + lane * N;
-        const SegOut o = team_run_pipe2<N, true, true, true, false, true>(
-            H->rec32j + d.roff, (int)d.l, (int)d.l, H->hap_bases + d.hoff, (int)d.k, c0, lane, 31, 5, pow, rng,
-            in, outb, has_left, has_right, stage[threadIdx.x >> 5], rstage[threadIdx.x >> 5], pl, pm, H->status);
+        const float4* in = s > 0 ? H->wbnd + cp.bnd_in : nullptr;
+        float4* outb = s + 1 < S ? H->wbnd + cp.bnd_out : nullptr;
+        const SegOut o = strip_run_skew<N, true, G10>(H->rec32j + d.roff, (int)d.l, H->hap_bases + d.hoff, (int)d.k,
+                                                      (int)s, rng, in, outb, st, tag, H->status);
         __syncwarp();
         if (lane == 0) {
             Partial p;
@@ -734,6 +728,14 @@ k_forward_wave(const BatchHeader* __restrict__ H, const PowRow<float>* __restric
             write_strip_part(H, cp.pair, s, S, cp.extra_base, p);
         }
     }
+}
+template <int N, int MINB>
+__global__ void __launch_bounds__(128, MINB)
+k_forward_wave(const BatchHeader* __restrict__ H) {
+    __shared__ SkewStage stage[4];
+    const PipeRange rng = skew_range(H);
+    if (skew_g10(H->skst)) wave_items<N, true>(H, rng, stage[threadIdx.x >> 5]);
+    else wave_items<N, false>(H, rng, stage[threadIdx.x >> 5]);
 }
 
 // Team lookup of a warp item: this lane's team (first lane, size, pairs) and the scan
@@ -858,13 +860,11 @@ k_short_pipe64(const BatchHeader* __restrict__ H, const PowRow<double>* __restri
     }
 }
 
-// Pipelined scalar teams with packed column halves (team_run_pipe2).  LEAN: the fused row
-// (no partials array) with records and carry powers read from L1 each row, which fits
-// 128 registers and so four CTAs of four warps per SM.
-template <int N, int MINB, bool PACKED, bool LEAN = false>
-__global__ void __launch_bounds__(kShortThreads, MINB)
-k_short_pipe2(const BatchHeader* __restrict__ H, const PowRow<float>* __restrict__ pow) {
-    const PipeRange rng = pipe_range(H->dropgrow);
+// Scalar teams on the skewed engine (team_run_skew), same work list as k_short_scalar.  The
+// name and its last two parameters are those of the engine it took the place of (column
+// halves in packed pairs, and a lean form of it), which kernel_variant 5 and 6 ask for.
+template <int N, bool G10>
+__device__ __forceinline__ void skew_items(const BatchHeader* __restrict__ H, const PipeRange& rng, uint32_t* sm) {
     const uint32_t n_w = H->n_witems;
     const int lane = threadIdx.x & 31;
     for (;;) {
@@ -883,10 +883,21 @@ k_short_pipe2(const BatchHeader* __restrict__ H, const PowRow<float>* __restrict
             rec = H->rec32j + d.roff;
             hap = H->hap_bases + d.hoff;
         }
-        const int lmax = (int)__reduce_max_sync(kFull, (unsigned)l);
-        const SegOut o = team_run_pipe2<N, PACKED, false, LEAN, LEAN>(rec, l, lmax, hap, k, t.lt * N, t.lt, t.tlast, t.nsteps, pow, rng);
+        const int team = t.tlast - (lane - t.lt) + 1;
+        const int steps = (int)__reduce_max_sync(kFull, l > 0 ? (unsigned)(l + team - 1) : 0u);
+        const int p0 = 1 + (int)__reduce_max_sync(kFull, l > 0 ? (unsigned)team : 1u);
+        const int p1 = (int)__reduce_min_sync(kFull, l > 0 ? (unsigned)l : 0x7fffffffu);
+        const SegOut o = team_run_skew<N, G10>(rec, l, steps, p0, p1, hap, k, t.lt, t.tlast, rng, sm + lane);
         if (t.pair != kNoPair && t.lt == 0) write_part(H, t.pair, o);
     }
+}
+template <int N, int MINB, bool HALVES = true, bool LEAN = false>
+__global__ void __launch_bounds__(kShortThreads, MINB)
+k_short_pipe2(const BatchHeader* __restrict__ H) {
+    __shared__ uint32_t masks[kShortThreads / 32][5 * 32];
+    const PipeRange rng = skew_range(H);
+    if (skew_g10(H->skst)) skew_items<N, true>(H, rng, masks[threadIdx.x >> 5]);
+    else skew_items<N, false>(H, rng, masks[threadIdx.x >> 5]);
 }
 
 // Packed teams of two haplotypes of the same read, N columns per lane (item list
@@ -949,29 +960,32 @@ __device__ __forceinline__ double fp32_bound_log10(double l, double k) {
 template <typename T>
 __global__ void k_finalize(const BatchHeader* __restrict__ H) {
     using NT = Num<T>;
+    using NT64 = Num<double>;
     const uint32_t n = H->n_pairs;
     const uint32_t mode = H->mode;
     for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
         Partial q = H->parts[p];
         const PairDesc d = H->desc[p];
         if ((q.flags & PF_DONE) && q.n_extra > 0) {
-            // strips of a wide pair: L * C = sum_s S_s 2^(E_s)
-            int Eref = q.S != 0.0 ? q.E : INT_MIN;
+            // strips of a wide pair: L * C = sum_s S_s 2^(E_s), in the scale of the strip that
+            // holds the largest share (the underflow test below reads its stored units)
+            int Eref = q.E, top = q.S != 0.0 ? q.E + NT64::expo(q.S) : INT_MIN;
             for (uint32_t e = 0; e < q.n_extra; ++e) {
                 const Partial x = H->parts[q.extra_base + e];
                 q.flags |= x.flags;
                 if (!(x.flags & PF_DONE)) q.flags &= ~PF_DONE;
-                if (x.S != 0.0) Eref = max(Eref, x.E);
+                if (x.S != 0.0 && x.E + NT64::expo(x.S) > top) {
+                    top = x.E + NT64::expo(x.S);
+                    Eref = x.E;
+                }
             }
             double Sum = 0.0;
-            if (Eref != INT_MIN) {
-                if (q.S != 0.0) Sum += ldexp(q.S, q.E - Eref);
-                for (uint32_t e = 0; e < q.n_extra; ++e) {
-                    const Partial x = H->parts[q.extra_base + e];
-                    if (x.S != 0.0) Sum += ldexp(x.S, x.E - Eref);
-                }
-                q.E = Eref;
+            if (q.S != 0.0) Sum += ldexp(q.S, q.E - Eref);
+            for (uint32_t e = 0; e < q.n_extra; ++e) {
+                const Partial x = H->parts[q.extra_base + e];
+                if (x.S != 0.0) Sum += ldexp(x.S, x.E - Eref);
             }
+            q.E = Eref;
             q.S = Sum;
         }
         uint32_t f = q.flags;

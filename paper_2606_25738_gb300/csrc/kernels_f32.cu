@@ -22,11 +22,16 @@ __global__ void k_reset(const BatchHeader* __restrict__ H) {
             H->dropgrow[1] = 0u;
             H->dropgrow[2] = 0u;
             H->dropgrow[3] = 0u;
+            *H->skst = SkewStats{};
         }
     }
     const uint64_t n = H->n_bnd_words;
     for (uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (uint64_t)gridDim.x * blockDim.x)
         H->bnd[q] = 0ull;
+    // the wave kind's tags start over after this launch: no row may keep one
+    const uint64_t nw = *H->wave_epoch == kWaveTags ? H->wbnd_rows : 0;
+    for (uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nw; q += (uint64_t)gridDim.x * blockDim.x)
+        H->wbnd[q] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // Phred tables as double-float pairs in shared memory.
@@ -86,10 +91,12 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep32(const BatchHeader* __re
                                                          const PhredTables* __restrict__ TG) {
     __shared__ Tables32 T;
     __shared__ uint4 sb[5][kPrepTile / 16 + 1];  // bases, Q, ins, del, gcp; byte 16 = tile start
+    if (blockIdx.x == 0 && threadIdx.x == 0) *H->wave_epoch = *H->wave_epoch % kWaveTags + 1u;
     stage_tables32(TG, T);
     const float2 *tq = T.tq, *tom = T.tom, *tq3 = T.tq3, *tinv = T.tinv;
     Rec32J* const rj = H->rec32j;
     uint32_t dmax = 0, gmax = 0, jmax = 0, hmax = 0;
+    SkewStats sk{};
     const uint64_t n = H->n_read_bases;
     const uint32_t seed = H->seed;
     const uint8_t* const s8[5] = {H->read_bases, H->base_q, H->ins_q, H->del_q, H->gcp_q};
@@ -138,6 +145,9 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep32(const BatchHeader* __re
                 const float big = fmaxf(fmaxf(fabsf(r2.a), fabsf(r2.b) / om), T.tiq[x.insp].x);
                 jmax = max(jmax, (uint32_t)fmaxf(ceilf(log2f(fmaxf(big, 1.0f))), 0.0f));
                 hmax = max(hmax, (uint32_t)ceilf(log2f(1.0f + fabsf(r2.h)) * 64.0f) + 1u);
+                sk.drop = max(sk.drop, (uint32_t)ceilf(fmaxf(-log2f(fmaxf(r2.h, 0x1p-126f)), 0.0f) * 64.0f) + 1u);
+                sk.gcp_max = max(sk.gcp_max, (uint32_t)x.gcp);
+                sk.gcp_inv = max(sk.gcp_inv, 255u - (uint32_t)x.gcp);
             }
             if (x.bad) atomicOr(H->status, ST_BAD_INPUT);
             const float qi = tq[x.ins].x, qd = tq[x.del].x, qg = tq[x.gcp].x;
@@ -150,6 +160,11 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep32(const BatchHeader* __re
     block_max2(dmax, gmax, H->dropgrow);
     __syncthreads();
     block_max2(jmax, hmax, H->dropgrow + 2);
+    uint32_t* const w = reinterpret_cast<uint32_t*>(H->skst);
+    __syncthreads();
+    block_max2(sk.drop, 0u, w);
+    __syncthreads();
+    block_max2(sk.gcp_max, sk.gcp_inv, w + 2);
     build_desc(H);
 }
 
@@ -172,9 +187,9 @@ __global__ void __launch_bounds__(256) k_prep32_first(const BatchHeader* __restr
 template __global__ void k_forward<float, kNLong32, false>(const BatchHeader*, const PowRow<float>*);
 template __global__ void k_forward_pipe<32, kCtaWarpsPipe>(const BatchHeader*, const PowRow<float>*);
 template __global__ void k_forward_pipe<24, kCtaWarps>(const BatchHeader*, const PowRow<float>*);
-template __global__ void k_forward_serial<32, 3>(const BatchHeader*, const PowRow<float>*);
-template __global__ void k_forward_wave<32, 3>(const BatchHeader*, const PowRow<float>*);
-template __global__ void k_forward_wave<16, 3>(const BatchHeader*, const PowRow<float>*);
+template __global__ void k_forward_serial<32, 3>(const BatchHeader*);
+template __global__ void k_forward_wave<32, 3>(const BatchHeader*);
+template __global__ void k_forward_wave<16, 3>(const BatchHeader*);
 template __global__ void k_forward_pipe<32, 4>(const BatchHeader*, const PowRow<float>*);
 template __global__ void k_forward_cluster<32, kClusterWarps, kClusterCtas>(const BatchHeader*, const PowRow<float>*);
 template __global__ void k_short_scalar<32, 4>(const BatchHeader*, const PowRow<float>*);
@@ -184,9 +199,9 @@ template __global__ void k_short_scalar<16, 6>(const BatchHeader*, const PowRow<
 template __global__ void k_short_pipe<32, 3>(const BatchHeader*, const PowRow<float>*);
 template __global__ void k_short_pipe<24, 4>(const BatchHeader*, const PowRow<float>*);
 template __global__ void k_short_pipe<16, 4>(const BatchHeader*, const PowRow<float>*);
-template __global__ void k_short_pipe2<32, 3, true>(const BatchHeader*, const PowRow<float>*);
-template __global__ void k_short_pipe2<24, 4, true>(const BatchHeader*, const PowRow<float>*);
-template __global__ void k_short_pipe2<32, 4, true, true>(const BatchHeader*, const PowRow<float>*);
+template __global__ void k_short_pipe2<32, 3>(const BatchHeader*);
+template __global__ void k_short_pipe2<24, 4>(const BatchHeader*);
+template __global__ void k_short_pipe2<32, 4, true, true>(const BatchHeader*);
 
 template __global__ void k_short_packed<12, 4>(const BatchHeader*, const PowRow<float>*);
 template __global__ void k_short_packed<16, 3>(const BatchHeader*, const PowRow<float>*);
@@ -249,9 +264,9 @@ void launch_forward32_long(const BatchHeader* H, const void* pow, int grid, cuda
 void launch_forward32_long_pipe(int kind, const BatchHeader* H, const void* pow, int grid, cudaStream_t s) {
     const PowRow<float>* p = static_cast<const PowRow<float>*>(pow);
     if (kind == 5) k_forward_cluster<32, kClusterWarps, kClusterCtas><<<grid, kClusterWarps * 32, 0, s>>>(H, p);
-    else if (kind == 3) k_forward_serial<32, 3><<<grid, kSerialThreads, 0, s>>>(H, p);
-    else if (kind == 6 || kind == 7) k_forward_wave<32, 3><<<grid, kSerialThreads, 0, s>>>(H, p);
-    else if (kind == 8) k_forward_wave<16, 3><<<grid, kSerialThreads, 0, s>>>(H, p);
+    else if (kind == 3) k_forward_serial<32, 3><<<grid, kSerialThreads, 0, s>>>(H);
+    else if (kind == 6 || kind == 7) k_forward_wave<32, 3><<<grid, kSerialThreads, 0, s>>>(H);
+    else if (kind == 8) k_forward_wave<16, 3><<<grid, kSerialThreads, 0, s>>>(H);
     else if (kind == 4) k_forward_pipe<32, 4><<<grid, 4 * 32, 0, s>>>(H, p);
     else if (kind == 2) k_forward_pipe<24, kCtaWarps><<<grid, kCtaWarps * 32, 0, s>>>(H, p);
     else k_forward_pipe<32, kCtaWarpsPipe><<<grid, kCtaWarpsPipe * 32, 0, s>>>(H, p);
@@ -280,9 +295,9 @@ void launch_short_scalar(int id, const BatchHeader* H, const void* pow, int grid
     case 4: k_short_pipe<32, 3><<<grid, kShortThreads, 0, s>>>(H, p); break;
     case 5: k_short_pipe<24, 4><<<grid, kShortThreads, 0, s>>>(H, p); break;
     case 6: k_short_pipe<16, 4><<<grid, kShortThreads, 0, s>>>(H, p); break;
-    case 7: k_short_pipe2<32, 3, true><<<grid, kShortThreads, 0, s>>>(H, p); break;
-    case 8: k_short_pipe2<24, 4, true><<<grid, kShortThreads, 0, s>>>(H, p); break;
-    case 9: k_short_pipe2<32, 4, true, true><<<grid, kShortThreads, 0, s>>>(H, p); break;
+    case 7: k_short_pipe2<32, 3><<<grid, kShortThreads, 0, s>>>(H); break;
+    case 8: k_short_pipe2<24, 4><<<grid, kShortThreads, 0, s>>>(H); break;
+    case 9: k_short_pipe2<32, 4, true, true><<<grid, kShortThreads, 0, s>>>(H); break;
 
     default: k_short_scalar<32, 4><<<grid, kShortThreads, 0, s>>>(H, p); break;
     }
@@ -302,8 +317,8 @@ int occupancy_short_scalar(int id) {
     case 4: return occ_of(k_short_pipe<32, 3>);
     case 5: return occ_of(k_short_pipe<24, 4>);
     case 6: return occ_of(k_short_pipe<16, 4>);
-    case 7: return occ_of(k_short_pipe2<32, 3, true>);
-    case 8: return occ_of(k_short_pipe2<24, 4, true>);
+    case 7: return occ_of(k_short_pipe2<32, 3>);
+    case 8: return occ_of(k_short_pipe2<24, 4>);
     case 9: return occ_of(k_short_pipe2<32, 4, true, true>);
 
     default: return occ_of(k_short_scalar<32, 4>);

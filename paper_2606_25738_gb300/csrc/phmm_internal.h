@@ -51,11 +51,19 @@ struct alignas(16) Rec64J {
     uint64_t meta;
 };
 
+// Batch statistics for the skewed engines (prep; zeroed per launch).
+struct SkewStats {
+    uint32_t drop;               // bits * 64: largest -log2 h
+    uint32_t unused;
+    uint32_t gcp_max, gcp_inv;   // largest gcp Phred, largest 255 - gcp Phred
+};
+
 constexpr uint32_t META_CODE_MASK = 0x7u;
 constexpr int META_GCP_SHIFT = 8;
 constexpr uint32_t META_DEGEN = 1u << 16;  // 1 - g_i too small for the factored form
 constexpr uint32_t META_BAD = 1u << 17;    // invalid base or quality > 93
 
+constexpr uint32_t kWaveTags = 63;  // tags of the wave kind's boundary rows (skew.cuh)
 constexpr int kMaxPhred = 93;
 constexpr int kPhredTab = 96;  // table rows (>= kMaxPhred + 1)
 
@@ -189,6 +197,7 @@ struct BatchHeader {
     PairDesc *desc;
     Rec32 *rec32;
     Rec32J *rec32j;  // pipelined-engine records (nullptr when no kernel of the plan uses them)
+    SkewStats *skst;
     Rec64 *rec64;
     Rec64J *rec64j;  // FP64 pipelined-engine records (FP64 mode, variant 2; else nullptr)
     // plan
@@ -206,6 +215,8 @@ struct BatchHeader {
     unsigned long long *rbnd;   // rescue / single-launch scratch: 2 boundaries per CTA
     uint64_t rbnd_words_per_cta;
     float4 *wbnd;            // strips of the wave kind: each strip's right boundary (l rows)
+    uint64_t wbnd_rows;      // rows the buffer holds (k_reset clears it when the tags wrap)
+    uint32_t *wave_epoch;    // tag of this launch's boundary rows, 1 .. kWaveTags (k_prep32 steps it)
     float4 *sbnd;            // serial multi-warp pairs: 2 strip boundaries of sbnd_rows rows
     uint32_t sbnd_rows;      // per resident warp of k_forward_serial (not cleared)
     uint32_t sbnd_warps;     // warps the scratch holds (the kernel's grid x warps per CTA)

@@ -103,15 +103,21 @@ struct Plan {
 };
 
 // Cost model constants (issue slots): per lane and cell of a row, and per lane and row
-// (scan, shuffles, record loads, checkpoint share).
+// (scan, shuffles, record loads, checkpoint share); those of the skewed engine (cycles of a
+// scheduler: 330 a step of 32 columns a lane, 290 of 24), whose lanes start one row apart.
 constexpr double kCellCost = 8.0;
 constexpr double kRowCost = 70.0;
+struct TeamCost {
+    double cell = kCellCost, row = kRowCost;
+    bool skew = false;  // a team of G lanes takes l + G steps
+};
+constexpr TeamCost kSkewCost{5.0, 170.0, true};
 
 // Bin-pack teams (G lanes each) into 32-lane warp items within runs of similar row
 // count; a warp item runs the max row count of its teams.  Appends to `teams` / `items`.
 static void pack_teams(std::vector<Team>& run_teams, std::vector<uint32_t>& run_l,
                        std::vector<Team>& teams, std::vector<WarpItem>& items, double cell_w,
-                       double& cost) {
+                       double& cost, const TeamCost& tc = TeamCost()) {
     // order by l descending, then G descending
     std::vector<uint32_t> ord(run_teams.size());
     for (size_t q = 0; q < ord.size(); ++q) ord[q] = (uint32_t)q;
@@ -163,7 +169,7 @@ static void pack_teams(std::vector<Team>& run_teams, std::vector<uint32_t>& run_
             else nxt[bins[b].tail] = id;
             bins[b].tail = id;
             bins[b].rem -= G;
-            bins[b].lmax = std::max(bins[b].lmax, run_l[ord[q]]);
+            bins[b].lmax = std::max(bins[b].lmax, run_l[ord[q]] + (tc.skew ? G : 0u));
             if (bins[b].rem > 0) open[bins[b].rem].push_back(b);
         }
         for (auto& bn : bins) {
@@ -175,7 +181,7 @@ static void pack_teams(std::vector<Team>& run_teams, std::vector<uint32_t>& run_
                 w.n_teams++;
             }
             items.push_back(w);
-            cost += (double)bn.lmax * 32.0 * (cell_w * kCellCost + kRowCost);
+            cost += (double)bn.lmax * 32.0 * (cell_w * tc.cell + tc.row);
         }
         i = j;
     }
@@ -187,7 +193,8 @@ static void pack_teams(std::vector<Team>& run_teams, std::vector<uint32_t>& run_
 // CTA, packed best-fit into CTAs of CW warps (wider pairs: strips of CW warps).  Items
 // are ordered longest first.
 void make_plan(const uint32_t* l, const uint32_t* k, const uint32_t* pr, uint32_t n, int Ns, int NP,
-               int Nl, Plan& P, int kw = 4, int CW = kCtaWarps, bool serial = false, bool wave = false) {
+               int Nl, Plan& P, int kw = 4, int CW = kCtaWarps, bool serial = false, bool wave = false,
+               const TeamCost& tc = TeamCost()) {
     P = Plan();
     P.N = Ns;
     P.NP = NP;
@@ -240,7 +247,7 @@ void make_plan(const uint32_t* l, const uint32_t* k, const uint32_t* pr, uint32_
     for (const Team& t : pt)
         P.cells_br[1] += (uint64_t)l[t.pair] * k[t.pair] + (uint64_t)l[t.pair2] * k[t.pair2];
     for (uint32_t p : lo) P.cells_br[2] += (uint64_t)l[p] * k[p];
-    pack_teams(st, sl, P.teams, P.witems, (double)Ns, P.cost);
+    pack_teams(st, sl, P.teams, P.witems, (double)Ns, P.cost, tc);
     pack_teams(pt, pl, P.teams, P.witems2, 2.0 * NP * 1.2, P.cost);
     // long pairs
     P.n_long = (uint32_t)lo.size();
@@ -266,12 +273,12 @@ void make_plan(const uint32_t* l, const uint32_t* k, const uint32_t* pr, uint32_
     if (wave) {
         // one item per strip of 32 Nl columns, the pairs largest first and each pair's
         // strips in order, so a strip is always dequeued after the strip it waits for.
-        // Strip s writes its right boundary (l float4 rows) at wave row bnd_out and
-        // publishes its progress in boundary word `pad`; strip s + 1 reads both.
+        // Strip s writes its right boundary (l float4 rows) at wave row bnd_out, which strip
+        // s + 1 reads.
         for (uint32_t p : lo) {
             const uint32_t Wt = W_of(p);
             const uint32_t extra = n + P.n_extra;
-            const uint64_t r0 = P.wave_rows, w0 = P.bnd_words;
+            const uint64_t r0 = P.wave_rows;
             for (uint32_t stp = 0; stp < Wt; ++stp) {
                 CtaPair cp = cpair(p, 0, 1);
                 cp.strip = (uint16_t)stp;
@@ -280,7 +287,6 @@ void make_plan(const uint32_t* l, const uint32_t* k, const uint32_t* pr, uint32_
                 cp.extra_base = extra;
                 cp.bnd_in = stp > 0 ? r0 + (uint64_t)(stp - 1) * l[p] : kNoBnd;
                 cp.bnd_out = stp + 1 < Wt ? r0 + (uint64_t)stp * l[p] : kNoBnd;
-                cp.pad = (uint32_t)(w0 + stp);
                 CtaItem it;
                 it.first = (uint32_t)P.cpairs.size();
                 it.n = 1;
@@ -288,7 +294,6 @@ void make_plan(const uint32_t* l, const uint32_t* k, const uint32_t* pr, uint32_
                 P.citems.push_back(it);
             }
             P.wave_rows += (uint64_t)(Wt - 1) * l[p];
-            P.bnd_words += Wt;
             P.n_extra += Wt - 1;
             P.cost += (double)l[p] * Wt * 32.0 * (Nl * kCellCost + kRowCost);
         }
@@ -473,10 +478,11 @@ void build_pow_table(int N, std::vector<PowRow<T>>& out) {
 // ------------------------------------------------------------------------------------
 // Context
 // ------------------------------------------------------------------------------------
+constexpr size_t kSmallBytes = 128;
 struct Slot {
     DevBuf in_bases, in_bq, in_iq, in_dq, in_gq, in_hap, in_roff, in_hoff, in_pr, in_ph;
     DevBuf desc, rec32, rec32j, rec64, rec64j, teams, witems, witems2, cpairs, citems, parts, out, oflags, rescue;
-    DevBuf small;  // counters[8], status[1], dropgrow[4]
+    DevBuf small;  // counters[8], status[1], dropgrow[4], skew statistics [4], wave tag (kSmallBytes)
     DevBuf bnd;    // strip boundaries of the batch
     DevBuf rbnd;   // rescue / launch-per-pair boundary scratch
     DevBuf sbnd;   // serial multi-warp pairs: two boundaries per resident warp
@@ -589,8 +595,13 @@ uint64_t serial_bytes(const phmm_ctx* ctx, const Plan& P) {
 }
 cudaError_t ensure_serial(const phmm_ctx* ctx, Slot& S, const Plan& P) {
     if (kLongWave[P.long_kind]) {  // the wave kind's strip boundaries
+        // a new buffer holds no tag
         S.sbnd_warps = S.sbnd_rows = 0;
-        return ensure(S.wbnd, std::max<uint64_t>(P.wave_rows, 1) * sizeof(float4));
+        const void* before = S.wbnd.p;
+        const size_t cap = S.wbnd.cap;
+        const cudaError_t e = ensure(S.wbnd, std::max<uint64_t>(P.wave_rows, 1) * sizeof(float4));
+        if (e != cudaSuccess || (S.wbnd.p == before && S.wbnd.cap == cap)) return e;
+        return cudaMemsetAsync(S.wbnd.p, 0, S.wbnd.cap, ctx->copy_stream);
     }
     const uint64_t b = serial_bytes(ctx, P);
     if (b == 0) {
@@ -724,8 +735,20 @@ cudaError_t upload_plan(Slot& S, const Plan& P, cudaStream_t cs) {
 // kernel only; without them prep skips it and the batch needs no arena for it (an idle
 // arena up to kKeepRec32Bytes is kept).
 constexpr uint64_t kKeepRec32Bytes = 1ull << 30;
+// Likewise the J-form records (every other FP32 kernel).
+bool plan_needs_rec32j(const Plan& P) {
+    return (kShortScalarPipe[P.scal_id] && !P.witems.empty()) || (!P.citems.empty() && P.long_kind > 0);
+}
 bool plan_needs_rec32(const Plan& P) {
     return P.pack_id >= 0 || !kShortScalarPipe[P.scal_id] || (P.long_kind == 0 && !P.citems.empty());
+}
+
+// The arenas of the record layouts that an FP32 plan reads.
+cudaError_t ensure_records(Slot& S, const Plan& P, uint64_t nbases) {
+    cudaError_t e = cudaSuccess;
+    if (plan_needs_rec32(P)) e = ensure(S.rec32, nbases * sizeof(Rec32));
+    if (e == cudaSuccess && plan_needs_rec32j(P)) e = ensure(S.rec32j, nbases * sizeof(Rec32J));
+    return e;
 }
 
 void plan_header(const Slot& S, const Plan& P, BatchHeader& hh) {
@@ -744,7 +767,11 @@ void plan_header(const Slot& S, const Plan& P, BatchHeader& hh) {
     hh.sbnd_rows = S.sbnd_rows;
     hh.sbnd_warps = S.sbnd_warps;
     hh.wbnd = (float4*)S.wbnd.p;
-    if (hh.rec32 || hh.rec32j) hh.rec32 = plan_needs_rec32(P) ? (Rec32*)S.rec32.p : nullptr;
+    hh.wbnd_rows = S.wbnd.cap / sizeof(float4);
+    if (!P.fp64) {
+        hh.rec32 = plan_needs_rec32(P) ? (Rec32*)S.rec32.p : nullptr;
+        hh.rec32j = plan_needs_rec32j(P) ? (Rec32J*)S.rec32j.p : nullptr;
+    }
     // FP64 J-form records: only the pipelined FP64 variant reads them
     hh.rec64j = P.fp64 && f64_pipelined(P.scal_id) ? (Rec64J*)S.rec64j.p : nullptr;
 }
@@ -762,9 +789,14 @@ std::vector<std::pair<int, int>> fp32_candidates(const phmm_config& cfg) {
             if (v == 4 && !kShortScalarPipe[si]) continue;
             if (v == 5 && !kShortScalarHalves[si]) continue;
             if (v == 6 && !kShortScalarLean[si]) continue;
-            // the lean engine only when asked for: it measured 15% slower than the
-            // three-CTA halves engine on the short-read batch (L1 reads on every row)
+            // four CTAs per SM only when asked for: the same time on the short-read batch
             if (v != 6 && kShortScalarLean[si]) continue;
+            // left to itself the library runs the skewed engine: on 400 short-read regions 2.10 ms
+            // against 2.57 ms (pipelined), 2.73 ms (packed teams) and more (lean); on equal lengths
+            // of 32 to 1000 bp it is never slower than any of them.  Packed teams run when their
+            // width is asked for.
+            if (v == 0 && !kShortScalarHalves[si]) continue;
+            if (v == 0 && pi >= 0 && n != 12 && n != 16) continue;
             if ((n == 24 || n == 32 || n == 16) && scal_only && kShortScalarN[si] != n) continue;
             if ((n == 24 || n == 32) && !scal_only && kShortScalarN[si] != n) continue;
             if ((n == 12 || n == 16) && !scal_only && (pi < 0 || kShortPackedN[pi] != n)) continue;
@@ -812,7 +844,8 @@ void cluster_links(Plan& P) {
 void make_plan_id(const uint32_t* l, const uint32_t* k, const uint32_t* pr, uint32_t n, int scal_id,
                   int pack_id, int long_kind, Plan& P) {
     make_plan(l, k, pr, n, kShortScalarN[scal_id], pack_id >= 0 ? kShortPackedN[pack_id] : 0,
-              kLongN[long_kind], P, 4, kLongCW[long_kind], kLongSerial[long_kind], kLongWave[long_kind]);
+              kLongN[long_kind], P, 4, kLongCW[long_kind], kLongSerial[long_kind], kLongWave[long_kind],
+              kShortScalarHalves[scal_id] ? kSkewCost : TeamCost());
     if (long_kind == 5) cluster_links(P);
     P.scal_id = scal_id;
     P.pack_id = pack_id;
@@ -834,17 +867,20 @@ std::vector<int> long_kinds_of(const phmm_config& cfg) {
     if (cfg.flags & PHMM_F_LONG_WAVE) return {6, 7, 8};  // the wave kernels
     if (cfg.flags & PHMM_F_LONG_WAVE16) return {8};
     if (cfg.kernel_variant == 3) return {0};
-    return {0, 1, 3, 4, 5, 6, 7, 8};  // kind 2 only when forced: measured slower than kind 1 everywhere
+    // the kinds on the skewed engine; the others run only when forced (64 long-read pairs: wave
+    // kinds 27 to 40 ms, 4-warp strips and clusters over 120 ms; 60,000 uneven pairs: serial
+    // 22 ms, lean and 12-warp CTAs over 40 ms)
+    return {3, 6, 7, 8};
 }
 // Without measurement: the serial kind when multi-warp pairs outnumber the resident
 // warps of k_forward_serial four times over (each warp then has several pairs to run),
-// else the pipelined 12-warp kernel.
+// else the 512-column wave strips.
 int default_long_kind(const phmm_config& cfg, uint64_t n_long = 0, uint64_t serial_warps = 0) {
     const std::vector<int> k = long_kinds_of(cfg);
     if (k.size() == 1) return k[0];
     const bool serial_ok = std::find(k.begin(), k.end(), 3) != k.end();
     if (serial_ok && serial_warps > 0 && n_long >= 4 * serial_warps) return 3;
-    return std::find(k.begin(), k.end(), 1) != k.end() ? 1 : k[0];
+    return std::find(k.begin(), k.end(), 8) != k.end() ? 8 : k[0];
 }
 
 // Coarse shape of a batch for the tuner cache: pair count, mean read and haplotype
@@ -863,6 +899,37 @@ uint64_t batch_signature(const uint32_t* l, const uint32_t* k, const uint32_t* p
     return q(n) | (q(sl / std::max(n, 1u)) << 8) | (q(sk / std::max(n, 1u)) << 16) | (fs << 24) |
            ((uint64_t)cfg.precision << 32) | ((uint64_t)cfg.kernel_variant << 36) |
            ((uint64_t)cfg.cols_per_lane << 40);
+}
+
+// Upper bound of the device bytes of a batch with host inputs (phmm_batch_footprint).  The
+// wave kinds' boundaries have no term of their own: the kind chosen without measurement is
+// one whose plan fits (submit).
+uint64_t footprint_bound(const phmm_ctx* ctx, uint64_t nbases, uint64_t nhb, uint32_t nr, uint32_t nh, uint32_t np,
+                         const uint32_t* L, const uint32_t* K) {
+    const int prec = ctx->cfg.precision;
+    const bool need64 = prec != PHMM_PREC_FP32_ONLY;
+    const uint64_t seg = 32ull * (prec == PHMM_PREC_FP64 ? kN64 : kNLong32);
+    uint64_t f = nbases * 5 + nhb + (nr + 1) * 8ull + (nh + 1) * 8ull + np * 8ull;
+    f += nbases * ((prec != PHMM_PREC_FP64 ? sizeof(Rec32) + sizeof(Rec32J) : sizeof(Rec64J)) +
+                   (need64 ? sizeof(Rec64) : 0));
+    f += (uint64_t)np * (sizeof(PairDesc) + sizeof(Partial) + 8 + 1 + 4 + sizeof(Team) + 2 * sizeof(WarpItem) +
+                         sizeof(CtaPair) + sizeof(CtaItem));
+    uint64_t lmax = 0;
+    for (uint32_t p = 0; p < np; ++p) {
+        const uint64_t l = L[p], k = K[p];
+        lmax = std::max(lmax, l);
+        const uint64_t Wt = (k + seg - 1) / seg;
+        // the narrowest CTA strips of any FP32 multi-warp kind bound the boundary words
+        const uint64_t cw = prec == PHMM_PREC_FP64 ? (uint64_t)kCtaWarps : (uint64_t)kLongCW[4];
+        if (Wt > cw) {  // strips of a very wide pair
+            const uint64_t S = (Wt + cw - 1) / cw;
+            f += (S - 1) * (l * (prec == PHMM_PREC_FP64 ? 8 : 4) * 8 + sizeof(Partial) + sizeof(CtaPair) + sizeof(CtaItem));
+        }
+    }
+    if (need64) f += (uint64_t)ctx->sms * ctx->occ64 * 2 * lmax * 8 * 8 + 16;
+    if (prec != PHMM_PREC_FP64)  // serial multi-warp kind: two boundaries per resident warp
+        f += (uint64_t)ctx->sms * ctx->occ_longk[3] * (kSerialThreads / 32) * 2 * lmax * sizeof(float4);
+    return f;
 }
 
 constexpr uint64_t kTuneMinCells = 200000000ull;  // smaller batches keep the cost model's pick
@@ -995,8 +1062,8 @@ int phmm_create(const phmm_config* cfg, phmm_ctx** out) {
         cudaStream_t* sts[] = {&S.sm, &S.sb2, &S.sb3};
         for (auto* q : sts)
             if (cudaStreamCreateWithFlags(q, cudaStreamNonBlocking) != cudaSuccess) return fail(PHMM_ECUDA);
-        if (ensure(S.small, 64) != cudaSuccess || ensure(S.h_small, 64) != cudaSuccess ||
-            ensure(S.hdr, sizeof(BatchHeader)) != cudaSuccess)
+        if (ensure(S.small, kSmallBytes) != cudaSuccess || ensure(S.h_small, 64) != cudaSuccess ||
+            ensure(S.hdr, sizeof(BatchHeader)) != cudaSuccess || cudaMemset(S.small.p, 0, kSmallBytes) != cudaSuccess)
             return fail(PHMM_ECUDA);
     }
     if (cudaGetLastError() != cudaSuccess) return fail(PHMM_ECUDA);
@@ -1194,26 +1261,61 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
     }
     N = P.N;
     const auto th_plan = std::chrono::steady_clock::now();
-    // footprint and admission (lean records only for a plan that reads them, or for the
+    // footprint and admission (each record layout only for a plan that reads it, or for the
     // tuner's trials, which may)
     const bool need64 = ctx->cfg.precision != PHMM_PREC_FP32_ONLY;
-    const bool need32 = ctx->cfg.precision != PHMM_PREC_FP64 &&
-                        (tune_short || tune_long || plan_needs_rec32(P));
+    const bool fp32 = ctx->cfg.precision != PHMM_PREC_FP64;
+    bool need32 = false, need32j = false;
+    auto needs_of = [&](const Plan& Q) {
+        need32 |= fp32 && plan_needs_rec32(Q);
+        need32j |= fp32 && plan_needs_rec32j(Q);
+    };
     uint32_t lmax_b = 0;
     for (uint32_t p = 0; p < np; ++p) lmax_b = std::max(lmax_b, L[p]);
     const uint64_t rb_words = (uint64_t)lmax_b * 8;  // FP64 boundary: 8 words per row
     const int rescue_ctas = ctx->sms * ctx->occ64;
     const uint64_t rb_bytes = (uint64_t)rescue_ctas * 2 * rb_words * 8ull + 16;
-    const uint64_t foot = (dev_in ? 0 : nbases * 5 + nhb + (nr + 1) * 8ull + (nh + 1) * 8ull + np * 8ull) +
-                          (ctx->cfg.precision != PHMM_PREC_FP32_ONLY ? rb_bytes : 0) +
-                          np * (sizeof(PairDesc) + sizeof(Partial) + 8 + 1 + 4) +
-                          (ctx->cfg.precision == PHMM_PREC_FP64 ? 0 : nbases * sizeof(Rec32J)) +
-                          (need32 ? nbases * sizeof(Rec32) : 0) +
-                          (need64 ? nbases * sizeof(Rec64) : 0) +
-                          (ctx->cfg.precision == PHMM_PREC_FP64 ? nbases * sizeof(Rec64J) : 0) +
-                          P.teams.size() * sizeof(Team) + (P.witems.size() + P.witems2.size()) * sizeof(WarpItem) +
-                          P.cpairs.size() * sizeof(CtaPair) + P.citems.size() * sizeof(CtaItem) +
-                          P.bnd_words * 8ull + P.n_extra * sizeof(Partial) + serial_bytes(ctx, P);
+    auto foot_of = [&]() {
+        need32 = need32j = false;
+        needs_of(P);
+        Plan probe;  // the kernels that the tuner may try
+        probe.witems = P.witems;
+        if (tune_short)
+            for (auto& cd : tune_cand) {
+                probe.scal_id = cd.first;
+                probe.pack_id = cd.second;
+                needs_of(probe);
+            }
+        if (tune_long) {
+            probe.scal_id = P.scal_id;
+            probe.pack_id = P.pack_id;
+            probe.citems = P.citems;
+            for (int lk : long_kinds_of(ctx->cfg)) {
+                probe.long_kind = lk;
+                needs_of(probe);
+            }
+        }
+        return (dev_in ? 0 : nbases * 5 + nhb + (nr + 1) * 8ull + (nh + 1) * 8ull + np * 8ull) +
+               (ctx->cfg.precision != PHMM_PREC_FP32_ONLY ? rb_bytes : 0) +
+               np * (sizeof(PairDesc) + sizeof(Partial) + 8 + 1 + 4) + (need32j ? nbases * sizeof(Rec32J) : 0) +
+               (need32 ? nbases * sizeof(Rec32) : 0) +
+               (need64 ? nbases * sizeof(Rec64) : 0) + (fp32 ? 0 : nbases * sizeof(Rec64J)) +
+               P.teams.size() * sizeof(Team) + (P.witems.size() + P.witems2.size()) * sizeof(WarpItem) +
+               P.cpairs.size() * sizeof(CtaPair) + P.citems.size() * sizeof(CtaItem) + P.bnd_words * 8ull +
+               P.n_extra * sizeof(Partial) + serial_bytes(ctx, P);
+    };
+    uint64_t foot = foot_of();
+    // A wave kind that nobody asked for keeps within the bound that phmm_batch_footprint gives
+    // and the budget: else wider strips, else CTA strips.
+    if (!reuse && fp32 && kLongWave[P.long_kind] && long_kinds_of(ctx->cfg).size() > 1) {
+        const uint64_t most = std::min<uint64_t>(ctx->budget, footprint_bound(ctx, nbases, nhb, nr, nh, np, L.data(), K.data()));
+        for (int lk : {6, 1}) {
+            if (foot <= most) break;
+            const int si = P.scal_id, pi = P.pack_id;
+            make_plan_id(L.data(), K.data(), pr, np, si, pi, lk, P);
+            foot = foot_of();
+        }
+    }
     if (foot > ctx->budget) return PHMM_ENOMEM;
     if (foot + ctx->inflight_foot > ctx->budget) return PHMM_EBUSY;  // admissible once others retire
     {
@@ -1263,9 +1365,9 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
         // a large arena this plan does not read (e.g. left from the tuner's trials) goes
         // back; a small one stays, so that batches alternating between plans that read it
         // and plans that do not pay no cudaFree (a device-wide synchronisation) each time
-        if (need32) CK(ensure(S->rec32, nbases * sizeof(Rec32)));
-        else if (S->rec32.cap > kKeepRec32Bytes) release(S->rec32);
-        CK(ensure(S->rec32j, nbases * sizeof(Rec32J)));
+        if (!need32 && S->rec32.cap > kKeepRec32Bytes) release(S->rec32);
+        if (!need32j && S->rec32j.cap > kKeepRec32Bytes) release(S->rec32j);
+        CK(ensure_records(*S, P, nbases));
     }
     if (need64) CK(ensure(S->rec64, nbases * sizeof(Rec64)));
     if (ctx->cfg.precision == PHMM_PREC_FP64) CK(ensure(S->rec64j, nbases * sizeof(Rec64J)));
@@ -1286,8 +1388,6 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
     hh.n_haps = nh;
     hh.n_pairs = np;
     hh.desc = (PairDesc*)S->desc.p;
-    hh.rec32 = (Rec32*)S->rec32.p;
-    hh.rec32j = ctx->cfg.precision != PHMM_PREC_FP64 ? (Rec32J*)S->rec32j.p : nullptr;
     hh.rec64 = (Rec64*)S->rec64.p;
     plan_header(*S, P, hh);
     hh.n_partials = np + P.n_extra;
@@ -1305,6 +1405,8 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
     hh.counters = (uint32_t*)S->small.p;          // words 0..7
     hh.status = (uint32_t*)S->small.p + 8;        // word 8
     hh.dropgrow = (uint32_t*)S->small.p + 9;      // words 9 .. 12
+    hh.skst = (SkewStats*)((uint32_t*)S->small.p + 16);  // words 16 .. 19
+    hh.wave_epoch = (uint32_t*)S->small.p + 24;   // word 24 (kept between launches)
     hh.seed = ctx->seed;
     hh.mode = (uint32_t)ctx->cfg.precision;
     CK(cudaMemcpyAsync(S->hdr.p, &hh, sizeof(hh), cudaMemcpyHostToDevice, cs));
@@ -1398,6 +1500,7 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
             CK(ensure(S->parts, (np + c.n_extra) * sizeof(Partial)));
             CK(ensure(S->bnd, c.bnd_words * 8ull));
             CK(ensure_serial(ctx, *S, c));
+            CK(ensure_records(*S, c, nbases));
             hh.parts = (Partial*)S->parts.p;
             plan_header(*S, c, hh);
             CK(cudaMemcpyAsync(S->hdr.p, &hh, sizeof(hh), cudaMemcpyHostToDevice, cs));
@@ -1435,6 +1538,7 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
         CK(ensure(S->parts, (np + P.n_extra) * sizeof(Partial)));
         CK(ensure(S->bnd, P.bnd_words * 8ull));
         CK(ensure_serial(ctx, *S, P));
+        CK(ensure_records(*S, P, nbases));
         hh.parts = (Partial*)S->parts.p;
         plan_header(*S, P, hh);
         CK(cudaMemcpyAsync(S->hdr.p, &hh, sizeof(hh), cudaMemcpyHostToDevice, cs));
@@ -1553,33 +1657,13 @@ int phmm_batch_footprint(phmm_ctx* ctx, const phmm_batch* b, uint64_t* bytes) {
         if (roff[r + 1] <= roff[r] || roff[r + 1] - roff[r] > 0xffffffull) return PHMM_EINVAL;
     for (uint32_t h = 0; h < nh; ++h)
         if (hoff[h + 1] <= hoff[h] || hoff[h + 1] - hoff[h] > 0xffffffull) return PHMM_EINVAL;
-    const int prec = ctx->cfg.precision;
-    const bool need64 = prec != PHMM_PREC_FP32_ONLY;
-    const uint64_t nbases = roff[nr], nhb = hoff[nh];
-    const uint64_t seg = 32ull * (prec == PHMM_PREC_FP64 ? kN64 : kNLong32);
-    uint64_t f = nbases * 5 + nhb + (nr + 1) * 8ull + (nh + 1) * 8ull + np * 8ull;
-    f += nbases * ((prec != PHMM_PREC_FP64 ? sizeof(Rec32) + sizeof(Rec32J) : sizeof(Rec64J)) +
-                   (need64 ? sizeof(Rec64) : 0));
-    f += (uint64_t)np * (sizeof(PairDesc) + sizeof(Partial) + 8 + 1 + 4 + sizeof(Team) + 2 * sizeof(WarpItem) +
-                         sizeof(CtaPair) + sizeof(CtaItem));
-    uint64_t lmax = 0;
+    std::vector<uint32_t> L(np), K(np);
     for (uint32_t p = 0; p < np; ++p) {
         if (b->pair_read[p] >= nr || b->pair_hap[p] >= nh) return PHMM_EINVAL;
-        const uint64_t l = roff[b->pair_read[p] + 1] - roff[b->pair_read[p]];
-        const uint64_t k = hoff[b->pair_hap[p] + 1] - hoff[b->pair_hap[p]];
-        lmax = std::max(lmax, l);
-        const uint64_t Wt = (k + seg - 1) / seg;
-        // the narrowest CTA strips of any FP32 multi-warp kind bound the boundary words
-        const uint64_t cw = prec == PHMM_PREC_FP64 ? (uint64_t)kCtaWarps : (uint64_t)kLongCW[4];
-        if (Wt > cw) {  // strips of a very wide pair
-            const uint64_t S = (Wt + cw - 1) / cw;
-            f += (S - 1) * (l * (prec == PHMM_PREC_FP64 ? 8 : 4) * 8 + sizeof(Partial) + sizeof(CtaPair) + sizeof(CtaItem));
-        }
+        L[p] = (uint32_t)(roff[b->pair_read[p] + 1] - roff[b->pair_read[p]]);
+        K[p] = (uint32_t)(hoff[b->pair_hap[p] + 1] - hoff[b->pair_hap[p]]);
     }
-    if (need64) f += (uint64_t)ctx->sms * ctx->occ64 * 2 * lmax * 8 * 8 + 16;
-    if (prec != PHMM_PREC_FP64)  // serial multi-warp kind: two boundaries per resident warp
-        f += (uint64_t)ctx->sms * ctx->occ_longk[3] * (kSerialThreads / 32) * 2 * lmax * sizeof(float4);
-    *bytes = f;
+    *bytes = footprint_bound(ctx, roff[nr], hoff[nh], nr, nh, np, L.data(), K.data());
     return PHMM_OK;
 }
 
@@ -1715,15 +1799,13 @@ int phmm_plan_check(const uint32_t* l, const uint32_t* k, const uint32_t* pair_r
     struct StripSeen {
         uint32_t nstrip = 0, count = 0, extra_base = 0;
         std::vector<int64_t> col0, width, item, w0;
-        std::vector<uint64_t> bin, bout, pad;
+        std::vector<uint64_t> bin, bout;
     };
     std::map<uint32_t, StripSeen> strips;
     std::vector<std::pair<uint64_t, uint64_t>> bnd_ranges, extra_ranges;
     const bool serial = precision != PHMM_PREC_FP64 && kLongSerial[long_kind];
-    // wave kind: one strip per item on one warp; boundaries are float4 rows of wbnd and
-    // each strip's progress is boundary word `pad` (consecutive within a pair)
+    // wave kind: one strip per item on one warp; boundaries are float4 rows of wbnd
     const bool wave = precision != PHMM_PREC_FP64 && kLongWave[long_kind];
-    std::vector<std::pair<uint64_t, uint64_t>> prog_ranges;
     for (size_t it = 0; it < P.citems.size(); ++it) {
         const CtaItem& ci = P.citems[it];
         uint32_t used = 0;
@@ -1767,7 +1849,6 @@ int phmm_plan_check(const uint32_t* l, const uint32_t* k, const uint32_t* pair_r
                 sv.w0.assign(cp.nstrip, -1);
                 sv.bin.assign(cp.nstrip, 0);
                 sv.bout.assign(cp.nstrip, 0);
-                sv.pad.assign(cp.nstrip, 0);
             }
             if (wave && (ci.n != 1 || cp.W != 1 || cp.w0 != 0)) return fail(31);
             if (cp.nstrip != sv.nstrip || cp.extra_base != sv.extra_base || cp.strip >= sv.nstrip ||
@@ -1779,7 +1860,6 @@ int phmm_plan_check(const uint32_t* l, const uint32_t* k, const uint32_t* pair_r
             sv.w0[cp.strip] = cp.w0;
             sv.bin[cp.strip] = cp.bnd_in;
             sv.bout[cp.strip] = cp.bnd_out;
-            sv.pad[cp.strip] = cp.pad;
             sv.count++;
         }
     }
@@ -1809,7 +1889,6 @@ int phmm_plan_check(const uint32_t* l, const uint32_t* k, const uint32_t* pair_r
                 }
             }
             if (wave) {
-                if (sv.pad[st] != sv.pad[0] + st) return fail(32);
                 if (st + 1 < sv.nstrip) {
                     const uint64_t a = sv.bout[st], b = a + (uint64_t)l[p];
                     if (b > P.wave_rows) return fail(25);
@@ -1824,10 +1903,6 @@ int phmm_plan_check(const uint32_t* l, const uint32_t* k, const uint32_t* pair_r
             }
         }
         if ((uint64_t)warps != (k[p] + seg - 1) / seg) return fail(26);
-        if (wave) {
-            if (sv.pad[0] + sv.nstrip > P.bnd_words) return fail(32);
-            prog_ranges.push_back({sv.pad[0], sv.pad[0] + sv.nstrip});
-        }
         if (sv.extra_base < n || sv.extra_base + sv.nstrip - 1 > n + P.n_extra) return fail(27);
         extra_ranges.push_back({sv.extra_base, sv.extra_base + sv.nstrip - 1});
         seen[p]++;
@@ -1840,7 +1915,6 @@ int phmm_plan_check(const uint32_t* l, const uint32_t* k, const uint32_t* pair_r
         return true;
     };
     if (!disjoint(bnd_ranges)) return fail(28);
-    if (!disjoint(prog_ranges)) return fail(32);
     if (!disjoint(extra_ranges)) return fail(29);
     for (uint32_t p = 0; p < n; ++p)
         if (seen[p] != 1) return fail(30);

@@ -1,0 +1,68 @@
+"""The skewed FP32 engine (csrc/skew.cuh) at its edges, against the CPU oracle: reads of one
+row and around the team's and the strip's start and end (a lane starts one step after its
+left neighbour), widths around multiples of a lane and of a strip, gcp Phred 10 throughout
+(a constant of the code) and other or mixed values, insertion qualities that jump between rows.
+
+Tolerance: the library's own a-priori FP32 bound for the pair, (6.5 sqrt(16 l + 4 k) 2^-23 +
+8 l 2^-46) / ln 10, plus one rounding of log10 L.  No pair may need the FP64 pass."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2606_25738_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def phmm():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2606_25738_gb300 import phmm as P
+    return P
+
+
+def _pairs(shapes, gcp, ins, seed):
+    rng = np.random.default_rng(seed)
+    out = []
+    for l, k in shapes:
+        hap = rng.choice(list(b"ACGT"), size=max(k, l)).astype(np.uint8)
+        read = hap[:l].copy()
+        m = rng.random(l) < 0.02
+        read[m] = rng.choice(list(b"ACGTN"), size=int(m.sum()))
+        i = np.arange(l)
+        g = {"ten": 10, "other": 13, "mixed": i % 7 + 7}[gcp]
+        q = {"flat": 45, "jumps": i * 7 % 30 + 20}[ins]
+        out.append((read.tobytes(), hap[:k].tobytes(), rng.integers(8, 41, l), q, 44, g))
+    return W.from_strings(out)
+
+
+def _check(phmm, b, **kw):
+    with phmm.Context(precision="fp32", **kw) as ctx:
+        out, flags, rc, st = ctx.run(b)
+    ref = oracle.batch(b)
+    l, k = W.pair_lengths(b)
+    tol = (6.5 * np.sqrt(16.0 * l + 4.0 * k) * 2.0 ** -23 + 8.0 * l * 2.0 ** -46) / np.log(10.0) + np.abs(ref) * 2.0 ** -52
+    assert rc == 0 and not np.any(flags & 0x79)
+    assert np.all(np.abs(out - ref) <= tol), np.max(np.abs(out - ref) / tol)
+    return st
+
+
+@pytest.mark.parametrize("gcp,ins", [("ten", "flat"), ("ten", "jumps"), ("other", "jumps"), ("mixed", "flat")])
+@pytest.mark.parametrize("N,variant", [(32, "pipe2"), (24, "pipe2"), (32, "pipe2lean")])
+def test_short_teams(phmm, N, variant, gcp, ins):
+    w = 32 * N
+    shapes = [(1, 1), (1, w), (2, N), (2, N + 1), (3, 2 * N - 1), (31, w), (32, w - 1), (33, w), (34, w - N), (35, 5),
+              (64, N * 16), (65, N * 16 + 1), (150, 431), (151, 250), (300, w), (700, 3 * N)]
+    st = _check(phmm, _pairs(shapes, gcp, ins, 5), variant=variant, cols_per_lane=N)
+    assert st["short_kernel"] == {("pipe2", 32): 7, ("pipe2", 24): 8, ("pipe2lean", 32): 9}[variant, N]
+
+
+@pytest.mark.parametrize("gcp,ins", [("ten", "flat"), ("ten", "jumps"), ("other", "jumps"), ("mixed", "flat")])
+@pytest.mark.parametrize("kind", ["serial", "wave", "wave16"])
+def test_strips(phmm, kind, gcp, ins):
+    flag = {"serial": phmm.F_LONG_SERIAL, "wave": phmm.F_LONG_WAVE, "wave16": phmm.F_LONG_WAVE16}[kind]
+    shapes = [(1, 1025), (2, 1025), (3, 2048), (16, 2049), (17, 3072), (31, 1536), (32, 1537), (33, 4097), (34, 2080),
+              (63, 5000), (64, 1100), (65, 3000), (96, 1056), (97, 1057), (400, 7000), (1500, 1100), (2000, 4100)]
+    st = _check(phmm, _pairs(shapes, gcp, ins, 6), flags=flag)
+    assert st["long_kernel"] in {"serial": (3,), "wave": (6, 7, 8), "wave16": (8,)}[kind]
