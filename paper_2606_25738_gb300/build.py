@@ -14,7 +14,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIBDIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(LIBDIR, "libphmm.so")
-SOURCES = ["kernels_f32.cu", "kernels_f64.cu", "runtime.cu", "noalloc.cu", "serve.cpp"]
+SOURCES = ["kernels_f32.cu", "kernels_f64.cu", "planner.cu", "runtime.cu", "noalloc.cu", "serve.cpp"]
 CPU_SOURCE = "cpu_rowwise.c"
 CPU_DEPS = ["cpu_rowwise.c", "cpu_engine.inc"]
 CPU_LIB = os.path.join(LIBDIR, "libphmm_cpu.so")

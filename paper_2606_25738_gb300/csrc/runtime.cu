@@ -17,6 +17,7 @@
 #include "launch.h"
 #include "phmm.h"
 #include "phmm_internal.h"
+#include "planner.cuh"
 
 using namespace phmm;
 
@@ -100,6 +101,14 @@ struct Plan {
     uint64_t wave_rows = 0;   // long kind 6: boundary rows of all strips (float4 each)
     uint64_t cells_br[3] = {0, 0, 0};  // cells of the scalar, packed and multi-warp branches
     bool fp64 = false;        // an FP64 plan (scal_id = the FP64 variant)
+    // A plan that the device builds (planner.cuh): its arrays are empty here, their sizes (an
+    // upper bound for the warp items) below.
+    bool dev = false;
+    uint64_t d_teams = 0, d_items = 0;  // short teams; strip items (= CTA pairs)
+    uint64_t n_teams() const { return dev ? d_teams : teams.size(); }
+    uint64_t n_witems() const { return dev ? d_teams : witems.size(); }
+    uint64_t n_cpairs() const { return dev ? d_items : cpairs.size(); }
+    uint64_t n_citems() const { return dev ? d_items : citems.size(); }
 };
 
 // Cost model constants (issue slots): per lane and cell of a row, and per lane and row
@@ -487,9 +496,10 @@ struct Slot {
     DevBuf rbnd;   // rescue / launch-per-pair boundary scratch
     DevBuf sbnd;   // serial multi-warp pairs: two boundaries per resident warp
     DevBuf wbnd;   // wave multi-warp pairs: each strip's right boundary
+    DevBuf pscan, pscratch;  // device planner: PlanScan, its scratch
     uint32_t sbnd_warps = 0, sbnd_rows = 0;  // what sbnd holds for the current plan
     DevBuf hdr;
-    HostBuf h_out, h_oflags, h_small, h_roff, h_hoff, h_pr, h_ph;
+    HostBuf h_out, h_oflags, h_small, h_roff, h_hoff, h_pr, h_ph, h_pscan;
     BatchHeader hh;
     cudaEvent_t ev_copy = nullptr, ev_start = nullptr, ev_fwd0 = nullptr, ev_fwd1 = nullptr,
                 ev_res0 = nullptr, ev_res1 = nullptr, ev_end = nullptr;
@@ -569,7 +579,7 @@ DevBuf* arena_bufs(Slot& S, int i) {
     DevBuf* d[] = {&S.in_bases, &S.in_bq, &S.in_iq, &S.in_dq, &S.in_gq, &S.in_hap, &S.in_roff, &S.in_hoff,
                    &S.in_pr, &S.in_ph, &S.desc, &S.rec32, &S.rec32j, &S.rec64, &S.rec64j, &S.teams, &S.witems, &S.witems2,
                    &S.cpairs, &S.citems, &S.parts, &S.out, &S.oflags, &S.rescue, &S.bnd, &S.rbnd, &S.sbnd,
-                   &S.wbnd};
+                   &S.wbnd, &S.pscan, &S.pscratch};
     return i < (int)(sizeof(d) / sizeof(d[0])) ? d[i] : nullptr;
 }
 
@@ -589,7 +599,7 @@ void release_arenas(Slot& S) {
 // for every warp of k_forward_serial's grid.
 uint64_t serial_bytes(const phmm_ctx* ctx, const Plan& P) {
     if (kLongWave[P.long_kind]) return P.wave_rows * sizeof(float4);
-    if (!kLongSerial[P.long_kind] || P.citems.empty()) return 0;
+    if (!kLongSerial[P.long_kind] || P.n_citems() == 0) return 0;
     const uint64_t warps = (uint64_t)ctx->sms * ctx->occ_longk[P.long_kind] * (kSerialThreads / 32);
     return warps * 2 * P.serial_rows * sizeof(float4);
 }
@@ -715,11 +725,12 @@ uint64_t u64(const void* p) { return (uint64_t)(uintptr_t)p; }
 // Copies a plan's arrays into the slot's device arenas (growing them as needed).
 cudaError_t upload_plan(Slot& S, const Plan& P, cudaStream_t cs) {
     cudaError_t e;
-    if ((e = ensure(S.teams, P.teams.size() * sizeof(Team))) != cudaSuccess) return e;
-    if ((e = ensure(S.witems, P.witems.size() * sizeof(WarpItem))) != cudaSuccess) return e;
+    if ((e = ensure(S.teams, P.n_teams() * sizeof(Team))) != cudaSuccess) return e;
+    if ((e = ensure(S.witems, P.n_witems() * sizeof(WarpItem))) != cudaSuccess) return e;
     if ((e = ensure(S.witems2, P.witems2.size() * sizeof(WarpItem))) != cudaSuccess) return e;
-    if ((e = ensure(S.cpairs, P.cpairs.size() * sizeof(CtaPair))) != cudaSuccess) return e;
-    if ((e = ensure(S.citems, P.citems.size() * sizeof(CtaItem))) != cudaSuccess) return e;
+    if ((e = ensure(S.cpairs, P.n_cpairs() * sizeof(CtaPair))) != cudaSuccess) return e;
+    if ((e = ensure(S.citems, P.n_citems() * sizeof(CtaItem))) != cudaSuccess) return e;
+    if (P.dev) return cudaSuccess;  // build_plan, once the header is there
     auto cp = [&](DevBuf& d, const void* src, size_t n) {
         return n ? cudaMemcpyAsync(d.p, src, n, cudaMemcpyHostToDevice, cs) : cudaSuccess;
     };
@@ -737,10 +748,10 @@ cudaError_t upload_plan(Slot& S, const Plan& P, cudaStream_t cs) {
 constexpr uint64_t kKeepRec32Bytes = 1ull << 30;
 // Likewise the J-form records (every other FP32 kernel).
 bool plan_needs_rec32j(const Plan& P) {
-    return (kShortScalarPipe[P.scal_id] && !P.witems.empty()) || (!P.citems.empty() && P.long_kind > 0);
+    return (kShortScalarPipe[P.scal_id] && P.n_witems() > 0) || (P.n_citems() > 0 && P.long_kind > 0);
 }
 bool plan_needs_rec32(const Plan& P) {
-    return P.pack_id >= 0 || !kShortScalarPipe[P.scal_id] || (P.long_kind == 0 && !P.citems.empty());
+    return P.pack_id >= 0 || !kShortScalarPipe[P.scal_id] || (P.long_kind == 0 && P.n_citems() > 0);
 }
 
 // The arenas of the record layouts that an FP32 plan reads.
@@ -758,8 +769,8 @@ void plan_header(const Slot& S, const Plan& P, BatchHeader& hh) {
     hh.teams = (const Team*)S.teams.p;
     hh.citems = (const CtaItem*)S.citems.p;
     hh.cpairs = (const CtaPair*)S.cpairs.p;
-    hh.n_witems = (uint32_t)P.witems.size();
-    hh.n_citems = (uint32_t)P.citems.size();
+    hh.n_witems = (uint32_t)P.witems.size();  // a device-built plan's: written by its last kernel but two
+    hh.n_citems = (uint32_t)P.n_citems();
     hh.n_partials = hh.n_pairs + P.n_extra;
     hh.bnd = (unsigned long long*)S.bnd.p;
     hh.n_bnd_words = P.bnd_words;
@@ -774,6 +785,24 @@ void plan_header(const Slot& S, const Plan& P, BatchHeader& hh) {
     }
     // FP64 J-form records: only the pipelined FP64 variant reads them
     hh.rec64j = P.fp64 && f64_pipelined(P.scal_id) ? (Rec64J*)S.rec64j.p : nullptr;
+}
+
+// Runs the device planner for plan P (its header is in place).
+cudaError_t build_plan(Slot& S, const Plan& P, const PlanInput& in, int sms, cudaStream_t cs) {
+    cudaError_t e = ensure(S.pscratch, plan_scratch_bytes(in.n_pairs));
+    if (e != cudaSuccess) return e;
+    PlanOutput o;
+    o.N = P.N;
+    o.Nl = kLongN[P.long_kind];
+    o.wave = kLongWave[P.long_kind] ? 1 : 0;
+    o.teams = (Team*)S.teams.p;
+    o.witems = (WarpItem*)S.witems.p;
+    o.cpairs = (CtaPair*)S.cpairs.p;
+    o.citems = (CtaItem*)S.citems.p;
+    o.H = (BatchHeader*)S.hdr.p;
+    o.scratch = S.pscratch.p;
+    launch_plan_build(in, o, sms, cs);
+    return cudaGetLastError();
 }
 
 // FP32 short-pair kernel candidates (scalar id, packed id or -1) allowed by the config.
@@ -872,6 +901,17 @@ std::vector<int> long_kinds_of(const phmm_config& cfg) {
     // 22 ms, lean and 12-warp CTAs over 40 ms)
     return {3, 6, 7, 8};
 }
+// Batches of at least this many pairs are planned on the device (when every kernel that may
+// run is on the skewed engines).
+constexpr uint32_t kDevPlanPairs = 4096;
+bool plans_on_device(const phmm_config& cfg, uint32_t np) {
+    if (cfg.precision == PHMM_PREC_FP64 || np < kDevPlanPairs) return false;
+    for (const auto& cd : fp32_candidates(cfg))
+        if (!kShortScalarHalves[cd.first] || cd.second >= 0) return false;
+    for (int lk : long_kinds_of(cfg))
+        if (!kLongSerial[lk] && !kLongWave[lk]) return false;
+    return true;
+}
 // Without measurement: the serial kind when multi-warp pairs outnumber the resident
 // warps of k_forward_serial four times over (each warp then has several pairs to run),
 // else the 512-column wave strips.
@@ -885,6 +925,13 @@ int default_long_kind(const phmm_config& cfg, uint64_t n_long = 0, uint64_t seri
 
 // Coarse shape of a batch for the tuner cache: pair count, mean read and haplotype
 // lengths (quarter-octave buckets), share of pairs whose read has other pairs.
+uint64_t batch_signature(double sl, double sk, uint32_t shared, uint32_t n, const phmm_config& cfg) {
+    auto q = [](double x) { return (uint64_t)std::max(0.0, std::floor(4.0 * std::log2(std::max(x, 1.0)))); };
+    const uint64_t fs = n ? (uint64_t)(8.0 * shared / n) : 0;
+    return q(n) | (q(sl / std::max(n, 1u)) << 8) | (q(sk / std::max(n, 1u)) << 16) | (fs << 24) |
+           ((uint64_t)cfg.precision << 32) | ((uint64_t)cfg.kernel_variant << 36) |
+           ((uint64_t)cfg.cols_per_lane << 40);
+}
 uint64_t batch_signature(const uint32_t* l, const uint32_t* k, const uint32_t* pr, uint32_t n,
                          const phmm_config& cfg) {
     double sl = 0, sk = 0;
@@ -894,42 +941,66 @@ uint64_t batch_signature(const uint32_t* l, const uint32_t* k, const uint32_t* p
         sk += k[p];
         if ((p > 0 && pr[p - 1] == pr[p]) || (p + 1 < n && pr[p + 1] == pr[p])) shared++;
     }
-    auto q = [](double x) { return (uint64_t)std::max(0.0, std::floor(4.0 * std::log2(std::max(x, 1.0)))); };
-    const uint64_t fs = n ? (uint64_t)(8.0 * shared / n) : 0;
-    return q(n) | (q(sl / std::max(n, 1u)) << 8) | (q(sk / std::max(n, 1u)) << 16) | (fs << 24) |
-           ((uint64_t)cfg.precision << 32) | ((uint64_t)cfg.kernel_variant << 36) |
-           ((uint64_t)cfg.cols_per_lane << 40);
+    return batch_signature(sl, sk, shared, n, cfg);
+}
+
+// A plan of the device planner: what the host knows of it (PlanScan).
+void dev_plan(const PlanScan& sc, uint32_t np, int scal_id, int long_kind, Plan& P) {
+    P = Plan();
+    const int w = kShortScalarN[scal_id] == 24 ? 1 : 0, z = kLongN[long_kind] == 16 ? 1 : 0;
+    P.dev = true;
+    P.N = kShortScalarN[scal_id];
+    P.scal_id = scal_id;
+    P.pack_id = -1;
+    P.long_kind = long_kind;
+    P.n_long = sc.n_long[w];
+    P.d_teams = np - sc.n_long[w];
+    P.d_items = kLongWave[long_kind] ? sc.strips[w][z] : sc.n_long[w];
+    P.n_extra = (uint32_t)(sc.strips[w][z] - sc.n_long[w]);
+    P.wave_rows = kLongWave[long_kind] ? sc.rows[w][z] : 0;
+    P.serial_rows = kLongSerial[long_kind] ? sc.lmax_long[w] : 0;
+    P.cells_br[0] = sc.short_cells[w];
+    P.cells_br[2] = sc.cells - sc.short_cells[w];
 }
 
 // Upper bound of the device bytes of a batch with host inputs (phmm_batch_footprint).  The
 // wave kinds' boundaries have no term of their own: the kind chosen without measurement is
 // one whose plan fits (submit).
-uint64_t footprint_bound(const phmm_ctx* ctx, uint64_t nbases, uint64_t nhb, uint32_t nr, uint32_t nh, uint32_t np,
-                         const uint32_t* L, const uint32_t* K) {
+struct FootSums {
+    uint64_t nbases, nhb;
+    uint32_t nr, nh, np;
+    uint64_t lmax = 0, rows = 0, strips = 0;  // longest read; sums over strips 1.. of CTA strips: l, 1
+};
+uint64_t footprint_bound(const phmm_ctx* ctx, const FootSums& q) {
     const int prec = ctx->cfg.precision;
     const bool need64 = prec != PHMM_PREC_FP32_ONLY;
-    const uint64_t seg = 32ull * (prec == PHMM_PREC_FP64 ? kN64 : kNLong32);
-    uint64_t f = nbases * 5 + nhb + (nr + 1) * 8ull + (nh + 1) * 8ull + np * 8ull;
-    f += nbases * ((prec != PHMM_PREC_FP64 ? sizeof(Rec32) + sizeof(Rec32J) : sizeof(Rec64J)) +
-                   (need64 ? sizeof(Rec64) : 0));
-    f += (uint64_t)np * (sizeof(PairDesc) + sizeof(Partial) + 8 + 1 + 4 + sizeof(Team) + 2 * sizeof(WarpItem) +
-                         sizeof(CtaPair) + sizeof(CtaItem));
-    uint64_t lmax = 0;
+    uint64_t f = q.nbases * 5 + q.nhb + (q.nr + 1) * 8ull + (q.nh + 1) * 8ull + q.np * 8ull;
+    f += q.nbases * ((prec != PHMM_PREC_FP64 ? sizeof(Rec32) + sizeof(Rec32J) : sizeof(Rec64J)) +
+                     (need64 ? sizeof(Rec64) : 0));
+    f += (uint64_t)q.np * (sizeof(PairDesc) + sizeof(Partial) + 8 + 1 + 4 + sizeof(Team) + 2 * sizeof(WarpItem) +
+                           sizeof(CtaPair) + sizeof(CtaItem));
+    f += q.rows * (prec == PHMM_PREC_FP64 ? 8 : 4) * 8 + q.strips * (sizeof(Partial) + sizeof(CtaPair) + sizeof(CtaItem));
+    if (need64) f += (uint64_t)ctx->sms * ctx->occ64 * 2 * q.lmax * 8 * 8 + 16;
+    if (prec != PHMM_PREC_FP64)  // serial multi-warp kind: two boundaries per resident warp
+        f += (uint64_t)ctx->sms * ctx->occ_longk[3] * (kSerialThreads / 32) * 2 * q.lmax * sizeof(float4);
+    return f;
+}
+uint64_t footprint_bound(const phmm_ctx* ctx, uint64_t nbases, uint64_t nhb, uint32_t nr, uint32_t nh, uint32_t np,
+                         const uint32_t* L, const uint32_t* K) {
+    FootSums q{nbases, nhb, nr, nh, np};
+    const uint64_t seg = 32ull * (ctx->cfg.precision == PHMM_PREC_FP64 ? kN64 : kNLong32);
+    // the narrowest CTA strips of any FP32 multi-warp kind bound the boundary words
+    const uint64_t cw = ctx->cfg.precision == PHMM_PREC_FP64 ? (uint64_t)kCtaWarps : (uint64_t)kLongCW[4];
     for (uint32_t p = 0; p < np; ++p) {
-        const uint64_t l = L[p], k = K[p];
-        lmax = std::max(lmax, l);
-        const uint64_t Wt = (k + seg - 1) / seg;
-        // the narrowest CTA strips of any FP32 multi-warp kind bound the boundary words
-        const uint64_t cw = prec == PHMM_PREC_FP64 ? (uint64_t)kCtaWarps : (uint64_t)kLongCW[4];
+        q.lmax = std::max<uint64_t>(q.lmax, L[p]);
+        const uint64_t Wt = (K[p] + seg - 1) / seg;
         if (Wt > cw) {  // strips of a very wide pair
             const uint64_t S = (Wt + cw - 1) / cw;
-            f += (S - 1) * (l * (prec == PHMM_PREC_FP64 ? 8 : 4) * 8 + sizeof(Partial) + sizeof(CtaPair) + sizeof(CtaItem));
+            q.rows += (S - 1) * L[p];
+            q.strips += S - 1;
         }
     }
-    if (need64) f += (uint64_t)ctx->sms * ctx->occ64 * 2 * lmax * 8 * 8 + 16;
-    if (prec != PHMM_PREC_FP64)  // serial multi-warp kind: two boundaries per resident warp
-        f += (uint64_t)ctx->sms * ctx->occ_longk[3] * (kSerialThreads / 32) * 2 * lmax * sizeof(float4);
-    return f;
+    return footprint_bound(ctx, q);
 }
 
 constexpr uint64_t kTuneMinCells = 200000000ull;  // smaller batches keep the cost model's pick
@@ -1085,9 +1156,10 @@ void phmm_destroy(phmm_ctx* ctx) {
         DevBuf* d[] = {&S.in_bases, &S.in_bq, &S.in_iq, &S.in_dq, &S.in_gq, &S.in_hap, &S.in_roff,
                        &S.in_hoff, &S.in_pr, &S.in_ph, &S.desc, &S.rec32, &S.rec32j, &S.rec64, &S.rec64j, &S.teams,
                        &S.witems, &S.witems2, &S.cpairs, &S.citems, &S.parts, &S.out, &S.oflags, &S.rescue,
-                       &S.small, &S.hdr, &S.bnd, &S.rbnd, &S.sbnd, &S.wbnd};
+                       &S.small, &S.hdr, &S.bnd, &S.rbnd, &S.sbnd, &S.wbnd,
+                       &S.pscan, &S.pscratch};
         for (auto* b : d) release(*b);
-        HostBuf* h[] = {&S.h_out, &S.h_oflags, &S.h_small, &S.h_roff, &S.h_hoff, &S.h_pr, &S.h_ph};
+        HostBuf* h[] = {&S.h_out, &S.h_oflags, &S.h_small, &S.h_roff, &S.h_hoff, &S.h_pr, &S.h_ph, &S.h_pscan};
         for (auto* b : h) release(*b);
         cudaEvent_t evs[] = {S.ev_copy, S.ev_start, S.ev_fwd0, S.ev_fwd1, S.ev_res0, S.ev_res1, S.ev_end,
                              S.ev_br[0], S.ev_br[1], S.ev_br[2], S.ev_br[3], S.ev_br[4], S.ev_br[5]};
@@ -1143,28 +1215,61 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
     // host views of offsets and the pair index
     const uint64_t *roff = b->read_off, *hoff = b->hap_off;
     const uint32_t *pr = b->pair_read, *ph = b->pair_hap;
+    cudaStream_t cs = ctx->copy_stream;
+    const bool on_dev = plans_on_device(ctx->cfg, np);
+    PlanInput pin{};
+    PlanScan sc{};
     if (dev_in && np > 0) {
         // device inputs are produced on the caller's stream: read them after its pending work
         CK(cudaEventRecord(S->ev_user, ctx->stream));
-        CK(cudaStreamWaitEvent(ctx->copy_stream, S->ev_user, 0));
+        CK(cudaStreamWaitEvent(cs, S->ev_user, 0));
+    }
+    if (on_dev) {
+        // device planner: the lengths are checked and summed there
+        if (!dev_in) {
+            CK(ensure(S->in_roff, (nr + 1) * 8ull));
+            CK(ensure(S->in_hoff, (nh + 1) * 8ull));
+            CK(ensure(S->in_pr, np * 4ull));
+            CK(ensure(S->in_ph, np * 4ull));
+            CK(cudaMemcpyAsync(S->in_roff.p, roff, (nr + 1) * 8ull, cudaMemcpyHostToDevice, cs));
+            CK(cudaMemcpyAsync(S->in_hoff.p, hoff, (nh + 1) * 8ull, cudaMemcpyHostToDevice, cs));
+            CK(cudaMemcpyAsync(S->in_pr.p, pr, np * 4ull, cudaMemcpyHostToDevice, cs));
+            CK(cudaMemcpyAsync(S->in_ph.p, ph, np * 4ull, cudaMemcpyHostToDevice, cs));
+        }
+        pin.read_off = dev_in ? roff : static_cast<const uint64_t*>(S->in_roff.p);
+        pin.hap_off = dev_in ? hoff : static_cast<const uint64_t*>(S->in_hoff.p);
+        pin.pair_read = dev_in ? pr : static_cast<const uint32_t*>(S->in_pr.p);
+        pin.pair_hap = dev_in ? ph : static_cast<const uint32_t*>(S->in_ph.p);
+        pin.n_reads = nr;
+        pin.n_haps = nh;
+        pin.n_pairs = np;
+        CK(ensure(S->pscan, sizeof(PlanScan)));
+        CK(ensure(S->h_pscan, sizeof(PlanScan)));
+        launch_plan_scan(pin, static_cast<PlanScan*>(S->pscan.p), ctx->sms, cs);
+        CK(cudaGetLastError());
+        CK(cudaMemcpyAsync(S->h_pscan.p, S->pscan.p, sizeof(PlanScan), cudaMemcpyDeviceToHost, cs));
+        CK(cudaStreamSynchronize(cs));
+        sc = *static_cast<const PlanScan*>(S->h_pscan.p);
+        if (sc.bad) return PHMM_EINVAL;
+    } else if (dev_in && np > 0) {
         CK(ensure(S->h_roff, (nr + 1) * 8ull));
         CK(ensure(S->h_hoff, (nh + 1) * 8ull));
         CK(ensure(S->h_pr, np * 4ull));
         CK(ensure(S->h_ph, np * 4ull));
-        CK(cudaMemcpyAsync(S->h_roff.p, b->read_off, (nr + 1) * 8ull, cudaMemcpyDeviceToHost, ctx->copy_stream));
-        CK(cudaMemcpyAsync(S->h_hoff.p, b->hap_off, (nh + 1) * 8ull, cudaMemcpyDeviceToHost, ctx->copy_stream));
-        CK(cudaMemcpyAsync(S->h_pr.p, b->pair_read, np * 4ull, cudaMemcpyDeviceToHost, ctx->copy_stream));
-        CK(cudaMemcpyAsync(S->h_ph.p, b->pair_hap, np * 4ull, cudaMemcpyDeviceToHost, ctx->copy_stream));
-        CK(cudaStreamSynchronize(ctx->copy_stream));
+        CK(cudaMemcpyAsync(S->h_roff.p, b->read_off, (nr + 1) * 8ull, cudaMemcpyDeviceToHost, cs));
+        CK(cudaMemcpyAsync(S->h_hoff.p, b->hap_off, (nh + 1) * 8ull, cudaMemcpyDeviceToHost, cs));
+        CK(cudaMemcpyAsync(S->h_pr.p, b->pair_read, np * 4ull, cudaMemcpyDeviceToHost, cs));
+        CK(cudaMemcpyAsync(S->h_ph.p, b->pair_hap, np * 4ull, cudaMemcpyDeviceToHost, cs));
+        CK(cudaStreamSynchronize(cs));
         roff = static_cast<const uint64_t*>(S->h_roff.p);
         hoff = static_cast<const uint64_t*>(S->h_hoff.p);
         pr = static_cast<const uint32_t*>(S->h_pr.p);
         ph = static_cast<const uint32_t*>(S->h_ph.p);
     }
     // validation: offsets non-decreasing with lengths >= 1, indices in range
-    std::vector<uint32_t> L(np), K(np);
-    uint64_t cells = 0;
-    if (np > 0) {
+    std::vector<uint32_t> L(on_dev ? 0 : np), K(on_dev ? 0 : np);
+    uint64_t cells = sc.cells;
+    if (np > 0 && !on_dev) {
         if (roff[0] != 0 || hoff[0] != 0) return PHMM_EINVAL;
         for (uint32_t r = 0; r < nr; ++r)
             if (roff[r + 1] <= roff[r] || roff[r + 1] - roff[r] > 0xffffffull) return PHMM_EINVAL;
@@ -1177,12 +1282,13 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
             cells += (uint64_t)L[p] * K[p];
         }
     }
-    const uint64_t nbases = np > 0 ? roff[nr] : 0, nhb = np > 0 ? hoff[nh] : 0;
+    const uint64_t nbases = on_dev ? sc.n_read_bases : np > 0 ? roff[nr] : 0;
+    const uint64_t nhb = on_dev ? sc.n_hap_bases : np > 0 ? hoff[nh] : 0;
     // plan (FP32: packed short width from the config or the cost model; FP64: kN64).
     // A batch with the same pair lengths as this slot's previous one reuses its plan.
     const auto th0 = std::chrono::steady_clock::now();
     uint64_t hsh = 1469598103934665603ull ^ ((uint64_t)ctx->cfg.precision << 32) ^ (uint64_t)ctx->cfg.cols_per_lane ^ ((uint64_t)ctx->cfg.kernel_variant << 40);
-    for (uint32_t p = 0; p < np; ++p) {
+    for (uint32_t p = 0; p < np && !on_dev; ++p) {
         hsh = (hsh ^ ((uint64_t)L[p] << 24 ^ K[p])) * 1099511628211ull;
     }
     hsh ^= np;
@@ -1191,7 +1297,12 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
     bool tune_short = false, tune_long = false, tune64 = false;
     uint64_t tune_sig = 0;
     std::vector<std::pair<int, int>> tune_cand;
-    const bool reuse = S->plan_valid && S->plan_hash == hsh && S->plan_np == np;
+    const bool reuse = !on_dev && S->plan_valid && S->plan_hash == hsh && S->plan_np == np;
+    // FP32 plan of given kernels, on the host or (its sizes) for the device planner
+    auto plan_of = [&](int si, int pi, int lk, Plan& Q) {
+        if (on_dev) dev_plan(sc, np, si, lk, Q);
+        else make_plan_id(L.data(), K.data(), pr, np, si, pi, lk, Q);
+    };
     if (!reuse) {
         if (ctx->cfg.precision == PHMM_PREC_FP64) {
             // FP64 variant: cached choice for this batch shape, else the cost model's (the
@@ -1221,21 +1332,24 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
             }
         } else {
             const std::vector<std::pair<int, int>> cand = fp32_candidates(ctx->cfg);
-            const uint64_t sig = batch_signature(L.data(), K.data(), pr, np, ctx->cfg);
+            const uint64_t sig = on_dev ? batch_signature((double)sc.sum_l, (double)sc.sum_k, sc.shared, np, ctx->cfg)
+                                        : batch_signature(L.data(), K.data(), pr, np, ctx->cfg);
             auto hit = ctx->tuned.find(sig);
             if (hit != ctx->tuned.end()) {
-                make_plan_id(L.data(), K.data(), pr, np, hit->second[0], hit->second[1], hit->second[2], P);
+                plan_of(hit->second[0], hit->second[1], hit->second[2], P);
             } else {
                 // cost-model choice first; measured tuning (below) may replace it
-                uint64_t n_wide = 0;  // pairs wider than one warp of 32 columns per lane
-                for (uint32_t p = 0; p < np; ++p) n_wide += K[p] > 1024u;
+                uint64_t n_wide = sc.n_long[0];  // pairs wider than one warp of 32 columns per lane
+                for (uint32_t p = 0; p < np && !on_dev; ++p) n_wide += K[p] > 1024u;
                 const int dlk = default_long_kind(ctx->cfg, n_wide,
                                                   (uint64_t)ctx->sms * ctx->occ_longk[3] * (kSerialThreads / 32));
                 Plan best;
                 bool have = false;
                 for (auto& cd : cand) {
                     Plan c;
-                    make_plan_id(L.data(), K.data(), pr, np, cd.first, cd.second, dlk, c);
+                    // (the device planner has no cost to compare: the widest teams, which are the
+                    // first candidate)
+                    plan_of(cd.first, cd.second, dlk, c);
                     const double cost = c.cost + (double)c.n_too_long * 1e18;
                     if (!have || cost < best.cost + (double)best.n_too_long * 1e18) {
                         best = std::move(c);
@@ -1245,9 +1359,9 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
                 P = std::move(best);
                 // measure the short-pair kernels when short pairs, and the multi-warp
                 // kernels when multi-warp pairs, hold a real share of the batch's cells
-                uint64_t short_cells = 0;
+                uint64_t short_cells = sc.short_cells[0];
                 const uint64_t wmax = 32ull * 32ull;  // widest short team: 32 lanes x 32 columns
-                for (uint32_t p = 0; p < np; ++p)
+                for (uint32_t p = 0; p < np && !on_dev; ++p)
                     if (K[p] <= wmax) short_cells += (uint64_t)L[p] * K[p];
                 const uint64_t long_cells = cells - short_cells;
                 const bool may_tune = !(ctx->cfg.flags & PHMM_F_NO_TUNE);
@@ -1270,8 +1384,8 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
         need32 |= fp32 && plan_needs_rec32(Q);
         need32j |= fp32 && plan_needs_rec32j(Q);
     };
-    uint32_t lmax_b = 0;
-    for (uint32_t p = 0; p < np; ++p) lmax_b = std::max(lmax_b, L[p]);
+    uint32_t lmax_b = sc.lmax;
+    for (uint32_t p = 0; p < np && !on_dev; ++p) lmax_b = std::max(lmax_b, L[p]);
     const uint64_t rb_words = (uint64_t)lmax_b * 8;  // FP64 boundary: 8 words per row
     const int rescue_ctas = ctx->sms * ctx->occ64;
     const uint64_t rb_bytes = (uint64_t)rescue_ctas * 2 * rb_words * 8ull + 16;
@@ -1279,7 +1393,8 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
         need32 = need32j = false;
         needs_of(P);
         Plan probe;  // the kernels that the tuner may try
-        probe.witems = P.witems;
+        probe.dev = true;
+        probe.d_teams = P.n_witems();
         if (tune_short)
             for (auto& cd : tune_cand) {
                 probe.scal_id = cd.first;
@@ -1289,7 +1404,7 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
         if (tune_long) {
             probe.scal_id = P.scal_id;
             probe.pack_id = P.pack_id;
-            probe.citems = P.citems;
+            probe.d_items = P.n_citems();
             for (int lk : long_kinds_of(ctx->cfg)) {
                 probe.long_kind = lk;
                 needs_of(probe);
@@ -1300,19 +1415,22 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
                np * (sizeof(PairDesc) + sizeof(Partial) + 8 + 1 + 4) + (need32j ? nbases * sizeof(Rec32J) : 0) +
                (need32 ? nbases * sizeof(Rec32) : 0) +
                (need64 ? nbases * sizeof(Rec64) : 0) + (fp32 ? 0 : nbases * sizeof(Rec64J)) +
-               P.teams.size() * sizeof(Team) + (P.witems.size() + P.witems2.size()) * sizeof(WarpItem) +
-               P.cpairs.size() * sizeof(CtaPair) + P.citems.size() * sizeof(CtaItem) + P.bnd_words * 8ull +
+               P.n_teams() * sizeof(Team) + (P.n_witems() + P.witems2.size()) * sizeof(WarpItem) +
+               P.n_cpairs() * sizeof(CtaPair) + P.n_citems() * sizeof(CtaItem) + P.bnd_words * 8ull +
                P.n_extra * sizeof(Partial) + serial_bytes(ctx, P);
     };
     uint64_t foot = foot_of();
     // A wave kind that nobody asked for keeps within the bound that phmm_batch_footprint gives
     // and the budget: else wider strips, else CTA strips.
     if (!reuse && fp32 && kLongWave[P.long_kind] && long_kinds_of(ctx->cfg).size() > 1) {
-        const uint64_t most = std::min<uint64_t>(ctx->budget, footprint_bound(ctx, nbases, nhb, nr, nh, np, L.data(), K.data()));
-        for (int lk : {6, 1}) {
+        FootSums q{nbases, nhb, nr, nh, np, lmax_b, sc.cta_rows, sc.cta_strips};
+        const uint64_t most = std::min<uint64_t>(
+            ctx->budget, on_dev ? footprint_bound(ctx, q) : footprint_bound(ctx, nbases, nhb, nr, nh, np, L.data(), K.data()));
+        for (int lk : {6, 3, 1}) {
             if (foot <= most) break;
+            if (on_dev && lk == 1) break;  // (serial strips always fit the bound)
             const int si = P.scal_id, pi = P.pack_id;
-            make_plan_id(L.data(), K.data(), pr, np, si, pi, lk, P);
+            plan_of(si, pi, lk, P);
             foot = foot_of();
         }
     }
@@ -1340,17 +1458,18 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
         CK(ensure(S->in_dq, nbases)); CK(ensure(S->in_gq, nbases)); CK(ensure(S->in_hap, nhb));
         CK(ensure(S->in_roff, (nr + 1) * 8ull)); CK(ensure(S->in_hoff, (nh + 1) * 8ull));
         CK(ensure(S->in_pr, np * 4ull)); CK(ensure(S->in_ph, np * 4ull));
-        cudaStream_t cs = ctx->copy_stream;
         CK(cudaMemcpyAsync(S->in_bases.p, b->read_bases, nbases, cudaMemcpyHostToDevice, cs));
         CK(cudaMemcpyAsync(S->in_bq.p, b->base_q, nbases, cudaMemcpyHostToDevice, cs));
         CK(cudaMemcpyAsync(S->in_iq.p, b->ins_q, nbases, cudaMemcpyHostToDevice, cs));
         CK(cudaMemcpyAsync(S->in_dq.p, b->del_q, nbases, cudaMemcpyHostToDevice, cs));
         CK(cudaMemcpyAsync(S->in_gq.p, b->gcp_q, nbases, cudaMemcpyHostToDevice, cs));
         CK(cudaMemcpyAsync(S->in_hap.p, b->hap_bases, nhb, cudaMemcpyHostToDevice, cs));
-        CK(cudaMemcpyAsync(S->in_roff.p, b->read_off, (nr + 1) * 8ull, cudaMemcpyHostToDevice, cs));
-        CK(cudaMemcpyAsync(S->in_hoff.p, b->hap_off, (nh + 1) * 8ull, cudaMemcpyHostToDevice, cs));
-        CK(cudaMemcpyAsync(S->in_pr.p, b->pair_read, np * 4ull, cudaMemcpyHostToDevice, cs));
-        CK(cudaMemcpyAsync(S->in_ph.p, b->pair_hap, np * 4ull, cudaMemcpyHostToDevice, cs));
+        if (!on_dev) {
+            CK(cudaMemcpyAsync(S->in_roff.p, b->read_off, (nr + 1) * 8ull, cudaMemcpyHostToDevice, cs));
+            CK(cudaMemcpyAsync(S->in_hoff.p, b->hap_off, (nh + 1) * 8ull, cudaMemcpyHostToDevice, cs));
+            CK(cudaMemcpyAsync(S->in_pr.p, b->pair_read, np * 4ull, cudaMemcpyHostToDevice, cs));
+            CK(cudaMemcpyAsync(S->in_ph.p, b->pair_hap, np * 4ull, cudaMemcpyHostToDevice, cs));
+        }
         if (getenv("PHMM_DEBUG"))
             fprintf(stderr, "phmm submit: input copies issued %.1f ms after the plan\n",
                     std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - th_plan).count());
@@ -1380,7 +1499,6 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
     CK(ensure(S->rescue, np * 4ull));
     CK(ensure(S->h_out, np * 8ull));
     CK(ensure(S->h_oflags, np * 1ull));
-    cudaStream_t cs = ctx->copy_stream;
     if (!reuse) CK(upload_plan(*S, P, cs));
     CK(cudaMemsetAsync(S->parts.p, 0, (np + P.n_extra) * sizeof(Partial), cs));
     hh.n_read_bases = nbases;
@@ -1410,6 +1528,7 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
     hh.seed = ctx->seed;
     hh.mode = (uint32_t)ctx->cfg.precision;
     CK(cudaMemcpyAsync(S->hdr.p, &hh, sizeof(hh), cudaMemcpyHostToDevice, cs));
+    if (P.dev) CK(build_plan(*S, P, pin, ctx->sms, cs));
     CK(cudaEventRecord(S->ev_copy, cs));
     // host inputs may be released when submit returns
     CK(cudaEventSynchronize(S->ev_copy));
@@ -1494,7 +1613,7 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
                 cd[1] = bp;
             }
             Plan c;
-            make_plan_id(L.data(), K.data(), pr, np, cd[0], cd[1], cd[2], c);
+            plan_of(cd[0], cd[1], cd[2], c);
             if (c.n_too_long) continue;
             CK(upload_plan(*S, c, cs));
             CK(ensure(S->parts, (np + c.n_extra) * sizeof(Partial)));
@@ -1504,13 +1623,14 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
             hh.parts = (Partial*)S->parts.p;
             plan_header(*S, c, hh);
             CK(cudaMemcpyAsync(S->hdr.p, &hh, sizeof(hh), cudaMemcpyHostToDevice, cs));
+            if (c.dev) CK(build_plan(*S, c, pin, ctx->sms, cs));
             CK(cudaStreamSynchronize(cs));
             // time the candidate; a short run is repeated and the faster kept (the first
             // launch of a kernel after a plan change runs cold).  The serial multi-warp kind
             // is always run twice: its first run after a plan change measured about 30%
             // slower than its steady state, which would bias the choice against it.
             float ms = 1e30f, first = 0.f;
-            const bool warm_twice = !c.citems.empty() && kLongSerial[c.long_kind];
+            const bool warm_twice = c.n_citems() > 0 && kLongSerial[c.long_kind];
             for (int rep = 0; rep < 2; ++rep) {
                 const int rc = launch_sequence(ctx, *S, c.scal_id, c.pack_id, c.long_kind, false);
                 if (rc != PHMM_OK) return rc;
@@ -1533,7 +1653,7 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
             }
         }
         ctx->tuned[tune_sig] = {bs, bp, bl};
-        make_plan_id(L.data(), K.data(), pr, np, bs, bp, bl, P);
+        plan_of(bs, bp, bl, P);
         CK(upload_plan(*S, P, cs));
         CK(ensure(S->parts, (np + P.n_extra) * sizeof(Partial)));
         CK(ensure(S->bnd, P.bnd_words * 8ull));
@@ -1542,6 +1662,7 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
         hh.parts = (Partial*)S->parts.p;
         plan_header(*S, P, hh);
         CK(cudaMemcpyAsync(S->hdr.p, &hh, sizeof(hh), cudaMemcpyHostToDevice, cs));
+        if (P.dev) CK(build_plan(*S, P, pin, ctx->sms, cs));
         CK(cudaMemsetAsync(S->parts.p, 0, (np + P.n_extra) * sizeof(Partial), cs));
         CK(cudaStreamSynchronize(cs));
         N = P.N;
@@ -1627,14 +1748,14 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
     {
         const bool f32 = ctx->cfg.precision != PHMM_PREC_FP64;
         // FP64: the forward variant (0: N 8 in 16-warp CTAs, 1: N 16 in 8-warp CTAs)
-        S->st.short_kernel = f32 ? (!P.witems.empty() ? P.scal_id : -1) : P.scal_id;
+        S->st.short_kernel = f32 ? (P.n_witems() > 0 ? P.scal_id : -1) : P.scal_id;
         S->st.packed_kernel = f32 && !P.witems2.empty() ? P.pack_id : -1;
-        S->st.long_kernel = f32 && !P.citems.empty() ? P.long_kind : -1;
+        S->st.long_kernel = f32 && P.n_citems() > 0 ? P.long_kind : -1;
         const bool branched = f32 || f64_pipelined(P.scal_id);  // the pipelined FP64 variants have two branches
         for (int q = 0; q < 3; ++q) S->st.cells_branch[q] = branched ? P.cells_br[q] : (q == 0 ? cells : 0);
     }
     S->host_status = P.n_too_long ? PHMM_EINVAL : PHMM_OK;
-    S->plan_valid = true;
+    S->plan_valid = !on_dev;
     S->plan_hash = hsh;
     S->plan_np = np;
     S->st.ms_host = (float)std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - th0).count();

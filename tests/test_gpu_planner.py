@@ -1,0 +1,101 @@
+"""Batches of many pairs are planned on the device (csrc/planner.cu).  Each pair's result
+does not depend on the plan, so the same pairs in batches small enough for the host planner
+must give the same bits; the oracle checks a sample.  Shapes: every team width, many run
+lengths, wide pairs with one item per pair or per strip, one class only, shared reads; and the
+index and offset errors that submit must refuse."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2606_25738_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+HOST = 4095  # pairs that the host planner still takes
+
+
+@pytest.fixture(scope="module")
+def phmm():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2606_25738_gb300 import phmm as P
+    return P
+
+
+def _batch(l, k, seed, reads=None):
+    """reads: number of reads (pairs share them, l[:reads] are their lengths)."""
+    rng = np.random.default_rng(seed)
+    n, nr = len(k), reads or len(k)
+    rl, hl = np.asarray(l[:nr], np.uint64), np.asarray(k, np.uint64)
+    roff = np.concatenate([[0], np.cumsum(rl)]).astype(np.uint64)
+    hoff = np.concatenate([[0], np.cumsum(hl)]).astype(np.uint64)
+    nb, nh = int(roff[-1]), int(hoff[-1])
+    acgt = np.frombuffer(b"ACGT", np.uint8)
+    return dict(read_bases=acgt[rng.integers(0, 4, nb)], read_off=roff, base_q=rng.integers(10, 41, nb).astype(np.uint8),
+                ins_q=rng.integers(40, 46, nb).astype(np.uint8), del_q=np.full(nb, 45, np.uint8),
+                gcp_q=np.full(nb, 10, np.uint8), hap_bases=acgt[rng.integers(0, 4, nh)], hap_off=hoff,
+                pair_read=(np.arange(n) % nr).astype(np.uint32), pair_hap=np.arange(n, dtype=np.uint32))
+
+
+def _shapes(name):
+    rng = np.random.default_rng(17)
+    n = 9000
+    if name == "widths":
+        return np.full(n, 3), rng.integers(1, 1025, n), None
+    if name == "runs":
+        return np.rint(np.exp(rng.uniform(0, np.log(700), n))).astype(int), rng.integers(1, 200, n), None
+    if name == "wide":
+        return rng.integers(1, 20, n), np.rint(np.exp(rng.uniform(np.log(30), np.log(5000), n))).astype(int), None
+    if name == "one_class":
+        return np.full(n, 20), np.full(n, 100), None
+    return np.full(n, 30), rng.integers(1, 1025, n), 40  # shared reads
+
+
+@pytest.mark.parametrize("kind", ["auto", "serial", "wave", "wave16"])
+@pytest.mark.parametrize("name", ["widths", "runs", "wide", "one_class", "shared"])
+def test_same_bits_as_host_plans(phmm, name, kind):
+    if kind != "auto" and name != "wide":
+        pytest.skip("no wide pairs")
+    l, k, reads = _shapes(name)
+    b = _batch(l, k, 3, reads)
+    n = len(k)
+    flag = {"auto": 0, "serial": phmm.F_LONG_SERIAL, "wave": phmm.F_LONG_WAVE, "wave16": phmm.F_LONG_WAVE16}[kind]
+    d = phmm.to_device(b)
+    import torch
+    for N in (32, 24):
+        kw = dict(precision="fp32", variant="pipe2", cols_per_lane=N, flags=flag | phmm.F_NO_TUNE)
+        with phmm.Context(**kw) as ctx:
+            out, flags, rc, st = ctx.run(b)
+            dout = torch.empty(n, dtype=torch.float64, device="cuda")
+            ctx.run(d, out=dout)
+            parts = [ctx.run(W.subset(b, np.arange(p, min(p + HOST, n)))) for p in range(0, n, HOST)]
+        assert rc == 0 and st["n_pairs"] == n and st["cells"] == W.cells(b)
+        assert st["n_long"] == int(np.sum(np.asarray(k) > 32 * N))
+        assert np.array_equal(out, dout.cpu().numpy())
+        if kind != "auto":  # the untuned choice of a wide kind depends on the batch
+            assert np.array_equal(out, np.concatenate([p[0] for p in parts]))
+            assert np.array_equal(flags, np.concatenate([p[1] for p in parts]))
+        else:
+            assert np.max(np.abs(out - np.concatenate([p[0] for p in parts]))) <= 1e-5
+        pick = np.random.default_rng(1).choice(n, 300, replace=False)
+        assert np.max(np.abs(out[pick] - oracle.batch(W.subset(b, pick)))) <= 1e-3
+
+
+def test_bad_batches_refused(phmm):
+    l, k, _ = _shapes("one_class")
+    n = len(k)
+    with phmm.Context(precision="fp32") as ctx:
+        for what in ("index", "offset", "first", "hap"):
+            b = _batch(l, k, 4)
+            if what == "index":
+                b["pair_read"][n - 1] = n
+            elif what == "offset":
+                b["read_off"][5000] = b["read_off"][4999]
+            elif what == "first":
+                b["read_off"][0] = 1
+            else:
+                b["pair_hap"][17] = 0xffffffff
+            with pytest.raises(phmm.PhmmError) as e:
+                ctx.run(b)
+            assert e.value.status == phmm.PHMM_EINVAL
+        out, flags, rc, st = ctx.run(_batch(l, k, 4))
+        assert rc == 0 and np.all(np.isfinite(out))
