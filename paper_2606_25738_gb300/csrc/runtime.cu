@@ -1005,198 +1005,8 @@ uint64_t footprint_bound(const phmm_ctx* ctx, uint64_t nbases, uint64_t nhb, uin
 
 constexpr uint64_t kTuneMinCells = 200000000ull;  // smaller batches keep the cost model's pick
 
-}  // namespace
-
-extern "C" {
-
-int phmm_abi_version(void) { return PHMM_ABI_VERSION; }
-
-const char* phmm_strerror(int s) {
-    switch (s) {
-    case PHMM_OK: return "ok";
-    case PHMM_PENDING: return "pending";
-    case PHMM_EINVAL: return "invalid argument or input";
-    case PHMM_ENOMEM: return "batch exceeds the device memory budget";
-    case PHMM_EBUSY: return "too many batches in flight";
-    case PHMM_ECUDA: return "CUDA error";
-    case PHMM_ETIMEOUT: return "timed out";
-    case PHMM_ECANCELED: return "cancelled";
-    case PHMM_ENOTFOUND: return "unknown ticket";
-    default: return "unknown status";
-    }
-}
-
-int phmm_create(const phmm_config* cfg, phmm_ctx** out) {
-    if (!cfg || !out) return PHMM_EINVAL;
-    *out = nullptr;
-    if (cfg->precision < 0 || cfg->precision > 2) return PHMM_EINVAL;
-    if (cfg->kernel_variant < 0 || cfg->kernel_variant > 6) return PHMM_EINVAL;
-    if (!(cfg->fp32_tolerance >= 0.0)) return PHMM_EINVAL;
-    {
-        const unsigned lk =
-            cfg->flags & (PHMM_F_LONG_LEAN | PHMM_F_LONG_PIPE32 | PHMM_F_LONG_PIPE24 | PHMM_F_LONG_SERIAL |
-                          PHMM_F_LONG_PIPE4 | PHMM_F_LONG_CLUSTER | PHMM_F_LONG_WAVE | PHMM_F_LONG_WAVE16);
-        if (lk & (lk - 1)) return PHMM_EINVAL;  // more than one forced multi-warp kernel
-    }
-    {
-        const int n = cfg->cols_per_lane;
-        const bool okp = n == 12 || n == 16;  // packed widths
-        const bool oks = n == 16 || n == 24 || n == 32;  // scalar widths
-        if (cfg->precision == PHMM_PREC_FP64) {
-            if (n != 0 && n != kF64N[0] && n != kF64N[1]) return PHMM_EINVAL;  // the FP64 variants
-        } else if (n != 0 && !(cfg->kernel_variant >= 2 ? oks : (okp || oks))) {
-            return PHMM_EINVAL;
-        }
-    }
-    int ndev = 0;
-    if (cudaGetDeviceCount(&ndev) != cudaSuccess || cfg->device < 0 || cfg->device >= ndev)
-        return PHMM_ECUDA;
-    phmm_ctx* ctx = new phmm_ctx();
-    ctx->dev = cfg->device;
-    ctx->cfg = *cfg;
-    if (ctx->cfg.max_inflight == 0) ctx->cfg.max_inflight = 4;
-    if (ctx->cfg.max_inflight > 64) ctx->cfg.max_inflight = 64;
-    auto fail = [&](int code) {
-        phmm_destroy(ctx);
-        return code;
-    };
-    if (cudaSetDevice(ctx->dev) != cudaSuccess) return fail(PHMM_ECUDA);
-    cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->dev);
-    int khz = 0;
-    cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, ctx->dev);
-    ctx->max_mhz = khz / 1000.0;
-    if (cfg->stream) {
-        ctx->stream = static_cast<cudaStream_t>(cfg->stream);
-    } else {
-        if (cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking) != cudaSuccess)
-            return fail(PHMM_ECUDA);
-        ctx->own_stream = true;
-    }
-    if (cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) != cudaSuccess)
-        return fail(PHMM_ECUDA);
-    size_t fr = 0, tot = 0;
-    cudaMemGetInfo(&fr, &tot);
-    ctx->budget = cfg->mem_budget_bytes ? cfg->mem_budget_bytes : (size_t)(0.9 * (double)fr);
-    // tables
-    PhredTables T;
-    build_phred_tables(T);
-    if (ensure(ctx->tables, sizeof(T)) != cudaSuccess) return fail(PHMM_ECUDA);
-    cudaMemcpy(ctx->tables.p, &T, sizeof(T), cudaMemcpyHostToDevice);
-    for (int q = 0; q < 5; ++q) {
-        std::vector<PowRow<float>> v;
-        build_pow_table<float>(kPowN[q], v);
-        if (ensure(ctx->pow32[q], v.size() * sizeof(v[0])) != cudaSuccess) return fail(PHMM_ECUDA);
-        cudaMemcpy(ctx->pow32[q].p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice);
-    }
-    for (int q = 0; q < kNumPacked; ++q) ctx->occ_packed[q] = occupancy_short_packed(q);
-    for (int q = 0; q < kNumScalar; ++q) ctx->occ_scalar[q] = occupancy_short_scalar(q);
-    ctx->occ_longk[0] = occupancy_forward32_long();
-    ctx->occ_longk[1] = occupancy_forward32_long_pipe(1);
-    ctx->occ_longk[2] = occupancy_forward32_long_pipe(2);
-    ctx->occ_longk[3] = occupancy_forward32_long_pipe(3);
-    ctx->occ_longk[4] = occupancy_forward32_long_pipe(4);
-    ctx->occ_longk[5] = occupancy_forward32_long_pipe(5);
-    ctx->occ_longk[6] = occupancy_forward32_long_pipe(6);
-    ctx->occ_longk[7] = occupancy_forward32_long_pipe(7);
-    ctx->occ_longk[8] = occupancy_forward32_long_pipe(8);
-    if (getenv("PHMM_DEBUG")) {
-        fprintf(stderr, "phmm: sms %d occupancy packed %d %d long %d %d %d %d %d fp64 %d scalar", ctx->sms,
-                ctx->occ_packed[0], ctx->occ_packed[1], ctx->occ_longk[0], ctx->occ_longk[1],
-                ctx->occ_longk[2], ctx->occ_longk[3], ctx->occ_longk[4], ctx->occ64);
-        for (int q = 0; q < kNumScalar; ++q) fprintf(stderr, " %d", ctx->occ_scalar[q]);
-        fprintf(stderr, "\n");
-    }
-    {
-        std::vector<PowRow<double>> v;
-        build_pow_table<double>(kN64, v);
-        if (ensure(ctx->pow64, v.size() * sizeof(v[0])) != cudaSuccess) return fail(PHMM_ECUDA);
-        cudaMemcpy(ctx->pow64.p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice);
-        build_pow_table<double>(kF64N[1], v);
-        if (ensure(ctx->pow64w, v.size() * sizeof(v[0])) != cudaSuccess) return fail(PHMM_ECUDA);
-        cudaMemcpy(ctx->pow64w.p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice);
-        build_pow_table<double>(kF64NS[3], v);
-        if (ensure(ctx->pow64x, v.size() * sizeof(v[0])) != cudaSuccess) return fail(PHMM_ECUDA);
-        cudaMemcpy(ctx->pow64x.p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice);
-        for (int q = 0; q < kNumF64; ++q) ctx->occ64v[q] = occupancy_forward64(q);
-        for (int q = 2; q < kNumF64; ++q) ctx->occ64s[q] = occupancy_short_pipe64(q);
-        ctx->occ64 = ctx->occ64v[0];
-    }
-    ctx->slots.resize(ctx->cfg.max_inflight);
-    for (auto& S : ctx->slots) {
-        cudaEvent_t* evs[] = {&S.ev_copy, &S.ev_start, &S.ev_fwd0, &S.ev_fwd1, &S.ev_res0, &S.ev_res1, &S.ev_end,
-                              &S.ev_br[0], &S.ev_br[1], &S.ev_br[2], &S.ev_br[3], &S.ev_br[4], &S.ev_br[5]};
-        for (auto* e : evs)
-            if (cudaEventCreate(e) != cudaSuccess) return fail(PHMM_ECUDA);
-        cudaEvent_t* evn[] = {&S.ev_fork, &S.ev_join, &S.ev_join3, &S.ev_user};
-        for (auto* e : evn)
-            if (cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) return fail(PHMM_ECUDA);
-        cudaStream_t* sts[] = {&S.sm, &S.sb2, &S.sb3};
-        for (auto* q : sts)
-            if (cudaStreamCreateWithFlags(q, cudaStreamNonBlocking) != cudaSuccess) return fail(PHMM_ECUDA);
-        if (ensure(S.small, kSmallBytes) != cudaSuccess || ensure(S.h_small, 64) != cudaSuccess ||
-            ensure(S.hdr, sizeof(BatchHeader)) != cudaSuccess || cudaMemset(S.small.p, 0, kSmallBytes) != cudaSuccess)
-            return fail(PHMM_ECUDA);
-    }
-    if (cudaGetLastError() != cudaSuccess) return fail(PHMM_ECUDA);
-    *out = ctx;
-    return PHMM_OK;
-}
-
-void phmm_destroy(phmm_ctx* ctx) {
-    if (!ctx) return;
-    cudaSetDevice(ctx->dev);
-    if (ctx->stream) cudaStreamSynchronize(ctx->stream);
-    if (ctx->copy_stream) cudaStreamSynchronize(ctx->copy_stream);
-    for (auto& S : ctx->slots) {
-        cudaStream_t sts[] = {S.sm, S.sb2, S.sb3};
-        for (auto q : sts)
-            if (q) cudaStreamSynchronize(q);
-    }
-    for (auto& S : ctx->slots) {
-        DevBuf* d[] = {&S.in_bases, &S.in_bq, &S.in_iq, &S.in_dq, &S.in_gq, &S.in_hap, &S.in_roff,
-                       &S.in_hoff, &S.in_pr, &S.in_ph, &S.desc, &S.rec32, &S.rec32j, &S.rec64, &S.rec64j, &S.teams,
-                       &S.witems, &S.witems2, &S.cpairs, &S.citems, &S.parts, &S.out, &S.oflags, &S.rescue,
-                       &S.small, &S.hdr, &S.bnd, &S.rbnd, &S.sbnd, &S.wbnd,
-                       &S.pscan, &S.pscratch};
-        for (auto* b : d) release(*b);
-        HostBuf* h[] = {&S.h_out, &S.h_oflags, &S.h_small, &S.h_roff, &S.h_hoff, &S.h_pr, &S.h_ph, &S.h_pscan};
-        for (auto* b : h) release(*b);
-        cudaEvent_t evs[] = {S.ev_copy, S.ev_start, S.ev_fwd0, S.ev_fwd1, S.ev_res0, S.ev_res1, S.ev_end,
-                             S.ev_br[0], S.ev_br[1], S.ev_br[2], S.ev_br[3], S.ev_br[4], S.ev_br[5]};
-        for (auto e : evs)
-            if (e) cudaEventDestroy(e);
-        cudaEvent_t evn[] = {S.ev_fork, S.ev_join, S.ev_join3, S.ev_user};
-        for (auto e : evn)
-            if (e) cudaEventDestroy(e);
-        if (S.gexec) cudaGraphExecDestroy(S.gexec);
-        cudaStream_t sts[] = {S.sm, S.sb2, S.sb3};
-        for (auto q : sts)
-            if (q) cudaStreamDestroy(q);
-    }
-    release(ctx->tables);
-    release(ctx->scan_row);
-    for (auto& b : ctx->pow32) release(b);
-    release(ctx->pow64);
-    release(ctx->pow64w);
-    release(ctx->pow64x);
-    if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
-    if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
-    delete ctx;
-}
-
-int phmm_device_info(phmm_ctx* ctx, int* sms, double* max_clock_mhz, double* cups) {
-    if (!ctx) return PHMM_EINVAL;
-    if (sms) *sms = ctx->sms;
-    if (max_clock_mhz) *max_clock_mhz = ctx->max_mhz;
-    if (cups) *cups = 2.0 * 128.0 * ctx->sms * ctx->max_mhz * 1e6 / 12.0;
-    return PHMM_OK;
-}
-
-int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
-    if (!ctx || !b || !ticket) return PHMM_EINVAL;
-    std::lock_guard<std::mutex> lock(ctx->mu);
-    if (ctx->dead) return PHMM_ECUDA;
-    if (cudaSetDevice(ctx->dev) != cudaSuccess) return PHMM_ECUDA;
+// host_plan: the plan is built on the host whatever the batch's size
+int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool host_plan) {
     if (b->n_pairs > 0 && (!b->read_bases || !b->read_off || !b->base_q || !b->ins_q || !b->del_q ||
                            !b->gcp_q || !b->hap_bases || !b->hap_off || !b->pair_read ||
                            !b->pair_hap || !b->out_log10))
@@ -1216,7 +1026,7 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
     const uint64_t *roff = b->read_off, *hoff = b->hap_off;
     const uint32_t *pr = b->pair_read, *ph = b->pair_hap;
     cudaStream_t cs = ctx->copy_stream;
-    const bool on_dev = plans_on_device(ctx->cfg, np);
+    const bool on_dev = !host_plan && plans_on_device(ctx->cfg, np);
     PlanInput pin{};
     PlanScan sc{};
     if (dev_in && np > 0) {
@@ -1428,7 +1238,10 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
             ctx->budget, on_dev ? footprint_bound(ctx, q) : footprint_bound(ctx, nbases, nhb, nr, nh, np, L.data(), K.data()));
         for (int lk : {6, 3, 1}) {
             if (foot <= most) break;
-            if (on_dev && lk == 1) break;  // (serial strips always fit the bound)
+            if (on_dev && lk == 1) {  // (serial strips always fit the bound)
+                if (foot <= ctx->budget) break;
+                return submit_locked(ctx, b, ticket, true);  // CTA strips are planned on the host
+            }
             const int si = P.scal_id, pi = P.pack_id;
             plan_of(si, pi, lk, P);
             foot = foot_of();
@@ -1764,6 +1577,201 @@ int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
                 std::chrono::duration<double, std::milli>(th_plan - th0).count(), S->st.ms_host);
     *ticket = S->ticket;
     return PHMM_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int phmm_abi_version(void) { return PHMM_ABI_VERSION; }
+
+const char* phmm_strerror(int s) {
+    switch (s) {
+    case PHMM_OK: return "ok";
+    case PHMM_PENDING: return "pending";
+    case PHMM_EINVAL: return "invalid argument or input";
+    case PHMM_ENOMEM: return "batch exceeds the device memory budget";
+    case PHMM_EBUSY: return "too many batches in flight";
+    case PHMM_ECUDA: return "CUDA error";
+    case PHMM_ETIMEOUT: return "timed out";
+    case PHMM_ECANCELED: return "cancelled";
+    case PHMM_ENOTFOUND: return "unknown ticket";
+    default: return "unknown status";
+    }
+}
+
+int phmm_create(const phmm_config* cfg, phmm_ctx** out) {
+    if (!cfg || !out) return PHMM_EINVAL;
+    *out = nullptr;
+    if (cfg->precision < 0 || cfg->precision > 2) return PHMM_EINVAL;
+    if (cfg->kernel_variant < 0 || cfg->kernel_variant > 6) return PHMM_EINVAL;
+    if (!(cfg->fp32_tolerance >= 0.0)) return PHMM_EINVAL;
+    {
+        const unsigned lk =
+            cfg->flags & (PHMM_F_LONG_LEAN | PHMM_F_LONG_PIPE32 | PHMM_F_LONG_PIPE24 | PHMM_F_LONG_SERIAL |
+                          PHMM_F_LONG_PIPE4 | PHMM_F_LONG_CLUSTER | PHMM_F_LONG_WAVE | PHMM_F_LONG_WAVE16);
+        if (lk & (lk - 1)) return PHMM_EINVAL;  // more than one forced multi-warp kernel
+    }
+    {
+        const int n = cfg->cols_per_lane;
+        const bool okp = n == 12 || n == 16;  // packed widths
+        const bool oks = n == 16 || n == 24 || n == 32;  // scalar widths
+        if (cfg->precision == PHMM_PREC_FP64) {
+            if (n != 0 && n != kF64N[0] && n != kF64N[1]) return PHMM_EINVAL;  // the FP64 variants
+        } else if (n != 0 && !(cfg->kernel_variant >= 2 ? oks : (okp || oks))) {
+            return PHMM_EINVAL;
+        }
+    }
+    int ndev = 0;
+    if (cudaGetDeviceCount(&ndev) != cudaSuccess || cfg->device < 0 || cfg->device >= ndev)
+        return PHMM_ECUDA;
+    phmm_ctx* ctx = new phmm_ctx();
+    ctx->dev = cfg->device;
+    ctx->cfg = *cfg;
+    if (ctx->cfg.max_inflight == 0) ctx->cfg.max_inflight = 4;
+    if (ctx->cfg.max_inflight > 64) ctx->cfg.max_inflight = 64;
+    auto fail = [&](int code) {
+        phmm_destroy(ctx);
+        return code;
+    };
+    if (cudaSetDevice(ctx->dev) != cudaSuccess) return fail(PHMM_ECUDA);
+    cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->dev);
+    int khz = 0;
+    cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, ctx->dev);
+    ctx->max_mhz = khz / 1000.0;
+    if (cfg->stream) {
+        ctx->stream = static_cast<cudaStream_t>(cfg->stream);
+    } else {
+        if (cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking) != cudaSuccess)
+            return fail(PHMM_ECUDA);
+        ctx->own_stream = true;
+    }
+    if (cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) != cudaSuccess)
+        return fail(PHMM_ECUDA);
+    size_t fr = 0, tot = 0;
+    cudaMemGetInfo(&fr, &tot);
+    ctx->budget = cfg->mem_budget_bytes ? cfg->mem_budget_bytes : (size_t)(0.9 * (double)fr);
+    // tables
+    PhredTables T;
+    build_phred_tables(T);
+    if (ensure(ctx->tables, sizeof(T)) != cudaSuccess) return fail(PHMM_ECUDA);
+    cudaMemcpy(ctx->tables.p, &T, sizeof(T), cudaMemcpyHostToDevice);
+    for (int q = 0; q < 5; ++q) {
+        std::vector<PowRow<float>> v;
+        build_pow_table<float>(kPowN[q], v);
+        if (ensure(ctx->pow32[q], v.size() * sizeof(v[0])) != cudaSuccess) return fail(PHMM_ECUDA);
+        cudaMemcpy(ctx->pow32[q].p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice);
+    }
+    for (int q = 0; q < kNumPacked; ++q) ctx->occ_packed[q] = occupancy_short_packed(q);
+    for (int q = 0; q < kNumScalar; ++q) ctx->occ_scalar[q] = occupancy_short_scalar(q);
+    ctx->occ_longk[0] = occupancy_forward32_long();
+    ctx->occ_longk[1] = occupancy_forward32_long_pipe(1);
+    ctx->occ_longk[2] = occupancy_forward32_long_pipe(2);
+    ctx->occ_longk[3] = occupancy_forward32_long_pipe(3);
+    ctx->occ_longk[4] = occupancy_forward32_long_pipe(4);
+    ctx->occ_longk[5] = occupancy_forward32_long_pipe(5);
+    ctx->occ_longk[6] = occupancy_forward32_long_pipe(6);
+    ctx->occ_longk[7] = occupancy_forward32_long_pipe(7);
+    ctx->occ_longk[8] = occupancy_forward32_long_pipe(8);
+    if (getenv("PHMM_DEBUG")) {
+        fprintf(stderr, "phmm: sms %d occupancy packed %d %d long %d %d %d %d %d fp64 %d scalar", ctx->sms,
+                ctx->occ_packed[0], ctx->occ_packed[1], ctx->occ_longk[0], ctx->occ_longk[1],
+                ctx->occ_longk[2], ctx->occ_longk[3], ctx->occ_longk[4], ctx->occ64);
+        for (int q = 0; q < kNumScalar; ++q) fprintf(stderr, " %d", ctx->occ_scalar[q]);
+        fprintf(stderr, "\n");
+    }
+    {
+        std::vector<PowRow<double>> v;
+        build_pow_table<double>(kN64, v);
+        if (ensure(ctx->pow64, v.size() * sizeof(v[0])) != cudaSuccess) return fail(PHMM_ECUDA);
+        cudaMemcpy(ctx->pow64.p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice);
+        build_pow_table<double>(kF64N[1], v);
+        if (ensure(ctx->pow64w, v.size() * sizeof(v[0])) != cudaSuccess) return fail(PHMM_ECUDA);
+        cudaMemcpy(ctx->pow64w.p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice);
+        build_pow_table<double>(kF64NS[3], v);
+        if (ensure(ctx->pow64x, v.size() * sizeof(v[0])) != cudaSuccess) return fail(PHMM_ECUDA);
+        cudaMemcpy(ctx->pow64x.p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice);
+        for (int q = 0; q < kNumF64; ++q) ctx->occ64v[q] = occupancy_forward64(q);
+        for (int q = 2; q < kNumF64; ++q) ctx->occ64s[q] = occupancy_short_pipe64(q);
+        ctx->occ64 = ctx->occ64v[0];
+    }
+    ctx->slots.resize(ctx->cfg.max_inflight);
+    for (auto& S : ctx->slots) {
+        cudaEvent_t* evs[] = {&S.ev_copy, &S.ev_start, &S.ev_fwd0, &S.ev_fwd1, &S.ev_res0, &S.ev_res1, &S.ev_end,
+                              &S.ev_br[0], &S.ev_br[1], &S.ev_br[2], &S.ev_br[3], &S.ev_br[4], &S.ev_br[5]};
+        for (auto* e : evs)
+            if (cudaEventCreate(e) != cudaSuccess) return fail(PHMM_ECUDA);
+        cudaEvent_t* evn[] = {&S.ev_fork, &S.ev_join, &S.ev_join3, &S.ev_user};
+        for (auto* e : evn)
+            if (cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) return fail(PHMM_ECUDA);
+        cudaStream_t* sts[] = {&S.sm, &S.sb2, &S.sb3};
+        for (auto* q : sts)
+            if (cudaStreamCreateWithFlags(q, cudaStreamNonBlocking) != cudaSuccess) return fail(PHMM_ECUDA);
+        if (ensure(S.small, kSmallBytes) != cudaSuccess || ensure(S.h_small, 64) != cudaSuccess ||
+            ensure(S.hdr, sizeof(BatchHeader)) != cudaSuccess || cudaMemset(S.small.p, 0, kSmallBytes) != cudaSuccess)
+            return fail(PHMM_ECUDA);
+    }
+    if (cudaGetLastError() != cudaSuccess) return fail(PHMM_ECUDA);
+    *out = ctx;
+    return PHMM_OK;
+}
+
+void phmm_destroy(phmm_ctx* ctx) {
+    if (!ctx) return;
+    cudaSetDevice(ctx->dev);
+    if (ctx->stream) cudaStreamSynchronize(ctx->stream);
+    if (ctx->copy_stream) cudaStreamSynchronize(ctx->copy_stream);
+    for (auto& S : ctx->slots) {
+        cudaStream_t sts[] = {S.sm, S.sb2, S.sb3};
+        for (auto q : sts)
+            if (q) cudaStreamSynchronize(q);
+    }
+    for (auto& S : ctx->slots) {
+        DevBuf* d[] = {&S.in_bases, &S.in_bq, &S.in_iq, &S.in_dq, &S.in_gq, &S.in_hap, &S.in_roff,
+                       &S.in_hoff, &S.in_pr, &S.in_ph, &S.desc, &S.rec32, &S.rec32j, &S.rec64, &S.rec64j, &S.teams,
+                       &S.witems, &S.witems2, &S.cpairs, &S.citems, &S.parts, &S.out, &S.oflags, &S.rescue,
+                       &S.small, &S.hdr, &S.bnd, &S.rbnd, &S.sbnd, &S.wbnd,
+                       &S.pscan, &S.pscratch};
+        for (auto* b : d) release(*b);
+        HostBuf* h[] = {&S.h_out, &S.h_oflags, &S.h_small, &S.h_roff, &S.h_hoff, &S.h_pr, &S.h_ph, &S.h_pscan};
+        for (auto* b : h) release(*b);
+        cudaEvent_t evs[] = {S.ev_copy, S.ev_start, S.ev_fwd0, S.ev_fwd1, S.ev_res0, S.ev_res1, S.ev_end,
+                             S.ev_br[0], S.ev_br[1], S.ev_br[2], S.ev_br[3], S.ev_br[4], S.ev_br[5]};
+        for (auto e : evs)
+            if (e) cudaEventDestroy(e);
+        cudaEvent_t evn[] = {S.ev_fork, S.ev_join, S.ev_join3, S.ev_user};
+        for (auto e : evn)
+            if (e) cudaEventDestroy(e);
+        if (S.gexec) cudaGraphExecDestroy(S.gexec);
+        cudaStream_t sts[] = {S.sm, S.sb2, S.sb3};
+        for (auto q : sts)
+            if (q) cudaStreamDestroy(q);
+    }
+    release(ctx->tables);
+    release(ctx->scan_row);
+    for (auto& b : ctx->pow32) release(b);
+    release(ctx->pow64);
+    release(ctx->pow64w);
+    release(ctx->pow64x);
+    if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
+    if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
+    delete ctx;
+}
+
+int phmm_device_info(phmm_ctx* ctx, int* sms, double* max_clock_mhz, double* cups) {
+    if (!ctx) return PHMM_EINVAL;
+    if (sms) *sms = ctx->sms;
+    if (max_clock_mhz) *max_clock_mhz = ctx->max_mhz;
+    if (cups) *cups = 2.0 * 128.0 * ctx->sms * ctx->max_mhz * 1e6 / 12.0;
+    return PHMM_OK;
+}
+
+int phmm_submit_batch(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket) {
+    if (!ctx || !b || !ticket) return PHMM_EINVAL;
+    std::lock_guard<std::mutex> lock(ctx->mu);
+    if (ctx->dead) return PHMM_ECUDA;
+    if (cudaSetDevice(ctx->dev) != cudaSuccess) return PHMM_ECUDA;
+    return submit_locked(ctx, b, ticket, false);
 }
 
 int phmm_batch_footprint(phmm_ctx* ctx, const phmm_batch* b, uint64_t* bytes) {

@@ -99,3 +99,15 @@ def test_bad_batches_refused(phmm):
             assert e.value.status == phmm.PHMM_EINVAL
         out, flags, rc, st = ctx.run(_batch(l, k, 4))
         assert rc == 0 and np.all(np.isfinite(out))
+
+
+def test_small_budget_takes_cta_strips(phmm):
+    """A memory budget that holds neither the waves' boundary rows (4096 x 1000 of 16 bytes) nor
+    two boundaries of 1000 rows per resident warp: the strips of a CTA need neither."""
+    n, l, k = 4096, 1000, 1100
+    b = _batch(np.full(n, l), np.full(n, k), 8, 4)
+    with phmm.Context(precision="fp32_only", mem_budget=16 << 20, flags=phmm.F_NO_TUNE) as ctx:
+        out, flags, rc, st = ctx.run(b)
+    assert rc == 0 and st["long_kernel"] == 1
+    with phmm.Context(precision="fp32_only", flags=phmm.F_NO_TUNE) as ctx:
+        assert np.max(np.abs(out - ctx.run(b)[0])) <= 1e-3
