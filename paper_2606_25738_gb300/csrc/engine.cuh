@@ -112,6 +112,15 @@ __device__ __forceinline__ T scale2(T x, int s) {
     return (x * NT::pow2(s1)) * NT::pow2(s - s1);
 }
 
+// log10(S 2^e) for finite S > 0.  The power of two is taken whole, so that no two large terms
+// cancel: log10(S) + e log10(2) lost up to 6e-14 for a likelihood near 1, whose S is near
+// 2^(initial scale).
+__device__ __forceinline__ double log10_scaled(double S, int e) {
+    const int x = Num<double>::expo(S);
+    if (x == INT_MIN) return log10(S) + (double)e * 0.30102999566398119521;  // subnormal
+    return fma((double)(x + e), 0.30102999566398119521, log10(scale2<double>(S, -x)));
+}
+
 __device__ __forceinline__ Rec32 load_rec(const Rec32* p) {
     const float4 a = __ldg(reinterpret_cast<const float4*>(p));
     const float4 b = __ldg(reinterpret_cast<const float4*>(p) + 1);
@@ -851,13 +860,13 @@ namespace phmm {
 // takes five steps (steps beyond the team width change nothing), so it is one basic
 // block that the compiler can interleave with phase A.
 // ------------------------------------------------------------------------------------
-template <int N, typename T = float, bool FUSE = false>
-__device__ SegOut team_run_pipe(const typename Num<T>::RecJ* __restrict__ rec, int l, int lmax,
+template <int N>
+__device__ SegOut team_run_pipe(const Rec32J* __restrict__ rec, int l, int lmax,
                                 const uint8_t* __restrict__ hap, int k, int col0, int lt,
-                                int tlast, int nsteps, const PowRow<T>* __restrict__ pow_tab,
+                                int tlast, int nsteps, const PowRow<float>* __restrict__ pow_tab,
                                 const PipeRange& rng) {
+    using T = float;
     using NT = Num<T>;
-    using RecJ = typename NT::RecJ;
     static_assert(N <= 32, "match masks hold 32 columns");
     uint32_t bmA = 0, bmC = 0, bmG = 0, bmT = 0, flags = rng.ok ? 0u : PF_DEGEN, mflags = 0;
     const int nvalid = max(0, min(k - col0, N));
@@ -874,8 +883,7 @@ __device__ SegOut team_run_pipe(const typename Num<T>::RecJ* __restrict__ rec, i
         }
     }
     T M[N], J[N];
-    T U[FUSE ? 1 : N];  // unfused: row i + 1's partials, formed after row i's scan
-    T nj = T(0);        // fused: row i's J at the column before the lane
+    T U[N];  // row i + 1's partials, formed after row i's scan
     int E = NT::kLog2C - rng.target;  // see cinit
     T ml = T(0), dt = T(0), gprev = T(0);
     T sp1[5], sp2[5], last1 = T(0), last2 = T(0);
@@ -888,10 +896,10 @@ __device__ SegOut team_run_pipe(const typename Num<T>::RecJ* __restrict__ rec, i
     // so that row 1 and the partials U formed from it start in range
     const T cinit = l > 0 && k > 0 ? (T)(ldexp(1.0, rng.target) / (double)k) : T(0);
     const int l1 = max(l, 1) - 1;
-    RecJ cur = load_recj(rec);
+    Rec32J cur = load_recj(rec);
     int until = 0;
     for (int i = 1; i <= lmax; ++i) {
-        RecJ nxt = cur;
+        Rec32J nxt = cur;
         if (i < lmax) nxt = load_recj(rec + min(i, l1));
         const uint32_t meta = (uint32_t)cur.meta;
         mflags |= meta;
@@ -921,23 +929,6 @@ __device__ SegOut team_run_pipe(const typename Num<T>::RecJ* __restrict__ rec, i
                 if (c == N - 1) yprev = y;
                 y = fma(rg, y, M[c]);
             }
-        } else if constexpr (FUSE) {
-            // Row i's partials U = a M' + J' and insertions J = M' + h J' (primes: row i - 1)
-            // formed column by column inside phase B, as in team_run_pipe2's fused row
-            const T rb = cur.b, na = cur.a, nh = cur.h;
-#pragma unroll
-            for (int c = 0; c < N; ++c) {
-                const T uq = fma(na, ml, c == 0 ? nj : J[c - 1]);
-                if (c > 0) J[c - 1] = fma(nh, J[c - 1], ml);
-                const T u = fma(rb, dt, uq);
-                dt = fma(gprev, dt, ml);
-                ml = M[c];
-                const T mn = (((mask >> c) & 1u) ? pim : pix) * u;
-                M[c] = mn;
-                if (c == N - 1) yprev = y;
-                y = fma(rg, y, mn);
-            }
-            J[N - 1] = fma(nh, J[N - 1], ml);
         } else {
             const T rb = cur.b;
 #pragma unroll
@@ -971,7 +962,7 @@ __device__ SegOut team_run_pipe(const typename Num<T>::RecJ* __restrict__ rec, i
         }
         // the deletion scan of row i and, independent of it, phase A of row i+1
         T nm = __shfl_up_sync(kFull, M[N - 1], 1);
-        nj = __shfl_up_sync(kFull, J[N - 1], 1);
+        T nj = __shfl_up_sync(kFull, J[N - 1], 1);
         T yp = __shfl_up_sync(kFull, yprev, 1);
         if (lt == 0) {
             nm = T(0);
@@ -985,28 +976,25 @@ __device__ SegOut team_run_pipe(const typename Num<T>::RecJ* __restrict__ rec, i
             const T up = __shfl_up_sync(kFull, Z, off);
             Z = fma(up * sp1[s], sp2[s], Z);
         }
-        if constexpr (!FUSE) {
-            const T na = nxt.a, nh = nxt.h;
+        const T na = nxt.a, nh = nxt.h;
 #pragma unroll
-            for (int c = N - 1; c >= 1; --c) {
-                U[c] = fma(na, M[c - 1], J[c - 1]);
-                J[c] = fma(nh, J[c], M[c]);
-            }
-            U[0] = fma(na, nm, nj);
-            J[0] = fma(nh, J[0], M[0]);
+        for (int c = N - 1; c >= 1; --c) {
+            U[c] = fma(na, M[c - 1], J[c - 1]);
+            J[c] = fma(nh, J[c], M[c]);
         }
+        U[0] = fma(na, nm, nj);
+        J[0] = fma(nh, J[0], M[0]);
         T zz = __shfl_up_sync(kFull, Z, 2);
         if (lt < 2) zz = T(0);
         if (until == 0) {
-            // checkpoint: M holds row i, J and U row i+1 when unfused (linear in row i, so
-            // they take the same power of two; U was formed before this test, which the
-            // headroom of the range bounds covers), J row i when fused
+            // checkpoint: M holds row i, J and U row i+1 (linear in row i, so they take the
+            // same power of two; U was formed before this test, which the headroom of the
+            // range bounds covers)
             until = rng.R;
             T m = T(0);
 #pragma unroll
             for (int c = 0; c < N; ++c) m = fmax(m, fmax(fabs(M[c]), fabs(J[c])));
-            if constexpr (sizeof(T) == 4) m = team_max_pos(m, lt, tlast);
-            else m = team_max<T>(m, lt, tlast, nsteps);
+            m = team_max_pos(m, lt, tlast);
             const int e = NT::expo(m);
             if (e == INT_MAX) {
                 flags |= PF_NONFINITE;
@@ -1020,7 +1008,7 @@ __device__ SegOut team_run_pipe(const typename Num<T>::RecJ* __restrict__ rec, i
                         for (int c = 0; c < N; ++c) {
                             M[c] *= f;
                             J[c] *= f;
-                            if constexpr (!FUSE) U[c] *= f;
+                            U[c] *= f;
                         }
                         nm *= f;
                         nj *= f;
@@ -1032,7 +1020,7 @@ __device__ SegOut team_run_pipe(const typename Num<T>::RecJ* __restrict__ rec, i
                         for (int c = 0; c < N; ++c) {
                             M[c] = (M[c] * f1) * f2v;
                             J[c] = (J[c] * f1) * f2v;
-                            if constexpr (!FUSE) U[c] = (U[c] * f1) * f2v;
+                            U[c] = (U[c] * f1) * f2v;
                         }
                         nm = (nm * f1) * f2v;
                         nj = (nj * f1) * f2v;

@@ -180,7 +180,7 @@ __device__ __forceinline__ Rec64J make_rec64j(const BaseQ& x, const PhredTables&
     r.px = T.q3[x.Q] * om_g * mi_p;
     r.a = (1.0 - T.q[x.ins] - T.q[x.del]) * T.inv[x.gcp] * imi_p;
     r.b = T.q[x.delp] * imi_p;
-    r.h = T.q[x.gcp] * mi_p * T.iq[x.ins];
+    r.h = first ? 0.0 : T.q[x.gcp] * mi_p * T.iq[x.ins];  // no insertion before row 1
     r.g = T.q[x.gcp];
     r.mi = T.q[x.ins];
     uint64_t meta = (uint64_t)x.code | ((uint64_t)x.gcp << META_GCP_SHIFT);
@@ -827,43 +827,10 @@ k_short_pipe(const BatchHeader* __restrict__ H, const PowRow<float>* __restrict_
     }
 }
 
-// FP64 mode, pipelined variant: short pairs on the pipelined engine in FP64
-// (team_run_pipe<N, double>, Rec64J records), same work list as k_short_scalar; the
-// multi-warp pairs run on k_forward<double> (CTA items) on the other branch.  A pair with a
-// degenerate row (1 - g = 0) or a range the engine cannot hold is flagged and goes to the
-// unfactored FP64 pass.
-template <int N, int MINB, bool FUSE = false>
-__global__ void __launch_bounds__(kShortThreads, MINB)
-k_short_pipe64(const BatchHeader* __restrict__ H, const PowRow<double>* __restrict__ pow) {
-    const PipeRange rng = pipe_range<double>(H->dropgrow);
-    const uint32_t n_w = H->n_witems;
-    const int lane = threadIdx.x & 31;
-    for (;;) {
-        uint32_t wi = 0;
-        if (lane == 0) wi = atomicAdd(&H->counters[1], 1u);
-        wi = __shfl_sync(kFull, wi, 0);
-        if (wi >= n_w) break;
-        const TeamOf t = team_of(H->teams, H->witems[wi]);
-        int l = 0, k = 0;
-        const Rec64J* rec = reinterpret_cast<const Rec64J*>(dummy_rec<double>());
-        const uint8_t* hap = H->hap_bases;
-        if (t.pair != kNoPair) {
-            const PairDesc d = H->desc[t.pair];
-            l = (int)d.l;
-            k = (int)d.k;
-            rec = H->rec64j + d.roff;
-            hap = H->hap_bases + d.hoff;
-        }
-        const int lmax = (int)__reduce_max_sync(kFull, (unsigned)l);
-        const SegOut o = team_run_pipe<N, double, FUSE>(rec, l, lmax, hap, k, t.lt * N, t.lt, t.tlast, t.nsteps, pow, rng);
-        if (t.pair != kNoPair && t.lt == 0) write_part(H, t.pair, o);
-    }
-}
-
 // Scalar teams on the skewed engine (team_run_skew), same work list as k_short_scalar.  The
 // name and its last two parameters are those of the engine it took the place of (column
 // halves in packed pairs, and a lean form of it), which kernel_variant 5 and 6 ask for.
-template <int N, bool G10>
+template <typename T, int N, bool G10>
 __device__ __forceinline__ void skew_items(const BatchHeader* __restrict__ H, const PipeRange& rng, uint32_t* sm) {
     const uint32_t n_w = H->n_witems;
     const int lane = threadIdx.x & 31;
@@ -874,20 +841,21 @@ __device__ __forceinline__ void skew_items(const BatchHeader* __restrict__ H, co
         if (wi >= n_w) break;
         const TeamOf t = team_of(H->teams, H->witems[wi]);
         int l = 0, k = 0;
-        const Rec32J* rec = reinterpret_cast<const Rec32J*>(dummy_rec<float>());
+        const typename Num<T>::RecJ* rec = reinterpret_cast<const typename Num<T>::RecJ*>(dummy_rec<T>());
         const uint8_t* hap = H->hap_bases;
         if (t.pair != kNoPair) {
             const PairDesc d = H->desc[t.pair];
             l = (int)d.l;
             k = (int)d.k;
-            rec = H->rec32j + d.roff;
+            if constexpr (std::is_same_v<T, float>) rec = H->rec32j + d.roff;
+            else rec = H->rec64j + d.roff;
             hap = H->hap_bases + d.hoff;
         }
         const int team = t.tlast - (lane - t.lt) + 1;
         const int steps = (int)__reduce_max_sync(kFull, l > 0 ? (unsigned)(l + team - 1) : 0u);
         const int p0 = 1 + (int)__reduce_max_sync(kFull, l > 0 ? (unsigned)team : 1u);
         const int p1 = (int)__reduce_min_sync(kFull, l > 0 ? (unsigned)l : 0x7fffffffu);
-        const SegOut o = team_run_skew<N, G10>(rec, l, steps, p0, p1, hap, k, t.lt, t.tlast, rng, sm + lane);
+        const SegOut o = team_run_skew<T, N, G10>(rec, l, steps, p0, p1, hap, k, t.lt, t.tlast, rng, sm + lane);
         if (t.pair != kNoPair && t.lt == 0) write_part(H, t.pair, o);
     }
 }
@@ -896,8 +864,18 @@ __global__ void __launch_bounds__(kShortThreads, MINB)
 k_short_pipe2(const BatchHeader* __restrict__ H) {
     __shared__ uint32_t masks[kShortThreads / 32][5 * 32];
     const PipeRange rng = skew_range(H);
-    if (skew_g10(H->skst)) skew_items<N, true>(H, rng, masks[threadIdx.x >> 5]);
-    else skew_items<N, false>(H, rng, masks[threadIdx.x >> 5]);
+    if (skew_g10(H->skst)) skew_items<float, N, true>(H, rng, masks[threadIdx.x >> 5]);
+    else skew_items<float, N, false>(H, rng, masks[threadIdx.x >> 5]);
+}
+
+// FP64 mode: short pairs on the skewed engine in FP64 (Rec64J records), same work list; the
+// multi-warp pairs run on the other branch.  A pair with a degenerate row (1 - g = 0) or a range
+// the engine cannot hold is flagged and goes to the unfactored FP64 pass.
+template <int N, int MINB>
+__global__ void __launch_bounds__(kShortThreads, MINB)
+k_short_pipe64(const BatchHeader* __restrict__ H) {
+    __shared__ uint32_t masks[kShortThreads / 32][5 * 32];
+    skew_items<double, N, false>(H, skew_range<double>(H), masks[threadIdx.x >> 5]);
 }
 
 // Packed teams of two haplotypes of the same read, N columns per lane (item list
@@ -1002,7 +980,7 @@ __global__ void k_finalize(const BatchHeader* __restrict__ H) {
             atomicOr(H->status, ST_BAD_INPUT);
         } else {
             if (q.S > 0.0 && isfinite(q.S))
-                v = log10(q.S) + (double)(q.E - NT::kLog2C) * 0.30102999566398119521;
+                v = log10_scaled(q.S, q.E - NT::kLog2C);
             else
                 v = q.S == 0.0 ? -INFINITY : NAN;
             if (f & PF_RESCALED) of |= 0x2u;

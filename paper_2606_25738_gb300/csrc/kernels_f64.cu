@@ -16,7 +16,7 @@ __global__ void __launch_bounds__(256) k_prep64_all(const BatchHeader* __restric
     __shared__ PhredTables T;
     load_tables(TG, T);
     __syncthreads();
-    uint32_t dmax = 0, gmax = 0, jmax = 0, hmax = 0;
+    uint32_t dmax = 0, gmax = 0, jmax = 0, hmax = 0, hdrop = 0;
     const uint64_t n = H->n_read_bases;
     Rec64J* const rj = H->rec64j;
     for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; b < n;
@@ -32,6 +32,7 @@ __global__ void __launch_bounds__(256) k_prep64_all(const BatchHeader* __restric
             const double big = fmax(fmax(fabs(r2.a), fabs(r2.b) / om), T.iq[x.insp]);
             jmax = max(jmax, (uint32_t)fmax(ceil(log2(fmax(big, 1.0))), 0.0));
             hmax = max(hmax, (uint32_t)ceil(log2(1.0 + fabs(r2.h)) * 64.0) + 1u);
+            hdrop = max(hdrop, (uint32_t)ceil(fmax(-log2(fmax(r2.h, 0x1p-126)), 0.0) * 64.0) + 1u);
         }
         if (x.bad) atomicOr(H->status, ST_BAD_INPUT);
         uint32_t d, g;
@@ -42,6 +43,8 @@ __global__ void __launch_bounds__(256) k_prep64_all(const BatchHeader* __restric
     block_max2(dmax, gmax, H->dropgrow);
     __syncthreads();
     block_max2(jmax, hmax, H->dropgrow + 2);
+    __syncthreads();
+    block_max2(hdrop, 0u, reinterpret_cast<uint32_t*>(H->skst));
     build_desc(H);
 }
 
@@ -80,13 +83,13 @@ __global__ void __launch_bounds__(256) k_prep64_list(const BatchHeader* __restri
 template __global__ void k_forward<double, kN64, true>(const BatchHeader*, const PowRow<double>*);
 template __global__ void k_forward<double, kF64N[1], true, kF64CW[1]>(const BatchHeader*, const PowRow<double>*);
 template __global__ void k_forward<double, kF64N[2], false, kF64CW[2]>(const BatchHeader*, const PowRow<double>*);
-template __global__ void k_short_pipe64<kF64NS[2], 2>(const BatchHeader*, const PowRow<double>*);
-template __global__ void k_short_pipe64<kF64NS[3], 1, true>(const BatchHeader*, const PowRow<double>*);
+template __global__ void k_short_pipe64<kF64NS[2], 2>(const BatchHeader*);
+template __global__ void k_short_pipe64<kF64NS[3], 2>(const BatchHeader*);
 template __global__ void k_finalize<double>(const BatchHeader*);
 
 __device__ __forceinline__ double log10_of(const Partial& q) {
     if (q.S > 0.0 && isfinite(q.S))
-        return log10(q.S) + (double)(q.E - Num<double>::kLog2C) * 0.30102999566398119521;
+        return log10_scaled(q.S, q.E - Num<double>::kLog2C);
     return q.S == 0.0 ? -INFINITY : NAN;
 }
 
@@ -140,14 +143,13 @@ void launch_forward64(int id, const BatchHeader* H, const void* pow, int grid, c
     else if (id == 1) k_forward<double, kF64N[1], true, kF64CW[1]><<<grid, kF64CW[1] * 32, 0, s>>>(H, p);
     else k_forward<double, kN64, true><<<grid, kCtaThreads, 0, s>>>(H, p);
 }
-void launch_short_pipe64(int id, const BatchHeader* H, const void* pow, int grid, cudaStream_t s) {
-    const PowRow<double>* p = static_cast<const PowRow<double>*>(pow);
-    if (id == 3) k_short_pipe64<kF64NS[3], 1, true><<<grid, kShortThreads, 0, s>>>(H, p);
-    else k_short_pipe64<kF64NS[2], 2><<<grid, kShortThreads, 0, s>>>(H, p);
+void launch_short_pipe64(int id, const BatchHeader* H, int grid, cudaStream_t s) {
+    if (id == 3) k_short_pipe64<kF64NS[3], 2><<<grid, kShortThreads, 0, s>>>(H);
+    else k_short_pipe64<kF64NS[2], 2><<<grid, kShortThreads, 0, s>>>(H);
 }
 int occupancy_short_pipe64(int id) {
     int b = 0;
-    if (id == 3) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_short_pipe64<kF64NS[3], 1, true>, kShortThreads, 0);
+    if (id == 3) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_short_pipe64<kF64NS[3], 2>, kShortThreads, 0);
     else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_short_pipe64<kF64NS[2], 2>, kShortThreads, 0);
     return b > 0 ? b : 1;
 }

@@ -63,7 +63,7 @@ constexpr int kF64NS[kNumF64] = {8, 16, 16, 32};  // short teams: columns per la
 constexpr int kF64CW[kNumF64] = {16, 8, 8, 8};
 constexpr bool f64_pipelined(int id) { return id >= 2; }
 void launch_forward64(int id, const BatchHeader* H, const void* pow, int grid, cudaStream_t s);
-void launch_short_pipe64(int id, const BatchHeader* H, const void* pow, int grid, cudaStream_t s);
+void launch_short_pipe64(int id, const BatchHeader* H, int grid, cudaStream_t s);
 int occupancy_short_pipe64(int id);
 void launch_prep64_first(const BatchHeader* H, const PhredTables* T, int grid, cudaStream_t s);
 void launch_finalize64(const BatchHeader* H, int grid, cudaStream_t s);

@@ -546,7 +546,6 @@ struct phmm_ctx {
     DevBuf pow32[5];                        // N = 12, 16, 20, 24 (packed short), 32 (long)
     DevBuf pow64;                           // FP64 powers, N = 8 (variant 0, rescue, comparator)
     DevBuf pow64w;                          // FP64 powers, N = 16 (variants 1-3)
-    DevBuf pow64x;                          // FP64 powers, N = 32 (variant 3's short teams)
     int occ64v[kNumF64] = {1, 1, 1, 1};     // resident CTAs per SM of the FP64 forward variants
     int occ64s[kNumF64] = {1, 1, 1, 1};     // ... and of the pipelined FP64 short-team kernels
     // resident CTAs per SM of each kernel (long kind 5: resident clusters of the GPU)
@@ -653,7 +652,7 @@ int launch_sequence(phmm_ctx* ctx, Slot& S, int scal_id, int pack_id, int long_k
             CK(rec_on(S.ev_br[5], S.sb2));
             CK(cudaEventRecord(S.ev_join, S.sb2));
             CK(rec(S.ev_br[0]));
-            launch_short_pipe64(scal_id, H, scal_id == 3 ? ctx->pow64x.p : pw, ctx->sms * ctx->occ64s[scal_id], s);
+            launch_short_pipe64(scal_id, H, ctx->sms * ctx->occ64s[scal_id], s);
             CK(rec(S.ev_br[1]));
             CK(cudaStreamWaitEvent(s, S.ev_join, 0));
             S.br_timed = true;
@@ -837,14 +836,15 @@ std::vector<std::pair<int, int>> fp32_candidates(const phmm_config& cfg) {
 // FP64 plan of variant id (launch.h: kF64N columns per lane, kF64CW-warp CTAs); the
 // variant travels in scal_id.
 void make_plan64(const uint32_t* l, const uint32_t* k, const uint32_t* pr, uint32_t n, int id, Plan& P) {
-    make_plan(l, k, pr, n, kF64NS[id], 0, kF64N[id], P, 8, kF64CW[id]);
+    make_plan(l, k, pr, n, kF64NS[id], 0, kF64N[id], P, 8, kF64CW[id], false, false,
+              f64_pipelined(id) ? kSkewCost : TeamCost());
     P.scal_id = id;
     P.pack_id = -1;
     P.long_kind = 0;
     P.fp64 = true;
-    // the pipelined engine does about 6 FP64 operations per cell of a short team against
-    // 8 for the unfactored one
-    if (f64_pipelined(id)) P.cost -= 0.25 * (double)P.cells_br[0] * 8.0;
+    // the skewed engine does 5 FP64 operations per cell of a short team against 8 for the
+    // unfactored one
+    if (f64_pipelined(id)) P.cost -= 0.375 * (double)P.cells_br[0] * 8.0;
 }
 
 // Cluster kind: CTA items are taken kClusterCtas at a time, item g kClusterCtas + r by CTA
@@ -1688,9 +1688,6 @@ int phmm_create(const phmm_config* cfg, phmm_ctx** out) {
         build_pow_table<double>(kF64N[1], v);
         if (ensure(ctx->pow64w, v.size() * sizeof(v[0])) != cudaSuccess) return fail(PHMM_ECUDA);
         cudaMemcpy(ctx->pow64w.p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice);
-        build_pow_table<double>(kF64NS[3], v);
-        if (ensure(ctx->pow64x, v.size() * sizeof(v[0])) != cudaSuccess) return fail(PHMM_ECUDA);
-        cudaMemcpy(ctx->pow64x.p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice);
         for (int q = 0; q < kNumF64; ++q) ctx->occ64v[q] = occupancy_forward64(q);
         for (int q = 2; q < kNumF64; ++q) ctx->occ64s[q] = occupancy_short_pipe64(q);
         ctx->occ64 = ctx->occ64v[0];
@@ -1752,7 +1749,6 @@ void phmm_destroy(phmm_ctx* ctx) {
     for (auto& b : ctx->pow32) release(b);
     release(ctx->pow64);
     release(ctx->pow64w);
-    release(ctx->pow64x);
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
     if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
     delete ctx;

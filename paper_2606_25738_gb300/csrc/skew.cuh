@@ -1,4 +1,4 @@
-// Skewed FP32 engines: the row-wise recurrence of Eq. 7 with the lanes of a team one row
+// Skewed engines: the row-wise recurrence of Eq. 7 with the lanes of a team one row
 // apart instead of in step, so that the deletion chain needs no scan.
 //
 // Each lane owns N consecutive columns; lane t of a team works on row s - t at step s.  What it
@@ -21,6 +21,9 @@
 //    the first: 160 to 195 instructions a step, which leave slots for the boundary traffic; the
 //    strip takes 64 steps more than its rows.  On 60,000 uneven pairs the serial kind took 22.0
 //    ms against 25.6 ms with the scalar form (28.6 ms on the scan engine).
+// The scalar form also runs FP64 short teams, where the FP64 pipe (2.1 FMAs a cycle and SM) is the
+// bound and 5 operations a cell take the place of 6.5: 40 regions of short reads, 6.15 ms
+// against 6.65 ms on the scan engine, with 32 columns a lane (16: 10.8 ms).
 // With g constant (G10: gcp Phred 10 throughout, the T_II = T_DD = 0.1 that Section 2 fixes) the
 // D-hat chain reads one operand less.
 //
@@ -39,26 +42,32 @@ namespace phmm {
 // Range control as pipe_range(), with the drop of a column's max(M, J): J[r] = h J[r-1] +
 // M[r-1] keeps at least min(1, h) of it a row (prep: the largest -log2 h of the batch), which
 // lets R be about three times what the drop of max(M, I) allows.
+template <typename T = float>
 __device__ __forceinline__ PipeRange skew_range(const BatchHeader* __restrict__ H) {
     const uint32_t dg[4] = {H->skst->drop, H->dropgrow[1], H->dropgrow[2], H->dropgrow[3]};
-    return pipe_range(dg);
+    return pipe_range<T>(dg);
 }
 // gcp Phred 10 throughout the batch
 __device__ __forceinline__ bool skew_g10(const SkewStats* st) { return st->gcp_max == 10u && st->gcp_inv == 245u; }
 constexpr float kG10 = 0.1f;
 
 // 2^d for d <= 0: exact down to the smallest subnormal, then 0.
-__device__ __forceinline__ float pow2_down(int d) {
-    return d >= -126 ? Num<float>::pow2(d) : d >= -149 ? __uint_as_float(1u << (d + 149)) : 0.f;
+template <typename T = float>
+__device__ __forceinline__ T pow2_down(int d) {
+    if constexpr (std::is_same_v<T, float>)
+        return d >= -126 ? Num<float>::pow2(d) : d >= -149 ? __uint_as_float(1u << (d + 149)) : 0.f;
+    else
+        return d >= -1022 ? Num<double>::pow2(d) : d >= -1074 ? __longlong_as_double(1ll << (d + 1074)) : 0.0;
 }
 
 // The exponent side of a checkpoint (see above), common to both forms.  x: the lane's largest
 // |M|, |J|; keep: the lane holds its exponent (not started: C / k must stay in range; or done);
 // Eb: the exponent of what enters the team's first lane from a strip to its left (INT_MIN:
 // none).  Returns the new exponent.
-__device__ __forceinline__ int skew_exponent(float x, int E, uint32_t& flags, int lt, bool keep, int Eb,
+template <typename T>
+__device__ __forceinline__ int skew_exponent(T x, int E, uint32_t& flags, int lt, bool keep, int Eb,
                                              const PipeRange& rng) {
-    using NT = Num<float>;
+    using NT = Num<T>;
     const int e = NT::expo(x);
     const bool first = lt == 0;
     const bool has_left = !first || Eb != INT_MIN;
@@ -81,15 +90,18 @@ __device__ __forceinline__ int skew_exponent(float x, int E, uint32_t& flags, in
     return En;
 }
 // 2^sh as one or two exact factors (sh beyond twice the format's range: 0, or the largest).
-__device__ __forceinline__ void skew_factors(int sh, float& f, float& g) {
-    const int s1 = max(-126, min(sh, 126)), s2 = sh - s1;
-    f = Num<float>::pow2(s1);
-    g = s2 < -126 ? 0.f : Num<float>::pow2(min(s2, 126));
+template <typename T>
+__device__ __forceinline__ void skew_factors(int sh, T& f, T& g) {
+    using NT = Num<T>;
+    const int s1 = max(NT::kMinExp, min(sh, -NT::kMinExp)), s2 = sh - s1;
+    f = NT::pow2(s1);
+    g = s2 < NT::kMinExp ? T(0) : NT::pow2(min(s2, -NT::kMinExp));
 }
 // Scale of what arrives from the left, 2^(E_left - E) <= 1.
-__device__ __forceinline__ float skew_left_scale(int E, int lt, int Eb) {
+template <typename T = float>
+__device__ __forceinline__ T skew_left_scale(int E, int lt, int Eb) {
     const int El = __shfl_up_sync(kFull, E, 1);
-    return lt == 0 && Eb == INT_MIN ? 1.f : pow2_down((lt == 0 ? Eb : El) - E);
+    return lt == 0 && Eb == INT_MIN ? T(1) : pow2_down<T>((lt == 0 ? Eb : El) - E);
 }
 
 // Sum over the team's lanes (s: the lane's, FP64, in scale E), in the scale of the lane that
@@ -122,8 +134,9 @@ __device__ __forceinline__ SegOut skew_sum(double s, int E, int E0, uint32_t fla
 }
 
 // C / k of Eq. 1 in the scale of a lane with exponent E >= E0
-__device__ __forceinline__ float skew_init(const PipeRange& rng, int k, int E0, int E) {
-    return (float)(ldexp(1.0, rng.target) / (double)k) * pow2_down(E0 - E);
+template <typename T = float>
+__device__ __forceinline__ T skew_init(const PipeRange& rng, int k, int E0, int E) {
+    return (T)(ldexp(1.0, rng.target) / (double)k) * pow2_down<T>(E0 - E);
 }
 
 // Match masks of a lane's columns (Eq. 3), by read base code (4: N, matches everything), at
@@ -157,33 +170,34 @@ __device__ __forceinline__ void skew_masks(const uint8_t* __restrict__ hap, int 
 // ------------------------------------------------------------------------------------
 // Short teams (scalar form).
 // ------------------------------------------------------------------------------------
+template <typename T>
 struct SkewLane {
-    float m, j, d;               // left of the lane (the row above its row)
-    float pm, px, a, b, h, g, gp;  // the lane's row; gp: g of the row above (not used with G10)
-    float lsc;                   // 2^(E of the left lane - E)
+    T m, j, d;               // left of the lane (the row above its row)
+    T pm, px, a, b, h, g, gp;  // the lane's row; gp: g of the row above (not used with G10)
+    T lsc;                       // 2^(E of the left lane - E)
     int E;
 };
 
 // The lane's columns of one step; m, j, d: in the values left of the lane, out those at its
 // last column (of the row above this one), which the lane to the right takes at the next step.
-template <int N, bool G10>
-__device__ __forceinline__ void skew_row(float (&M)[N], float (&J)[N], SkewLane& L, uint32_t mask) {
-    const float gp = G10 ? kG10 : L.gp;
-    const float mo = M[N - 1], jo = J[N - 1];
+template <typename T, int N, bool G10>
+__device__ __forceinline__ void skew_row(T (&M)[N], T (&J)[N], SkewLane<T>& L, uint32_t mask) {
+    const T gp = G10 ? (T)kG10 : L.gp;
+    const T mo = M[N - 1], jo = J[N - 1];
     // column q's old M and J have their last uses (column q + 1's partial t and D-hat, its own
     // J) before its new M is formed, so the new values take the old ones' registers
-    float t = fmaf(L.a, L.m, L.j);
-    float dA = L.d, dB = fmaf(gp, L.d, L.m);
+    T t = fma(L.a, L.m, L.j);
+    T dA = L.d, dB = fma(gp, L.d, L.m);
 #pragma unroll
     for (int q = 0; q < N; ++q) {
-        const float u = fmaf(L.b, dA, t);
-        const float o = M[q];
+        const T u = fma(L.b, dA, t);
+        const T o = M[q];
         if (q + 1 < N) {
             dA = dB;
-            dB = fmaf(gp, dB, o);
-            t = fmaf(L.a, o, J[q]);
+            dB = fma(gp, dB, o);
+            t = fma(L.a, o, J[q]);
         }
-        J[q] = fmaf(L.h, J[q], o);
+        J[q] = fma(L.h, J[q], o);
         M[q] = (((mask >> q) & 1u) ? L.pm : L.px) * u;
     }
     L.m = mo;
@@ -196,36 +210,36 @@ __device__ __forceinline__ void skew_row(float (&M)[N], float (&J)[N], SkewLane&
 // steps plain0 .. plain1.  A lane starts as M = 0, J = C / k and keeps that before row 1 (P' = 0,
 // h = 1); row 1's record has h = 0, so that J = 0 and M = P' C / k follow; after row l a lane
 // does nothing.  Records come through L1, one step ahead.
-template <int N, bool G10>
-__device__ SegOut team_run_skew(const Rec32J* __restrict__ rec, int l, int steps, int plain0, int plain1,
+template <typename T, int N, bool G10>
+__device__ SegOut team_run_skew(const typename Num<T>::RecJ* __restrict__ rec, int l, int steps, int plain0, int plain1,
                                 const uint8_t* __restrict__ hap, int k, int lt, int tlast, const PipeRange& rng,
                                 uint32_t* sm) {
     static_assert(N <= 32, "match masks hold 32 columns");
     uint32_t flags = rng.ok ? 0u : PF_DEGEN, mflags = 0;
     skew_masks<N, false>(hap, k, lt * N, sm, flags);
-    const int E0 = Num<float>::kLog2C - rng.target;
-    const float cin = l > 0 && k > 0 ? skew_init(rng, k, E0, E0) : 0.f;
-    float M[N], J[N];
+    const int E0 = Num<T>::kLog2C - rng.target;
+    const T cin = l > 0 && k > 0 ? skew_init<T>(rng, k, E0, E0) : T(0);
+    T M[N], J[N];
 #pragma unroll
     for (int q = 0; q < N; ++q) {
-        M[q] = 0.f;
+        M[q] = T(0);
         J[q] = cin;
     }
-    SkewLane L;
-    L.m = L.d = L.g = 0.f;
+    SkewLane<T> L;
+    L.m = L.d = L.g = T(0);
     L.j = cin;
-    L.lsc = 1.f;
+    L.lsc = T(1);
     L.E = E0;
     const int l1 = max(l, 1) - 1;
     int r = 1 - lt;  // the lane's row
-    Rec32J nxt = load_recj(rec + max(0, min(r - 1, l1)));
+    typename Num<T>::RecJ nxt = load_recj(rec + max(0, min(r - 1, l1)));
     int ck = rng.R;  // checkpoint after step ck
     // EDGE: some lane is before row 2 or past row l
     auto run = [&](auto edge, int& s, int e) {
         constexpr bool EDGE = decltype(edge)::value;
 #pragma unroll 1
         for (; s <= e; ++s, ++r) {
-            const float um = __shfl_up_sync(kFull, L.m, 1), uj = __shfl_up_sync(kFull, L.j, 1),
+            const T um = __shfl_up_sync(kFull, L.m, 1), uj = __shfl_up_sync(kFull, L.j, 1),
                         ud = __shfl_up_sync(kFull, L.d, 1);
             L.pm = nxt.pm;
             L.px = nxt.px;
@@ -236,19 +250,19 @@ __device__ SegOut team_run_skew(const Rec32J* __restrict__ rec, int l, int steps
                 L.gp = L.g;
                 L.g = nxt.g;
             }
-            mflags |= nxt.meta;
-            const uint32_t mask = sm[(nxt.meta & META_CODE_MASK) * 32];
+            mflags |= (uint32_t)nxt.meta;
+            const uint32_t mask = sm[((uint32_t)nxt.meta & META_CODE_MASK) * 32];
             if constexpr (EDGE) {
                 if (r < 1) {  // not started: hold
-                    L.pm = L.px = 0.f;
-                    L.h = 1.f;
+                    L.pm = L.px = T(0);
+                    L.h = T(1);
                 }
             }
             if (!EDGE || r <= l) {
-                L.m = lt == 0 ? 0.f : um * L.lsc;
-                L.j = lt == 0 ? (EDGE && r == 1 ? cin : 0.f) : uj * L.lsc;
-                L.d = lt == 0 ? 0.f : ud * L.lsc;
-                skew_row<N, G10>(M, J, L, mask);
+                L.m = lt == 0 ? T(0) : um * L.lsc;
+                L.j = lt == 0 ? (EDGE && r == 1 ? cin : T(0)) : uj * L.lsc;
+                L.d = lt == 0 ? T(0) : ud * L.lsc;
+                skew_row<T, N, G10>(M, J, L, mask);
             }
             nxt = load_recj(rec + (EDGE ? max(0, min(r, l1)) : min(r, l1)));
         }
@@ -262,15 +276,15 @@ __device__ SegOut team_run_skew(const Rec32J* __restrict__ rec, int l, int steps
         else run(std::true_type{}, s, e);
         if (s > ck && s <= steps) {
             ck += rng.R;
-            float x0 = 0.f, x1 = 0.f;
+            T x0 = 0, x1 = 0;
 #pragma unroll
             for (int q = 0; q < N; ++q) {
-                if (q & 1) x1 = fmaxf(x1, fmaxf(fabsf(M[q]), fabsf(J[q])));
-                else x0 = fmaxf(x0, fmaxf(fabsf(M[q]), fabsf(J[q])));
+                if (q & 1) x1 = fmax(x1, fmax(fabs(M[q]), fabs(J[q])));
+                else x0 = fmax(x0, fmax(fabs(M[q]), fabs(J[q])));
             }
-            const int En = skew_exponent(fmaxf(x0, x1), L.E, flags, lt, r - 1 < 1 || r - 1 > l, INT_MIN, rng);
+            const int En = skew_exponent(fmax(x0, x1), L.E, flags, lt, r - 1 < 1 || r - 1 > l, INT_MIN, rng);
             if (En != L.E) {
-                float f, g;
+                T f, g;
                 skew_factors(L.E - En, f, g);
                 for (;;) {
 #pragma unroll
@@ -281,13 +295,13 @@ __device__ SegOut team_run_skew(const Rec32J* __restrict__ rec, int l, int steps
                     L.m *= f;
                     L.j *= f;
                     L.d *= f;
-                    if (g == 1.f) break;  // one factor, nearly always
+                    if (g == T(1)) break;  // one factor, nearly always
                     f = g;
-                    g = 1.f;
+                    g = T(1);
                 }
                 L.E = En;
             }
-            L.lsc = skew_left_scale(L.E, lt, INT_MIN);
+            L.lsc = skew_left_scale<T>(L.E, lt, INT_MIN);
         }
     }
     double s = 0.0;

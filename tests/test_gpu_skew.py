@@ -1,4 +1,4 @@
-"""The skewed FP32 engine (csrc/skew.cuh) at its edges, against the CPU oracle: reads of one
+"""The skewed engines (csrc/skew.cuh) at its edges, against the CPU oracle: reads of one
 row and around the team's and the strip's start and end (a lane starts one step after its
 left neighbour), widths around multiples of a lane and of a strip, gcp Phred 10 throughout
 (a constant of the code) and other or mixed values, insertion qualities that jump between rows.
@@ -66,3 +66,22 @@ def test_strips(phmm, kind, gcp, ins):
               (63, 5000), (64, 1100), (65, 3000), (96, 1056), (97, 1057), (400, 7000), (1500, 1100), (2000, 4100)]
     st = _check(phmm, _pairs(shapes, gcp, ins, 6), flags=flag)
     assert st["long_kernel"] in {"serial": (3,), "wave": (6, 7, 8), "wave16": (8,)}[kind]
+
+
+# FP64: every path through the matrices adds positive terms, with at most 16 roundings (2^-53 each)
+# per row or column in the engine and as many in the oracle, plus one of log10 L
+@pytest.mark.parametrize("gcp,ins", [("ten", "flat"), ("other", "jumps"), ("mixed", "flat")])
+@pytest.mark.parametrize("variant", [4, 5])
+def test_short_teams_fp64(phmm, variant, gcp, ins):
+    N = {4: 16, 5: 32}[variant]
+    w = 32 * N
+    shapes = [(1, 1), (1, w), (2, N), (2, N + 1), (3, 2 * N - 1), (31, w), (32, w - 1), (33, w), (34, w - N), (35, 5),
+              (64, N * 16), (65, N * 16 + 1), (150, 431), (700, 3 * N), (1500, 90)]
+    b = _pairs(shapes, gcp, ins, 5)
+    with phmm.Context(precision="fp64", variant={4: "pipe", 5: "pipe2"}[variant]) as ctx:
+        out, flags, rc, st = ctx.run(b)
+    ref = oracle.batch(b)
+    l, k = W.pair_lengths(b)
+    tol = 32.0 * (l + k) * 2.0 ** -53 / np.log(10.0) + np.abs(ref) * 2.0 ** -51
+    assert rc == 0 and not np.any(flags & 0x79) and st["short_kernel"] == {4: 2, 5: 3}[variant]
+    assert np.all(np.abs(out - ref) <= tol), np.max(np.abs(out - ref) / tol)
