@@ -118,15 +118,13 @@ typedef struct {
                                  teams; 2 = scalar teams only (lean or pipelined engine);
                                  3 = lean scalar engine only; 4 = pipelined scalar engine
                                  only (the next row's scan-independent work overlaps the
-                                 deletion scan); 5 = pipelined engine with each lane's two
-                                 column halves in packed FP32 pairs; 6 = its lean form
-                                 (the next row's partials formed inside the row, records
-                                 and carry powers read from L1: four CTAs per SM).  With
-                                 PHMM_PREC_FP64, 4 fixes the pipelined FP64 variant with
-                                 16-column short teams (pairs up to 512 columns on the
-                                 J-form engine, six FP64 operations per cell), 5 or 6 the
-                                 one with 32-column fused teams (pairs up to 1024
-                                 columns) */
+                                 deletion scan); 5 = scalar teams on skewed lanes (each lane
+                                 one row behind its left neighbour: no deletion scan); 6 =
+                                 the same in four CTAs per SM.  With PHMM_PREC_FP64, 4
+                                 fixes the skewed FP64 variant with 16-column short teams
+                                 (pairs up to 512 columns; J-form records, five FP64
+                                 operations per cell), 5 or 6 the one with 32-column teams
+                                 (pairs up to 1024 columns) */
     double fp32_tolerance;    /* largest |error of log10 L| accepted from the FP32 pass
                                  (0 = 1e-3): with PHMM_PREC_FP32_RESCUE a pair whose
                                  a-priori FP32 rounding bound exceeds it is recomputed in

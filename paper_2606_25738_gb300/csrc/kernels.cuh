@@ -738,6 +738,30 @@ k_forward_wave(const BatchHeader* __restrict__ H) {
     else wave_items<N, false>(H, rng, stage[threadIdx.x >> 5]);
 }
 
+// The same for FP64 (mode FP64's multi-warp pairs), a strip of 128 N columns on each CTA.
+template <int N>
+__global__ void __launch_bounds__(kStrip64Lanes)
+k_forward_wave64(const BatchHeader* __restrict__ H) {
+    __shared__ SkewStage64 st;
+    const PipeRange rng = skew_range<double>(H);
+    const uint32_t n_c = H->n_citems;
+    const uint32_t tag = *H->wave_epoch;
+    for (;;) {
+        if (threadIdx.x == 0) st.item = atomicAdd(&H->counters[0], 1u);
+        __syncthreads();
+        const uint32_t wi = st.item;
+        if (wi >= n_c) break;
+        const CtaPair cp = H->cpairs[H->citems[wi].first];
+        const PairDesc d = H->desc[cp.pair];
+        const uint32_t s = cp.strip, S = cp.nstrip;
+        const Partial p = strip_run_skew64<N>(H->rec64j + d.roff, (int)d.l, H->hap_bases + d.hoff, (int)d.k, (int)s, rng,
+                                              s > 0 ? H->wbnd + cp.bnd_in : nullptr,
+                                              s + 1 < S ? H->wbnd + cp.bnd_out : nullptr, st, tag, H->status);
+        if (threadIdx.x == 0) write_strip_part(H, cp.pair, s, S, cp.extra_base, p);
+        __syncthreads();
+    }
+}
+
 // Team lookup of a warp item: this lane's team (first lane, size, pairs) and the scan
 // steps of the widest team.
 struct TeamOf {

@@ -1,6 +1,8 @@
 // FP64 instantiation: prep of FP64 records (all reads, or only the reads of pairs
 // selected for rescue), the FP64 forward kernel, the rescue pass, the one-launch-per-
 // pair comparator kernel and finalize.
+#include <algorithm>
+
 #include "kernels.cuh"
 #include "launch.h"
 
@@ -16,6 +18,7 @@ __global__ void __launch_bounds__(256) k_prep64_all(const BatchHeader* __restric
     __shared__ PhredTables T;
     load_tables(TG, T);
     __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *H->wave_epoch = *H->wave_epoch % kWaveTags + 1u;
     uint32_t dmax = 0, gmax = 0, jmax = 0, hmax = 0, hdrop = 0;
     const uint64_t n = H->n_read_bases;
     Rec64J* const rj = H->rec64j;
@@ -85,6 +88,7 @@ template __global__ void k_forward<double, kF64N[1], true, kF64CW[1]>(const Batc
 template __global__ void k_forward<double, kF64N[2], false, kF64CW[2]>(const BatchHeader*, const PowRow<double>*);
 template __global__ void k_short_pipe64<kF64NS[2], 2>(const BatchHeader*);
 template __global__ void k_short_pipe64<kF64NS[3], 2>(const BatchHeader*);
+template __global__ void k_forward_wave64<kF64WaveN>(const BatchHeader*);
 template __global__ void k_finalize<double>(const BatchHeader*);
 
 __device__ __forceinline__ double log10_of(const Partial& q) {
@@ -100,6 +104,7 @@ k_rescue(const BatchHeader* __restrict__ H, const PowRow<double>* __restrict__ p
     __shared__ CtaShared<double> sh;
     const int R = checkpoint_interval<double>(H->dropgrow);
     const uint32_t n = H->counters[2];
+    if (blockIdx.x >= H->rbnd_ctas) return;
     unsigned long long* scratch = H->rbnd + (size_t)blockIdx.x * 2 * H->rbnd_words_per_cta;
     for (;;) {
         if (threadIdx.x == 0) sh.item = atomicAdd(&H->counters[3], 1u);
@@ -112,6 +117,13 @@ k_rescue(const BatchHeader* __restrict__ H, const PowRow<double>* __restrict__ p
         if (threadIdx.x == 0) {
             uint8_t of = (uint8_t)((H->out_flags[p] & 0x78u) | 0x1u | 0x4u);
             const double v = log10_of(q);
+            if (H->mode == 1 && H->desc[p].k > H->wave64_k) {
+                // the unfactored engine is a wide FP64 pair's own: what the strips could not
+                // hold is no property of the pair
+                of = 0x4u;
+                if (q.flags & PF_DANGER) of |= 0x9u;
+                if ((q.flags & PF_NONFINITE) || !isfinite(q.S)) of |= 0x11u;
+            }
             if (q.flags & PF_RESCALED) of |= 0x2u;
             if (q.flags & (PF_TIMEOUT | PF_BAD)) of |= 0x80u;
             if (!isfinite(q.S)) atomicOr(H->status, ST_NONFINITE);
@@ -146,6 +158,14 @@ void launch_forward64(int id, const BatchHeader* H, const void* pow, int grid, c
 void launch_short_pipe64(int id, const BatchHeader* H, int grid, cudaStream_t s) {
     if (id == 3) k_short_pipe64<kF64NS[3], 2><<<grid, kShortThreads, 0, s>>>(H);
     else k_short_pipe64<kF64NS[2], 2><<<grid, kShortThreads, 0, s>>>(H);
+}
+void launch_forward_wave64(const BatchHeader* H, int grid, cudaStream_t s) {
+    k_forward_wave64<kF64WaveN><<<grid, kStrip64Lanes, 0, s>>>(H);
+}
+int occupancy_forward_wave64() {
+    int b = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_forward_wave64<kF64WaveN>, kStrip64Lanes, 0);
+    return std::max(1, std::min(b, kF64WaveCtas));
 }
 int occupancy_short_pipe64(int id) {
     int b = 0;

@@ -52,19 +52,25 @@ void launch_prep64_list(const BatchHeader* H, const PhredTables* T, int grid, cu
 // FP64 forward kernels (precision FP64): variant 0 = N 8 in 16-warp CTAs, 1 = N 16 in
 // 8-warp CTAs (fewer padded columns and per-row operations per cell for pairs up to 512
 // columns; the same 4096-column CTA width for wider pairs), both on the unfactored engine;
-// 2 = short pairs (up to 512 columns) on the pipelined FP64 engine (J-form records, six
-// FP64 operations per cell) and multi-warp pairs on the unfactored engine in 8-warp CTAs
-// (CTA items only), two concurrent branches; 3 = as 2 with 32-column short teams (pairs
-// up to 1024 columns) on the fused pipelined engine (no partials array).  pow: the FP64
-// power table of that N (kF64N for the multi-warp kernel, kF64NS for the short teams).
+// 2 = short pairs (up to 512 columns) on the skewed engine in FP64 (J-form records, five
+// FP64 operations per cell) and multi-warp pairs on its strips or on the unfactored engine in
+// 8-warp CTAs (CTA items only), two concurrent branches; 3 = as 2 with 32-column short teams
+// (pairs up to 1024 columns).  pow: the FP64 power table of kF64N columns.
 constexpr int kNumF64 = 4;
 constexpr int kF64N[kNumF64] = {8, 16, 16, 16};   // multi-warp (CTA) kernel: columns per lane
 constexpr int kF64NS[kNumF64] = {8, 16, 16, 32};  // short teams: columns per lane
 constexpr int kF64CW[kNumF64] = {16, 8, 8, 8};
 constexpr bool f64_pipelined(int id) { return id >= 2; }
+// Variants 2 and 3: multi-warp pairs as waves of strips of 512 columns on the skewed engine
+// (k_forward_wave64), where their boundary rows fit (32 bytes a row and strip) in what
+// phmm_batch_footprint promises, else on CTAs (24 pairs of 1 to 10 kbp: 11 ms against 72 to 84 ms).
+constexpr int kF64WaveN = 4;  // columns per lane, 128 lanes
+constexpr int kF64WaveCtas = 1;  // resident CTAs per SM: two share its FP64 units, 16 ms
 void launch_forward64(int id, const BatchHeader* H, const void* pow, int grid, cudaStream_t s);
 void launch_short_pipe64(int id, const BatchHeader* H, int grid, cudaStream_t s);
 int occupancy_short_pipe64(int id);
+void launch_forward_wave64(const BatchHeader* H, int grid, cudaStream_t s);
+int occupancy_forward_wave64();
 void launch_prep64_first(const BatchHeader* H, const PhredTables* T, int grid, cudaStream_t s);
 void launch_finalize64(const BatchHeader* H, int grid, cudaStream_t s);
 void launch_rescue64(const BatchHeader* H, const void* pow, int grid, cudaStream_t s);

@@ -214,6 +214,8 @@ struct BatchHeader {
     uint64_t n_bnd_words;
     unsigned long long *rbnd;   // rescue / single-launch scratch: 2 boundaries per CTA
     uint64_t rbnd_words_per_cta;
+    uint32_t rbnd_ctas;         // CTAs that have one (the others have nothing to do)
+    uint32_t wave64_k;          // FP64: wider pairs run on the skewed strips; else 0xffffffff
     float4 *wbnd;            // strips of the wave kind: each strip's right boundary (l rows)
     uint64_t wbnd_rows;      // rows the buffer holds (k_reset clears it when the tags wrap)
     uint32_t *wave_epoch;    // tag of this launch's boundary rows, 1 .. kWaveTags (k_prep32 steps it)

@@ -547,7 +547,8 @@ struct phmm_ctx {
     DevBuf pow64;                           // FP64 powers, N = 8 (variant 0, rescue, comparator)
     DevBuf pow64w;                          // FP64 powers, N = 16 (variants 1-3)
     int occ64v[kNumF64] = {1, 1, 1, 1};     // resident CTAs per SM of the FP64 forward variants
-    int occ64s[kNumF64] = {1, 1, 1, 1};     // ... and of the pipelined FP64 short-team kernels
+    int occ64s[kNumF64] = {1, 1, 1, 1};     // ... and of the skewed FP64 short-team kernels
+    int occ64w = 1;                         // ... and of k_forward_wave64
     // resident CTAs per SM of each kernel (long kind 5: resident clusters of the GPU)
     int occ_packed[kNumPacked] = {}, occ_scalar[kNumScalar] = {}, occ_longk[kNumLong] = {1, 1, 1, 1, 1, 1, 1, 1, 1}, occ64 = 1;
     std::map<uint64_t, std::array<int, 3>> tuned;  // batch signature -> (scalar id, packed id, long kind)
@@ -643,12 +644,13 @@ int launch_sequence(phmm_ctx* ctx, Slot& S, int scal_id, int pack_id, int long_k
         CK(rec(S.ev_fwd0));
         const void* pw = scal_id == 0 ? ctx->pow64.p : ctx->pow64w.p;
         if (f64_pipelined(scal_id)) {
-            // two branches: short teams on the pipelined engine here, multi-warp CTA items
-            // on the unfactored engine on sb2
+            // two branches: short teams on the skewed engine here, multi-warp pairs on sb2 (the
+            // strips of that engine, or CTA items on the unfactored one)
             CK(cudaEventRecord(S.ev_fork, s));
             CK(cudaStreamWaitEvent(S.sb2, S.ev_fork, 0));
             CK(rec_on(S.ev_br[4], S.sb2));
-            launch_forward64(2, H, pw, ctx->sms * ctx->occ64v[2], S.sb2);
+            if (long_kind == 6) launch_forward_wave64(H, ctx->sms * ctx->occ64w, S.sb2);
+            else launch_forward64(2, H, pw, ctx->sms * ctx->occ64v[2], S.sb2);
             CK(rec_on(S.ev_br[5], S.sb2));
             CK(cudaEventRecord(S.ev_join, S.sb2));
             CK(rec(S.ev_br[0]));
@@ -776,6 +778,7 @@ void plan_header(const Slot& S, const Plan& P, BatchHeader& hh) {
     hh.sbnd = (float4*)S.sbnd.p;
     hh.sbnd_rows = S.sbnd_rows;
     hh.sbnd_warps = S.sbnd_warps;
+    hh.wave64_k = P.fp64 && P.long_kind == 6 ? 32u * (uint32_t)kF64NS[P.scal_id] : 0xffffffffu;
     hh.wbnd = (float4*)S.wbnd.p;
     hh.wbnd_rows = S.wbnd.cap / sizeof(float4);
     if (!P.fp64) {
@@ -835,16 +838,24 @@ std::vector<std::pair<int, int>> fp32_candidates(const phmm_config& cfg) {
 
 // FP64 plan of variant id (launch.h: kF64N columns per lane, kF64CW-warp CTAs); the
 // variant travels in scal_id.
-void make_plan64(const uint32_t* l, const uint32_t* k, const uint32_t* pr, uint32_t n, int id, Plan& P) {
-    make_plan(l, k, pr, n, kF64NS[id], 0, kF64N[id], P, 8, kF64CW[id], false, false,
+// wave: multi-warp pairs of the skewed variants as waves (long_kind 6) rather than CTA items
+void make_plan64(const uint32_t* l, const uint32_t* k, const uint32_t* pr, uint32_t n, int id, Plan& P,
+                 bool wave = false) {
+    wave = wave && f64_pipelined(id);
+    make_plan(l, k, pr, n, kF64NS[id], 0, wave ? 4 * kF64WaveN : kF64N[id], P, 8, wave ? 1 : kF64CW[id], false, wave,
               f64_pipelined(id) ? kSkewCost : TeamCost());
     P.scal_id = id;
     P.pack_id = -1;
-    P.long_kind = 0;
+    P.long_kind = wave ? 6 : 0;
     P.fp64 = true;
-    // the skewed engine does 5 FP64 operations per cell of a short team against 8 for the
-    // unfactored one
-    if (f64_pipelined(id)) P.cost -= 0.375 * (double)P.cells_br[0] * 8.0;
+    // the skewed engine does 5 FP64 operations per cell against 8 for the unfactored one
+    if (f64_pipelined(id)) P.cost -= 0.375 * (double)(P.cells_br[0] + (wave ? P.cells_br[2] : 0)) * 8.0;
+    if (!wave) return;
+    P.wave_rows *= 2;  // a boundary row takes two float4
+    for (CtaPair& cp : P.cpairs) {
+        if (cp.bnd_in != kNoBnd) cp.bnd_in *= 2;
+        if (cp.bnd_out != kNoBnd) cp.bnd_out *= 2;
+    }
 }
 
 // Cluster kind: CTA items are taken kClusterCtas at a time, item g kClusterCtas + r by CTA
@@ -1119,6 +1130,7 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
             // smaller plan cost), measured below for large batches
             const uint64_t sig = batch_signature(L.data(), K.data(), pr, np, ctx->cfg);
             auto hit = ctx->tuned.find(sig);
+            const bool waves = !(ctx->cfg.flags & PHMM_F_LAUNCH_PER_PAIR);
             // forced: cols_per_lane 8 / 16 = the unfactored variants, kernel_variant 4 (the
             // pipelined engine, 16-column teams) = variant 2, 5 or 6 (32-column fused
             // teams) = variant 3
@@ -1126,18 +1138,17 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
                              : ctx->cfg.cols_per_lane == kF64N[0] ? 0
                              : ctx->cfg.cols_per_lane == kF64N[1] ? 1 : -1;
             if (forced >= 0) {
-                make_plan64(L.data(), K.data(), pr, np, forced, P);
+                make_plan64(L.data(), K.data(), pr, np, forced, P, waves);
             } else if (hit != ctx->tuned.end()) {
-                make_plan64(L.data(), K.data(), pr, np, hit->second[0], P);
+                make_plan64(L.data(), K.data(), pr, np, hit->second[0], P, waves);
             } else {
-                make_plan64(L.data(), K.data(), pr, np, 0, P);
-                for (int id = 1; id < kNumF64; ++id) {
+                tune64 = !(ctx->cfg.flags & PHMM_F_NO_TUNE) && waves && cells >= kTuneMinCells;
+                make_plan64(L.data(), K.data(), pr, np, tune64 ? 3 : 0, P, waves);
+                for (int id = 1; id < kNumF64 && !tune64; ++id) {
                     Plan c;
-                    make_plan64(L.data(), K.data(), pr, np, id, c);
+                    make_plan64(L.data(), K.data(), pr, np, id, c, waves);
                     if (c.cost < P.cost) P = std::move(c);
                 }
-                tune64 = !(ctx->cfg.flags & PHMM_F_NO_TUNE) && !(ctx->cfg.flags & PHMM_F_LAUNCH_PER_PAIR) &&
-                         cells >= kTuneMinCells;
                 tune_sig = sig;
             }
         } else {
@@ -1196,8 +1207,14 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     };
     uint32_t lmax_b = sc.lmax;
     for (uint32_t p = 0; p < np && !on_dev; ++p) lmax_b = std::max(lmax_b, L[p]);
-    const uint64_t rb_words = (uint64_t)lmax_b * 8;  // FP64 boundary: 8 words per row
-    const int rescue_ctas = ctx->sms * ctx->occ64;
+    // scratch of the FP64 pass: two boundaries (8 words a row) for each CTA that may get a pair;
+    // FP64 mode knows on the host whether a pair is wider than its CTA
+    uint64_t rb_words = (uint64_t)lmax_b * 8;
+    uint64_t rescue_ctas = (uint64_t)ctx->sms * ctx->occ64;
+    if (!fp32) {
+        rescue_ctas = std::min<uint64_t>(rescue_ctas, std::max(np, 1u));
+        if (np == 0 || *std::max_element(K.begin(), K.end()) <= (uint32_t)kCtaWarps * 32u * kN64) rb_words = 0;
+    }
     const uint64_t rb_bytes = (uint64_t)rescue_ctas * 2 * rb_words * 8ull + 16;
     auto foot_of = [&]() {
         need32 = need32j = false;
@@ -1246,6 +1263,15 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
             plan_of(si, pi, lk, P);
             foot = foot_of();
         }
+    }
+    // FP64 waves likewise, else CTA strips
+    bool wave64 = !fp32 && P.long_kind == 6;
+    if (!reuse && wave64 &&
+        foot > std::min<uint64_t>(ctx->budget, footprint_bound(ctx, nbases, nhb, nr, nh, np, L.data(), K.data()))) {
+        const int id = P.scal_id;
+        make_plan64(L.data(), K.data(), pr, np, id, P);
+        foot = foot_of();
+        wave64 = false;
     }
     if (foot > ctx->budget) return PHMM_ENOMEM;
     if (foot + ctx->inflight_foot > ctx->budget) return PHMM_EBUSY;  // admissible once others retire
@@ -1326,6 +1352,7 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     hh.n_bnd_words = P.bnd_words;
     hh.rbnd = (unsigned long long*)S->rbnd.p;
     hh.rbnd_words_per_cta = rb_words;
+    hh.rbnd_ctas = (uint32_t)rescue_ctas;
     hh.l_max = lmax_b;
     hh.force_rescue = (ctx->cfg.flags & PHMM_F_FORCE_RESCUE) ? 1u : 0u;
     hh.tol32 = ctx->cfg.fp32_tolerance > 0.0 ? ctx->cfg.fp32_tolerance : 1e-3;
@@ -1356,18 +1383,19 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
         int best = P.scal_id;
         for (int id = 0; id < kNumF64; ++id) {
             Plan c;
-            make_plan64(L.data(), K.data(), pr, np, id, c);
+            make_plan64(L.data(), K.data(), pr, np, id, c, wave64);
             if (c.n_too_long) continue;
             CK(upload_plan(*S, c, cs));
             CK(ensure(S->parts, (np + c.n_extra) * sizeof(Partial)));
             CK(ensure(S->bnd, c.bnd_words * 8ull));
+            CK(ensure_serial(ctx, *S, c));
             hh.parts = (Partial*)S->parts.p;
             plan_header(*S, c, hh);
             CK(cudaMemcpyAsync(S->hdr.p, &hh, sizeof(hh), cudaMemcpyHostToDevice, cs));
             CK(cudaStreamSynchronize(cs));
             float ms = 1e30f;
             for (int rep = 0; rep < 2; ++rep) {
-                const int rc = launch_sequence(ctx, *S, id, -1, 0, false);
+                const int rc = launch_sequence(ctx, *S, id, -1, c.long_kind, false);
                 if (rc != PHMM_OK) return rc;
                 CK(cudaStreamSynchronize(S->sm));
                 float m1 = 0.f;
@@ -1384,10 +1412,11 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
             }
         }
         ctx->tuned[tune_sig] = {best, -1, 0};
-        make_plan64(L.data(), K.data(), pr, np, best, P);
+        make_plan64(L.data(), K.data(), pr, np, best, P, wave64);
         CK(upload_plan(*S, P, cs));
         CK(ensure(S->parts, (np + P.n_extra) * sizeof(Partial)));
         CK(ensure(S->bnd, P.bnd_words * 8ull));
+        CK(ensure_serial(ctx, *S, P));
         hh.parts = (Partial*)S->parts.p;
         plan_header(*S, P, hh);
         CK(cudaMemcpyAsync(S->hdr.p, &hh, sizeof(hh), cudaMemcpyHostToDevice, cs));
@@ -1690,6 +1719,7 @@ int phmm_create(const phmm_config* cfg, phmm_ctx** out) {
         cudaMemcpy(ctx->pow64w.p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice);
         for (int q = 0; q < kNumF64; ++q) ctx->occ64v[q] = occupancy_forward64(q);
         for (int q = 2; q < kNumF64; ++q) ctx->occ64s[q] = occupancy_short_pipe64(q);
+        ctx->occ64w = occupancy_forward_wave64();
         ctx->occ64 = ctx->occ64v[0];
     }
     ctx->slots.resize(ctx->cfg.max_inflight);

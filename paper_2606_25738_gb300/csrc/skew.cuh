@@ -413,9 +413,6 @@ constexpr int kWaveBlock = 16;  // boundary rows taken at a time
 // WAVE: the left strip runs at the same time on another warp (boundary rows tagged `tag`);
 // else its boundary is complete.  in: the left strip's boundary (index = row, 1 .. l - 1),
 // null for none; out: this strip's, null for none.
-// WAVE: the left strip runs at the same time on another warp (boundary rows tagged `tag`);
-// else its boundary is complete.  in: the left strip's boundary (index = row, 1 .. l - 1),
-// null for none; out: this strip's, null for none.
 template <int N, bool WAVE, bool G10>
 __device__ SegOut strip_run_skew(const Rec32J* __restrict__ rec, int l, const uint8_t* __restrict__ hap, int k,
                                  int strip, const PipeRange& rng, const float4* in, float4* out, SkewStage& st,
@@ -649,6 +646,323 @@ __device__ SegOut strip_run_skew(const Rec32J* __restrict__ rec, int l, const ui
         if (q + H < nvalid) s += (double)J[q].y;
     }
     return skew_sum(s, L.E, E0, flags, lane, 31);
+}
+
+// ------------------------------------------------------------------------------------
+// FP64 strips of wide pairs (scalar form): a CTA of four warps runs 128 N columns, thread t on
+// row s - t at step s.  A scheduler's FP64 unit takes about 60 cycles for one warp's FMA, so a
+// strip's step lasts as long as its warps' 5 N operations each: four warps side by side, with few
+// columns a lane, advance a row chain four times as fast as one warp with all of them.  They
+// step together: a barrier a step, and the last lane of a warp hands over through shared memory.
+// 24 pairs of 1 to 10 kbp: 10.9 ms with 4 columns a lane (3: 10.9, 2: 11.9), 17.3 ms on strips of
+// one warp with 8, 72 to 84 ms on CTAs of the unfactored engine; 1600 cycles a step, of which the
+// FP64 unit takes 1200.
+// As strip_run_skew<.., WAVE> otherwise, with one virtual lane a lane: checkpoints 128 steps earlier
+// than the left strip's, and a boundary row of 32 bytes, two 16-byte accesses that both carry
+// the tag (M and half of J; the other half and D-hat).
+// ------------------------------------------------------------------------------------
+constexpr int kStrip64Warps = 4, kStrip64Lanes = 32 * kStrip64Warps;
+struct SkewStage64 {
+    double2 pp[2 * kStrip64Lanes], ab[2 * kStrip64Lanes], hg[2 * kStrip64Lanes];  // pm px, a b, h g
+    uint32_t meta[2 * kStrip64Lanes];
+    uint4 bndA[64], bndB[64];                                     // boundary rows (warp 0)
+    double xch[2][kStrip64Warps][4];                              // a warp's last m, j, d by step parity
+    int E[kStrip64Warps];
+    double S[kStrip64Warps];                                      // the warps' sums
+    uint32_t item, flags[kStrip64Warps];
+    uint32_t mask[5 * kStrip64Lanes];
+};
+// x 2^d for d <= 0 on the integer side (the FP64 unit is what the strips wait for); what
+// would be subnormal becomes 0 (values are held above 2^-950).
+__device__ __forceinline__ double skew_shift(double x, int d) {
+    const int hi = __double2hiint(x);
+    const bool ok = ((hi >> 20) & 0x7ff) + d > 0;
+    return __hiloint2double(ok ? hi + d * (1 << 20) : 0, ok ? __double2loint(x) : 0);
+}
+
+template <int N>
+__device__ Partial strip_run_skew64(const Rec64J* __restrict__ rec, int l, const uint8_t* __restrict__ hap, int k,
+                                    int strip, const PipeRange& rng, const float4* in, float4* out, SkewStage64& st,
+                                    uint32_t tag, uint32_t* __restrict__ status) {
+    static_assert(N <= 32, "match masks hold 32 columns");
+    constexpr int G = kStrip64Lanes, kRows = 2 * G;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int scol = strip * G * N;
+    uint32_t flags = rng.ok ? 0u : PF_DEGEN, mflags = 0;
+    const bool has_left = in != nullptr, has_right = out != nullptr;
+    const double mil = __ldg(&rec[l - 1].mi);
+    __syncthreads();  // the CTA's previous strip is done with the stage
+    {
+        uint32_t bm[4] = {0u, 0u, 0u, 0u};
+        const int nv = max(0, min(k - (scol + t * N), N));
+        for (int c = 0; c < nv; ++c) {
+            const int code = base_code(hap[scol + t * N + c]);
+            if (code < 0) flags |= PF_BAD;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (code == q || code == 4) bm[q] |= 1u << c;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) st.mask[q * G + t] = bm[q];
+        st.mask[4 * G + t] = 0xffffffffu;
+    }
+    // row l + 1 collects M + I, other rows outside 1 .. l hold
+    auto fetch = [&](int row) {
+        const int sl = row & (kRows - 1);
+        if (row >= 1 && row <= l) {
+            const double2* src = reinterpret_cast<const double2*>(rec + (row - 1));
+            cp_async16_cg(&st.pp[sl], src);
+            cp_async16_cg(&st.ab[sl], src + 1);
+            cp_async16_cg(&st.hg[sl], src + 2);
+            st.meta[sl] = (uint32_t)__ldg(&rec[row - 1].meta);
+        } else {
+            st.pp[sl] = st.ab[sl] = make_double2(0.0, 0.0);
+            st.hg[sl] = make_double2(row == l + 1 ? mil : 1.0, 0.0);
+            st.meta[sl] = 4u;
+        }
+        cp_async_commit();
+    };
+    // boundary rows kWaveBlock b .. (warp 0): lane & 15 the row, lane >> 4 the part
+    uint4 pv = make_uint4(0u, 0u, 0u, 0u);
+    auto load_bnd = [&](int b) {
+        const int i = kWaveBlock * b + (lane & (kWaveBlock - 1));
+        if (has_left && i >= 1 && i < l) pv = ld_row_relaxed(in + 2 * i + (lane >> 4));
+    };
+    auto take_bnd = [&](int b) {
+        const int i = kWaveBlock * b + (lane & (kWaveBlock - 1));
+        const bool mine = has_left && i >= 1, need = mine && i < l;
+        long long spins = 0;
+        // (after one wait has run out the strip waits no more: its result is an error already)
+        while (__any_sync(kFull, need && (pv.w & kWaveTagMask) != tag) && !(flags & PF_TIMEOUT)) {
+            if (++spins > kSpinLimit) {
+                flags |= PF_TIMEOUT;
+                if (lane == 0) atomicOr(status, ST_TIMEOUT);
+                break;
+            }
+            if (spins > kSpinFast) __nanosleep(64);
+            if (need && (pv.w & kWaveTagMask) != tag) pv = ld_row_relaxed(in + 2 * i + (lane >> 4));
+        }
+        if (mine) (lane < kWaveBlock ? st.bndA : st.bndB)[i & 63] = need ? pv : make_uint4(0u, 0u, 0u, 0u);
+        __syncwarp();
+    };
+    if (t < 64) st.bndA[t] = st.bndB[t] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    fetch(t - (G - 1));
+    if (warp == 0) {
+        load_bnd(0);
+        take_bnd(0);
+        load_bnd(1);
+    }
+    if (t < 64) fetch(1 + t);
+    cp_async_wait_0();
+    __syncthreads();
+
+    const int E0 = Num<double>::kLog2C - rng.target;
+    // the left strip's exponent: that of boundary row 1 up to the first checkpoint, where it
+    // may change next
+    int Eb = has_left && l > 1 ? (int)st.bndA[1].w >> kWaveTagBits : INT_MIN;
+    SkewLane<double> L;
+    L.m = L.d = L.g = 0.0;
+    L.E = max(E0, Eb);
+    int lsh = t == 0 && Eb != INT_MIN ? Eb - L.E : 0;  // exponent of what comes from the left
+    double M[N], J[N];
+    {
+        const double c = skew_init<double>(rng, k, E0, L.E);
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            M[q] = 0.0;
+            J[q] = c;
+        }
+        L.j = c;
+        // boundary row 0 (Eb >= E0: a strip keeps its first exponent until its last lane started)
+        const double j0 = Eb == INT_MIN ? c : scale2(c, L.E - Eb);
+        __syncthreads();
+        if (t == 0) {
+            st.bndA[0] = make_uint4(0u, 0u, (uint32_t)__double2loint(j0), 0u);
+            st.bndB[0] = make_uint4((uint32_t)__double2hiint(j0), 0u, 0u, 0u);
+        }
+        if (lane == 31) {
+            st.xch[0][warp][0] = 0.0;
+            st.xch[0][warp][1] = c;
+            st.xch[0][warp][2] = 0.0;
+        }
+        __syncthreads();
+    }
+    const int nl = min(G, (k - scol + N - 1) / N);
+    const int steps = l + nl;
+    const bool sends = has_right && t == G - 1;
+    int ck = rng.R - (int)(((long long)G * strip) % rng.R);  // checkpoint after step ck
+    int sl = (1 - t) & (kRows - 1);
+    double2 n0 = st.pp[sl], n1 = st.ab[sl], n2 = st.hg[sl];
+    uint32_t meta = st.meta[sl];
+    for (int s = 1; s <= steps;) {
+        const int e = min(min(min(ck, (s + kWaveBlock - 1) & ~(kWaveBlock - 1)), steps), s <= G + 1 ? G + 1 : steps);
+        const bool send = sends && s > G + 1;
+        // (the steps between events in a loop of their own, as in team_run_skew)
+#pragma unroll 1
+        for (; s <= e; ++s) {
+            if (send) {  // row s - G - 1 at the strip's last column
+                const uint32_t w = ((uint32_t)L.E << kWaveTagBits) | tag;
+                float4* o = out + 2 * (s - G - 1);
+                st_row_relaxed(o, __int_as_float(__double2loint(L.m)), __int_as_float(__double2hiint(L.m)),
+                               __int_as_float(__double2loint(L.j)), w);
+                st_row_relaxed(o + 1, __int_as_float(__double2hiint(L.j)), __int_as_float(__double2loint(L.d)),
+                               __int_as_float(__double2hiint(L.d)), w);
+            }
+            double um = __shfl_up_sync(kFull, L.m, 1), uj = __shfl_up_sync(kFull, L.j, 1),
+                   ud = __shfl_up_sync(kFull, L.d, 1);
+            if (lane == 0) {
+                if (warp == 0) {
+                    const uint4 va = st.bndA[(s - 1) & 63], vb = st.bndB[(s - 1) & 63];
+                    um = __hiloint2double((int)va.y, (int)va.x);
+                    uj = __hiloint2double((int)vb.x, (int)va.z);
+                    ud = __hiloint2double((int)vb.z, (int)vb.y);
+                } else {
+                    um = st.xch[(s - 1) & 1][warp - 1][0];
+                    uj = st.xch[(s - 1) & 1][warp - 1][1];
+                    ud = st.xch[(s - 1) & 1][warp - 1][2];
+                }
+            }
+            L.m = skew_shift(um, lsh);
+            L.j = skew_shift(uj, lsh);
+            L.d = skew_shift(ud, lsh);
+            L.pm = n0.x;
+            L.px = n0.y;
+            L.a = n1.x;
+            L.b = n1.y;
+            L.h = n2.x;
+            L.gp = L.g;
+            L.g = n2.y;
+            mflags |= meta;
+            skew_row<double, N, false>(M, J, L, st.mask[(meta & META_CODE_MASK) * G + t]);
+            if (lane == 31) {
+                st.xch[s & 1][warp][0] = L.m;
+                st.xch[s & 1][warp][1] = L.j;
+                st.xch[s & 1][warp][2] = L.d;
+            }
+            sl = (s + 1 - t) & (kRows - 1);
+            n0 = st.pp[sl];
+            n1 = st.ab[sl];
+            n2 = st.hg[sl];
+            meta = st.meta[sl];
+            __syncthreads();
+        }
+        // after step e
+        if ((e & 31) == 0) {
+            // rows up to e + 32 have landed, rows before e - 126 are done with; every lane takes its
+            // next row again (lane 0's is one of those)
+            cp_async_wait_0();
+            __syncthreads();
+            n0 = st.pp[sl];
+            n1 = st.ab[sl];
+            n2 = st.hg[sl];
+            meta = st.meta[sl];
+            if (warp == ((e >> 5) & (kStrip64Warps - 1))) fetch(e + 33 + lane);
+        }
+        if (warp == 0 && (e & (kWaveBlock - 1)) == 0) {
+            if (e == 32 && t == 0) st.bndA[0] = st.bndB[0] = make_uint4(0u, 0u, 0u, 0u);
+            __syncwarp();
+            take_bnd(e / kWaveBlock);
+            load_bnd(e / kWaveBlock + 1);
+        }
+        if (e == ck) {
+            ck += rng.R;
+            __syncthreads();  // the boundary rows that warp 0 took
+            if (has_left && e < l) Eb = (int)st.bndA[e & 63].w >> kWaveTagBits;
+            const int r = e - t;
+            const bool keep = r < 1 || r > l;
+            double x = 0.0;
+#pragma unroll
+            for (int q = 0; q < N; ++q) x = fmax(x, fmax(fabs(M[q]), fabs(J[q])));
+            // as skew_exponent, over the CTA's lanes
+            using NT = Num<double>;
+            const int ex = NT::expo(x);
+            int want = L.E;
+            if (!keep) {
+                if (ex == INT_MAX) flags |= PF_NONFINITE;
+                else if (ex == INT_MIN) want = t > 0 || Eb != INT_MIN ? INT_MIN : L.E;
+                else if (ex > rng.hi || ex <= NT::kLo) want = L.E + (ex - rng.target);
+            }
+            int En = t == 0 ? max(want, Eb) : want;
+#pragma unroll
+            for (int q = 0; q < 5; ++q) {
+                const int up = __shfl_up_sync(kFull, En, 1 << q);
+                if (lane >= (1 << q)) En = max(En, up);
+            }
+            if (lane == 31) st.E[warp] = En;
+            __syncthreads();
+            int left = t == 0 ? Eb : INT_MIN;  // exponent of the lane to the left
+            int before = INT_MIN;
+            for (int q = 0; q < warp; ++q) before = max(before, st.E[q]);
+            En = max(En, before);
+            if (En == INT_MIN) En = L.E;
+            if (!keep && En == want && ex <= rng.danger) flags |= PF_DANGER;
+            __syncthreads();
+            if (lane == 31) st.E[warp] = En;
+            __syncthreads();
+            const int up = __shfl_up_sync(kFull, En, 1);
+            if (lane > 0) left = up;
+            else if (warp > 0) left = st.E[warp - 1];
+            if (En != L.E) {
+                double f, g;
+                skew_factors(L.E - En, f, g);
+                for (;;) {
+#pragma unroll
+                    for (int q = 0; q < N; ++q) {
+                        M[q] *= f;
+                        J[q] *= f;
+                    }
+                    L.m *= f;
+                    L.j *= f;
+                    L.d *= f;
+                    if (g == 1.0) break;  // one factor, nearly always
+                    f = g;
+                    g = 1.0;
+                }
+                L.E = En;
+                if (lane == 31) {
+                    st.xch[e & 1][warp][0] = L.m;
+                    st.xch[e & 1][warp][1] = L.j;
+                    st.xch[e & 1][warp][2] = L.d;
+                }
+            }
+            lsh = left == INT_MIN ? 0 : max(left - L.E, -2047);
+            if (L.E > kWaveMaxE || L.E < -kWaveMaxE) flags |= PF_DANGER;  // does not fit beside the tag
+            __syncthreads();
+        }
+    }
+    if (mflags & META_BAD) flags |= PF_BAD;
+    if (mflags & META_DEGEN) flags |= PF_DEGEN;
+    const int nvalid = max(0, min(k - (scol + t * N), N));
+    double sum = 0.0;
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+        if (q < nvalid) sum += J[q];
+    const SegOut o = skew_sum(sum, L.E, E0, flags, lane, 31);
+    if (lane == 0) {
+        st.S[warp] = o.S;
+        st.E[warp] = o.E;
+        st.flags[warp] = o.flags;
+    }
+    cp_async_wait_0();  // nothing may land in the stage after this strip
+    __syncthreads();
+    // the warps' sums in the scale of the largest
+    Partial p;
+    p.S = 0.0;
+    p.E = st.E[0];
+    p.flags = PF_DONE;
+    int top = INT_MIN;
+    for (int q = 0; q < kStrip64Warps; ++q) {
+        p.flags |= st.flags[q];
+        const int x = st.S[q] != 0.0 ? st.E[q] + Num<double>::expo(st.S[q]) : INT_MIN;
+        if (x > top) {
+            top = x;
+            p.E = st.E[q];
+        }
+    }
+    for (int q = 0; q < kStrip64Warps; ++q)
+        if (st.S[q] != 0.0) p.S += ldexp(st.S[q], st.E[q] - p.E);
+    return p;
 }
 
 }  // namespace phmm

@@ -85,3 +85,35 @@ def test_short_teams_fp64(phmm, variant, gcp, ins):
     tol = 32.0 * (l + k) * 2.0 ** -53 / np.log(10.0) + np.abs(ref) * 2.0 ** -51
     assert rc == 0 and not np.any(flags & 0x79) and st["short_kernel"] == {4: 2, 5: 3}[variant]
     assert np.all(np.abs(out - ref) <= tol), np.max(np.abs(out - ref) / tol)
+
+
+@pytest.mark.parametrize("gcp,ins", [("ten", "flat"), ("other", "jumps"), ("mixed", "flat")])
+@pytest.mark.parametrize("variant", ["pipe", "pipe2"])
+def test_strips_fp64(phmm, variant, gcp, ins):
+    shapes = [(1, 1025), (2, 1025), (3, 1280), (16, 1281), (17, 3072), (31, 1536), (32, 1537), (33, 4097), (34, 2080),
+              (63, 5000), (64, 1100), (65, 3000), (96, 1056), (97, 1057), (400, 7000), (1500, 1100), (2000, 4100), (60, 900)]
+    b = _pairs(shapes, gcp, ins, 6)
+    with phmm.Context(precision="fp64", variant=variant) as ctx:
+        need = ctx.footprint(b)
+        out, flags, rc, st = ctx.run(b)
+    ref = oracle.batch(b)
+    l, k = W.pair_lengths(b)
+    tol = 32.0 * (l + k) * 2.0 ** -53 / np.log(10.0) + np.abs(ref) * 2.0 ** -51
+    assert rc == 0 and not np.any(flags & 0x79) and st["n_long"] == len(shapes) - (1 if variant == "pipe2" else 0)
+    assert np.all(np.abs(out - ref) <= tol), np.max(np.abs(out - ref) / tol)
+    # the footprint's bound is enough, whichever strips fit in it
+    with phmm.Context(precision="fp64", variant=variant, mem_budget=need) as ctx:
+        small = ctx.run(b)[0]
+    assert np.all(np.abs(small - ref) <= tol)
+
+
+def test_degenerate_strips_fp64(phmm):
+    """gcp Phred 0 (T_DD = 1), which the strips cannot hold: a wide pair's flags stay those of
+    the unfactored engine."""
+    b = _pairs([(50, 2000), (200, 1500)], "other", "flat", 3)
+    b["gcp_q"] = np.zeros_like(b["gcp_q"])
+    with phmm.Context(precision="fp64", variant="pipe2") as ctx:
+        out, flags, rc, st = ctx.run(b)
+    with phmm.Context(precision="fp64", cols_per_lane=8) as ctx:
+        out8, flags8, _, _ = ctx.run(b)
+    assert rc == 0 and np.array_equal(flags, flags8) and np.array_equal(out, out8)
