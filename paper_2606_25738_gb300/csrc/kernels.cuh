@@ -649,6 +649,26 @@ k_forward_cluster(const BatchHeader* __restrict__ H, const PowRow<float>* __rest
     }
 }
 
+// Order in which a persistent kernel's CTAs begin to take items: those that are first on their
+// SM, then those that are second, and so on, so that the longest items, which the lists have
+// first, spread over all SMs, and items fewer than the warps leave no SM with two of them while
+// another has none.  (Left to chance, 64 strips of one pair took 6.3 ms or, three to a scheduler,
+// 11 to 14 ms.)  False: enough CTAs stand before this one.  The wait is a matter of speed only,
+// and short: 20 us at most, where another kernel holds SMs.  list: 0 multi-warp, 1 short.
+__device__ __forceinline__ bool sm_turn(const BatchHeader* __restrict__ H, int list, uint32_t n_items, uint32_t per_cta) {
+    __shared__ uint32_t before;
+    if (threadIdx.x == 0) {
+        uint32_t sm;
+        asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
+        const uint32_t rank = atomicAdd(H->sm_rank + list * kSmSlots + (sm & (kSmSlots - 1)), 1u);
+        before = rank * H->sms * per_cta;
+        if (n_items > before)
+            for (int q = 0; q < 200 && *(volatile uint32_t*)&H->counters[list] < before; ++q) __nanosleep(100);
+    }
+    __syncthreads();
+    return n_items > before;
+}
+
 // Multi-warp pairs one warp at a time (long kind 3): each warp takes a whole pair and
 // runs its strips of 32 N columns one after another (strip_run_skew), strip s reading the
 // boundary strip s - 1 left in this warp's scratch.  No warp ever waits on another; the
@@ -690,6 +710,7 @@ k_forward_serial(const BatchHeader* __restrict__ H) {
     __shared__ SkewStage stage[4];
     const PipeRange rng = skew_range(H);
     const uint32_t gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (!sm_turn(H, 0, H->n_citems, blockDim.x >> 5)) return;
     if (gw >= H->sbnd_warps) return;  // no scratch for this warp (grid larger than planned)
     if (skew_g10(H->skst)) serial_items<N, true>(H, rng, stage[threadIdx.x >> 5]);
     else serial_items<N, false>(H, rng, stage[threadIdx.x >> 5]);
@@ -733,6 +754,7 @@ template <int N, int MINB>
 __global__ void __launch_bounds__(128, MINB)
 k_forward_wave(const BatchHeader* __restrict__ H) {
     __shared__ SkewStage stage[4];
+    if (!sm_turn(H, 0, H->n_citems, blockDim.x >> 5)) return;
     const PipeRange rng = skew_range(H);
     if (skew_g10(H->skst)) wave_items<N, true>(H, rng, stage[threadIdx.x >> 5]);
     else wave_items<N, false>(H, rng, stage[threadIdx.x >> 5]);
@@ -887,6 +909,7 @@ template <int N, int MINB, bool HALVES = true, bool LEAN = false>
 __global__ void __launch_bounds__(kShortThreads, MINB)
 k_short_pipe2(const BatchHeader* __restrict__ H) {
     __shared__ uint32_t masks[kShortThreads / 32][5 * 32];
+    if (!sm_turn(H, 1, H->n_witems, blockDim.x >> 5)) return;
     const PipeRange rng = skew_range(H);
     if (skew_g10(H->skst)) skew_items<float, N, true>(H, rng, masks[threadIdx.x >> 5]);
     else skew_items<float, N, false>(H, rng, masks[threadIdx.x >> 5]);
@@ -899,6 +922,7 @@ template <int N, int MINB>
 __global__ void __launch_bounds__(kShortThreads, MINB)
 k_short_pipe64(const BatchHeader* __restrict__ H) {
     __shared__ uint32_t masks[kShortThreads / 32][5 * 32];
+    if (!sm_turn(H, 1, H->n_witems, blockDim.x >> 5)) return;
     skew_items<double, N, false>(H, skew_range<double>(H), masks[threadIdx.x >> 5]);
 }
 

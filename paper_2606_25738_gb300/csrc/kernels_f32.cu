@@ -15,6 +15,7 @@ __device__ const Rec32* dummy_rec<float>() { return &g_dummy32; }
 // row tags must not survive from an earlier launch).
 __global__ void k_reset(const BatchHeader* __restrict__ H) {
     if (blockIdx.x == 0) {
+        for (uint32_t q = threadIdx.x; q < 2 * kSmSlots; q += blockDim.x) H->sm_rank[q] = 0u;
         if (threadIdx.x < 8) H->counters[threadIdx.x] = 0u;
         if (threadIdx.x == 0) {
             H->status[0] = 0u;

@@ -63,6 +63,7 @@ constexpr int META_GCP_SHIFT = 8;
 constexpr uint32_t META_DEGEN = 1u << 16;  // 1 - g_i too small for the factored form
 constexpr uint32_t META_BAD = 1u << 17;    // invalid base or quality > 93
 
+constexpr uint32_t kSmSlots = 512;  // SM ids (more than there are)
 constexpr uint32_t kWaveTags = 63;  // tags of the wave kind's boundary rows (skew.cuh)
 constexpr int kMaxPhred = 93;
 constexpr int kPhredTab = 96;  // table rows (>= kMaxPhred + 1)
@@ -218,6 +219,8 @@ struct BatchHeader {
     uint32_t wave64_k;          // FP64: wider pairs run on the skewed strips; else 0xffffffff
     float4 *wbnd;            // strips of the wave kind: each strip's right boundary (l rows)
     uint64_t wbnd_rows;      // rows the buffer holds (k_reset clears it when the tags wrap)
+    uint32_t *sm_rank;       // [2][kSmSlots]: CTAs that started on each SM (multi-warp, short kernels)
+    uint32_t sms;
     uint32_t *wave_epoch;    // tag of this launch's boundary rows, 1 .. kWaveTags (k_prep32 steps it)
     float4 *sbnd;            // serial multi-warp pairs: 2 strip boundaries of sbnd_rows rows
     uint32_t sbnd_rows;      // per resident warp of k_forward_serial (not cleared)

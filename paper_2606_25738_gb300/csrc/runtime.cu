@@ -487,11 +487,11 @@ void build_pow_table(int N, std::vector<PowRow<T>>& out) {
 // ------------------------------------------------------------------------------------
 // Context
 // ------------------------------------------------------------------------------------
-constexpr size_t kSmallBytes = 128;
+constexpr size_t kSmallBytes = 128 + 2 * kSmSlots * 4;
 struct Slot {
     DevBuf in_bases, in_bq, in_iq, in_dq, in_gq, in_hap, in_roff, in_hoff, in_pr, in_ph;
     DevBuf desc, rec32, rec32j, rec64, rec64j, teams, witems, witems2, cpairs, citems, parts, out, oflags, rescue;
-    DevBuf small;  // counters[8], status[1], dropgrow[4], skew statistics [4], wave tag (kSmallBytes)
+    DevBuf small;  // counters[8], status[1], dropgrow[4], skew statistics [4], wave tag, CTAs by SM (kSmallBytes)
     DevBuf bnd;    // strip boundaries of the batch
     DevBuf rbnd;   // rescue / launch-per-pair boundary scratch
     DevBuf sbnd;   // serial multi-warp pairs: two boundaries per resident warp
@@ -838,10 +838,30 @@ std::vector<std::pair<int, int>> fp32_candidates(const phmm_config& cfg) {
 
 // FP64 plan of variant id (launch.h: kF64N columns per lane, kF64CW-warp CTAs); the
 // variant travels in scal_id.
+// Whether a batch's FP64 multi-warp pairs (wider than `wide`) are done sooner as waves: cycles
+// over all SMs and of the longest row chain, from what both kernels measured.  A 512-column
+// strip takes l + 128 steps of 1600 cycles, starting 150 steps after its left neighbour (24 pairs
+// of 1 to 10 kbp: 10.9 ms); CTA items do 8 operations a cell at 1.1 cells x operations a cycle
+// and SM, and 7700 cycles a row for each four warps of 512 columns (84 ms).  Many short reads
+// against 513 to 1024 columns are the other end (5,000 pairs of 150 rows: 28 ms and 10.8).
+bool waves64_pay(const uint32_t* l, const uint32_t* k, uint32_t n, uint32_t wide) {
+    const double sms = 152.0;
+    double wave = 0, wchain = 0, cta = 0, cchain = 0;
+    for (uint32_t p = 0; p < n; ++p) {
+        if (k[p] <= wide) continue;
+        const double W = (double)((k[p] + 128u * kF64WaveN - 1) / (128u * kF64WaveN));
+        wave += W * (l[p] + 144.0) * 1600.0 / sms;
+        wchain = std::max(wchain, (l[p] + 150.0 * W) * 1600.0);
+        cta += (double)l[p] * k[p] * 8.0 / 1.1 / sms;
+        cchain = std::max(cchain, l[p] * 7700.0 * std::min(2.0, std::ceil(W / 4.0)));
+    }
+    return std::max(wave, wchain) < std::max(cta, cchain);
+}
+
 // wave: multi-warp pairs of the skewed variants as waves (long_kind 6) rather than CTA items
 void make_plan64(const uint32_t* l, const uint32_t* k, const uint32_t* pr, uint32_t n, int id, Plan& P,
                  bool wave = false) {
-    wave = wave && f64_pipelined(id);
+    wave = wave && f64_pipelined(id) && waves64_pay(l, k, n, 32u * (uint32_t)kF64NS[id]);
     make_plan(l, k, pr, n, kF64NS[id], 0, wave ? 4 * kF64WaveN : kF64N[id], P, 8, wave ? 1 : kF64CW[id], false, wave,
               f64_pipelined(id) ? kSkewCost : TeamCost());
     P.scal_id = id;
@@ -1365,6 +1385,8 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     hh.dropgrow = (uint32_t*)S->small.p + 9;      // words 9 .. 12
     hh.skst = (SkewStats*)((uint32_t*)S->small.p + 16);  // words 16 .. 19
     hh.wave_epoch = (uint32_t*)S->small.p + 24;   // word 24 (kept between launches)
+    hh.sm_rank = (uint32_t*)S->small.p + 32;      // words 32 ..
+    hh.sms = (uint32_t)ctx->sms;
     hh.seed = ctx->seed;
     hh.mode = (uint32_t)ctx->cfg.precision;
     CK(cudaMemcpyAsync(S->hdr.p, &hh, sizeof(hh), cudaMemcpyHostToDevice, cs));

@@ -117,3 +117,11 @@ def test_degenerate_strips_fp64(phmm):
     with phmm.Context(precision="fp64", cols_per_lane=8) as ctx:
         out8, flags8, _, _ = ctx.run(b)
     assert rc == 0 and np.array_equal(flags, flags8) and np.array_equal(out, out8)
+
+
+@pytest.mark.parametrize("shape", [(3, 1025), (2, 1000)])
+@pytest.mark.parametrize("n", [1, 607, 609, 1217, 1825])
+def test_items_around_the_warps(phmm, shape, n):
+    """Items one fewer and one more than the warps that are first on their SM, second, all."""
+    st = _check(phmm, _pairs([shape] * n, "ten", "flat", 2), flags=phmm.F_LONG_SERIAL)
+    assert st["n_long"] == (n if shape[1] > 1024 else 0)
