@@ -123,5 +123,5 @@ def test_degenerate_strips_fp64(phmm):
 @pytest.mark.parametrize("n", [1, 607, 609, 1217, 1825])
 def test_items_around_the_warps(phmm, shape, n):
     """Items one fewer and one more than the warps that are first on their SM, second, all."""
-    st = _check(phmm, _pairs([shape] * n, "ten", "flat", 2), flags=phmm.F_LONG_SERIAL)
+    st = _check(phmm, _pairs([shape] * n, "ten", "flat", 2), flags=phmm.F_LONG_SERIAL, variant="pipe2", cols_per_lane=32)
     assert st["n_long"] == (n if shape[1] > 1024 else 0)
