@@ -905,14 +905,38 @@ __device__ __forceinline__ void skew_items(const BatchHeader* __restrict__ H, co
         if (t.pair != kNoPair && t.lt == 0) write_part(H, t.pair, o);
     }
 }
+// Pairs no more than the resident warps: one warp each.
+template <int N, bool G10>
+__device__ __forceinline__ void solo_items(const BatchHeader* __restrict__ H, const PipeRange& rng, SoloStage& st) {
+    const uint32_t n = H->n_solo;
+    const int lane = threadIdx.x & 31;
+    for (;;) {
+        uint32_t wi = 0;
+        if (lane == 0) wi = atomicAdd(&H->counters[1], 1u);
+        wi = __shfl_sync(kFull, wi, 0);
+        if (wi >= n) break;
+        const uint32_t pair = H->teams[wi].pair;
+        const PairDesc d = H->desc[pair];
+        const SegOut o = pair_run_skew<N, G10, kSolo>(H->rec32j + d.roff, (int)d.l, H->hap_bases + d.hoff, (int)d.k, rng, st);
+        if (lane == 0) write_part(H, pair, o);
+    }
+}
 template <int N, int MINB, bool HALVES = true, bool LEAN = false>
 __global__ void __launch_bounds__(kShortThreads, MINB)
 k_short_pipe2(const BatchHeader* __restrict__ H) {
-    __shared__ uint32_t masks[kShortThreads / 32][5 * 32];
-    if (!sm_turn(H, 1, H->n_witems, blockDim.x >> 5)) return;
+    __shared__ SoloStage stage[kShortThreads / 32];
+    SoloStage& st = stage[threadIdx.x >> 5];
+    const bool solo = H->n_solo > 0;
+    if (!sm_turn(H, 1, solo ? H->n_solo : H->n_witems, blockDim.x >> 5)) return;
     const PipeRange rng = skew_range(H);
-    if (skew_g10(H->skst)) skew_items<float, N, true>(H, rng, masks[threadIdx.x >> 5]);
-    else skew_items<float, N, false>(H, rng, masks[threadIdx.x >> 5]);
+    const bool g10 = skew_g10(H->skst);
+    if (solo) {
+        if (g10) solo_items<N, true>(H, rng, st);
+        else solo_items<N, false>(H, rng, st);
+    } else {
+        if (g10) skew_items<float, N, true>(H, rng, st.mask);
+        else skew_items<float, N, false>(H, rng, st.mask);
+    }
 }
 
 // FP64 mode: short pairs on the skewed engine in FP64 (Rec64J records), same work list; the

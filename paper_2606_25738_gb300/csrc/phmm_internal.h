@@ -208,6 +208,7 @@ struct BatchHeader {
     const CtaItem *citems;
     const CtaPair *cpairs;
     uint32_t n_witems, n_citems, n_witems2;
+    uint32_t n_solo;           // > 0: every short team (of n_solo) on a warp of its own
     uint32_t n_partials;
     uint32_t force_rescue;   // 1: every pair goes to the FP64 rescue pass
     Partial *parts;          // n_pairs slots, then extra slots of strips 1.. of wide pairs

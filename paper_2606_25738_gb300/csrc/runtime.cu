@@ -771,6 +771,11 @@ void plan_header(const Slot& S, const Plan& P, BatchHeader& hh) {
     hh.citems = (const CtaItem*)S.citems.p;
     hh.cpairs = (const CtaPair*)S.cpairs.p;
     hh.n_witems = (uint32_t)P.witems.size();  // a device-built plan's: written by its last kernel but two
+    // short pairs no more than 12 to an SM have a warp each, of few columns a lane: the step of a
+    // scheduler's only warp is latency (20 pairs of 150 rows: forward 54 us against 84 in teams;
+    // from about three warps a scheduler on, teams take fewer slots)
+    hh.n_solo = !P.fp64 && !P.dev && kShortScalarHalves[P.scal_id] && P.witems2.empty() &&
+                P.teams.size() <= 12u * hh.sms ? (uint32_t)P.teams.size() : 0u;
     hh.n_citems = (uint32_t)P.n_citems();
     hh.n_partials = hh.n_pairs + P.n_extra;
     hh.bnd = (unsigned long long*)S.bnd.p;
@@ -1366,6 +1371,7 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     hh.n_pairs = np;
     hh.desc = (PairDesc*)S->desc.p;
     hh.rec64 = (Rec64*)S->rec64.p;
+    hh.sms = (uint32_t)ctx->sms;
     plan_header(*S, P, hh);
     hh.n_partials = np + P.n_extra;
     hh.bnd = (unsigned long long*)S->bnd.p;
@@ -1386,7 +1392,6 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     hh.skst = (SkewStats*)((uint32_t*)S->small.p + 16);  // words 16 .. 19
     hh.wave_epoch = (uint32_t*)S->small.p + 24;   // word 24 (kept between launches)
     hh.sm_rank = (uint32_t*)S->small.p + 32;      // words 32 ..
-    hh.sms = (uint32_t)ctx->sms;
     hh.seed = ctx->seed;
     hh.mode = (uint32_t)ctx->cfg.precision;
     CK(cudaMemcpyAsync(S->hdr.p, &hh, sizeof(hh), cudaMemcpyHostToDevice, cs));

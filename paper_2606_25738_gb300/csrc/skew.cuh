@@ -173,6 +173,7 @@ __device__ __forceinline__ void skew_masks(const uint8_t* __restrict__ hap, int 
 template <typename T>
 struct SkewLane {
     T m, j, d;               // left of the lane (the row above its row)
+    T mi;                        // (lean form)
     T pm, px, a, b, h, g, gp;  // the lane's row; gp: g of the row above (not used with G10)
     T lsc;                       // 2^(E of the left lane - E)
     int E;
@@ -205,17 +206,60 @@ __device__ __forceinline__ void skew_row(T (&M)[N], T (&J)[N], SkewLane<T>& L, u
     L.d = dB;
 }
 
+// The same in the lean engine's order of operations, on its records (Rec32): I in the place of
+// J, with L.mi = T_MI; one operation more a cell.
+template <int N>
+__device__ __forceinline__ void skew_row_lean(float (&M)[N], float (&I)[N], SkewLane<float>& L, uint32_t mask) {
+    float ml = L.m, il = L.j, d = L.d;
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+        const float u = fmaf(L.a, ml, fmaf(L.b, d, il));
+        d = fmaf(L.gp, d, ml);
+        ml = M[q];
+        il = I[q];
+        I[q] = fmaf(L.mi, ml, L.h * il);
+        M[q] = (((mask >> q) & 1u) ? L.pm : L.px) * u;
+    }
+    L.m = ml;
+    L.j = il;
+    L.d = d;
+}
+
+// Records of one pair's rows in shared memory, two blocks of 32 rows ahead of the team's first
+// lane: slot row & 127.
+struct SoloStage {
+    float4 r0[128], r1[128];
+    uint32_t mask[5 * 32];
+};
+
 // Lane lt of a team of tlast - (first lane) + 1 lanes runs columns lt N .. of its pair; steps =
 // the largest l + team size - 1 of the warp's teams; every lane of a team is at rows 2 .. l at
 // steps plain0 .. plain1.  A lane starts as M = 0, J = C / k and keeps that before row 1 (P' = 0,
 // h = 1); row 1's record has h = 0, so that J = 0 and M = P' C / k follow; after row l a lane
-// does nothing.  Records come through L1, one step ahead.
-template <typename T, int N, bool G10>
-__device__ SegOut team_run_skew(const typename Num<T>::RecJ* __restrict__ rec, int l, int steps, int plain0, int plain1,
+// does nothing.  Records come through L1, one step ahead, or (FORM solo and lean: the warp has one
+// team, all 32 lanes) through shared memory: the first lane's record is new to L1 at every
+// step, which is what a scheduler's only warp waits for (a step of 900 cycles).
+enum SkewForm { kTeams, kSolo, kLean };
+template <typename T, int N, bool G10, SkewForm FORM = kTeams>
+__device__ SegOut team_run_skew(const std::conditional_t<FORM == kLean, Rec32, typename Num<T>::RecJ>* __restrict__ rec, int l, int steps, int plain0, int plain1,
                                 const uint8_t* __restrict__ hap, int k, int lt, int tlast, const PipeRange& rng,
-                                uint32_t* sm) {
+                                uint32_t* sm, SoloStage* st = nullptr, int rows = 0) {
     static_assert(N <= 32, "match masks hold 32 columns");
+    using Rec = std::conditional_t<FORM == kLean, Rec32, typename Num<T>::RecJ>;
     uint32_t flags = rng.ok ? 0u : PF_DEGEN, mflags = 0;
+    auto fetch = [&](int row) {  // solo: the pair's rows, by every lane
+        if (row <= rows) {
+            const float4* src = reinterpret_cast<const float4*>(rec + (row - 1));
+            cp_async16_cg(&st->r0[row & 127], src);
+            cp_async16_cg(&st->r1[row & 127], src + 1);
+        }
+        cp_async_commit();
+    };
+    if constexpr (FORM != kTeams) {
+        __syncwarp();  // the warp's previous pair is done with the stage
+        fetch(1 + (threadIdx.x & 31));
+        fetch(33 + (threadIdx.x & 31));
+    }
     skew_masks<N, false>(hap, k, lt * N, sm, flags);
     const int E0 = Num<T>::kLog2C - rng.target;
     const T cin = l > 0 && k > 0 ? skew_init<T>(rng, k, E0, E0) : T(0);
@@ -232,7 +276,24 @@ __device__ SegOut team_run_skew(const typename Num<T>::RecJ* __restrict__ rec, i
     L.E = E0;
     const int l1 = max(l, 1) - 1;
     int r = 1 - lt;  // the lane's row
-    typename Num<T>::RecJ nxt = load_recj(rec + max(0, min(r - 1, l1)));
+    auto load = [&](int i) {  // record of row i + 1
+        if constexpr (FORM == kTeams) {
+            return load_recj(rec + i);
+        } else {
+            const float4 a = st->r0[(i + 1) & 127], b = st->r1[(i + 1) & 127];
+            Rec x;
+            x.pm = a.x; x.px = a.y; x.a = a.z; x.b = a.w;
+            if constexpr (FORM == kLean) { x.mi = b.x; x.g = b.y; x.gm = b.z; }
+            else { x.h = b.x; x.g = b.y; x.mi = b.z; }
+            x.meta = __float_as_uint(b.w);
+            return x;
+        }
+    };
+    if constexpr (FORM != kTeams) {
+        cp_async_wait_0();
+        __syncwarp();
+    }
+    Rec nxt = load(max(0, min(r - 1, l1)));
     int ck = rng.R;  // checkpoint after step ck
     // EDGE: some lane is before row 2 or past row l
     auto run = [&](auto edge, int& s, int e) {
@@ -245,7 +306,12 @@ __device__ SegOut team_run_skew(const typename Num<T>::RecJ* __restrict__ rec, i
             L.px = nxt.px;
             L.a = nxt.a;
             L.b = nxt.b;
-            L.h = nxt.h;
+            if constexpr (FORM == kLean) {
+                L.mi = nxt.mi;
+                L.h = EDGE && r == 1 ? 0.f : nxt.g;
+            } else {
+                L.h = nxt.h;
+            }
             if constexpr (!G10) {
                 L.gp = L.g;
                 L.g = nxt.g;
@@ -256,24 +322,36 @@ __device__ SegOut team_run_skew(const typename Num<T>::RecJ* __restrict__ rec, i
                 if (r < 1) {  // not started: hold
                     L.pm = L.px = T(0);
                     L.h = T(1);
+                    if constexpr (FORM == kLean) L.mi = 0.f;
                 }
             }
             if (!EDGE || r <= l) {
                 L.m = lt == 0 ? T(0) : um * L.lsc;
                 L.j = lt == 0 ? (EDGE && r == 1 ? cin : T(0)) : uj * L.lsc;
                 L.d = lt == 0 ? T(0) : ud * L.lsc;
-                skew_row<T, N, G10>(M, J, L, mask);
+                if constexpr (FORM == kLean) skew_row_lean<N>(M, J, L, mask);
+                else skew_row<T, N, G10>(M, J, L, mask);
             }
-            nxt = load_recj(rec + (EDGE ? max(0, min(r, l1)) : min(r, l1)));
+            nxt = load(EDGE ? max(0, min(r, l1)) : min(r, l1));
         }
     };
     for (int s = 1; s <= steps;) {
         // (steps between events run in a loop of their own, in which nothing but the row writes
         // M and J: with the checkpoint inside it every step copied both)
-        const int e = min(ck, steps);
+        const int e = FORM == kTeams ? min(ck, steps) : min(min(ck, steps), (s + 31) & ~31);
         if (s < plain0) run(std::true_type{}, s, min(e, plain0 - 1));
         else if (s <= plain1) run(std::false_type{}, s, min(e, plain1));
         else run(std::true_type{}, s, e);
+        if constexpr (FORM != kTeams) {
+            if (((s - 1) & 31) == 0) {
+                // rows up to s + 31 have landed, rows before s - 31 are done with; a lane's next record may
+                // have been taken before it landed
+                cp_async_wait_0();
+                __syncwarp();
+                nxt = load(max(0, min(r - 1, l1)));
+                fetch(s + 32 + (threadIdx.x & 31));
+            }
+        }
         if (s > ck && s <= steps) {
             ck += rng.R;
             T x0 = 0, x1 = 0;
@@ -309,13 +387,32 @@ __device__ SegOut team_run_skew(const typename Num<T>::RecJ* __restrict__ rec, i
         // Eq. 4 (I = T_MI J on the last row)
         if (mflags & META_BAD) flags |= PF_BAD;
         if (mflags & META_DEGEN) flags |= PF_DEGEN;
-        const double mi = (double)__ldg(&rec[l1].mi);
+        const double mi = FORM == kLean ? 1.0 : (double)__ldg(&rec[l1].mi);
         const int nvalid = max(0, min(k - lt * N, N));
 #pragma unroll
         for (int q = 0; q < N; ++q)
             if (q < nvalid) s += (double)M[q] + mi * (double)J[q];
     }
+    if constexpr (FORM != kTeams) cp_async_wait_0();  // nothing may land in the stage after this pair
     return skew_sum(s, L.E, E0, flags, lt, tlast);
+}
+
+// One pair on one warp: the fewer columns a lane, the shorter a step.
+template <int N, bool G10, SkewForm FORM>
+__device__ __forceinline__ SegOut pair_run_skew(const std::conditional_t<FORM == kLean, Rec32, Rec32J>* __restrict__ rec, int l,
+                                                const uint8_t* __restrict__ hap, int k, const PipeRange& rng,
+                                                SoloStage& st) {
+    const int lane = threadIdx.x & 31;
+    auto go = [&](auto n) {
+        constexpr int Nl = decltype(n)::value;
+        const int g = (k + Nl - 1) / Nl;
+        const bool in = lane < g;  // (the others are teams of no rows)
+        return team_run_skew<float, Nl, G10, FORM>(rec, in ? l : 0, l + g - 1, g + 1, l, hap, in ? k : 0, in ? lane : 0,
+                                                   in ? g - 1 : lane, rng, st.mask + lane, &st, l);
+    };
+    if (k <= 32 * 8) return go(std::integral_constant<int, 8>{});
+    if (k <= 32 * 16) return go(std::integral_constant<int, 16>{});
+    return go(std::integral_constant<int, N>{});
 }
 
 // ------------------------------------------------------------------------------------

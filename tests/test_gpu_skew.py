@@ -37,11 +37,12 @@ def _pairs(shapes, gcp, ins, seed):
     return W.from_strings(out)
 
 
-def _check(phmm, b, **kw):
+def _check(phmm, b, copies=1, **kw):
+    pick = np.arange(len(b["pair_read"]))
     with phmm.Context(precision="fp32", **kw) as ctx:
-        out, flags, rc, st = ctx.run(b)
-    ref = oracle.batch(b)
-    l, k = W.pair_lengths(b)
+        out, flags, rc, st = ctx.run(W.subset(b, np.tile(pick, copies)) if copies > 1 else b)
+    ref = np.tile(oracle.batch(b), copies)
+    l, k = (np.tile(x, copies) for x in W.pair_lengths(b))
     tol = (6.5 * np.sqrt(16.0 * l + 4.0 * k) * 2.0 ** -23 + 8.0 * l * 2.0 ** -46) / np.log(10.0) + np.abs(ref) * 2.0 ** -52
     assert rc == 0 and not np.any(flags & 0x79)
     assert np.all(np.abs(out - ref) <= tol), np.max(np.abs(out - ref) / tol)
@@ -49,12 +50,13 @@ def _check(phmm, b, **kw):
 
 
 @pytest.mark.parametrize("gcp,ins", [("ten", "flat"), ("ten", "jumps"), ("other", "jumps"), ("mixed", "flat")])
+@pytest.mark.parametrize("copies", [1, 120])  # a warp for each pair; more pairs than warps: teams
 @pytest.mark.parametrize("N,variant", [(32, "pipe2"), (24, "pipe2"), (32, "pipe2lean")])
-def test_short_teams(phmm, N, variant, gcp, ins):
+def test_short_teams(phmm, N, variant, gcp, ins, copies):
     w = 32 * N
     shapes = [(1, 1), (1, w), (2, N), (2, N + 1), (3, 2 * N - 1), (31, w), (32, w - 1), (33, w), (34, w - N), (35, 5),
-              (64, N * 16), (65, N * 16 + 1), (150, 431), (151, 250), (300, w), (700, 3 * N)]
-    st = _check(phmm, _pairs(shapes, gcp, ins, 5), variant=variant, cols_per_lane=N)
+              (64, N * 16), (65, N * 16 + 1), (150, 431), (151, 250), (300, w), (700, 3 * N), (40, 256), (97, 257), (96, 513)]
+    st = _check(phmm, _pairs(shapes, gcp, ins, 5), copies, variant=variant, cols_per_lane=N)
     assert st["short_kernel"] == {("pipe2", 32): 7, ("pipe2", 24): 8, ("pipe2lean", 32): 9}[variant, N]
 
 
