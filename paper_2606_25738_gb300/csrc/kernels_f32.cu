@@ -11,8 +11,8 @@ __device__ __align__(16) Rec32 g_dummy32;  // read as two float4
 template <>
 __device__ const Rec32* dummy_rec<float>() { return &g_dummy32; }
 
-// Zeroes the work counters and status words, and clears the strip boundary buffer (its
-// row tags must not survive from an earlier launch).
+// Zeroes the work counters and status words and the partials, and clears the strip boundary
+// buffer (its row tags must not survive from an earlier launch).
 __global__ void k_reset(const BatchHeader* __restrict__ H) {
     if (blockIdx.x == 0) {
         for (uint32_t q = threadIdx.x; q < 2 * kSmSlots; q += blockDim.x) H->sm_rank[q] = 0u;
@@ -29,6 +29,10 @@ __global__ void k_reset(const BatchHeader* __restrict__ H) {
     const uint64_t n = H->n_bnd_words;
     for (uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (uint64_t)gridDim.x * blockDim.x)
         H->bnd[q] = 0ull;
+    uint4* const pp = reinterpret_cast<uint4*>(H->parts);
+    const uint64_t np = (uint64_t)H->n_partials * (sizeof(Partial) / 16);
+    for (uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; q < np; q += (uint64_t)gridDim.x * blockDim.x)
+        pp[q] = make_uint4(0u, 0u, 0u, 0u);
     // the wave kind's tags start over after this launch: no row may keep one
     const uint64_t nw = *H->wave_epoch == kWaveTags ? H->wbnd_rows : 0;
     for (uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nw; q += (uint64_t)gridDim.x * blockDim.x)

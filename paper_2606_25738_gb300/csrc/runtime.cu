@@ -487,10 +487,14 @@ void build_pow_table(int N, std::vector<PowRow<T>>& out) {
 // ------------------------------------------------------------------------------------
 // Context
 // ------------------------------------------------------------------------------------
+// Host arrays of a small batch (inputs, plan) go to the device with its header in one copy from
+// pinned memory, up to this many bytes; beyond, each array is copied by itself.
+constexpr size_t kPackBytes = 1u << 20;
+constexpr size_t kPackStart = (sizeof(BatchHeader) + 255) / 256 * 256;
 constexpr size_t kSmallBytes = 128 + 2 * kSmSlots * 4;
 struct Slot {
     DevBuf in_bases, in_bq, in_iq, in_dq, in_gq, in_hap, in_roff, in_hoff, in_pr, in_ph;
-    DevBuf desc, rec32, rec32j, rec64, rec64j, teams, witems, witems2, cpairs, citems, parts, out, oflags, rescue;
+    DevBuf desc, rec32, rec32j, rec64, rec64j, teams, witems, witems2, cpairs, citems, parts, out, rescue;  // out: log10 L, then the flags
     DevBuf small;  // counters[8], status[1], dropgrow[4], skew statistics [4], wave tag, CTAs by SM (kSmallBytes)
     DevBuf bnd;    // strip boundaries of the batch
     DevBuf rbnd;   // rescue / launch-per-pair boundary scratch
@@ -499,7 +503,7 @@ struct Slot {
     DevBuf pscan, pscratch;  // device planner: PlanScan, its scratch
     uint32_t sbnd_warps = 0, sbnd_rows = 0;  // what sbnd holds for the current plan
     DevBuf hdr;
-    HostBuf h_out, h_oflags, h_small, h_roff, h_hoff, h_pr, h_ph, h_pscan;
+    HostBuf h_out, h_small, h_pack, h_roff, h_hoff, h_pr, h_ph, h_pscan;
     BatchHeader hh;
     cudaEvent_t ev_copy = nullptr, ev_start = nullptr, ev_fwd0 = nullptr, ev_fwd1 = nullptr,
                 ev_res0 = nullptr, ev_res1 = nullptr, ev_end = nullptr;
@@ -519,6 +523,12 @@ struct Slot {
     int state = 0;  // 0 free, 1 pending
     double* user_out = nullptr;
     uint8_t* user_flags = nullptr;
+    // the plan's arrays (in their arenas, or beside the header)
+    const Team* d_teams = nullptr;
+    const WarpItem *d_witems = nullptr, *d_witems2 = nullptr;
+    const CtaItem* d_citems = nullptr;
+    const CtaPair* d_cpairs = nullptr;
+    bool plan_packed = false;
     bool out_on_dev = false;
     uint32_t n_pairs = 0;
     phmm_stats st{};
@@ -578,7 +588,7 @@ int pow_index(int N) { return N == 12 ? 0 : N == 16 ? 1 : N == 20 ? 2 : N == 24 
 DevBuf* arena_bufs(Slot& S, int i) {
     DevBuf* d[] = {&S.in_bases, &S.in_bq, &S.in_iq, &S.in_dq, &S.in_gq, &S.in_hap, &S.in_roff, &S.in_hoff,
                    &S.in_pr, &S.in_ph, &S.desc, &S.rec32, &S.rec32j, &S.rec64, &S.rec64j, &S.teams, &S.witems, &S.witems2,
-                   &S.cpairs, &S.citems, &S.parts, &S.out, &S.oflags, &S.rescue, &S.bnd, &S.rbnd, &S.sbnd,
+                   &S.cpairs, &S.citems, &S.parts, &S.out, &S.rescue, &S.bnd, &S.rbnd, &S.sbnd,
                    &S.wbnd, &S.pscan, &S.pscratch};
     return i < (int)(sizeof(d) / sizeof(d[0])) ? d[i] : nullptr;
 }
@@ -731,6 +741,11 @@ cudaError_t upload_plan(Slot& S, const Plan& P, cudaStream_t cs) {
     if ((e = ensure(S.witems2, P.witems2.size() * sizeof(WarpItem))) != cudaSuccess) return e;
     if ((e = ensure(S.cpairs, P.n_cpairs() * sizeof(CtaPair))) != cudaSuccess) return e;
     if ((e = ensure(S.citems, P.n_citems() * sizeof(CtaItem))) != cudaSuccess) return e;
+    S.d_teams = (const Team*)S.teams.p;
+    S.d_witems = (const WarpItem*)S.witems.p;
+    S.d_witems2 = (const WarpItem*)S.witems2.p;
+    S.d_citems = (const CtaItem*)S.citems.p;
+    S.d_cpairs = (const CtaPair*)S.cpairs.p;
     if (P.dev) return cudaSuccess;  // build_plan, once the header is there
     auto cp = [&](DevBuf& d, const void* src, size_t n) {
         return n ? cudaMemcpyAsync(d.p, src, n, cudaMemcpyHostToDevice, cs) : cudaSuccess;
@@ -764,12 +779,12 @@ cudaError_t ensure_records(Slot& S, const Plan& P, uint64_t nbases) {
 }
 
 void plan_header(const Slot& S, const Plan& P, BatchHeader& hh) {
-    hh.witems = (const WarpItem*)S.witems.p;
-    hh.witems2 = (const WarpItem*)S.witems2.p;
+    hh.witems = S.d_witems;
+    hh.witems2 = S.d_witems2;
     hh.n_witems2 = (uint32_t)P.witems2.size();
-    hh.teams = (const Team*)S.teams.p;
-    hh.citems = (const CtaItem*)S.citems.p;
-    hh.cpairs = (const CtaPair*)S.cpairs.p;
+    hh.teams = S.d_teams;
+    hh.citems = S.d_citems;
+    hh.cpairs = S.d_cpairs;
     hh.n_witems = (uint32_t)P.witems.size();  // a device-built plan's: written by its last kernel but two
     // short pairs no more than 12 to an SM have a warp each, of few columns a lane: the step of a
     // scheduler's only warp is latency (20 pairs of 150 rows: forward 54 us against 84 in teams;
@@ -1065,6 +1080,17 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     const bool on_dev = !host_plan && plans_on_device(ctx->cfg, np);
     PlanInput pin{};
     PlanScan sc{};
+    uint8_t* const hpk = static_cast<uint8_t*>(S->h_pack.p);
+    size_t pk = kPackStart;  // packed so far
+    auto packed = [](size_t n) { return (n + 255) / 256 * 256; };
+    auto pack = [&](const void* src, size_t n) {
+        const size_t at = pk;
+        if (n) memcpy(hpk + at, src, n);
+        pk += packed(n);
+        return static_cast<uint8_t*>(S->hdr.p) + at;
+    };
+    const size_t index_bytes = packed((nr + 1) * 8ull) + packed((nh + 1) * 8ull) + 2 * packed(np * 4ull);
+    bool index_packed = false;
     if (dev_in && np > 0) {
         // device inputs are produced on the caller's stream: read them after its pending work
         CK(cudaEventRecord(S->ev_user, ctx->stream));
@@ -1072,7 +1098,15 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     }
     if (on_dev) {
         // device planner: the lengths are checked and summed there
-        if (!dev_in) {
+        if (!dev_in && index_bytes <= kPackBytes / 2) {
+            index_packed = true;
+            pin.read_off = (const uint64_t*)pack(roff, (nr + 1) * 8ull);
+            pin.hap_off = (const uint64_t*)pack(hoff, (nh + 1) * 8ull);
+            pin.pair_read = (const uint32_t*)pack(pr, np * 4ull);
+            pin.pair_hap = (const uint32_t*)pack(ph, np * 4ull);
+            CK(cudaMemcpyAsync(static_cast<uint8_t*>(S->hdr.p) + kPackStart, hpk + kPackStart, pk - kPackStart,
+                               cudaMemcpyHostToDevice, cs));
+        } else if (!dev_in) {
             CK(ensure(S->in_roff, (nr + 1) * 8ull));
             CK(ensure(S->in_hoff, (nh + 1) * 8ull));
             CK(ensure(S->in_pr, np * 4ull));
@@ -1082,10 +1116,12 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
             CK(cudaMemcpyAsync(S->in_pr.p, pr, np * 4ull, cudaMemcpyHostToDevice, cs));
             CK(cudaMemcpyAsync(S->in_ph.p, ph, np * 4ull, cudaMemcpyHostToDevice, cs));
         }
-        pin.read_off = dev_in ? roff : static_cast<const uint64_t*>(S->in_roff.p);
-        pin.hap_off = dev_in ? hoff : static_cast<const uint64_t*>(S->in_hoff.p);
-        pin.pair_read = dev_in ? pr : static_cast<const uint32_t*>(S->in_pr.p);
-        pin.pair_hap = dev_in ? ph : static_cast<const uint32_t*>(S->in_ph.p);
+        if (!index_packed) {
+            pin.read_off = dev_in ? roff : static_cast<const uint64_t*>(S->in_roff.p);
+            pin.hap_off = dev_in ? hoff : static_cast<const uint64_t*>(S->in_hoff.p);
+            pin.pair_read = dev_in ? pr : static_cast<const uint32_t*>(S->in_pr.p);
+            pin.pair_hap = dev_in ? ph : static_cast<const uint32_t*>(S->in_ph.p);
+        }
         pin.n_reads = nr;
         pin.n_haps = nh;
         pin.n_pairs = np;
@@ -1312,11 +1348,25 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     // device arenas
     BatchHeader& hh = S->hh;
     memset(&hh, 0, sizeof(hh));
+    const size_t base_bytes = dev_in ? 0 : 5 * packed(nbases) + packed(nhb) + (on_dev ? 0 : index_bytes);
+    const size_t plan_bytes = P.dev ? 0 : packed(P.teams.size() * sizeof(Team)) + packed(P.witems.size() * sizeof(WarpItem)) +
+                                              packed(P.witems2.size() * sizeof(WarpItem)) +
+                                              packed(P.cpairs.size() * sizeof(CtaPair)) +
+                                              packed(P.citems.size() * sizeof(CtaItem));
+    const bool all_packed = np > 0 && (!on_dev || dev_in || index_packed) && pk + base_bytes + plan_bytes <= kPackStart + kPackBytes;
     if (dev_in) {
         hh.read_bases = b->read_bases; hh.base_q = b->base_q; hh.ins_q = b->ins_q;
         hh.del_q = b->del_q; hh.gcp_q = b->gcp_q; hh.hap_bases = b->hap_bases;
         hh.read_off = b->read_off; hh.hap_off = b->hap_off;
         hh.pair_read = b->pair_read; hh.pair_hap = b->pair_hap;
+    } else if (all_packed) {
+        hh.read_bases = pack(b->read_bases, nbases); hh.base_q = pack(b->base_q, nbases);
+        hh.ins_q = pack(b->ins_q, nbases); hh.del_q = pack(b->del_q, nbases);
+        hh.gcp_q = pack(b->gcp_q, nbases); hh.hap_bases = pack(b->hap_bases, nhb);
+        hh.read_off = on_dev ? pin.read_off : (const uint64_t*)pack(b->read_off, (nr + 1) * 8ull);
+        hh.hap_off = on_dev ? pin.hap_off : (const uint64_t*)pack(b->hap_off, (nh + 1) * 8ull);
+        hh.pair_read = on_dev ? pin.pair_read : (const uint32_t*)pack(b->pair_read, np * 4ull);
+        hh.pair_hap = on_dev ? pin.pair_hap : (const uint32_t*)pack(b->pair_hap, np * 4ull);
     } else if (np > 0) {
         CK(ensure(S->in_bases, nbases)); CK(ensure(S->in_bq, nbases)); CK(ensure(S->in_iq, nbases));
         CK(ensure(S->in_dq, nbases)); CK(ensure(S->in_gq, nbases)); CK(ensure(S->in_hap, nhb));
@@ -1340,8 +1390,10 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
         hh.read_bases = (const uint8_t*)S->in_bases.p; hh.base_q = (const uint8_t*)S->in_bq.p;
         hh.ins_q = (const uint8_t*)S->in_iq.p; hh.del_q = (const uint8_t*)S->in_dq.p;
         hh.gcp_q = (const uint8_t*)S->in_gq.p; hh.hap_bases = (const uint8_t*)S->in_hap.p;
-        hh.read_off = (const uint64_t*)S->in_roff.p; hh.hap_off = (const uint64_t*)S->in_hoff.p;
-        hh.pair_read = (const uint32_t*)S->in_pr.p; hh.pair_hap = (const uint32_t*)S->in_ph.p;
+        hh.read_off = on_dev ? pin.read_off : (const uint64_t*)S->in_roff.p;
+        hh.hap_off = on_dev ? pin.hap_off : (const uint64_t*)S->in_hoff.p;
+        hh.pair_read = on_dev ? pin.pair_read : (const uint32_t*)S->in_pr.p;
+        hh.pair_hap = on_dev ? pin.pair_hap : (const uint32_t*)S->in_ph.p;
     }
     CK(ensure(S->desc, np * sizeof(PairDesc)));
     if (ctx->cfg.precision != PHMM_PREC_FP64) {
@@ -1358,13 +1410,20 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     CK(ensure(S->bnd, P.bnd_words * 8ull));
     CK(ensure_serial(ctx, *S, P));
     if (ctx->cfg.precision != PHMM_PREC_FP32_ONLY) CK(ensure(S->rbnd, rb_bytes));
-    CK(ensure(S->out, np * 8ull));
-    CK(ensure(S->oflags, np * 1ull));
+    CK(ensure(S->out, np * 9ull));
     CK(ensure(S->rescue, np * 4ull));
-    CK(ensure(S->h_out, np * 8ull));
-    CK(ensure(S->h_oflags, np * 1ull));
-    if (!reuse) CK(upload_plan(*S, P, cs));
-    CK(cudaMemsetAsync(S->parts.p, 0, (np + P.n_extra) * sizeof(Partial), cs));
+    CK(ensure(S->h_out, np * 9ull));
+    if (all_packed && !P.dev) {
+        S->d_teams = (const Team*)pack(P.teams.data(), P.teams.size() * sizeof(Team));
+        S->d_witems = (const WarpItem*)pack(P.witems.data(), P.witems.size() * sizeof(WarpItem));
+        S->d_witems2 = (const WarpItem*)pack(P.witems2.data(), P.witems2.size() * sizeof(WarpItem));
+        S->d_cpairs = (const CtaPair*)pack(P.cpairs.data(), P.cpairs.size() * sizeof(CtaPair));
+        S->d_citems = (const CtaItem*)pack(P.citems.data(), P.citems.size() * sizeof(CtaItem));
+        S->plan_packed = true;
+    } else if (!reuse || S->plan_packed) {
+        CK(upload_plan(*S, P, cs));
+        S->plan_packed = false;
+    }
     hh.n_read_bases = nbases;
     hh.n_reads = nr;
     hh.n_haps = nh;
@@ -1384,7 +1443,7 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     hh.tol32 = ctx->cfg.fp32_tolerance > 0.0 ? ctx->cfg.fp32_tolerance : 1e-3;
     hh.parts = (Partial*)S->parts.p;
     hh.out = (double*)S->out.p;
-    hh.out_flags = (uint8_t*)S->oflags.p;
+    hh.out_flags = (uint8_t*)S->out.p + np * 8ull;
     hh.rescue_list = (uint32_t*)S->rescue.p;
     hh.counters = (uint32_t*)S->small.p;          // words 0..7
     hh.status = (uint32_t*)S->small.p + 8;        // word 8
@@ -1394,11 +1453,12 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     hh.sm_rank = (uint32_t*)S->small.p + 32;      // words 32 ..
     hh.seed = ctx->seed;
     hh.mode = (uint32_t)ctx->cfg.precision;
-    CK(cudaMemcpyAsync(S->hdr.p, &hh, sizeof(hh), cudaMemcpyHostToDevice, cs));
+    memcpy(hpk, &hh, sizeof(hh));
+    CK(cudaMemcpyAsync(S->hdr.p, hpk, all_packed ? pk : sizeof(hh), cudaMemcpyHostToDevice, cs));
     if (P.dev) CK(build_plan(*S, P, pin, ctx->sms, cs));
     CK(cudaEventRecord(S->ev_copy, cs));
-    // host inputs may be released when submit returns
-    CK(cudaEventSynchronize(S->ev_copy));
+    // host inputs may be released when submit returns (packed ones already are)
+    if (!all_packed) CK(cudaEventSynchronize(S->ev_copy));
     // this slot's pipeline runs after the caller's pending work and the uploads
     CK(cudaEventRecord(S->ev_user, ctx->stream));
     CK(cudaStreamWaitEvent(S->sm, S->ev_user, 0));
@@ -1441,13 +1501,13 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
         ctx->tuned[tune_sig] = {best, -1, 0};
         make_plan64(L.data(), K.data(), pr, np, best, P, wave64);
         CK(upload_plan(*S, P, cs));
+        S->plan_packed = false;
         CK(ensure(S->parts, (np + P.n_extra) * sizeof(Partial)));
         CK(ensure(S->bnd, P.bnd_words * 8ull));
         CK(ensure_serial(ctx, *S, P));
         hh.parts = (Partial*)S->parts.p;
         plan_header(*S, P, hh);
         CK(cudaMemcpyAsync(S->hdr.p, &hh, sizeof(hh), cudaMemcpyHostToDevice, cs));
-        CK(cudaMemsetAsync(S->parts.p, 0, (np + P.n_extra) * sizeof(Partial), cs));
         CK(cudaStreamSynchronize(cs));
     }
     if (tune_short || tune_long) {
@@ -1524,6 +1584,7 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
         ctx->tuned[tune_sig] = {bs, bp, bl};
         plan_of(bs, bp, bl, P);
         CK(upload_plan(*S, P, cs));
+        S->plan_packed = false;
         CK(ensure(S->parts, (np + P.n_extra) * sizeof(Partial)));
         CK(ensure(S->bnd, P.bnd_words * 8ull));
         CK(ensure_serial(ctx, *S, P));
@@ -1532,7 +1593,6 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
         plan_header(*S, P, hh);
         CK(cudaMemcpyAsync(S->hdr.p, &hh, sizeof(hh), cudaMemcpyHostToDevice, cs));
         if (P.dev) CK(build_plan(*S, P, pin, ctx->sms, cs));
-        CK(cudaMemsetAsync(S->parts.p, 0, (np + P.n_extra) * sizeof(Partial), cs));
         CK(cudaStreamSynchronize(cs));
         N = P.N;
     }
@@ -1582,11 +1642,10 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
         }
         // outputs
         if (b->outputs_on_device) {
-            CK(cudaMemcpyAsync(b->out_log10, S->out.p, np * 8ull, cudaMemcpyDeviceToDevice, s));
-            if (b->out_flags) CK(cudaMemcpyAsync(b->out_flags, S->oflags.p, np, cudaMemcpyDeviceToDevice, s));
+            CK(cudaMemcpyAsync(b->out_log10, hh.out, np * 8ull, cudaMemcpyDeviceToDevice, s));
+            if (b->out_flags) CK(cudaMemcpyAsync(b->out_flags, hh.out_flags, np, cudaMemcpyDeviceToDevice, s));
         } else {
-            CK(cudaMemcpyAsync(S->h_out.p, S->out.p, np * 8ull, cudaMemcpyDeviceToHost, s));
-            CK(cudaMemcpyAsync(S->h_oflags.p, S->oflags.p, np, cudaMemcpyDeviceToHost, s));
+            CK(cudaMemcpyAsync(S->h_out.p, S->out.p, np * 9ull, cudaMemcpyDeviceToHost, s));
         }
         CK(cudaMemcpyAsync(S->h_small.p, S->small.p, 64, cudaMemcpyDeviceToHost, s));
     } else {
@@ -1762,7 +1821,8 @@ int phmm_create(const phmm_config* cfg, phmm_ctx** out) {
         for (auto* q : sts)
             if (cudaStreamCreateWithFlags(q, cudaStreamNonBlocking) != cudaSuccess) return fail(PHMM_ECUDA);
         if (ensure(S.small, kSmallBytes) != cudaSuccess || ensure(S.h_small, 64) != cudaSuccess ||
-            ensure(S.hdr, sizeof(BatchHeader)) != cudaSuccess || cudaMemset(S.small.p, 0, kSmallBytes) != cudaSuccess)
+            ensure(S.hdr, kPackStart + kPackBytes) != cudaSuccess ||
+            ensure(S.h_pack, kPackStart + kPackBytes) != cudaSuccess || cudaMemset(S.small.p, 0, kSmallBytes) != cudaSuccess)
             return fail(PHMM_ECUDA);
     }
     if (cudaGetLastError() != cudaSuccess) return fail(PHMM_ECUDA);
@@ -1783,11 +1843,11 @@ void phmm_destroy(phmm_ctx* ctx) {
     for (auto& S : ctx->slots) {
         DevBuf* d[] = {&S.in_bases, &S.in_bq, &S.in_iq, &S.in_dq, &S.in_gq, &S.in_hap, &S.in_roff,
                        &S.in_hoff, &S.in_pr, &S.in_ph, &S.desc, &S.rec32, &S.rec32j, &S.rec64, &S.rec64j, &S.teams,
-                       &S.witems, &S.witems2, &S.cpairs, &S.citems, &S.parts, &S.out, &S.oflags, &S.rescue,
+                       &S.witems, &S.witems2, &S.cpairs, &S.citems, &S.parts, &S.out, &S.rescue,
                        &S.small, &S.hdr, &S.bnd, &S.rbnd, &S.sbnd, &S.wbnd,
                        &S.pscan, &S.pscratch};
         for (auto* b : d) release(*b);
-        HostBuf* h[] = {&S.h_out, &S.h_oflags, &S.h_small, &S.h_roff, &S.h_hoff, &S.h_pr, &S.h_ph, &S.h_pscan};
+        HostBuf* h[] = {&S.h_out, &S.h_small, &S.h_pack, &S.h_roff, &S.h_hoff, &S.h_pr, &S.h_ph, &S.h_pscan};
         for (auto* b : h) release(*b);
         cudaEvent_t evs[] = {S.ev_copy, S.ev_start, S.ev_fwd0, S.ev_fwd1, S.ev_res0, S.ev_res1, S.ev_end,
                              S.ev_br[0], S.ev_br[1], S.ev_br[2], S.ev_br[3], S.ev_br[4], S.ev_br[5]};
@@ -1872,12 +1932,14 @@ int phmm_poll(phmm_ctx* ctx, uint64_t ticket, int timeout_ms) {
             const double el = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
             if (el >= timeout_ms) return PHMM_PENDING;
         }
-        std::this_thread::sleep_for(std::chrono::microseconds(50));
+        // a small batch is done within this time, where a sleep would cost as much as its kernels
+        if (std::chrono::steady_clock::now() - t0 < std::chrono::microseconds(400)) std::this_thread::yield();
+        else std::this_thread::sleep_for(std::chrono::microseconds(50));
     }
     std::lock_guard<std::mutex> lock(ctx->mu);
     if (!S->out_on_dev && S->n_pairs > 0) {
         memcpy(S->user_out, S->h_out.p, S->n_pairs * 8ull);
-        if (S->user_flags) memcpy(S->user_flags, S->h_oflags.p, S->n_pairs);
+        if (S->user_flags) memcpy(S->user_flags, static_cast<const uint8_t*>(S->h_out.p) + S->n_pairs * 8ull, S->n_pairs);
     }
     const uint32_t* sm = static_cast<const uint32_t*>(S->h_small.p);
     S->st.n_rescued = sm[2];

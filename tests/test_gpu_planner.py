@@ -10,7 +10,7 @@ import oracle
 from paper_2606_25738_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
-HOST = 4095  # pairs that the host planner still takes
+HOST = 3000  # pairs of a host plan: more short ones than resident warps, so in teams too
 
 
 @pytest.fixture(scope="module")
@@ -111,3 +111,20 @@ def test_small_budget_takes_cta_strips(phmm):
     assert rc == 0 and st["long_kernel"] == 1
     with phmm.Context(precision="fp32_only", flags=phmm.F_NO_TUNE) as ctx:
         assert np.max(np.abs(out - ctx.run(b)[0])) <= 1e-3
+
+
+@pytest.mark.parametrize("where", ["host", "device"])
+@pytest.mark.parametrize("l", [195, 200, 205, 210])
+def test_packed_and_separate_copies(phmm, l, where):
+    """1000 reads whose host arrays come to a little less and a little more than what goes to the
+    device in one copy (1 MiB); twice in a row on one slot, so the plan moves or is reused."""
+    n = 1000
+    b = _batch(np.full(n, l), np.full(n, 40), l)
+    pick = np.arange(0, n, 37)
+    ref = oracle.batch(W.subset(b, pick))
+    with phmm.Context(precision="fp32", max_inflight=1, flags=phmm.F_NO_TUNE) as ctx:
+        small = _batch(np.full(n, 20), np.full(n, 40), 1)
+        for x in (b, b, small, b):
+            out, flags, rc, st = ctx.run(phmm.to_device(x) if where == "device" else x)
+            assert rc == 0
+    assert np.max(np.abs(out[pick] - ref)) <= 1e-3
