@@ -70,10 +70,10 @@ __device__ __forceinline__ void store_rec32j(Rec32J* dst, const Rec32J& r) {
 // at unaligned or ragged edges, zeros outside), so each thread then reads its bases from
 // shared memory and the records it writes stay consecutive across the warp.
 constexpr int kPrepThreads = 256, kPrepTile = kPrepThreads * 16;
-__device__ __forceinline__ void stage_bytes(const uint8_t* __restrict__ src, uint64_t n, uint64_t t0,
+__device__ __forceinline__ void stage_bytes(const uint8_t* __restrict__ src, uint64_t n, uint64_t t0, int tile,
                                             uint4* __restrict__ dst) {
     const bool al = ((uintptr_t)src & 15u) == 0;
-    for (int c = threadIdx.x; c < kPrepTile / 16 + 1; c += blockDim.x) {
+    for (int c = threadIdx.x; c < tile / 16 + 1; c += blockDim.x) {
         const int64_t g = (int64_t)t0 - 16 + 16 * (int64_t)c;  // first byte of chunk c
         uint4 v;
         if (al && g >= 0 && g + 16 <= (int64_t)n) {
@@ -92,10 +92,29 @@ __device__ __forceinline__ void stage_bytes(const uint8_t* __restrict__ src, uin
     }
 }
 
+// First index of the non-decreasing a[0 .. n - 1] with a[i] >= v, by the whole block (256
+// probes a round).
+__device__ __forceinline__ uint32_t block_lower_bound(const uint64_t* __restrict__ a, uint32_t n, uint64_t v) {
+    uint32_t lo = 0, hi = n;
+    while (lo < hi) {
+        const uint32_t step = (hi - lo + kPrepThreads - 1) / kPrepThreads, at = lo + threadIdx.x * step;
+        const uint32_t c = (uint32_t)__syncthreads_count(at < hi && a[at] < v);  // a[lo + (c - 1) step] < v
+        hi = min(hi, lo + c * step);
+        if (c == 0) break;
+        lo += (c - 1) * step + 1;
+    }
+    return lo;
+}
+
+// A tile has as few bases a thread (1 to 16) as give every block one: 1,500 read bases took 19 us in
+// one tile of 4096, 75,000 took 31 us.  Row 1 of a read (the previous row's T_MI is 1 there) is known
+// by a bit per base, set from the offsets that lie in the tile; a kernel of its own for these rows
+// took 8 us more.
 __global__ void __launch_bounds__(kPrepThreads) k_prep32(const BatchHeader* __restrict__ H,
                                                          const PhredTables* __restrict__ TG) {
     __shared__ Tables32 T;
     __shared__ uint4 sb[5][kPrepTile / 16 + 1];  // bases, Q, ins, del, gcp; byte 16 = tile start
+    __shared__ uint32_t starts[kPrepTile / 32];
     if (blockIdx.x == 0 && threadIdx.x == 0) *H->wave_epoch = *H->wave_epoch % kWaveTags + 1u;
     stage_tables32(TG, T);
     const float2 *tq = T.tq, *tom = T.tom, *tq3 = T.tq3, *tinv = T.tinv;
@@ -105,17 +124,29 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep32(const BatchHeader* __re
     const uint64_t n = H->n_read_bases;
     const uint32_t seed = H->seed;
     const uint8_t* const s8[5] = {H->read_bases, H->base_q, H->ins_q, H->del_q, H->gcp_q};
-    for (uint64_t t0 = (uint64_t)blockIdx.x * kPrepTile; t0 < n; t0 += (uint64_t)gridDim.x * kPrepTile) {
+    const uint64_t once = (uint64_t)gridDim.x * kPrepThreads;
+    const int per = (int)min((n + once - 1) / once, (uint64_t)(kPrepTile / kPrepThreads)), tile = per * kPrepThreads;
+    for (uint64_t t0 = (uint64_t)blockIdx.x * tile; t0 < n; t0 += (uint64_t)gridDim.x * tile) {
         __syncthreads();  // the previous tile's reads are done
 #pragma unroll
-        for (int q = 0; q < 5; ++q) stage_bytes(s8[q], n, t0, sb[q]);
+        for (int q = 0; q < 5; ++q) stage_bytes(s8[q], n, t0, tile, sb[q]);
+        if (rj) {
+            if (threadIdx.x < kPrepTile / 32) starts[threadIdx.x] = 0u;
+            const uint32_t r0 = block_lower_bound(H->read_off, H->n_reads, t0);
+            __syncthreads();
+            for (uint32_t r = r0 + threadIdx.x; r < H->n_reads; r += kPrepThreads) {
+                const uint64_t o = H->read_off[r] - t0;
+                if (o >= (uint64_t)tile) break;
+                atomicOr(&starts[o >> 5], 1u << (o & 31));
+            }
+        }
         __syncthreads();
         const uint8_t* const sbase = reinterpret_cast<const uint8_t*>(sb[0]);
         const uint8_t* const sq = reinterpret_cast<const uint8_t*>(sb[1]);
         const uint8_t* const si = reinterpret_cast<const uint8_t*>(sb[2]);
         const uint8_t* const sd = reinterpret_cast<const uint8_t*>(sb[3]);
         const uint8_t* const sg = reinterpret_cast<const uint8_t*>(sb[4]);
-        for (int m = 0; m < kPrepTile / kPrepThreads; ++m) {
+        for (int m = 0; m < per; ++m) {
             const int o = 16 + m * kPrepThreads + (int)threadIdx.x;  // byte of base b in the stage
             const uint64_t b = t0 + (uint64_t)(o - 16);
             if (b >= n) break;
@@ -144,7 +175,10 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep32(const BatchHeader* __re
             }
             if (rj) {
                 const Rec32J r2 = make_rec32j(x, tq, tom, tq3, tinv, T.tiq, seed, b, false);
-                store_rec32j(rj + b, r2);
+                const uint32_t at = (uint32_t)(o - 16);
+                if (starts[at >> 5] >> (at & 31) & 1u)
+                    store_rec32j(rj + b, make_rec32j(x, tq, tom, tq3, tinv, T.tiq, seed, b, true));
+                else store_rec32j(rj + b, r2);
                 // range of the pipelined engine's intermediates relative to the row maximum
                 const float om = fmaxf(1.0f - r2.g, 0x1p-60f);
                 const float big = fmaxf(fmaxf(fabsf(r2.a), fabsf(r2.b) / om), T.tiq[x.insp].x);
@@ -171,22 +205,6 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep32(const BatchHeader* __re
     __syncthreads();
     block_max2(sk.gcp_max, sk.gcp_inv, w + 2);
     build_desc(H);
-}
-
-// Row 1 of every read in the pipelined-engine records: the previous row's T_MI is 1
-// there (k_prep32 used the previous base of the batch).  Runs after k_prep32.
-__global__ void __launch_bounds__(256) k_prep32_first(const BatchHeader* __restrict__ H,
-                                                      const PhredTables* __restrict__ TG) {
-    __shared__ Tables32 T;
-    stage_tables32(TG, T);
-    Rec32J* const rj = H->rec32j;
-    if (!rj) return;
-    for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < H->n_reads; r += gridDim.x * blockDim.x) {
-        const uint64_t b = H->read_off[r];
-        if (b >= H->read_off[r + 1]) continue;
-        const BaseQ x = base_inputs(H, b);
-        store_rec32j(rj + b, make_rec32j(x, T.tq, T.tom, T.tq3, T.tinv, T.tiq, H->seed, b, true));
-    }
 }
 
 template __global__ void k_forward<float, kNLong32, false>(const BatchHeader*, const PowRow<float>*);
@@ -257,11 +275,6 @@ void launch_reset(const BatchHeader* H, int grid, cudaStream_t s) { k_reset<<<gr
 void launch_prep32(const BatchHeader* H, const PhredTables* T, int grid, cudaStream_t s) {
     k_prep32<<<grid, kPrepThreads, 0, s>>>(H, T);
 }
-
-void launch_prep32_first(const BatchHeader* H, const PhredTables* T, int grid, cudaStream_t s) {
-    k_prep32_first<<<grid, 256, 0, s>>>(H, T);
-}
-
 void launch_forward32_long(const BatchHeader* H, const void* pow, int grid, cudaStream_t s) {
     k_forward<float, kNLong32, false><<<grid, kCtaThreads, 0, s>>>(H, static_cast<const PowRow<float>*>(pow));
 }

@@ -12,7 +12,6 @@ struct PhredTables;
 // FP32 unit
 void launch_reset(const BatchHeader* H, int grid, cudaStream_t s);
 void launch_prep32(const BatchHeader* H, const PhredTables* T, int grid, cudaStream_t s);
-void launch_prep32_first(const BatchHeader* H, const PhredTables* T, int grid, cudaStream_t s);
 void launch_forward32_long(const BatchHeader* H, const void* pow, int grid, cudaStream_t s);
 // FP32 multi-warp kernels: kind 0 = lean engine (N 32, 16-warp CTAs), 1 = pipelined
 // (N 32, 12-warp CTAs), 2 = pipelined (N 24, 16-warp CTAs), 3 = pipelined with packed

@@ -681,7 +681,6 @@ int launch_sequence(phmm_ctx* ctx, Slot& S, int scal_id, int pack_id, int long_k
         CK(rec(S.ev_res1));
     } else {
         launch_prep32(H, T, grid_pre, s);
-        launch_prep32_first(H, T, grid_pre, s);
         CK(rec(S.ev_fwd0));
         // fork: multi-warp pairs and packed teams on two more branches, scalar teams here
         CK(cudaEventRecord(S.ev_fork, s));
@@ -727,8 +726,9 @@ int launch_sequence(phmm_ctx* ctx, Slot& S, int scal_id, int pack_id, int long_k
 
 int kernels_per_launch(int prec, int NP, int fp64_id = 0) {
     const int packed = NP > 0 ? 1 : 0;
-    // FP64: reset, prep, [first-row prep, short teams], forward, finalize, rescue
-    return prec == PHMM_PREC_FP64 ? (f64_pipelined(fp64_id) ? 7 : 5) : prec == PHMM_PREC_FP32_RESCUE ? 8 + packed : 6 + packed;
+    // FP32: reset, prep, multi-warp, [packed,] scalar, finalize, [rescue prep, rescue]; FP64: reset, prep,
+    // [first-row prep, short teams], forward, finalize, rescue
+    return prec == PHMM_PREC_FP64 ? (f64_pipelined(fp64_id) ? 7 : 5) : prec == PHMM_PREC_FP32_RESCUE ? 7 + packed : 5 + packed;
 }
 
 uint64_t u64(const void* p) { return (uint64_t)(uintptr_t)p; }
