@@ -517,8 +517,7 @@ struct Slot {
     bool br_timed = false;
     unsigned br_mask = 0;  // branches whose events the last launch sequence recorded
     uint64_t foot = 0;  // admitted device footprint while pending
-    cudaGraphExec_t gexec = nullptr;
-    int g_key = -1;
+    std::map<int, cudaGraphExec_t> graphs;  // by kernel choice (its arguments are the slot's own)
     uint64_t ticket = 0;
     int state = 0;  // 0 free, 1 pending
     double* user_out = nullptr;
@@ -1616,9 +1615,8 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
             launches = np + 3;
         } else if (use_graph) {
             const int key = P.long_kind * 100000 + ctx->cfg.precision * 10000 + P.scal_id * 100 + (P.pack_id + 1);
-            if (!S->gexec || S->g_key != key) {
-                if (S->gexec) cudaGraphExecDestroy(S->gexec);
-                S->gexec = nullptr;
+            cudaGraphExec_t& gexec = S->graphs[key];
+            if (!gexec) {
                 cudaGraph_t g = nullptr;
                 CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
                 const int rc = launch_sequence(ctx, *S, P.scal_id, P.pack_id, P.long_kind, true);
@@ -1628,12 +1626,11 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
                     ctx->dead = true;
                     return PHMM_ECUDA;
                 }
-                cudaError_t e3 = cudaGraphInstantiate(&S->gexec, g, 0);
+                cudaError_t e3 = cudaGraphInstantiate(&gexec, g, 0);
                 cudaGraphDestroy(g);
                 CK(e3);
-                S->g_key = key;
             }
-            CK(cudaGraphLaunch(S->gexec, s));
+            CK(cudaGraphLaunch(gexec, s));
             launches = (uint32_t)kernels_per_launch(ctx->cfg.precision, P.NP, P.scal_id);
         } else {
             const int rc = launch_sequence(ctx, *S, P.scal_id, P.pack_id, P.long_kind, false);
@@ -1856,7 +1853,8 @@ void phmm_destroy(phmm_ctx* ctx) {
         cudaEvent_t evn[] = {S.ev_fork, S.ev_join, S.ev_join3, S.ev_user};
         for (auto e : evn)
             if (e) cudaEventDestroy(e);
-        if (S.gexec) cudaGraphExecDestroy(S.gexec);
+        for (auto& g : S.graphs)
+            if (g.second) cudaGraphExecDestroy(g.second);
         cudaStream_t sts[] = {S.sm, S.sb2, S.sb3};
         for (auto q : sts)
             if (q) cudaStreamDestroy(q);
