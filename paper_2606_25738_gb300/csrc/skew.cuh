@@ -512,12 +512,11 @@ constexpr int kWaveBlock = 16;  // boundary rows taken at a time
 // null for none; out: this strip's, null for none.
 template <int N, bool WAVE, bool G10>
 __device__ SegOut strip_run_skew(const Rec32J* __restrict__ rec, int l, const uint8_t* __restrict__ hap, int k,
-                                 int strip, const PipeRange& rng, const float4* in, float4* out, SkewStage& st,
+                                 int strip, int scol, const PipeRange& rng, const float4* in, float4* out, SkewStage& st,
                                  uint32_t tag, uint32_t* __restrict__ status) {
     static_assert(N <= 32 && N % 2 == 0, "match masks hold 32 columns; two halves");
     constexpr int H = N / 2;
     const int lane = threadIdx.x & 31;
-    const int scol = strip * 32 * N;
     uint32_t flags = rng.ok ? 0u : PF_DEGEN, mflags = 0;
     skew_masks<N, true>(hap, k, scol + lane * N, st.mask + lane, flags);
     const bool has_left = in != nullptr, has_right = out != nullptr;
