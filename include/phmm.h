@@ -86,7 +86,7 @@ typedef enum {
  * strips exchanging their boundary rows through distributed shared memory. */
 #define PHMM_F_LONG_CLUSTER 0x400u
 /* ... or every strip of a pair on its own warp at the same time, strips linked through
- * global memory in blocks of 32 rows (a strip waits for its left neighbour once per
+ * global memory in blocks of 16 rows (a strip waits for its left neighbour once per
  * block: for a few very wide pairs); the tuner picks the strip width and grid (1024
  * columns on the resident maximum or on two CTAs per SM, or 512 columns). */
 #define PHMM_F_LONG_WAVE 0x800u

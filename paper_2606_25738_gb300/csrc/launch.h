@@ -14,14 +14,14 @@ void launch_reset(const BatchHeader* H, int grid, cudaStream_t s);
 void launch_prep32(const BatchHeader* H, const PhredTables* T, int grid, cudaStream_t s);
 void launch_forward32_long(const BatchHeader* H, const void* pow, int grid, cudaStream_t s);
 // FP32 multi-warp kernels: kind 0 = lean engine (N 32, 16-warp CTAs), 1 = pipelined
-// (N 32, 12-warp CTAs), 2 = pipelined (N 24, 16-warp CTAs), 3 = pipelined with packed
+// (N 32, 12-warp CTAs), 2 = pipelined (N 24, 16-warp CTAs), 3 = skewed with packed
 // column halves, one warp per pair running its 1024-column strips one after another
 // (k_forward_serial, 4-warp CTAs), 4 = pipelined in 4-warp CTAs (3 per SM): strips of
 // 4096 columns, so that a few very wide pairs spread over many SMs, 5 = the same 4-warp
 // strips taken eight at a time by thread-block clusters, neighbouring strips linked
 // through distributed shared memory (k_forward_cluster), 6 = every 1024-column strip of a
 // pair on its own warp at the same time, the strips linked through global memory in blocks
-// of 32 rows (a strip waits for its left neighbour's progress counter once per block,
+// of 16 rows (a strip waits for its left neighbour once per block,
 // k_forward_wave), 7 = kind 6 on a grid of two CTAs per SM (fewer warps share each
 // scheduler, so a long strip chain's row step is shorter), 8 = kind 6 with 16 columns per
 // lane (512-column strips: twice the strips, each row step with half the in-lane chain).
@@ -81,12 +81,11 @@ constexpr int kNLong32 = 32;  // columns per lane of FP32 multi-warp pairs
 // FP32 short-pair kernel variants: columns per lane of scalar teams / packed teams.
 constexpr int kNumScalar = 10;
 constexpr int kShortScalarN[kNumScalar] = {32, 24, 24, 16, 32, 24, 16, 32, 24, 32};
-// scalar ids whose kernel is the pipelined engine (Rec32J records)
+// scalar ids whose kernel reads Rec32J records (the pipelined and the skewed engine)
 constexpr bool kShortScalarPipe[kNumScalar] = {false, false, false, false, true, true, true, true, true, true};
-// scalar ids whose pipelined engine packs the two column halves of a lane (FFMA2)
+// scalar ids of the skewed engine
 constexpr bool kShortScalarHalves[kNumScalar] = {false, false, false, false, false, false, false, true, true, true};
-// scalar ids of the lean halves engine: fused row, records and carry powers from L1, four
-// CTAs per SM
+// scalar ids of the skewed engine in four CTAs per SM
 constexpr bool kShortScalarLean[kNumScalar] = {false, false, false, false, false, false, false, false, false, true};
 constexpr int kNumPacked = 2;
 constexpr int kShortPackedN[kNumPacked] = {12, 16};
