@@ -1179,6 +1179,8 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     uint64_t tune_sig = 0;
     std::vector<std::pair<int, int>> tune_cand;
     const bool reuse = !on_dev && S->plan_valid && S->plan_hash == hsh && S->plan_np == np;
+    // (S->plan is written from here on; a batch refused below leaves a plan of no batch)
+    if (!reuse) S->plan_valid = false;
     // FP32 plan of given kernels, on the host or (its sizes) for the device planner
     auto plan_of = [&](int si, int pi, int lk, Plan& Q) {
         if (on_dev) dev_plan(sc, np, si, lk, Q);

@@ -106,11 +106,13 @@ def test_small_budget_takes_cta_strips(phmm):
     two boundaries of 1000 rows per resident warp: the strips of a CTA need neither."""
     n, l, k = 4096, 1000, 1100
     b = _batch(np.full(n, l), np.full(n, k), 8, 4)
-    with phmm.Context(precision="fp32_only", mem_budget=16 << 20, flags=phmm.F_NO_TUNE) as ctx:
-        out, flags, rc, st = ctx.run(b)
-    assert rc == 0 and st["long_kernel"] == 1
     with phmm.Context(precision="fp32_only", flags=phmm.F_NO_TUNE) as ctx:
-        assert np.max(np.abs(out - ctx.run(b)[0])) <= 1e-3
+        ref = ctx.run(b)[0]
+    with phmm.Context(precision="fp32_only", mem_budget=16 << 20, max_inflight=1, flags=phmm.F_NO_TUNE) as ctx:
+        for _ in range(2):  # what was accepted once is accepted again
+            out, flags, rc, st = ctx.run(b)
+            assert rc == 0 and st["long_kernel"] == 1
+            assert np.max(np.abs(out - ref)) <= 1e-3
 
 
 @pytest.mark.parametrize("where", ["host", "device"])
@@ -128,3 +130,20 @@ def test_packed_and_separate_copies(phmm, l, where):
             out, flags, rc, st = ctx.run(phmm.to_device(x) if where == "device" else x)
             assert rc == 0
     assert np.max(np.abs(out[pick] - ref)) <= 1e-3
+
+
+@pytest.mark.parametrize("planned", ["host", "device"])
+def test_refused_batch_leaves_no_plan(phmm, planned):
+    """A batch over the memory budget between two of the same lengths, on one slot: its plan, of
+    more pairs, is not taken for theirs."""
+    small = _batch(np.full(100, 60), np.full(100, 200), 5)
+    n = {"host": 2000, "device": 5000}[planned]
+    big = _batch(np.full(n, 3000), np.full(n, 300), 6)
+    with phmm.Context(precision="fp32_only", mem_budget=64 << 20, max_inflight=1, flags=phmm.F_NO_TUNE) as ctx:
+        first = ctx.run(small)[0]
+        for _ in range(2):
+            with pytest.raises(phmm.PhmmError) as e:
+                ctx.run(big)
+            assert e.value.status == phmm.PHMM_ENOMEM
+            out, flags, rc, st = ctx.run(small)
+            assert rc == 0 and st["n_pairs"] == 100 and np.array_equal(out, first)
