@@ -1166,11 +1166,16 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     const uint64_t nbases = on_dev ? sc.n_read_bases : np > 0 ? roff[nr] : 0;
     const uint64_t nhb = on_dev ? sc.n_hap_bases : np > 0 ? hoff[nh] : 0;
     // plan (FP32: packed short width from the config or the cost model; FP64: kN64).
-    // A batch with the same pair lengths as this slot's previous one reuses its plan.
+    // A batch with the same pair lengths as this slot's previous one reuses its plan (and the same
+    // reads, where packed teams, whose two pairs share one, may be in it).
     const auto th0 = std::chrono::steady_clock::now();
     uint64_t hsh = 1469598103934665603ull ^ ((uint64_t)ctx->cfg.precision << 32) ^ (uint64_t)ctx->cfg.cols_per_lane ^ ((uint64_t)ctx->cfg.kernel_variant << 40);
+    bool may_pack = false;
+    if (ctx->cfg.precision != PHMM_PREC_FP64)
+        for (const auto& cd : fp32_candidates(ctx->cfg)) may_pack |= cd.second >= 0;
     for (uint32_t p = 0; p < np && !on_dev; ++p) {
         hsh = (hsh ^ ((uint64_t)L[p] << 24 ^ K[p])) * 1099511628211ull;
+        if (may_pack) hsh = (hsh ^ pr[p]) * 1099511628211ull;
     }
     hsh ^= np;
     Plan& P = S->plan;

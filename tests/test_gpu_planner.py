@@ -147,3 +147,18 @@ def test_refused_batch_leaves_no_plan(phmm, planned):
             assert e.value.status == phmm.PHMM_ENOMEM
             out, flags, rc, st = ctx.run(small)
             assert rc == 0 and st["n_pairs"] == 100 and np.array_equal(out, first)
+
+
+@pytest.mark.parametrize("cols", [12, 16])
+def test_same_lengths_other_reads(phmm, cols):
+    """Packed teams hold two pairs of one read: a batch of the same lengths whose pairs come in
+    another order does not take the earlier batch's teams."""
+    b = _batch(np.full(320, 60), np.full(320, 150), 7, 40)
+    rng = np.random.default_rng(2)
+    order = [np.sort(b["pair_read"]), b["pair_read"], rng.permutation(b["pair_read"])]
+    with phmm.Context(precision="fp32", cols_per_lane=cols, variant="packed", max_inflight=1, flags=phmm.F_NO_TUNE) as ctx:
+        for pr in order:
+            x = dict(b, pair_read=pr.astype(np.uint32))
+            out, flags, rc, st = ctx.run(x)
+            assert rc == 0 and st["packed_kernel"] >= 0
+            assert np.max(np.abs(out - oracle.batch(x))) <= 1e-3
