@@ -1263,15 +1263,9 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     }
     N = P.N;
     const auto th_plan = std::chrono::steady_clock::now();
-    // footprint and admission (each record layout only for a plan that reads it, or for the
-    // tuner's trials, which may)
+    // footprint and admission (each record layout only for a plan that reads it)
     const bool need64 = ctx->cfg.precision != PHMM_PREC_FP32_ONLY;
     const bool fp32 = ctx->cfg.precision != PHMM_PREC_FP64;
-    bool need32 = false, need32j = false;
-    auto needs_of = [&](const Plan& Q) {
-        need32 |= fp32 && plan_needs_rec32(Q);
-        need32j |= fp32 && plan_needs_rec32j(Q);
-    };
     uint32_t lmax_b = sc.lmax;
     for (uint32_t p = 0; p < np && !on_dev; ++p) lmax_b = std::max(lmax_b, L[p]);
     // scratch of the FP64 pass: two boundaries (8 words a row) for each CTA that may get a pair;
@@ -1283,43 +1277,28 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
         if (np == 0 || *std::max_element(K.begin(), K.end()) <= (uint32_t)kCtaWarps * 32u * kN64) rb_words = 0;
     }
     const uint64_t rb_bytes = (uint64_t)rescue_ctas * 2 * rb_words * 8ull + 16;
-    auto foot_of = [&]() {
-        need32 = need32j = false;
-        needs_of(P);
-        Plan probe;  // the kernels that the tuner may try
-        probe.dev = true;
-        probe.d_teams = P.n_witems();
-        if (tune_short)
-            for (auto& cd : tune_cand) {
-                probe.scal_id = cd.first;
-                probe.pack_id = cd.second;
-                needs_of(probe);
-            }
-        if (tune_long) {
-            probe.scal_id = P.scal_id;
-            probe.pack_id = P.pack_id;
-            probe.d_items = P.n_citems();
-            for (int lk : long_kinds_of(ctx->cfg)) {
-                probe.long_kind = lk;
-                needs_of(probe);
-            }
-        }
+    auto foot_of = [&](const Plan& Q) {
         return (dev_in ? 0 : nbases * 5 + nhb + (nr + 1) * 8ull + (nh + 1) * 8ull + np * 8ull) +
                (ctx->cfg.precision != PHMM_PREC_FP32_ONLY ? rb_bytes : 0) +
-               np * (sizeof(PairDesc) + sizeof(Partial) + 8 + 1 + 4) + (need32j ? nbases * sizeof(Rec32J) : 0) +
-               (need32 ? nbases * sizeof(Rec32) : 0) +
+               np * (sizeof(PairDesc) + sizeof(Partial) + 8 + 1 + 4) +
+               (fp32 && plan_needs_rec32j(Q) ? nbases * sizeof(Rec32J) : 0) +
+               (fp32 && plan_needs_rec32(Q) ? nbases * sizeof(Rec32) : 0) +
                (need64 ? nbases * sizeof(Rec64) : 0) + (fp32 ? 0 : nbases * sizeof(Rec64J)) +
-               P.n_teams() * sizeof(Team) + (P.n_witems() + P.witems2.size()) * sizeof(WarpItem) +
-               P.n_cpairs() * sizeof(CtaPair) + P.n_citems() * sizeof(CtaItem) + P.bnd_words * 8ull +
-               P.n_extra * sizeof(Partial) + serial_bytes(ctx, P);
+               Q.n_teams() * sizeof(Team) + (Q.n_witems() + Q.witems2.size()) * sizeof(WarpItem) +
+               Q.n_cpairs() * sizeof(CtaPair) + Q.n_citems() * sizeof(CtaItem) + Q.bnd_words * 8ull +
+               Q.n_extra * sizeof(Partial) + serial_bytes(ctx, Q);
     };
-    uint64_t foot = foot_of();
-    // A wave kind that nobody asked for keeps within the bound that phmm_batch_footprint gives
-    // and the budget: else wider strips, else CTA strips.
-    if (!reuse && fp32 && kLongWave[P.long_kind] && long_kinds_of(ctx->cfg).size() > 1) {
+    uint64_t foot = foot_of(P);
+    // A kind that nobody asked for keeps within the bound that phmm_batch_footprint gives and the
+    // budget: a wave kind gives way to wider strips, those to CTA strips.
+    const bool choose_kind = fp32 && long_kinds_of(ctx->cfg).size() > 1;
+    uint64_t most = ctx->budget;
+    if (choose_kind || (!fp32 && (tune64 || P.long_kind == 6))) {
         FootSums q{nbases, nhb, nr, nh, np, lmax_b, sc.cta_rows, sc.cta_strips};
-        const uint64_t most = std::min<uint64_t>(
-            ctx->budget, on_dev ? footprint_bound(ctx, q) : footprint_bound(ctx, nbases, nhb, nr, nh, np, L.data(), K.data()));
+        most = std::min<uint64_t>(
+            most, on_dev ? footprint_bound(ctx, q) : footprint_bound(ctx, nbases, nhb, nr, nh, np, L.data(), K.data()));
+    }
+    if (!reuse && choose_kind && kLongWave[P.long_kind]) {
         for (int lk : {6, 3, 1}) {
             if (foot <= most) break;
             if (on_dev && lk == 1) {  // (serial strips always fit the bound)
@@ -1328,17 +1307,17 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
             }
             const int si = P.scal_id, pi = P.pack_id;
             plan_of(si, pi, lk, P);
-            foot = foot_of();
+            foot = foot_of(P);
         }
+        // (CTA strips are what is left: none of the kinds that would be measured fits.  Nothing is
+        // kept of such a batch, whose shape others with more room may have.)
+        if (P.long_kind == 1) tune_short = tune_long = false;
     }
     // FP64 waves likewise, else CTA strips
-    bool wave64 = !fp32 && P.long_kind == 6;
-    if (!reuse && wave64 &&
-        foot > std::min<uint64_t>(ctx->budget, footprint_bound(ctx, nbases, nhb, nr, nh, np, L.data(), K.data()))) {
+    if (!reuse && !fp32 && P.long_kind == 6 && foot > most) {
         const int id = P.scal_id;
         make_plan64(L.data(), K.data(), pr, np, id, P);
-        foot = foot_of();
-        wave64 = false;
+        foot = foot_of(P);
     }
     if (foot > ctx->budget) return PHMM_ENOMEM;
     if (foot + ctx->inflight_foot > ctx->budget) return PHMM_EBUSY;  // admissible once others retire
@@ -1406,8 +1385,8 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
         // a large arena this plan does not read (e.g. left from the tuner's trials) goes
         // back; a small one stays, so that batches alternating between plans that read it
         // and plans that do not pay no cudaFree (a device-wide synchronisation) each time
-        if (!need32 && S->rec32.cap > kKeepRec32Bytes) release(S->rec32);
-        if (!need32j && S->rec32j.cap > kKeepRec32Bytes) release(S->rec32j);
+        if (!plan_needs_rec32(P) && S->rec32.cap > kKeepRec32Bytes) release(S->rec32);
+        if (!plan_needs_rec32j(P) && S->rec32j.cap > kKeepRec32Bytes) release(S->rec32j);
         CK(ensure_records(*S, P, nbases));
     }
     if (need64) CK(ensure(S->rec64, nbases * sizeof(Rec64)));
@@ -1469,15 +1448,31 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     CK(cudaEventRecord(S->ev_user, ctx->stream));
     CK(cudaStreamWaitEvent(S->sm, S->ev_user, 0));
     CK(cudaStreamWaitEvent(S->sm, S->ev_copy, 0));
+    // What a trial may hold: the bound and budget of the admitted plan, beside the batches in flight.
+    // Arenas of other trials that this one does not read make room for its own.
+    const uint64_t room = std::min<uint64_t>(most, ctx->budget - ctx->inflight_foot);
+    auto make_room = [&](const Plan& Q) {
+        if (slot_capacity(*S) + serial_bytes(ctx, Q) + (fp32 ? nbases * sizeof(Rec32J) : 0) <= room) return;
+        if (!kLongWave[Q.long_kind]) release(S->wbnd);
+        if (!kLongSerial[Q.long_kind]) release(S->sbnd);
+        if (fp32 && !plan_needs_rec32(Q)) release(S->rec32);
+        if (fp32 && !plan_needs_rec32j(Q)) release(S->rec32j);
+    };
     if (tune64) {
         // Measured choice of the FP64 variant: the forward pass of each, twice (the first
         // launch after a plan change runs cold), the faster kept for this batch shape.
         float best_ms = 1e30f;
         int best = P.scal_id;
+        // (variant 2 has waves for more pairs than the admitted plan of variant 3)
+        auto plan64_of = [&](int id, Plan& Q) {
+            make_plan64(L.data(), K.data(), pr, np, id, Q, true);
+            if (Q.long_kind == 6 && foot_of(Q) > most) make_plan64(L.data(), K.data(), pr, np, id, Q);
+        };
         for (int id = 0; id < kNumF64; ++id) {
             Plan c;
-            make_plan64(L.data(), K.data(), pr, np, id, c, wave64);
-            if (c.n_too_long) continue;
+            plan64_of(id, c);
+            if (c.n_too_long || foot_of(c) > room) continue;
+            make_room(c);
             CK(upload_plan(*S, c, cs));
             CK(ensure(S->parts, (np + c.n_extra) * sizeof(Partial)));
             CK(ensure(S->bnd, c.bnd_words * 8ull));
@@ -1505,7 +1500,9 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
             }
         }
         ctx->tuned[tune_sig] = {best, -1, 0};
-        make_plan64(L.data(), K.data(), pr, np, best, P, wave64);
+        plan64_of(best, P);
+        foot = foot_of(P);
+        make_room(P);
         CK(upload_plan(*S, P, cs));
         S->plan_packed = false;
         CK(ensure(S->parts, (np + P.n_extra) * sizeof(Partial)));
@@ -1527,6 +1524,7 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
         if (tune_short)
             for (auto& cd : tune_cand) runs.push_back({cd.first, cd.second, bl});
         const size_t n_short = runs.size();
+        bool long_ran = false;
         if (tune_long) {
             // the serial kind needs about one multi-warp pair per resident warp or more:
             // with far fewer it leaves most of the GPU idle, so it is not worth a (long)
@@ -1549,7 +1547,9 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
             }
             Plan c;
             plan_of(cd[0], cd[1], cd[2], c);
-            if (c.n_too_long) continue;
+            if (c.n_too_long || foot_of(c) > room) continue;
+            long_ran |= ri >= n_short;
+            make_room(c);
             CK(upload_plan(*S, c, cs));
             CK(ensure(S->parts, (np + c.n_extra) * sizeof(Partial)));
             CK(ensure(S->bnd, c.bnd_words * 8ull));
@@ -1587,8 +1587,11 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
                 bl = cd[2];
             }
         }
-        ctx->tuned[tune_sig] = {bs, bp, bl};
+        // (a kind that was never run against another is no choice to keep)
+        if (!tune_long || long_ran) ctx->tuned[tune_sig] = {bs, bp, bl};
         plan_of(bs, bp, bl, P);
+        foot = foot_of(P);
+        make_room(P);
         CK(upload_plan(*S, P, cs));
         S->plan_packed = false;
         CK(ensure(S->parts, (np + P.n_extra) * sizeof(Partial)));

@@ -101,18 +101,41 @@ def test_bad_batches_refused(phmm):
         assert rc == 0 and np.all(np.isfinite(out))
 
 
-def test_small_budget_takes_cta_strips(phmm):
+@pytest.mark.parametrize("tuned", [False, True])
+def test_small_budget_takes_cta_strips(phmm, tuned):
     """A memory budget that holds neither the waves' boundary rows (4096 x 1000 of 16 bytes) nor
-    two boundaries of 1000 rows per resident warp: the strips of a CTA need neither."""
+    two boundaries of 1000 rows per resident warp: the strips of a CTA need neither, and the tuner
+    does not bring back what did not fit."""
     n, l, k = 4096, 1000, 1100
     b = _batch(np.full(n, l), np.full(n, k), 8, 4)
     with phmm.Context(precision="fp32_only", flags=phmm.F_NO_TUNE) as ctx:
         ref = ctx.run(b)[0]
-    with phmm.Context(precision="fp32_only", mem_budget=16 << 20, max_inflight=1, flags=phmm.F_NO_TUNE) as ctx:
+    with phmm.Context(precision="fp32_only", mem_budget=16 << 20, max_inflight=1, flags=0 if tuned else phmm.F_NO_TUNE) as ctx:
         for _ in range(2):  # what was accepted once is accepted again
             out, flags, rc, st = ctx.run(b)
             assert rc == 0 and st["long_kernel"] == 1
             assert np.max(np.abs(out - ref)) <= 1e-3
+
+
+@pytest.mark.parametrize("precision", ["fp32_only", "fp64"])
+def test_tuner_keeps_to_the_budget(phmm, precision):
+    """FP32: the 512-column wave strips need 960 MB of boundary rows, the 1024-column ones 384 MB.
+    FP64: waves of the pairs up to 1024 columns, which only variant 2 makes, 290 MB.  Neither
+    trial may take what the budget does not hold (64 MB: two megabytes a buffer)."""
+    import torch
+    if precision == "fp64":
+        n, l, k, budget = 3010, 3000, np.concatenate([np.full(3000, 800), np.full(10, 2000)]), 150 << 20
+    else:
+        n, l, k, budget = 600, 20000, np.full(600, 3000), 500 << 20
+    b = _batch(np.full(n, l), k, 9, 10)
+    with phmm.Context(precision=precision, mem_budget=budget, max_inflight=1) as ctx:
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        out, flags, rc, st = ctx.run(b)
+        assert rc == 0 and np.all(np.isfinite(out))
+        assert free - torch.cuda.mem_get_info()[0] <= budget + (64 << 20)
+        if precision != "fp64":
+            assert st["long_kernel"] in (6, 7)
 
 
 @pytest.mark.parametrize("where", ["host", "device"])
