@@ -1290,17 +1290,19 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     };
     uint64_t foot = foot_of(P);
     // A kind that nobody asked for keeps within the bound that phmm_batch_footprint gives and the
-    // budget: a wave kind gives way to wider strips, those to CTA strips.
+    // budget: a wave kind gives way to wider strips, those to CTA strips.  (Wave kinds that were asked for:
+    // the budget only, and wider strips.)
     const bool choose_kind = fp32 && long_kinds_of(ctx->cfg).size() > 1;
+    const bool wave_asked = (ctx->cfg.flags & PHMM_F_LONG_WAVE) != 0;
     uint64_t most = ctx->budget;
-    if (choose_kind || (!fp32 && (tune64 || P.long_kind == 6))) {
+    if ((choose_kind && !wave_asked) || (!fp32 && (tune64 || P.long_kind == 6))) {
         FootSums q{nbases, nhb, nr, nh, np, lmax_b, sc.cta_rows, sc.cta_strips};
         most = std::min<uint64_t>(
             most, on_dev ? footprint_bound(ctx, q) : footprint_bound(ctx, nbases, nhb, nr, nh, np, L.data(), K.data()));
     }
     if (!reuse && choose_kind && kLongWave[P.long_kind]) {
         for (int lk : {6, 3, 1}) {
-            if (foot <= most) break;
+            if (foot <= most || (wave_asked && lk != 6)) break;
             if (on_dev && lk == 1) {  // (serial strips always fit the bound)
                 if (foot <= ctx->budget) break;
                 return submit_locked(ctx, b, ticket, true);  // CTA strips are planned on the host

@@ -185,3 +185,17 @@ def test_same_lengths_other_reads(phmm, cols):
             out, flags, rc, st = ctx.run(x)
             assert rc == 0 and st["packed_kernel"] >= 0
             assert np.max(np.abs(out - oracle.batch(x))) <= 1e-3
+
+
+@pytest.mark.parametrize("n", [2400, 4096])
+def test_asked_waves_stay_waves(phmm, n):
+    """F_LONG_WAVE fixes the wave kinds, also where their boundary rows are beyond what the library
+    would take by itself; the budget only decides the width of the strips."""
+    b = _batch(np.full(n, 300), np.full(n, 4200), 12, 4)
+    ref = oracle.batch(W.subset(b, np.arange(0, n, 200)))
+    rows = n * 300 * 16  # bytes a boundary: 4 with strips of 1024 columns, 8 with 512
+    for budget, kinds in ((0, (8,)), (6 * rows, (6,))):
+        with phmm.Context(precision="fp32_only", mem_budget=budget, flags=phmm.F_LONG_WAVE | phmm.F_NO_TUNE) as ctx:
+            out, flags, rc, st = ctx.run(b)
+        assert rc == 0 and st["long_kernel"] in kinds
+        assert np.max(np.abs(out[::200] - ref)) <= 1e-3
