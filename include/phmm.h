@@ -229,7 +229,9 @@ int phmm_submit_batch(phmm_ctx *ctx, const phmm_batch *batch, uint64_t *ticket);
 
 /* Upper bound of the device bytes a batch with host inputs needs while in flight (inputs,
  * per-base coefficient records, per-pair descriptors and work items, strip boundaries
- * of very wide pairs, FP64 rescue scratch), as counted against the memory budget.
+ * of very wide pairs, FP64 rescue scratch, the device planner's scratch), as counted against
+ * the memory budget.  What a context holds from phmm_create on (tables; a header of 1 MiB a
+ * slot, in which a small batch's inputs travel) is not part of a batch.
  * Offsets and pair indices must be valid (PHMM_EINVAL otherwise); bases and qualities
  * are not read. */
 int phmm_batch_footprint(phmm_ctx *ctx, const phmm_batch *batch, uint64_t *bytes);

@@ -1013,6 +1013,9 @@ void dev_plan(const PlanScan& sc, uint32_t np, int scal_id, int long_kind, Plan&
     P.cells_br[2] = sc.cells - sc.short_cells[w];
 }
 
+// What the device planner holds beside the plan.
+uint64_t planner_bytes(uint32_t np) { return sizeof(PlanScan) + plan_scratch_bytes(np); }
+
 // Upper bound of the device bytes of a batch with host inputs (phmm_batch_footprint).  The
 // wave kinds' boundaries have no term of their own: the kind chosen without measurement is
 // one whose plan fits (submit).
@@ -1033,6 +1036,7 @@ uint64_t footprint_bound(const phmm_ctx* ctx, const FootSums& q) {
     if (need64) f += (uint64_t)ctx->sms * ctx->occ64 * 2 * q.lmax * 8 * 8 + 16;
     if (prec != PHMM_PREC_FP64)  // serial multi-warp kind: two boundaries per resident warp
         f += (uint64_t)ctx->sms * ctx->occ_longk[3] * (kSerialThreads / 32) * 2 * q.lmax * sizeof(float4);
+    if (plans_on_device(ctx->cfg, q.np)) f += planner_bytes(q.np);
     return f;
 }
 uint64_t footprint_bound(const phmm_ctx* ctx, uint64_t nbases, uint64_t nhb, uint32_t nr, uint32_t nh, uint32_t np,
@@ -1286,7 +1290,7 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
                (need64 ? nbases * sizeof(Rec64) : 0) + (fp32 ? 0 : nbases * sizeof(Rec64J)) +
                Q.n_teams() * sizeof(Team) + (Q.n_witems() + Q.witems2.size()) * sizeof(WarpItem) +
                Q.n_cpairs() * sizeof(CtaPair) + Q.n_citems() * sizeof(CtaItem) + Q.bnd_words * 8ull +
-               Q.n_extra * sizeof(Partial) + serial_bytes(ctx, Q);
+               Q.n_extra * sizeof(Partial) + serial_bytes(ctx, Q) + (Q.dev ? planner_bytes(np) : 0);
     };
     uint64_t foot = foot_of(P);
     // A kind that nobody asked for keeps within the bound that phmm_batch_footprint gives and the
@@ -1321,6 +1325,8 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
         make_plan64(L.data(), K.data(), pr, np, id, P);
         foot = foot_of(P);
     }
+    // (a budget that holds all but the device planner's scratch)
+    if (on_dev && foot > ctx->budget && foot - planner_bytes(np) <= ctx->budget) return submit_locked(ctx, b, ticket, true);
     if (foot > ctx->budget) return PHMM_ENOMEM;
     if (foot + ctx->inflight_foot > ctx->budget) return PHMM_EBUSY;  // admissible once others retire
     {

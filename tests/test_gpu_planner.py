@@ -199,3 +199,19 @@ def test_asked_waves_stay_waves(phmm, n):
             out, flags, rc, st = ctx.run(b)
         assert rc == 0 and st["long_kernel"] in kinds
         assert np.max(np.abs(out[::200] - ref)) <= 1e-3
+
+
+def test_footprint_counts_the_planner(phmm):
+    """The device planner's scratch (over 5 MB) is part of a batch's footprint, and a budget that
+    holds all but it still takes the batch, planned on the host."""
+    n = 5000
+    b = _batch(np.full(n, 20), np.full(n, 100), 13)
+    with phmm.Context(precision="fp32_only") as ctx:
+        below, need = (ctx.footprint(W.subset(b, np.arange(m))) for m in (4095, 4096))
+        assert need - below > 5 << 20
+        need = ctx.footprint(b)
+        ref = ctx.run(b)[0]
+    for budget in (need, 7 << 20):
+        with phmm.Context(precision="fp32_only", mem_budget=budget) as ctx:
+            out, flags, rc, st = ctx.run(b)
+        assert rc == 0 and np.array_equal(out, ref)
