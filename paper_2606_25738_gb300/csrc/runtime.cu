@@ -514,8 +514,7 @@ struct Slot {
     // FP32 forward branches, each timed on its own stream: [0, 1] scalar short teams (sm),
     // [2, 3] packed teams (sb3), [4, 5] multi-warp pairs (sb2)
     cudaEvent_t ev_br[6] = {};
-    bool br_timed = false;
-    unsigned br_mask = 0;  // branches whose events the last launch sequence recorded
+    unsigned br_mask = 0;  // branches whose events the batch's launch sequence records (0: it has none)
     uint64_t foot = 0;  // admitted device footprint while pending
     std::map<int, cudaGraphExec_t> graphs;  // by kernel choice (its arguments are the slot's own)
     uint64_t ticket = 0;
@@ -666,11 +665,8 @@ int launch_sequence(phmm_ctx* ctx, Slot& S, int scal_id, int pack_id, int long_k
             launch_short_pipe64(scal_id, H, ctx->sms * ctx->occ64s[scal_id], s);
             CK(rec(S.ev_br[1]));
             CK(cudaStreamWaitEvent(s, S.ev_join, 0));
-            S.br_timed = true;
-            S.br_mask = 0x5u;  // no packed branch in FP64
         } else {
             launch_forward64(scal_id, H, pw, ctx->sms * ctx->occ64v[scal_id], s);
-            S.br_timed = false;
         }
         CK(rec(S.ev_fwd1));
         launch_finalize64(H, grid_pre, s);
@@ -706,8 +702,6 @@ int launch_sequence(phmm_ctx* ctx, Slot& S, int scal_id, int pack_id, int long_k
         launch_short_scalar(scal_id, H, ctx->pow32[pow_index(kShortScalarN[scal_id])].p,
                             ctx->sms * ctx->occ_scalar[scal_id], s);
         CK(rec(S.ev_br[1]));
-        S.br_timed = true;
-        S.br_mask = 0x7u;
         CK(cudaStreamWaitEvent(s, S.ev_join, 0));
         CK(cudaStreamWaitEvent(s, S.ev_join3, 0));
         CK(rec(S.ev_fwd1));
@@ -1616,9 +1610,13 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     cudaStream_t s = S->sm;
     CK(cudaEventRecord(S->ev_start, s));
     uint32_t launches = 0;
+    S->br_mask = 0;
     if (np > 0) {
         const bool per_pair = ctx->cfg.precision == PHMM_PREC_FP64 && (ctx->cfg.flags & PHMM_F_LAUNCH_PER_PAIR);
         const bool use_graph = !(ctx->cfg.flags & PHMM_F_NO_GRAPH) && !per_pair;
+        // (a replayed graph records the events of its own branches, whichever graph was captured last;
+        // FP64 has no packed branch)
+        if (!per_pair) S->br_mask = fp32 ? 0x7u : f64_pipelined(P.scal_id) ? 0x5u : 0u;
         if (per_pair) {
             const BatchHeader* H = static_cast<const BatchHeader*>(S->hdr.p);
             launch_reset(H, ctx->sms * 4, s);
@@ -1971,10 +1969,10 @@ int phmm_poll(phmm_ctx* ctx, uint64_t ticket, int timeout_ms) {
     S->st.ms_rescue = ms;
     for (int q = 0; q < 3; ++q) {
         ms = 0.f;
-        if (S->br_timed && (S->br_mask >> q & 1u)) cudaEventElapsedTime(&ms, S->ev_br[2 * q], S->ev_br[2 * q + 1]);
+        if (S->br_mask >> q & 1u) cudaEventElapsedTime(&ms, S->ev_br[2 * q], S->ev_br[2 * q + 1]);
         S->st.ms_branch[q] = ms;
     }
-    if (!S->br_timed) S->st.ms_branch[0] = S->st.ms_forward;  // FP64: one forward kernel
+    if (!S->br_mask) S->st.ms_branch[0] = S->st.ms_forward;  // FP64: one forward kernel
     ctx->last_stats = S->st;
     ctx->last_retired = S->ticket;
     ctx->inflight_foot -= S->foot;

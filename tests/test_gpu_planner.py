@@ -215,3 +215,18 @@ def test_footprint_counts_the_planner(phmm):
         with phmm.Context(precision="fp32_only", mem_budget=budget) as ctx:
             out, flags, rc, st = ctx.run(b)
         assert rc == 0 and np.array_equal(out, ref)
+
+
+def test_branch_times_of_alternating_fp64_variants(phmm):
+    """One slot, batches that the cost model gives to the variants of one kernel and of two
+    branches by turns, replayed from graphs: each batch's branch times are its own."""
+    one = _batch(np.full(300, 50), np.full(300, 16), 14)
+    two = _batch(np.full(300, 200), np.full(300, 1020), 15)
+    with phmm.Context(precision="fp64", max_inflight=1, flags=phmm.F_NO_TUNE) as ctx:
+        for _ in range(3):
+            st = ctx.run(one)[3]
+            assert st["short_kernel"] in (0, 1) and st["ms_branch"] == [st["ms_forward"], 0.0, 0.0]
+            st = ctx.run(two)[3]
+            assert st["short_kernel"] in (2, 3)
+            # its short kernel is shorter than the forward pass, its other branch took a time of its own
+            assert 0.0 < st["ms_branch"][0] < st["ms_forward"] and st["ms_branch"][1] == 0.0 < st["ms_branch"][2]
