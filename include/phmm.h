@@ -269,10 +269,12 @@ int phmm_device_info(phmm_ctx *ctx, int *sms, double *max_clock_mhz, double *cup
 int phmm_scan_test(phmm_ctx *ctx, const float *y, float *z, int n, float a);
 
 /*
- * Test entry: the bounded device-side wait that links column strips (and, in shared
- * memory, warp segments) run on a boundary that is never written.  The wait gives up
- * after its poll limit (about a second) instead of hanging, and the call returns
- * PHMM_ETIMEOUT; the context stays usable.  Runs synchronously on the context's stream.
+ * Test entry: the bounded device-side waits that link column strips (and, in shared
+ * memory, warp segments) run on boundaries that are never written: the scan engines' words,
+ * and the tagged rows of the FP32 and FP64 wave kinds, whose one CTA also waits for CTAs
+ * that never come to take items before it.  Each wait gives up after its limit (a few seconds
+ * at most) instead of hanging, and the call returns PHMM_ETIMEOUT; the context stays usable.
+ * PHMM_OK: one of them did not give up as designed.  Runs synchronously on the context's stream.
  */
 int phmm_wait_test(phmm_ctx *ctx);
 

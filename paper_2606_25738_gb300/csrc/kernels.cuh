@@ -653,20 +653,32 @@ k_forward_cluster(const BatchHeader* __restrict__ H, const PowRow<float>* __rest
 // SM, then those that are second, and so on, so that the longest items, which the lists have
 // first, spread over all SMs, and items fewer than the warps leave no SM with two of them while
 // another has none.  (Left to chance, 64 strips of one pair took 6.3 ms or, three to a scheduler,
-// 11 to 14 ms.)  False: enough CTAs stand before this one.  The wait is a matter of speed only,
-// and short: 20 us at most, where another kernel holds SMs.  list: 0 multi-warp, 1 short.
+// 11 to 14 ms.)  A CTA waits until as many items are taken as the CTAs before it take at first,
+// kTurnNs at most: where other kernels hold SMs, those CTAs may not come, and the ones that did
+// start take every item.  list: 0 multi-warp, 1 short.
+constexpr unsigned long long kTurnNs = 20000;
+__device__ __forceinline__ unsigned long long global_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+// False: every item is taken.
 __device__ __forceinline__ bool sm_turn(const BatchHeader* __restrict__ H, int list, uint32_t n_items, uint32_t per_cta) {
-    __shared__ uint32_t before;
+    __shared__ uint32_t taken;
     if (threadIdx.x == 0) {
         uint32_t sm;
         asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
         const uint32_t rank = atomicAdd(H->sm_rank + list * kSmSlots + (sm & (kSmSlots - 1)), 1u);
-        before = rank * H->sms * per_cta;
-        if (n_items > before)
-            for (int q = 0; q < 200 && *(volatile uint32_t*)&H->counters[list] < before; ++q) __nanosleep(100);
+        const uint32_t before = min(rank * H->sms * per_cta, n_items);
+        const unsigned long long t0 = global_ns();
+        taken = *(volatile uint32_t*)&H->counters[list];
+        for (int q = 0; q < 1000 && taken < before && global_ns() - t0 < kTurnNs; ++q) {
+            __nanosleep(100);
+            taken = *(volatile uint32_t*)&H->counters[list];
+        }
     }
     __syncthreads();
-    return n_items > before;
+    return taken < n_items;
 }
 
 // Multi-warp pairs one warp at a time (long kind 3): each warp takes a whole pair and

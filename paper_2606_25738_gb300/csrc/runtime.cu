@@ -2200,7 +2200,74 @@ int phmm_wait_test(phmm_ctx* ctx) {
     CK(cudaMemcpyAsync(&st, status, sizeof(st), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     release(buf);
-    return (st & ST_TIMEOUT) ? PHMM_ETIMEOUT : PHMM_OK;
+    if (!(st & ST_TIMEOUT)) return PHMM_OK;
+    // The wave kinds' strips: the second strip of a pair whose first one no CTA runs, its boundary
+    // rows without a tag; and the one CTA started as if seven were before it on its SM.
+    constexpr uint32_t l = 40, k = 600;
+    constexpr size_t at_small = 4096, at_rec = 16384, at_hap = 20480, at_bnd = 24576, bytes = 32768;
+    static_assert(sizeof(BatchHeader) <= at_small &&
+                      at_small + kSmallBytes + 1024 <= at_rec && at_rec + l * sizeof(Rec64J) <= at_hap && at_bnd + l * 32 <= bytes, "layout");
+    std::vector<uint8_t> img(bytes);
+    CK(ensure(buf, bytes));
+    uint8_t* const d = static_cast<uint8_t*>(buf.p);
+    for (int fp64 = 0; fp64 < 2; ++fp64) {
+        std::fill(img.begin(), img.end(), (uint8_t)0);
+        uint32_t* const w = reinterpret_cast<uint32_t*>(img.data() + at_small);
+        uint32_t* const dw = reinterpret_cast<uint32_t*>(d + at_small);
+        w[24] = 1u;  // the launch's tag
+        for (uint32_t q = 0; q < 2 * kSmSlots; ++q) w[32 + q] = 7u;
+        const size_t at_desc = (at_small + kSmallBytes + 255) / 256 * 256;
+        PairDesc pd{};
+        pd.l = l;
+        pd.k = k;
+        CtaPair cp{};
+        cp.W = 1;
+        cp.strip = 1;
+        cp.nstrip = 2;
+        cp.col0 = 512;
+        cp.extra_base = 1;
+        cp.bnd_out = kNoBnd;
+        const CtaItem ci{0u, 1u};
+        memcpy(img.data() + at_desc, &pd, sizeof(pd));
+        memcpy(img.data() + at_desc + 64, &cp, sizeof(cp));
+        memcpy(img.data() + at_desc + 128, &ci, sizeof(ci));
+        memset(img.data() + at_hap, 'A', k);
+        BatchHeader hh;
+        memset(&hh, 0, sizeof(hh));
+        hh.n_pairs = 1;
+        hh.hap_bases = d + at_hap;
+        hh.desc = (PairDesc*)(d + at_desc);
+        hh.cpairs = (const CtaPair*)(d + at_desc + 64);
+        hh.citems = (const CtaItem*)(d + at_desc + 128);
+        hh.n_citems = 1;
+        hh.parts = (Partial*)(d + at_desc + 256);  // two
+        hh.rec32j = (Rec32J*)(d + at_rec);
+        hh.rec64j = (Rec64J*)(d + at_rec);
+        hh.wbnd = (float4*)(d + at_bnd);
+        hh.counters = dw;
+        hh.status = dw + 8;
+        hh.dropgrow = dw + 9;
+        hh.skst = (SkewStats*)(dw + 16);
+        hh.wave_epoch = dw + 24;
+        hh.sm_rank = dw + 32;
+        hh.sms = (uint32_t)ctx->sms;
+        memcpy(img.data(), &hh, sizeof(hh));
+        CK(cudaMemcpyAsync(d, img.data(), bytes, cudaMemcpyHostToDevice, ctx->stream));
+        const BatchHeader* H = reinterpret_cast<const BatchHeader*>(d);
+        if (fp64) launch_forward_wave64(H, 1, ctx->stream);
+        else launch_forward32_long_pipe(8, H, nullptr, 1, ctx->stream);
+        CK(cudaGetLastError());
+        CK(cudaMemcpyAsync(img.data(), d, bytes, cudaMemcpyDeviceToHost, ctx->stream));
+        CK(cudaStreamSynchronize(ctx->stream));
+        Partial p;
+        memcpy(&p, img.data() + at_desc + 256 + sizeof(Partial), sizeof(p));
+        if (!(w[8] & ST_TIMEOUT) || !(p.flags & PF_DONE) || !(p.flags & PF_TIMEOUT)) {
+            release(buf);
+            return PHMM_OK;
+        }
+    }
+    release(buf);
+    return PHMM_ETIMEOUT;
 }
 
 int phmm_scan_test(phmm_ctx* ctx, const float* y, float* z, int n, float a) {

@@ -429,7 +429,8 @@ def test_rounding_bound_triggers_fp64_rescue(phmm):
 
 
 def test_bounded_wait_times_out_and_context_survives(phmm):
-    """A device-side wait that can never be satisfied gives up within its poll limit and
+    """Device-side waits that can never be satisfied (scan engine, FP32 and FP64 wave strips, a CTA
+    whose turn never comes) give up within their limits and the call
     reports PHMM_ETIMEOUT; the same context then still scores a batch correctly."""
     import time
     b = W.plain_pairs(8, seed=40)
