@@ -518,6 +518,7 @@ struct Slot {
     uint64_t foot = 0;  // admitted device footprint while pending
     std::map<int, cudaGraphExec_t> graphs;  // by kernel choice (its arguments are the slot's own)
     uint64_t ticket = 0;
+    std::chrono::steady_clock::time_point submitted;
     int state = 0;  // 0 free, 1 pending
     double* user_out = nullptr;
     uint8_t* user_flags = nullptr;
@@ -1703,6 +1704,7 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     if (getenv("PHMM_DEBUG"))
         fprintf(stderr, "phmm submit: plan %s %.1f ms, host total %.1f ms\n", reuse ? "reused" : "built",
                 std::chrono::duration<double, std::milli>(th_plan - th0).count(), S->st.ms_host);
+    S->submitted = std::chrono::steady_clock::now();
     *ticket = S->ticket;
     return PHMM_OK;
 }
@@ -1946,8 +1948,9 @@ int phmm_poll(phmm_ctx* ctx, uint64_t ticket, int timeout_ms) {
             const double el = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
             if (el >= timeout_ms) return PHMM_PENDING;
         }
-        // a small batch is done within this time, where a sleep would cost as much as its kernels
-        if (std::chrono::steady_clock::now() - t0 < std::chrono::microseconds(400)) std::this_thread::yield();
+        // a small batch is done within this time of its submission, where a sleep (some 100 us) would cost as
+        // much as its kernels; a long one, polled in however short slices, is slept on
+        if (std::chrono::steady_clock::now() - S->submitted < std::chrono::milliseconds(1)) std::this_thread::yield();
         else std::this_thread::sleep_for(std::chrono::microseconds(50));
     }
     std::lock_guard<std::mutex> lock(ctx->mu);

@@ -230,3 +230,23 @@ def test_branch_times_of_alternating_fp64_variants(phmm):
             assert st["short_kernel"] in (2, 3)
             # its short kernel is shorter than the forward pass, its other branch took a time of its own
             assert 0.0 < st["ms_branch"][0] < st["ms_forward"] and st["ms_branch"][1] == 0.0 < st["ms_branch"][2]
+
+
+def _long_batch(n=20000, l=6000):
+    """n pairs of 8 reads and 8 haplotypes of l bases: about 0.2 s of the serial kernel."""
+    b = _batch(np.full(8, l), np.full(8, l), 20)
+    i = np.arange(n)
+    return dict(b, pair_read=(i % 8).astype(np.uint32), pair_hap=(i // 8 % 8).astype(np.uint32))
+
+
+def test_polling_in_slices_leaves_the_core(phmm):
+    """A long batch polled a millisecond at a time: the thread sleeps, but for the first millisecond."""
+    import time
+    with phmm.Context(precision="fp32", flags=phmm.F_NO_TUNE) as ctx:
+        ctx.run(_long_batch())
+        t = ctx.submit(_long_batch())
+        w0, c0 = time.perf_counter(), time.thread_time()
+        while (rc := ctx.poll(t, 1)) == phmm.PHMM_PENDING:
+            pass
+        wall, cpu = time.perf_counter() - w0, time.thread_time() - c0
+    assert rc == 0 and wall > 0.1 and cpu < 0.2 * wall, (wall, cpu)
