@@ -74,42 +74,17 @@ __global__ void __launch_bounds__(256) k_plan_scan(PlanInput in, PlanScan* __res
         const uint64_t a = in.hap_off[h], b = in.hap_off[h + 1];
         bad |= b <= a || b - a > 0xffffffull;
     }
-    unsigned long long cells = 0, sl = 0, sk = 0, shc[2] = {0, 0}, rows[2][2] = {{0, 0}, {0, 0}}, str[2][2] = {{0, 0}, {0, 0}};
-    unsigned long long crows = 0, cstr = 0;
-    uint32_t nl[2] = {0, 0}, lmax = 0, lml[2] = {0, 0}, shared = 0;
+    PlanScan q{};
     for (uint32_t p = t0; p < in.n_pairs; p += st) {
         const uint32_t r = in.pair_read[p], h = in.pair_hap[p];
         if (r >= in.n_reads || h >= in.n_haps) {
             bad = true;
             continue;
         }
-        const uint64_t l64 = in.read_off[r + 1] - in.read_off[r], k64 = in.hap_off[h + 1] - in.hap_off[h];
-        if (l64 > 0xffffffull || k64 > 0xffffffull) continue;  // found bad above
-        const uint32_t l = (uint32_t)l64, k = (uint32_t)k64;
-        const unsigned long long c = (unsigned long long)l * k;
-        cells += c;
-        sl += l;
-        sk += k;
-        lmax = max(lmax, l);
-        const uint32_t C = (k + 4095u) / 4096u;  // strips of 4-warp CTAs of 1024 columns a warp
-        crows += (unsigned long long)(C - 1) * l;
-        cstr += C - 1;
-        shared += (p > 0 && in.pair_read[p - 1] == r) || (p + 1 < in.n_pairs && in.pair_read[p + 1] == r);
-#pragma unroll
-        for (int w = 0; w < 2; ++w) {
-            if (k <= (w ? 768u : 1024u)) {
-                shc[w] += c;
-                continue;
-            }
-            nl[w]++;
-            lml[w] = max(lml[w], l);
-#pragma unroll
-            for (int z = 0; z < 2; ++z) {
-                const uint32_t W = z ? (k + 511u) / 512u : (k + 1023u) / 1024u;
-                rows[w][z] += (unsigned long long)(W - 1) * l;
-                str[w][z] += W;
-            }
-        }
+        const uint64_t l = in.read_off[r + 1] - in.read_off[r], k = in.hap_off[h + 1] - in.hap_off[h];
+        if (l > 0xffffffull || k > 0xffffffull) continue;  // found bad above
+        plan_scan_pair(q, (uint32_t)l, (uint32_t)k,
+                       (p > 0 && in.pair_read[p - 1] == r) || (p + 1 < in.n_pairs && in.pair_read[p + 1] == r));
     }
     const bool lead = (threadIdx.x & 31) == 0;
     auto add = [&](unsigned long long v, unsigned long long* to) {
@@ -124,24 +99,24 @@ __global__ void __launch_bounds__(256) k_plan_scan(PlanInput in, PlanScan* __res
         v = __reduce_max_sync(kFull, v);
         if (lead && v) atomicMax(to, v);
     };
-    add(cells, &out->cells);
-    add(sl, &out->sum_l);
-    add(sk, &out->sum_k);
-    add(crows, &out->cta_rows);
-    add(cstr, &out->cta_strips);
+    add(q.cells, &out->cells);
+    add(q.sum_l, &out->sum_l);
+    add(q.sum_k, &out->sum_k);
+    add(q.cta_rows, &out->cta_rows);
+    add(q.cta_strips, &out->cta_strips);
 #pragma unroll
     for (int w = 0; w < 2; ++w) {
-        add(shc[w], &out->short_cells[w]);
-        add32(nl[w], &out->n_long[w]);
-        top(lml[w], &out->lmax_long[w]);
+        add(q.short_cells[w], &out->short_cells[w]);
+        add32(q.n_long[w], &out->n_long[w]);
+        top(q.lmax_long[w], &out->lmax_long[w]);
 #pragma unroll
         for (int z = 0; z < 2; ++z) {
-            add(rows[w][z], &out->rows[w][z]);
-            add(str[w][z], &out->strips[w][z]);
+            add(q.rows[w][z], &out->rows[w][z]);
+            add(q.strips[w][z], &out->strips[w][z]);
         }
     }
-    top(lmax, &out->lmax);
-    add32(shared, &out->shared);
+    top(q.lmax, &out->lmax);
+    add32(q.shared, &out->shared);
     if (__any_sync(kFull, bad) && lead) atomicOr(&out->bad, 1u);
 }
 
@@ -388,6 +363,27 @@ void launch_plan_scan(const PlanInput& in, PlanScan* out, int sms, cudaStream_t 
     cudaMemsetAsync(out, 0, sizeof(PlanScan), s);
     const uint32_t n = in.n_pairs > in.n_reads ? in.n_pairs : in.n_reads;
     k_plan_scan<<<blocks_for(n, 256, sms * 4), 256, 0, s>>>(in, out);
+}
+
+PlanScan plan_scan_host(const PlanInput& in) {
+    PlanScan bad{}, s{};
+    bad.bad = 1;
+    if (in.read_off[0] != 0 || in.hap_off[0] != 0) return bad;
+    for (uint32_t r = 0; r < in.n_reads; ++r)
+        if (in.read_off[r + 1] <= in.read_off[r] || in.read_off[r + 1] - in.read_off[r] > 0xffffffull) return bad;
+    for (uint32_t h = 0; h < in.n_haps; ++h)
+        if (in.hap_off[h + 1] <= in.hap_off[h] || in.hap_off[h + 1] - in.hap_off[h] > 0xffffffull) return bad;
+    s.n_read_bases = in.read_off[in.n_reads];
+    s.n_hap_bases = in.hap_off[in.n_haps];
+    uint32_t last = 0xffffffffu;
+    for (uint32_t p = 0; p < in.n_pairs; ++p) {
+        const uint32_t r = in.pair_read[p], h = in.pair_hap[p];
+        if (r >= in.n_reads || h >= in.n_haps) return bad;
+        plan_scan_pair(s, (uint32_t)(in.read_off[r + 1] - in.read_off[r]), (uint32_t)(in.hap_off[h + 1] - in.hap_off[h]),
+                       r == last || (p + 1 < in.n_pairs && in.pair_read[p + 1] == r));
+        last = r;
+    }
+    return s;
 }
 
 void launch_plan_build(const PlanInput& in, const PlanOutput& out, int sms, cudaStream_t s) {

@@ -27,6 +27,40 @@ struct PlanScan {
     uint32_t pad;
 };
 
+// A pair's part of the sums.  shared: its neighbour in the list has the same read.
+__host__ __device__ inline void plan_scan_pair(PlanScan& s, uint32_t l, uint32_t k, bool shared) {
+    const unsigned long long c = (unsigned long long)l * k;
+    s.cells += c;
+    s.sum_l += l;
+    s.sum_k += k;
+    s.lmax = l > s.lmax ? l : s.lmax;
+    s.shared += shared;
+    if (k > 4096u) {  // strips of 4-warp CTAs of 1024 columns a warp
+        const uint32_t C = (k + 4095u) / 4096u;
+        s.cta_rows += (unsigned long long)(C - 1) * l;
+        s.cta_strips += C - 1;
+    }
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int w = 0; w < 2; ++w) {
+        if (k <= (w ? 768u : 1024u)) {
+            s.short_cells[w] += c;
+            continue;
+        }
+        s.n_long[w]++;
+        s.lmax_long[w] = l > s.lmax_long[w] ? l : s.lmax_long[w];
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+        for (int z = 0; z < 2; ++z) {
+            const uint32_t W = z ? (k + 511u) / 512u : (k + 1023u) / 1024u;
+            s.rows[w][z] += (unsigned long long)(W - 1) * l;
+            s.strips[w][z] += W;
+        }
+    }
+}
+
 struct PlanInput {
     const uint64_t *read_off, *hap_off;
     const uint32_t *pair_read, *pair_hap;
@@ -46,6 +80,8 @@ struct PlanOutput {
 
 size_t plan_scratch_bytes(uint32_t n_pairs);
 void launch_plan_scan(const PlanInput& in, PlanScan* out, int sms, cudaStream_t s);
+// The same on the host, for arrays there.
+PlanScan plan_scan_host(const PlanInput& in);
 // The batch is known to be valid (PlanScan.bad == 0).
 void launch_plan_build(const PlanInput& in, const PlanOutput& out, int sms, cudaStream_t s);
 

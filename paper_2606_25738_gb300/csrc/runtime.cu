@@ -620,7 +620,7 @@ cudaError_t ensure_serial(const phmm_ctx* ctx, Slot& S, const Plan& P) {
         const size_t cap = S.wbnd.cap;
         const cudaError_t e = ensure(S.wbnd, std::max<uint64_t>(P.wave_rows, 1) * sizeof(float4));
         if (e != cudaSuccess || (S.wbnd.p == before && S.wbnd.cap == cap)) return e;
-        return cudaMemsetAsync(S.wbnd.p, 0, S.wbnd.cap, ctx->copy_stream);
+        return cudaMemsetAsync(S.wbnd.p, 0, S.wbnd.cap, S.sm);
     }
     const uint64_t b = serial_bytes(ctx, P);
     if (b == 0) {
@@ -1075,6 +1075,7 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     const uint64_t *roff = b->read_off, *hoff = b->hap_off;
     const uint32_t *pr = b->pair_read, *ph = b->pair_hap;
     cudaStream_t cs = ctx->copy_stream;
+    auto th0 = std::chrono::steady_clock::now();  // planning starts (with the lengths on the host)
     const bool on_dev = !host_plan && plans_on_device(ctx->cfg, np);
     PlanInput pin{};
     PlanScan sc{};
@@ -1095,7 +1096,24 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
         CK(cudaStreamWaitEvent(cs, S->ev_user, 0));
     }
     if (on_dev) {
-        // device planner: the lengths are checked and summed there
+        // device planner: the lengths are checked and summed on the device, unless a batch in flight may
+        // fill the SMs until it drains: then on the host, so that submit waits for copies only (device inputs
+        // wait for the caller's stream anyway).  455,000 pairs of host arrays: 12.1 ms a call with the
+        // sums on an idle device, 12.8 with them on the host.
+        bool scan_dev = true;
+        for (auto& o : ctx->slots) scan_dev &= o.state == 0;
+        scan_dev |= dev_in;
+        pin.read_off = roff;
+        pin.hap_off = hoff;
+        pin.pair_read = pr;
+        pin.pair_hap = ph;
+        pin.n_reads = nr;
+        pin.n_haps = nh;
+        pin.n_pairs = np;
+        if (!scan_dev) {
+            sc = plan_scan_host(pin);
+            if (sc.bad) return PHMM_EINVAL;
+        }
         if (!dev_in && index_bytes <= kPackBytes / 2) {
             index_packed = true;
             pin.read_off = (const uint64_t*)pack(roff, (nr + 1) * 8ull);
@@ -1113,24 +1131,22 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
             CK(cudaMemcpyAsync(S->in_hoff.p, hoff, (nh + 1) * 8ull, cudaMemcpyHostToDevice, cs));
             CK(cudaMemcpyAsync(S->in_pr.p, pr, np * 4ull, cudaMemcpyHostToDevice, cs));
             CK(cudaMemcpyAsync(S->in_ph.p, ph, np * 4ull, cudaMemcpyHostToDevice, cs));
+            pin.read_off = static_cast<const uint64_t*>(S->in_roff.p);
+            pin.hap_off = static_cast<const uint64_t*>(S->in_hoff.p);
+            pin.pair_read = static_cast<const uint32_t*>(S->in_pr.p);
+            pin.pair_hap = static_cast<const uint32_t*>(S->in_ph.p);
         }
-        if (!index_packed) {
-            pin.read_off = dev_in ? roff : static_cast<const uint64_t*>(S->in_roff.p);
-            pin.hap_off = dev_in ? hoff : static_cast<const uint64_t*>(S->in_hoff.p);
-            pin.pair_read = dev_in ? pr : static_cast<const uint32_t*>(S->in_pr.p);
-            pin.pair_hap = dev_in ? ph : static_cast<const uint32_t*>(S->in_ph.p);
+        if (scan_dev) {
+            CK(ensure(S->pscan, sizeof(PlanScan)));
+            CK(ensure(S->h_pscan, sizeof(PlanScan)));
+            launch_plan_scan(pin, static_cast<PlanScan*>(S->pscan.p), ctx->sms, cs);
+            CK(cudaGetLastError());
+            CK(cudaMemcpyAsync(S->h_pscan.p, S->pscan.p, sizeof(PlanScan), cudaMemcpyDeviceToHost, cs));
+            CK(cudaStreamSynchronize(cs));
+            sc = *static_cast<const PlanScan*>(S->h_pscan.p);
+            if (dev_in) th0 = std::chrono::steady_clock::now();
+            if (sc.bad) return PHMM_EINVAL;
         }
-        pin.n_reads = nr;
-        pin.n_haps = nh;
-        pin.n_pairs = np;
-        CK(ensure(S->pscan, sizeof(PlanScan)));
-        CK(ensure(S->h_pscan, sizeof(PlanScan)));
-        launch_plan_scan(pin, static_cast<PlanScan*>(S->pscan.p), ctx->sms, cs);
-        CK(cudaGetLastError());
-        CK(cudaMemcpyAsync(S->h_pscan.p, S->pscan.p, sizeof(PlanScan), cudaMemcpyDeviceToHost, cs));
-        CK(cudaStreamSynchronize(cs));
-        sc = *static_cast<const PlanScan*>(S->h_pscan.p);
-        if (sc.bad) return PHMM_EINVAL;
     } else if (dev_in && np > 0) {
         CK(ensure(S->h_roff, (nr + 1) * 8ull));
         CK(ensure(S->h_hoff, (nh + 1) * 8ull));
@@ -1145,6 +1161,7 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
         hoff = static_cast<const uint64_t*>(S->h_hoff.p);
         pr = static_cast<const uint32_t*>(S->h_pr.p);
         ph = static_cast<const uint32_t*>(S->h_ph.p);
+        th0 = std::chrono::steady_clock::now();
     }
     // validation: offsets non-decreasing with lengths >= 1, indices in range
     std::vector<uint32_t> L(on_dev ? 0 : np), K(on_dev ? 0 : np);
@@ -1167,7 +1184,6 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     // plan (FP32: packed short width from the config or the cost model; FP64: kN64).
     // A batch with the same pair lengths as this slot's previous one reuses its plan (and the same
     // reads, where packed teams, whose two pairs share one, may be in it).
-    const auto th0 = std::chrono::steady_clock::now();
     uint64_t hsh = 1469598103934665603ull ^ ((uint64_t)ctx->cfg.precision << 32) ^ (uint64_t)ctx->cfg.cols_per_lane ^ ((uint64_t)ctx->cfg.kernel_variant << 40);
     bool may_pack = false;
     if (ctx->cfg.precision != PHMM_PREC_FP64)
@@ -1443,7 +1459,6 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     hh.mode = (uint32_t)ctx->cfg.precision;
     memcpy(hpk, &hh, sizeof(hh));
     CK(cudaMemcpyAsync(S->hdr.p, hpk, all_packed ? pk : sizeof(hh), cudaMemcpyHostToDevice, cs));
-    if (P.dev) CK(build_plan(*S, P, pin, ctx->sms, cs));
     CK(cudaEventRecord(S->ev_copy, cs));
     // host inputs may be released when submit returns (packed ones already are)
     if (!all_packed) CK(cudaEventSynchronize(S->ev_copy));
@@ -1451,6 +1466,8 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
     CK(cudaEventRecord(S->ev_user, ctx->stream));
     CK(cudaStreamWaitEvent(S->sm, S->ev_user, 0));
     CK(cudaStreamWaitEvent(S->sm, S->ev_copy, 0));
+    // (kernels run on the slot's stream: in the copies' one the next submit would wait for them)
+    if (P.dev && !tune_short && !tune_long) CK(build_plan(*S, P, pin, ctx->sms, S->sm));
     // What a trial may hold: the bound and budget of the admitted plan, beside the batches in flight.
     // Arenas of other trials that this one does not read make room for its own.
     const uint64_t room = std::min<uint64_t>(most, ctx->budget - ctx->inflight_foot);
@@ -1561,8 +1578,8 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
             hh.parts = (Partial*)S->parts.p;
             plan_header(*S, c, hh);
             CK(cudaMemcpyAsync(S->hdr.p, &hh, sizeof(hh), cudaMemcpyHostToDevice, cs));
-            if (c.dev) CK(build_plan(*S, c, pin, ctx->sms, cs));
             CK(cudaStreamSynchronize(cs));
+            if (c.dev) CK(build_plan(*S, c, pin, ctx->sms, S->sm));
             // time the candidate; a short run is repeated and the faster kept (the first
             // launch of a kernel after a plan change runs cold).  The serial multi-warp kind
             // is always run twice: its first run after a plan change measured about 30%
@@ -1604,8 +1621,8 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
         hh.parts = (Partial*)S->parts.p;
         plan_header(*S, P, hh);
         CK(cudaMemcpyAsync(S->hdr.p, &hh, sizeof(hh), cudaMemcpyHostToDevice, cs));
-        if (P.dev) CK(build_plan(*S, P, pin, ctx->sms, cs));
         CK(cudaStreamSynchronize(cs));
+        if (P.dev) CK(build_plan(*S, P, pin, ctx->sms, S->sm));
         N = P.N;
     }
     cudaStream_t s = S->sm;

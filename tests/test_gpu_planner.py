@@ -250,3 +250,32 @@ def test_polling_in_slices_leaves_the_core(phmm):
             pass
         wall, cpu = time.perf_counter() - w0, time.thread_time() - c0
     assert rc == 0 and wall > 0.1 and cpu < 0.2 * wall, (wall, cpu)
+
+
+def test_submit_does_not_wait_for_a_batch_in_flight(phmm):
+    """A batch of many pairs from host arrays is planned and uploaded while another one fills the
+    GPU: submit waits for copies only."""
+    import time
+    big = _long_batch()
+    rng = np.random.default_rng(21)
+    small = [_batch(np.full(5000, 100), rng.integers(50, 1500, 5000), s) for s in (22, 23)]
+    with phmm.Context(precision="fp32", max_inflight=2, flags=phmm.F_NO_TUNE) as ctx:
+        alone = [ctx.run(b)[0] for b in small]
+        for _ in range(2):  # the first round allocates
+            t0 = time.perf_counter()
+            a = ctx.submit(big)
+            t1 = time.perf_counter()
+            out = np.empty(5000)
+            c = ctx.submit(small[0], out)
+            t2 = time.perf_counter()
+            assert ctx.poll(a) == 0
+            t3 = time.perf_counter()
+            assert ctx.poll(c) == 0
+            assert np.array_equal(out, alone[0])
+        assert t3 - t0 > 0.1 and t2 - t1 < 0.25 * (t3 - t0), (t1 - t0, t2 - t1, t3 - t0)
+        # plans of two slots, the second made while the first one's batch runs
+        outs = [np.empty(5000) for _ in small]
+        for _ in range(3):
+            tk = [ctx.submit(b, o) for b, o in zip(small, outs)]
+            assert [ctx.poll(t) for t in tk] == [0, 0]
+            assert all(np.array_equal(o, x) for o, x in zip(outs, alone))
