@@ -282,7 +282,8 @@ int phmm_wait_test(phmm_ctx *ctx);
  * Test entry (host only, no device needed): builds the work plan the runtime would use
  * for a batch with read lengths l[p], haplotype lengths k[p] and read index pair_read[p]
  * (n pairs), for precision (PHMM_PREC_*) and, in FP32, the short-pair kernel ids (scalar
- * 0..9, packed -1..1) and the multi-warp kernel kind (0..8, as phmm_stats.long_kernel),
+ * 0..9, packed -1..1) and the multi-warp kernel kind (0..8, as phmm_stats.long_kernel; in
+ * FP64 scal_id is the variant, and kind 6 makes waves of variants 2 and 3's wide pairs),
  * and checks it: every pair scheduled exactly once; teams inside their warp, disjoint and
  * wide enough, packed pairs sharing a read; CTA warp ranges inside the CTA and disjoint; a
  * wide pair's strips tiling its columns in order, never placed in an earlier work item

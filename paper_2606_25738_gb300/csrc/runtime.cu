@@ -858,8 +858,7 @@ std::vector<std::pair<int, int>> fp32_candidates(const phmm_config& cfg) {
 // of 1 to 10 kbp: 10.9 ms); CTA items do 8 operations a cell at 1.1 cells x operations a cycle
 // and SM, and 7700 cycles a row for each four warps of 512 columns (84 ms).  Many short reads
 // against 513 to 1024 columns are the other end (5,000 pairs of 150 rows: 28 ms and 10.8).
-bool waves64_pay(const uint32_t* l, const uint32_t* k, uint32_t n, uint32_t wide) {
-    const double sms = 152.0;
+bool waves64_pay(const uint32_t* l, const uint32_t* k, uint32_t n, uint32_t wide, double sms) {
     double wave = 0, wchain = 0, cta = 0, cchain = 0;
     for (uint32_t p = 0; p < n; ++p) {
         if (k[p] <= wide) continue;
@@ -872,10 +871,13 @@ bool waves64_pay(const uint32_t* l, const uint32_t* k, uint32_t n, uint32_t wide
     return std::max(wave, wchain) < std::max(cta, cchain);
 }
 
-// wave: multi-warp pairs of the skewed variants as waves (long_kind 6) rather than CTA items
+// waves: multi-warp pairs of the skewed variants as waves (long_kind 6) rather than CTA items, never, where
+// they pay on a GPU of that many SMs, or always
+enum class Waves64 { kNone, kPaying, kAll };
 void make_plan64(const uint32_t* l, const uint32_t* k, const uint32_t* pr, uint32_t n, int id, Plan& P,
-                 bool wave = false) {
-    wave = wave && f64_pipelined(id) && waves64_pay(l, k, n, 32u * (uint32_t)kF64NS[id]);
+                 Waves64 waves = Waves64::kNone, int sms = 0) {
+    const bool wave = f64_pipelined(id) && waves != Waves64::kNone &&
+                      (waves == Waves64::kAll || waves64_pay(l, k, n, 32u * (uint32_t)kF64NS[id], (double)sms));
     make_plan(l, k, pr, n, kF64NS[id], 0, wave ? 4 * kF64WaveN : kF64N[id], P, 8, wave ? 1 : kF64CW[id], false, wave,
               f64_pipelined(id) ? kSkewCost : TeamCost());
     P.scal_id = id;
@@ -1212,7 +1214,8 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
             // smaller plan cost), measured below for large batches
             const uint64_t sig = batch_signature(L.data(), K.data(), pr, np, ctx->cfg);
             auto hit = ctx->tuned.find(sig);
-            const bool waves = !(ctx->cfg.flags & PHMM_F_LAUNCH_PER_PAIR);
+            const bool per_pair = (ctx->cfg.flags & PHMM_F_LAUNCH_PER_PAIR) != 0;
+            const Waves64 waves = per_pair ? Waves64::kNone : Waves64::kPaying;
             // forced: cols_per_lane 8 / 16 = the unfactored variants, kernel_variant 4 (the
             // pipelined engine, 16-column teams) = variant 2, 5 or 6 (32-column fused
             // teams) = variant 3
@@ -1220,15 +1223,15 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
                              : ctx->cfg.cols_per_lane == kF64N[0] ? 0
                              : ctx->cfg.cols_per_lane == kF64N[1] ? 1 : -1;
             if (forced >= 0) {
-                make_plan64(L.data(), K.data(), pr, np, forced, P, waves);
+                make_plan64(L.data(), K.data(), pr, np, forced, P, waves, ctx->sms);
             } else if (hit != ctx->tuned.end()) {
-                make_plan64(L.data(), K.data(), pr, np, hit->second[0], P, waves);
+                make_plan64(L.data(), K.data(), pr, np, hit->second[0], P, waves, ctx->sms);
             } else {
-                tune64 = !(ctx->cfg.flags & PHMM_F_NO_TUNE) && waves && cells >= kTuneMinCells;
-                make_plan64(L.data(), K.data(), pr, np, tune64 ? 3 : 0, P, waves);
+                tune64 = !(ctx->cfg.flags & PHMM_F_NO_TUNE) && !per_pair && cells >= kTuneMinCells;
+                make_plan64(L.data(), K.data(), pr, np, tune64 ? 3 : 0, P, waves, ctx->sms);
                 for (int id = 1; id < kNumF64 && !tune64; ++id) {
                     Plan c;
-                    make_plan64(L.data(), K.data(), pr, np, id, c, waves);
+                    make_plan64(L.data(), K.data(), pr, np, id, c, waves, ctx->sms);
                     if (c.cost < P.cost) P = std::move(c);
                 }
                 tune_sig = sig;
@@ -1485,7 +1488,7 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
         int best = P.scal_id;
         // (variant 2 has waves for more pairs than the admitted plan of variant 3)
         auto plan64_of = [&](int id, Plan& Q) {
-            make_plan64(L.data(), K.data(), pr, np, id, Q, true);
+            make_plan64(L.data(), K.data(), pr, np, id, Q, Waves64::kPaying, ctx->sms);
             if (Q.long_kind == 6 && foot_of(Q) > most) make_plan64(L.data(), K.data(), pr, np, id, Q);
         };
         for (int id = 0; id < kNumF64; ++id) {
@@ -2028,9 +2031,9 @@ int phmm_plan_check(const uint32_t* l, const uint32_t* k, const uint32_t* pair_r
     int CW = kCtaWarps, Nl = kN64, kw = 8;
     if (precision == PHMM_PREC_FP64) {
         if (scal_id < 0 || scal_id >= kNumF64) return PHMM_EINVAL;  // the FP64 variant
-        make_plan64(l, k, pair_read, n, scal_id, P);
-        CW = kF64CW[scal_id];
-        Nl = kF64N[scal_id];
+        make_plan64(l, k, pair_read, n, scal_id, P, long_kind == 6 ? Waves64::kAll : Waves64::kNone);
+        CW = P.long_kind == 6 ? 1 : kF64CW[scal_id];
+        Nl = P.long_kind == 6 ? 4 * kF64WaveN : kF64N[scal_id];
     } else {
         if (scal_id < 0 || scal_id >= kNumScalar || pack_id < -1 || pack_id >= kNumPacked || long_kind < 0 ||
             long_kind >= kNumLong)
@@ -2082,8 +2085,10 @@ int phmm_plan_check(const uint32_t* l, const uint32_t* k, const uint32_t* pair_r
     std::map<uint32_t, StripSeen> strips;
     std::vector<std::pair<uint64_t, uint64_t>> bnd_ranges, extra_ranges;
     const bool serial = precision != PHMM_PREC_FP64 && kLongSerial[long_kind];
-    // wave kind: one strip per item on one warp; boundaries are float4 rows of wbnd
-    const bool wave = precision != PHMM_PREC_FP64 && kLongWave[long_kind];
+    // wave kind: one strip per item on one warp (FP64: on one CTA, W = 1); boundaries are rows of wbnd, a float4
+    // each (FP64: two)
+    const bool wave = kLongWave[P.long_kind];
+    const uint64_t row_f4 = precision == PHMM_PREC_FP64 ? 2 : 1;
     for (size_t it = 0; it < P.citems.size(); ++it) {
         const CtaItem& ci = P.citems[it];
         uint32_t used = 0;
@@ -2168,7 +2173,7 @@ int phmm_plan_check(const uint32_t* l, const uint32_t* k, const uint32_t* pair_r
             }
             if (wave) {
                 if (st + 1 < sv.nstrip) {
-                    const uint64_t a = sv.bout[st], b = a + (uint64_t)l[p];
+                    const uint64_t a = sv.bout[st], b = a + (uint64_t)l[p] * row_f4;
                     if (b > P.wave_rows) return fail(25);
                     bnd_ranges.push_back({a, b});
                 }

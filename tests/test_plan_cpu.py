@@ -62,6 +62,17 @@ def test_fp64_plans_valid(P, shape, variant):
     assert P.plan_check(l, k, pr, "fp64", 4)[0] == P.PHMM_EINVAL
 
 
+@pytest.mark.parametrize("shape", sorted(SHAPES))
+@pytest.mark.parametrize("variant", [2, 3])
+def test_fp64_wave_plans_valid(P, shape, variant):
+    """Waves of variants 2 and 3: a strip of 512 columns per item, boundary rows of two float4."""
+    l, k, pr = SHAPES[shape]
+    rc, st = P.plan_check(l, k, pr, "fp64", variant, long_kind=6)
+    assert rc == P.PHMM_OK, st
+    wide = np.asarray(k)[np.asarray(k) > {2: 512, 3: 1024}[variant]]
+    assert st["cta_items"] == int(np.sum((wide + 511) // 512)) == st["cta_pairs"]
+
+
 def test_wide_pairs_are_striped_and_packed(P):
     l, k, pr = SHAPES["very_wide"]
     rc, st = P.plan_check(l, k, pr, "fp32", 4, -1, 1)
