@@ -127,3 +127,20 @@ def test_items_around_the_warps(phmm, shape, n):
     """Items one fewer and one more than the warps that are first on their SM, second, all."""
     st = _check(phmm, _pairs([shape] * n, "ten", "flat", 2), flags=phmm.F_LONG_SERIAL, variant="pipe2", cols_per_lane=32)
     assert st["n_long"] == (n if shape[1] > 1024 else 0)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_tags_start_over(phmm, precision):
+    """Boundary rows carry one of 63 tags, stepped at every launch.  140 launches on one slot, two
+    batches by turns, so that a row's tag comes back under the other batch's layout, whose row it
+    must not pass for."""
+    bs = [_pairs(shapes, "mixed", "jumps", s) for s, shapes in
+          ((7, [(90, 5000), (33, 1100), (150, 2600)]), (8, [(40, 1300), (200, 4200), (17, 1025), (77, 3000)]))]
+    kw = dict(flags=phmm.F_LONG_WAVE16) if precision == "fp32" else dict(variant="pipe2")
+    with phmm.Context(precision=precision, max_inflight=1, **kw) as ctx:
+        first = [ctx.run(b)[0] for b in bs]
+        for i in range(138):
+            out, flags, rc, st = ctx.run(bs[i % 2])
+            assert rc == 0 and np.array_equal(out, first[i % 2]), i
+    for b, out in zip(bs, first):
+        assert np.max(np.abs(out - oracle.batch(b))) <= {"fp32": 1e-3, "fp64": 1e-9}[precision]
