@@ -1287,7 +1287,7 @@ __device__ SegOut seg_link_pipe(const Rec32J* __restrict__ rec, int l, const uin
 // ------------------------------------------------------------------------------------
 // Packed FP32 team for two haplotypes of the SAME read (pair A in x, pair B in y halves).
 // Both halves share the row records and the scan powers, so the per-row work is that of
-// one pair while every cell operation (FFMA2 / FMUL2) serves two cells.  Match masks of
+// one pair while every cell operation (`__ffma2_rn`, `__fmul2_rn`) serves two cells.  Match masks of
 // both haplotypes live in one register per base (bits 0..15: A, 16..31: B; N <= 16).
 // ------------------------------------------------------------------------------------
 template <int N>

@@ -23,7 +23,10 @@ constexpr int kRuns = 272;           // log2(2^24) * 11.2 runs, and one spare
 constexpr int kG = 33;               // class of G lanes: run * kG + G
 constexpr int kClasses = kRuns * kG;
 constexpr int kLongClasses = 512;
-constexpr int kMaxPatterns = 96;     // per run (a pattern exhausts at least one of 32 counts; see pack_run)
+// Patterns of a run.  Most exhaust a class, but one that takes m teams of a class an item can leave up
+// to m - 1 of it; from pattern 63 on each is one team an item and exhausts its class, so the 32
+// classes take no more than 32 further ones (pack_run).
+constexpr int kMaxPatterns = 96;
 constexpr int kSlots = 32;
 
 struct Pattern {

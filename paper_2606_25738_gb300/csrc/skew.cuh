@@ -12,15 +12,16 @@
 // tables.  A pair of l rows on G lanes takes l + G steps.
 //
 // What bounds them: the register file's read ports.  A scheduler reads about two operands a
-// thread and cycle (clock64 around loops of each, 1 to 4 warps a scheduler): an FFMA with three
-// fresh operands takes 1.5 cycles, with one reused or constant 1.0 to 1.25; an FFMA2 takes 3.0
+// thread and cycle (clock64 around loops of each, 1 to 4 warps a scheduler): an fmaf with three
+// fresh operands takes 1.5 cycles, with one reused or constant 1.0 to 1.25; a __ffma2_rn takes 3.0
 // and 2.0 to 2.3.  Packing therefore saves no FMA time, only issue slots.  Two forms:
 //  - team_run_skew, scalar, for short teams: the fewest steps (l + G).  A bare step of 32
-//    columns takes 295 cycles a scheduler (224 instructions).
-//  - strip_run_skew, a lane's column halves in float2 (FFMA2), the second half one row behind
-//    the first: 160 to 195 instructions a step, which leave slots for the boundary traffic; the
-//    strip takes 64 steps more than its rows.  On 60,000 uneven pairs the serial kind took 22.0
-//    ms against 25.6 ms with the scalar form (28.6 ms on the scan engine).
+//    columns takes 295 cycles a scheduler.
+//  - strip_run_skew, a lane's column halves in float2, the second half one row behind the first:
+//    7.1 warp instructions issued per 32 cells (ncu; 8.5 on the scan engine, 9.8 in short teams), which
+//    leaves slots for the boundary traffic; the strip takes 64 steps more than its rows.  On 60,000
+//    uneven pairs the serial kind took 22.0 ms against 25.6 ms with the scalar form (28.6 ms on
+//    the scan engine).
 // The scalar form also runs FP64 short teams, where the FP64 pipe (2.1 FMAs a cycle and SM) is the
 // bound and 5 operations a cell take the place of 6.5: 40 regions of short reads, 6.15 ms
 // against 6.65 ms on the scan engine, with 32 columns a lane (16: 10.8 ms).
@@ -337,7 +338,7 @@ __device__ SegOut team_run_skew(const std::conditional_t<FORM == kLean, Rec32, t
     };
     for (int s = 1; s <= steps;) {
         // (steps between events run in a loop of their own, in which nothing but the row writes
-        // M and J: with the checkpoint inside it every step copied both)
+        // M and J)
         const int e = FORM == kTeams ? min(ck, steps) : min(min(ck, steps), (s + 31) & ~31);
         if (s < plain0) run(std::true_type{}, s, min(e, plain0 - 1));
         else if (s <= plain1) run(std::false_type{}, s, min(e, plain1));
@@ -463,9 +464,8 @@ __device__ __forceinline__ void skew_row2(float2 (&M)[H], float2 (&J)[H], SkewLa
 }
 
 // Match bits of the halves' rows: even bits from .x's row, odd bits from .y's (the row
-// before).  Opaque to the optimiser: seen through, each bit is tested in the word it came from
-// and costs an instruction of its own, where one word gives seven predicates at a time (310
-// against 340 cycles a step).
+// before), in one word that the optimiser cannot see through: 310 cycles a step, against 340 with
+// the same merge in C++.
 __device__ __forceinline__ uint32_t skew_mask2(SkewLane2& L, uint32_t mk) {
     uint32_t m;
     asm("lop3.b32 %0, %1, %2, 0x55555555, 0xe4;" : "=r"(m) : "r"(mk), "r"(L.mprev));
@@ -672,7 +672,7 @@ __device__ SegOut strip_run_skew(const Rec32J* __restrict__ rec, int l, const ui
             L.pmy = n2.z;
             L.pxy = n2.w;
             skew_row2<H, G10>(M, J, L, skew_mask2(L, mk));
-            // (after the row: before it they would be copied, 13 moves a step)
+            // (after the row, which has had its last use of the ones they replace)
             sl = skew_slot(s + 1 - 2 * lane);
             n0 = st.c0[sl];
             n1 = st.c1[sl];
