@@ -187,12 +187,12 @@ typedef struct {
     float ms_host;            /* host time of phmm_submit_batch's planning and enqueue */
     /* Kernels the plan ran (-1: that branch had no work).  FP64 precision: short_kernel =
      * the FP64 forward variant (0: 8 columns per lane in 16-warp CTAs, 1: 16 columns per
-     * lane in 8-warp CTAs, 2: short pairs on the pipelined FP64 engine, 16 columns per
-     * lane, and multi-warp pairs as in 1, 3: as 2 with 32-column fused short teams), the
-     * other two -1.  FP32:
+     * lane in 8-warp CTAs, 2: short pairs on the skewed FP64 engine, 16 columns per
+     * lane, and multi-warp pairs on its strips or as in 1, 3: as 2 with 32-column short teams),
+     * the other two -1.  FP32:
      * short_kernel = scalar-team variant 0..9 (k_short_scalar<32,4>, <24,4>, <24,5>,
-     * <16,6>, k_short_pipe<32,3>, <24,4>, <16,4>, k_short_pipe2<32,3>, <24,4>, and the
-     * lean k_short_pipe2<32,4>);
+     * <16,6>, k_short_pipe<32,3>, <24,4>, <16,4>, k_short_pipe2<32,3>, <24,4> and
+     * <32,4>, the skewed engine);
      * packed_kernel = packed-team variant 0..1 (k_short_packed<12,4>, <16,3>);
      * long_kernel = multi-warp kind 0..8 (lean k_forward<32>, k_forward_pipe<32,12>,
      * k_forward_pipe<24,16>, k_forward_serial<32,3>, k_forward_pipe<32,4>,
@@ -204,8 +204,8 @@ typedef struct {
     /* The FP32 forward pass runs three branches concurrently, each a persistent kernel on
      * its own stream: [0] scalar short teams, [1] packed short teams, [2] multi-warp pairs.
      * cells_branch = sum of l * k over the pairs each branch scored; ms_branch = device time
-     * of each branch's kernel (CUDA events on its stream).  FP64: [0] holds the whole
-     * forward pass. */
+     * of each branch's kernel (CUDA events on its stream).  FP64: variants 2 and 3 have
+     * branches [0] and [2]; with 0 and 1 [0] holds the whole forward pass. */
     uint64_t cells_branch[3];
     float ms_branch[3];
 } phmm_stats;

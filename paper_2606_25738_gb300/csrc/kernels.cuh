@@ -891,9 +891,8 @@ k_short_pipe(const BatchHeader* __restrict__ H, const PowRow<float>* __restrict_
     }
 }
 
-// Scalar teams on the skewed engine (team_run_skew), same work list as k_short_scalar.  The
-// name and its last two parameters are those of the engine it took the place of (column
-// halves in packed pairs, and a lean form of it), which kernel_variant 5 and 6 ask for.
+// Scalar teams on the skewed engine (team_run_skew), same work list as k_short_scalar
+// (k_short_pipe2: the name of the engine it took the place of, which kernel_variant 5 and 6 ask for).
 template <typename T, int N, bool G10>
 __device__ __forceinline__ void skew_items(const BatchHeader* __restrict__ H, const PipeRange& rng, uint32_t* sm) {
     const uint32_t n_w = H->n_witems;
@@ -939,7 +938,7 @@ __device__ __forceinline__ void solo_items(const BatchHeader* __restrict__ H, co
         if (lane == 0) write_part(H, pair, o);
     }
 }
-template <int N, int MINB, bool HALVES = true, bool LEAN = false>
+template <int N, int MINB>
 __global__ void __launch_bounds__(kShortThreads, MINB)
 k_short_pipe2(const BatchHeader* __restrict__ H) {
     __shared__ SoloStage stage[kShortThreads / 32];

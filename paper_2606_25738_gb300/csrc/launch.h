@@ -84,9 +84,9 @@ constexpr int kShortScalarN[kNumScalar] = {32, 24, 24, 16, 32, 24, 16, 32, 24, 3
 // scalar ids whose kernel reads Rec32J records (the pipelined and the skewed engine)
 constexpr bool kShortScalarPipe[kNumScalar] = {false, false, false, false, true, true, true, true, true, true};
 // scalar ids of the skewed engine
-constexpr bool kShortScalarHalves[kNumScalar] = {false, false, false, false, false, false, false, true, true, true};
+constexpr bool kShortScalarSkew[kNumScalar] = {false, false, false, false, false, false, false, true, true, true};
 // scalar ids of the skewed engine in four CTAs per SM
-constexpr bool kShortScalarLean[kNumScalar] = {false, false, false, false, false, false, false, false, false, true};
+constexpr bool kShortScalarFour[kNumScalar] = {false, false, false, false, false, false, false, false, false, true};
 constexpr int kNumPacked = 2;
 constexpr int kShortPackedN[kNumPacked] = {12, 16};
 

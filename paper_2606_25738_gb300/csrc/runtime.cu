@@ -783,7 +783,7 @@ void plan_header(const Slot& S, const Plan& P, BatchHeader& hh) {
     // short pairs no more than 12 to an SM have a warp each, of few columns a lane: the step of a
     // scheduler's only warp is latency (20 pairs of 150 rows: forward 54 us against 84 in teams;
     // from about three warps a scheduler on, teams take fewer slots)
-    hh.n_solo = !P.fp64 && !P.dev && kShortScalarHalves[P.scal_id] && P.witems2.empty() &&
+    hh.n_solo = !P.fp64 && !P.dev && kShortScalarSkew[P.scal_id] && P.witems2.empty() &&
                 P.teams.size() <= 12u * hh.sms ? (uint32_t)P.teams.size() : 0u;
     hh.n_citems = (uint32_t)P.n_citems();
     hh.n_partials = hh.n_pairs + P.n_extra;
@@ -832,15 +832,17 @@ std::vector<std::pair<int, int>> fp32_candidates(const phmm_config& cfg) {
             if (v == 1 && pi < 0) continue;
             if (v == 3 && kShortScalarPipe[si]) continue;
             if (v == 4 && !kShortScalarPipe[si]) continue;
-            if (v == 5 && !kShortScalarHalves[si]) continue;
-            if (v == 6 && !kShortScalarLean[si]) continue;
+            if (v == 5 && !kShortScalarSkew[si]) continue;
+            if (v == 6 && !kShortScalarFour[si]) continue;
             // four CTAs per SM only when asked for: the same time on the short-read batch
-            if (v != 6 && kShortScalarLean[si]) continue;
-            // left to itself the library runs the skewed engine: on 400 short-read regions 2.10 ms
-            // against 2.57 ms (pipelined), 2.73 ms (packed teams) and more (lean); on equal lengths
-            // of 32 to 1000 bp it is never slower than any of them.  Packed teams run when their
-            // width is asked for.
-            if (v == 0 && !kShortScalarHalves[si]) continue;
+            if (v != 6 && kShortScalarFour[si]) continue;
+            // left to itself the library runs the skewed engine: on 400 short-read regions 2.11 ms
+            // against 2.57 ms (pipelined), 2.73 ms (packed teams) and more (lean).  Against the best that
+            // the tuner found among the scan engines, gcp Phred 10: equal lengths of 32 bp 1.65 ms for 1.65,
+            // 48 bp 2.19 for 2.94, 128 bp 1.53 for 1.80, 512 bp 1.36 for 1.59, 1000 bp 1.43 for 1.63; with another
+            // gcp (an operand more a column): 400 regions 2.30 for 2.32, mixed values 2.30 for 2.50, 512 bp 1.86
+            // for 2.03, 1000 bp 2.75 for 3.01.  Packed teams run when their width is asked for.
+            if (v == 0 && !kShortScalarSkew[si]) continue;
             if (v == 0 && pi >= 0 && n != 12 && n != 16) continue;
             if ((n == 24 || n == 32 || n == 16) && scal_only && kShortScalarN[si] != n) continue;
             if ((n == 24 || n == 32) && !scal_only && kShortScalarN[si] != n) continue;
@@ -921,7 +923,7 @@ void make_plan_id(const uint32_t* l, const uint32_t* k, const uint32_t* pr, uint
                   int pack_id, int long_kind, Plan& P) {
     make_plan(l, k, pr, n, kShortScalarN[scal_id], pack_id >= 0 ? kShortPackedN[pack_id] : 0,
               kLongN[long_kind], P, 4, kLongCW[long_kind], kLongSerial[long_kind], kLongWave[long_kind],
-              kShortScalarHalves[scal_id] ? kSkewCost : TeamCost());
+              kShortScalarSkew[scal_id] ? kSkewCost : TeamCost());
     if (long_kind == 5) cluster_links(P);
     P.scal_id = scal_id;
     P.pack_id = pack_id;
@@ -945,7 +947,8 @@ std::vector<int> long_kinds_of(const phmm_config& cfg) {
     if (cfg.kernel_variant == 3) return {0};
     // the kinds on the skewed engine; the others run only when forced (64 long-read pairs: wave
     // kinds 27 to 40 ms, 4-warp strips and clusters over 120 ms; 60,000 uneven pairs: serial
-    // 22 ms, lean and 12-warp CTAs over 40 ms)
+    // 22 ms, lean and 12-warp CTAs over 40 ms).  With other gcp values than Phred 10 they keep 0.92 to
+    // 0.97 of their rate: 8,000 uneven pairs 6.1 ms where the scan engines took 7.5, 24 long pairs 9.6 and 30.4
     return {3, 6, 7, 8};
 }
 // Batches of at least this many pairs are planned on the device (when every kernel that may
@@ -954,7 +957,7 @@ constexpr uint32_t kDevPlanPairs = 4096;
 bool plans_on_device(const phmm_config& cfg, uint32_t np) {
     if (cfg.precision == PHMM_PREC_FP64 || np < kDevPlanPairs) return false;
     for (const auto& cd : fp32_candidates(cfg))
-        if (!kShortScalarHalves[cd.first] || cd.second >= 0) return false;
+        if (!kShortScalarSkew[cd.first] || cd.second >= 0) return false;
     for (int lk : long_kinds_of(cfg))
         if (!kLongSerial[lk] && !kLongWave[lk]) return false;
     return true;
@@ -1553,11 +1556,11 @@ int submit_locked(phmm_ctx* ctx, const phmm_batch* b, uint64_t* ticket, bool hos
             // with far fewer it leaves most of the GPU idle, so it is not worth a (long)
             // trial run (at half as many pairs as warps it can still win: measured)
             const uint64_t swarps = (uint64_t)ctx->sms * ctx->occ_longk[3] * (kSerialThreads / 32);
-            // the 4-warp-CTA kind pays off only for a few very wide pairs (it spreads them over
-            // more SMs); with many wide pairs it is not worth a trial run either
+            // the wave kinds pay off only for a few very wide pairs (their strips spread over the
+            // SMs); with many wide pairs they are not worth a trial run either
             for (int lk : long_kinds_of(ctx->cfg)) {
                 if (kLongSerial[lk] && 2 * (uint64_t)P.n_long < swarps) continue;
-                if ((lk == 4 || lk == 5 || kLongWave[lk]) && (uint64_t)P.n_long >= swarps) continue;
+                if (kLongWave[lk] && (uint64_t)P.n_long >= swarps) continue;
                 runs.push_back({-1, -1, lk});
             }
         }

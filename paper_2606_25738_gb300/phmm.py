@@ -65,11 +65,11 @@ ABI_VERSION = 3  # PHMM_ABI_VERSION of include/phmm.h
 # Kernel names behind phmm_stats.short_kernel / packed_kernel / long_kernel.
 SHORT_KERNELS = ["k_short_scalar<32, 4>", "k_short_scalar<24, 4>", "k_short_scalar<24, 5>",
                  "k_short_scalar<16, 6>", "k_short_pipe<32, 3>", "k_short_pipe<24, 4>",
-                 "k_short_pipe<16, 4>", "k_short_pipe2<32, 3, 1, 0>", "k_short_pipe2<24, 4, 1, 0>",
-                 "k_short_pipe2<32, 4, 1, 1>"]
+                 "k_short_pipe<16, 4>", "k_short_pipe2<32, 3>", "k_short_pipe2<24, 4>",
+                 "k_short_pipe2<32, 4>"]
 PACKED_KERNELS = ["k_short_packed<12, 4>", "k_short_packed<16, 3>"]
 LONG_KERNELS = ["k_forward<float, 32, 0>", "k_forward_pipe<32, 12>", "k_forward_pipe<24, 16>",
-                "k_forward_serial<32, 3, 0>", "k_forward_pipe<32, 4>", "k_forward_cluster<32, 4, 8>",
+                "k_forward_serial<32, 3>", "k_forward_pipe<32, 4>", "k_forward_cluster<32, 4, 8>",
                 "k_forward_wave<32, 3>", "k_forward_wave<32, 3> (2 CTAs/SM)", "k_forward_wave<16, 3>"]
 # FP64 forward variant behind phmm_stats.short_kernel when the precision is FP64.
 FP64_KERNELS = ["k_forward<double, 8, 1, 16>", "k_forward<double, 16, 1, 8>",
@@ -297,8 +297,8 @@ class Context:
         return v.value
 
     def wait_test(self) -> int:
-        """phmm_wait_test: a bounded device wait on a boundary nothing writes; returns
-        PHMM_ETIMEOUT when the wait gave up as designed."""
+        """phmm_wait_test: bounded device waits on boundaries nothing writes; returns
+        PHMM_ETIMEOUT when each of them gave up as designed."""
         return _lib.phmm_wait_test(self._h)
 
     def scan_test(self, y, a: float):

@@ -487,7 +487,7 @@ def test_stats_name_the_kernels_and_no_tune(phmm):
     with phmm.Context(precision="fp32", variant="pipe2", cols_per_lane=32, flags=phmm.F_LONG_SERIAL) as ctx:
         out, flags, rc, st = ctx.run(b)
     assert phmm.SHORT_KERNELS[st["short_kernel"]].startswith("k_short_pipe2<32")
-    assert phmm.LONG_KERNELS[st["long_kernel"]] == "k_forward_serial<32, 3, 0>"
+    assert phmm.LONG_KERNELS[st["long_kernel"]] == "k_forward_serial<32, 3>"
     assert st["packed_kernel"] == -1
     _check(out, flags, ref)
     with phmm.Context(precision="fp32", flags=phmm.F_NO_TUNE) as ctx:
