@@ -240,7 +240,7 @@ def _long_batch(n=20000, l=6000):
 
 
 def test_polling_in_slices_leaves_the_core(phmm):
-    """A long batch polled a millisecond at a time: the thread sleeps, but for the first millisecond."""
+    """A long batch polled a millisecond at a time: the thread sleeps, but for the first two milliseconds."""
     import time
     with phmm.Context(precision="fp32", flags=phmm.F_NO_TUNE) as ctx:
         ctx.run(_long_batch())
